@@ -195,7 +195,7 @@ int ensure_dx32(fsi_mesh* m) {
 int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigned flags) {
   m->applies++;
   m->dof_applied += b.n;
-  if (m->tet) return tet_op(m, b, 1, dx, y, flags & ~OP_DX32_READY);
+  if (m->tet) return tet_op(m, b, 1, dx, y, flags & ~(OP_DX32_READY | OP_REUSED));
   const bool f32 = flags & FSI_FP32;
   if (f32) {  // float copy of the increment for the float32 kernels (unless the caller wrote it)
     if (int rc = ensure_dx32(m)) return rc;
@@ -206,6 +206,7 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
   if (b.kind == 0) {
     // recorded (batched) launches take the per-element kernel; single launches the
     // product from the quadrature-point coefficients
+    if (m->rec) flags &= ~OP_REUSED;
     if (m->rec) return f32 ? launch_ns<float>(m, 1, dx, y, flags) : launch_ns<double>(m, 1, dx, y, flags);
     return f32 ? launch_nsq<float>(m, dx, y, flags) : launch_nsq<double>(m, dx, y, flags);
   }
@@ -215,8 +216,10 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
 }
 
 int op_diag(fsi_mesh* m, const BlockInfo& b, double* d, unsigned flags) {
-  if (m->tet) return tet_op(m, b, 2, nullptr, d, flags);
+  if (m->tet) return tet_op(m, b, 2, nullptr, d, flags & ~OP_REUSED);
   const bool f32 = flags & FSI_FP32;
+  if (b.kind == 0 && !f32 && !m->rec && (flags & OP_REUSED)) return nsa_diag(m, d, flags);
+  flags &= ~OP_REUSED;
   if (b.kind == 0)
     return f32 ? launch_ns<float>(m, 2, nullptr, d, flags) : launch_ns<double>(m, 2, nullptr, d, flags);
   if (b.kind == 1)
@@ -382,6 +385,7 @@ int fsi_destroy_mesh(fsi_mesh* m) {
   cudaFree(m->Z);
   cudaFree(m->cq64);
   cudaFree(m->cq32);
+  cudaFree(m->na64);
   cudaFree(m->ke64);
   cudaFree(m->ke_e);
   cudaFree(m->tma_err);
@@ -461,7 +465,7 @@ int fsi_jvp(fsi_mesh* m, int32_t block, const fsi_state* st, const double* dx, d
   int rc = block_info(m, block, &b);
   if (rc) return rc;
   if ((rc = stage(m, st, flags & FSI_FP32))) return rc;
-  return op_jvp(m, b, dx, y, flags & ~OP_DX32_READY);
+  return op_jvp(m, b, dx, y, flags & ~(OP_DX32_READY | OP_REUSED));
 }
 
 int fsi_diag(fsi_mesh* m, int32_t block, const fsi_state* st, double* d, uint32_t flags) {
@@ -470,7 +474,7 @@ int fsi_diag(fsi_mesh* m, int32_t block, const fsi_state* st, double* d, uint32_
   int rc = block_info(m, block, &b);
   if (rc) return rc;
   if ((rc = stage(m, st, flags & FSI_FP32))) return rc;
-  return op_diag(m, b, d, flags);
+  return op_diag(m, b, d, flags & ~OP_REUSED);
 }
 
 int fsi_update_ac_coeffs(fsi_mesh* m, int32_t phase, const fsi_state* st, double* out) {

@@ -80,15 +80,16 @@ struct fsi_mesh {
   alignas(64) unsigned char cq_tmap[256] = {};
   const void* cq_tmap_base = nullptr;
   int* tma_err = nullptr;
-  // float64 element matrices of the NS product (nse_elem_kernel), built from the coefficients once
-  // a state has taken NSE_AFTER float64 products
-  double* ke64 = nullptr;
+  // assembled float64 NS operator (nsa.cu), and the element matrices it is summed from
+  double* na64 = nullptr;
+  int64_t na_len = 0;
+  int64_t na_gen = -1;               // stage_gen of the last build
+  unsigned na_flags = 0;             // FSI_ELASTIC_AUG of the last build
+  double* ke64 = nullptr;            // some layers of element matrices
   int64_t ke_len = 0;
   double* ke_e = nullptr;            // [slots][elements] corner contributions of the element-centric products
   int64_t ke_e_len = 0;
-  int64_t ke_gen = -1;               // cq_gen they were built from
-  int64_t f64_gen = -1, f64_count = 0;  // float64 NS products applied at coefficient build f64_gen
-  int64_t cq_builds = 0;             // coefficient builds so far (a new build invalidates ke64)
+  int64_t f64_gen = -1, f64_count = 0;  // float64 NS products applied at staging f64_gen
   // float64 Allen-Cahn element matrices (ace_elem_kernel) of one phase at one staging
   double* ake64 = nullptr;
   int64_t ake_len = 0;
@@ -163,6 +164,9 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
 // op_jvp flag, internal only: with FSI_FP32, the float32 increment is already in m->dx32
 // (the Krylov solver's preconditioner kernel wrote it) and dx is not read
 constexpr unsigned OP_DX32_READY = 0x80000000u;
+// op_jvp and op_diag flag, internal only: the state stays for a whole solve, so the float64 NS operator
+// is assembled
+constexpr unsigned OP_REUSED = 0x40000000u;
 int ensure_dx32(fsi_mesh* m);  // allocates m->dx32 (6 x nn floats) on first use
 int op_diag(fsi_mesh* m, const BlockInfo& b, double* d, unsigned flags);
 int op_coeffs(fsi_mesh* m, int phase, double* gamma_beta);  // synchronises
@@ -210,13 +214,19 @@ int nsq_batch_launch(bool f64, const NSQBatchRec* recs, const int4* eitems, int 
 constexpr int NSQ_TBX = 64, NSQ_TBY = 2;  // element tile of the TMA product
 // [slots][elements] scratch of the element-centric products, grown on demand (ops_f64.cu)
 int ensure_elem_scratch(fsi_mesh* m, int slots, int64_t nxyp);
-// float64 NS product through element matrices (built first when stale), ops_f64.cu
-int launch_nse(fsi_mesh* m, const double* dx, double* y, unsigned flags);
+// assembled float64 NS operator of the staged state (built when stale): build, product and
+// diagonal (nsa.cu)
+int nsa_build(fsi_mesh* m, unsigned flags);
+int launch_nsa(fsi_mesh* m, const double* dx, double* y, unsigned flags);
+int nsa_diag(fsi_mesh* m, double* d, unsigned flags);
 // float64 Allen-Cahn product of one phase through element matrices (ops_f64.cu)
 int launch_ace(fsi_mesh* m, int phase, const double* dx, double* y);
 // float64 B product of one solid through the split operator (ops_f64.cu)
 int launch_be(fsi_mesh* m, int solid, const double* dx, double* y);
-constexpr int NSE_AFTER = 8;  // float64 products on one coefficient build before the matrices pay
+// float64 NS products at one staging after which the assembled operator is built; a solve that may
+// take more builds it at once (OP_REUSED).  At 64^3 the build takes as long as NSA_AFTER
+// products from the coefficients.
+constexpr int NSA_AFTER = 8;
 // Allen-Cahn element matrices: a build costs about three re-interpolating products and
 // each matrix product a fifteenth of one; the B split operator's build costs less than one
 // re-interpolating product, so it is built at the first product of a solve

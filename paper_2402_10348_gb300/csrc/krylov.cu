@@ -1056,8 +1056,11 @@ int gmres_solve(fsi_mesh* m, const BlockInfo& blk, const double* rhs, double* x,
   if (o.precond == FSI_PC_LEARNED && blk.kind == 0 && !pc)
     return set_error(FSI_EINVAL, "GMRES: FSI_PC_LEARNED without an attached preconditioner (fsi_set_pc)");
   fsi_pc* harvest = ((o.flags & FSI_HARVEST) && blk.kind == 0 && m->pc && m->pc->cap > 0) ? m->pc : nullptr;
-  const unsigned opflags =
-      o.flags & ~(FSI_HARVEST | FSI_PC_ALTERNATE | FSI_NO_STALL_STOP | FSI_PINNED_SOLVE | OP_DX32_READY);
+  unsigned opflags = o.flags & ~(FSI_HARVEST | FSI_PC_ALTERNATE | FSI_NO_STALL_STOP | FSI_PINNED_SOLVE | OP_DX32_READY |
+                                 OP_REUSED);
+  // a float64 solve that may take many products assembles the operator before the first one (its
+  // diagonal comes with it)
+  if (o.precision == FSI_PREC_FP64 && o.max_iter > NSA_AFTER) opflags |= OP_REUSED;
   // read by the solver loop only: network/Jacobi alternation, and no stop on stagnation
   const unsigned alt = o.flags & (FSI_PC_ALTERNATE | FSI_NO_STALL_STOP);
   const bool stall_stop = (o.flags & FSI_NO_STALL_STOP) == 0;

@@ -544,17 +544,6 @@ struct CoefRef {
 };
 
 
-// ------------------------------------------- float64 NS product from element matrices
-// GB300 issues float64 FMAs at 1/64 of the float32 rate, so a float64 solve that
-// applies the product hundreds of times on one state stores each element's 32 x 32
-// matrix (rows and columns ordered field-major: 8 corners of dv_x, dv_y, dv_z, dp) once
-// and applies it with 1024 FMAs per element, against about 2400 for the coefficient
-// form.  Layout: K[((ez * 1024 + i * 32 + j) * nxyp + ey * nxp + ex], unweighted (W
-// per node as above).  Column j is the coefficient product of the unit increment j, so
-// both forms are the same operator up to summation order.
-constexpr int NKE = 32 * 32;
-
-
 // ----------------------------------------------------------------- AC block
 // fields: [dphi (JVP)], v(3), phi, dphi/dt
 template <typename TT, int MODE>

@@ -335,16 +335,15 @@ __global__ void __launch_bounds__(128) nsq_elem_kernel(const T* __restrict__ cq,
 template <typename T>
 int launch_nsq(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   const unsigned eflags = flags & FSI_ELASTIC_AUG;
-  if (m->cq_gen != m->stage_gen || m->cq_flags != eflags || !m->cq64) {
-    if (int rc = ns_build(m, flags)) return rc;
-  }
   if constexpr (sizeof(T) == 8) {
-    // a float64 solve on this state: after NSE_AFTER products switch to element matrices
-    if (m->f64_gen != m->cq_builds) {
-      m->f64_gen = m->cq_builds;
+    if (m->f64_gen != m->stage_gen) {
+      m->f64_gen = m->stage_gen;
       m->f64_count = 0;
     }
-    if (++m->f64_count > NSE_AFTER) return launch_nse(m, dx, y, flags);
+    if ((flags & OP_REUSED) || ++m->f64_count > NSA_AFTER) return launch_nsa(m, dx, y, flags);
+  }
+  if (m->cq_gen != m->stage_gen || m->cq_flags != eflags || !m->cq64) {
+    if (int rc = ns_build(m, flags)) return rc;
   }
   const Geom& g = m->g;
   const int64_t nn = m->nn;

@@ -29,7 +29,7 @@ struct TetData {
   int32_t* nlist = nullptr; // 4 e + a of every (element, corner) at a node, by element
   double* E = nullptr;      // [24][ne] element contributions, slot (a * ncomp + eq)
   // float64 NS element matrices [256][ne], row a * 4 + eq, column b * 4 + f, built once a
-  // solve has taken NSE_AFTER products on one staging (k_stage) with one elastic flag
+  // solve has taken NSA_AFTER products on one staging (k_stage) with one elastic flag
   double* K = nullptr;
   int64_t k_stage = -1;
   int k_elastic = -1, k_count = 0, k_built = 0;
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(128) tet_nsk_apply(const int32_t* __restrict__
 int tet_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
   if (flags & FSI_FP32) return set_error(FSI_EINVAL, "tetrahedral meshes: float64 operators only");
   if (mode == 1 && !m->rec) {
-    // a float64 solve on one staging: after NSE_AFTER products switch to element matrices
+    // a float64 solve on one staging: after NSA_AFTER products switch to element matrices
     TetData* t = m->tet;
     const int elastic = ((flags & FSI_ELASTIC_AUG) && m->ns > 0) ? 1 : 0;
     if (t->k_stage != m->stage_gen || t->k_elastic != elastic) {
@@ -371,7 +371,7 @@ int tet_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
       t->k_count = 0;
       t->k_built = 0;
     }
-    if (++t->k_count > NSE_AFTER) {
+    if (++t->k_count > NSA_AFTER) {
       const unsigned grid = (unsigned)((t->ne + 127) / 128);
       if (!t->k_built) {
         if (!t->K) FSI_CUDA(cudaMalloc(&t->K, sizeof(double) * 256 * (size_t)t->ne));
