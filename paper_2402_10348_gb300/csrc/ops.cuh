@@ -73,9 +73,7 @@ struct OutDesc {
   double* y;            // output block [NC][nn]
   const double* dx;     // JVP input block (Dirichlet rows copy it), or null
   const float* dx32;    // its float copy: the rows copy this one when dx is null
-  const double* x;      // state x^{n+1} (residual Dirichlet rows), or null
   const uint8_t* mask;  // Dirichlet mask (NS only): bits 0-2 velocity, bit 3 pressure
-  const double* vD;     // Dirichlet velocity values [3][nn]
   int accumulate;       // add into y instead of writing (later solid passes)
   int dirichlet;        // apply Dirichlet rows
   int pin;              // NS: the pressure pin row is active (mask bit 3); 0: the node keeps
@@ -85,7 +83,7 @@ struct OutDesc {
 // ----------------------------------------------------------------- NS block
 // Field layout (NSField): state v(3), p, dv/dt(3), rho, mu, then per solid in the
 // pass: alpha^s, B^s(6); JVP: the input dv(3), dp first.
-template <typename TT, int MODE>  // MODE 0: residual, 1: JVP, 2: diagonal
+template <typename TT, int MODE>  // MODE 1: JVP, 2: diagonal (residuals: hexq_ops.cu)
 struct NSOp {
   using T = TT;
   static constexpr int NC = 4;
@@ -138,41 +136,8 @@ struct NSOp {
       const T dt2 = T(4.0) / (T(P.dt) * T(P.dt));
       const T tau_m = T(1) / sqrt(dt2 + vGv + T(P.c_i) * nu * nu * T(P.GG));
       const T tau_c = T(1) / (T(P.trG) * tau_m);
-      const T Rc = L[0][0] + L[1][1] + L[2][2];
 
-      if (MODE == 0) {
-        T E[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-        for (int s = s0; s < s1; ++s) {
-          const int fs = fsol + 7 * (s - s0);
-          cr.get(fs, u);
-          const T a = interp_v(u, w) * T(P.muL[P.solid_phase[s]]);
-#pragma unroll
-          for (int cc = 0; cc < 6; ++cc) {
-            cr.get(fs + 1 + cc, u);
-            E[cc] += a * (interp_v(u, w) - (cc < 3 ? T(1) : T(0)));
-          }
-        }
-        const T W = T(this->W);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          T gk[3];
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            T s = E[sym_idx(k, j)];
-            if (fluid) {
-              s += mu * (L[k][j] + L[j][k]) + tau_m * v[j] * Rm[k];
-              if (j == k) s += -pr.v + tau_c * rho * Rc;
-            }
-            gk[j] = W * s;
-          }
-          const T fk = fluid ? W * (Rm[k] - gp[k]) : T(0);  // rho (acc_k - g_k)
-          scatter_vg(c[k], w, fk, gk[0], gk[1], gk[2], rhx, rhy, rhz);
-        }
-        if (fluid) {
-          const T r = W * tau_m / rho;
-          scatter_vg(c[3], w, W * Rc, r * Rm[0], r * Rm[1], r * Rm[2], rhx, rhy, rhz);
-        }
-      } else if (MODE == 1) {
+      if (MODE == 1) {
         T dv[3], dL[3][3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -317,9 +282,7 @@ struct NSOp {
       const bool dir = ((m >> k) & 1) && (k < 3 || out.pin);
       if (dir) {
         if (!out.dirichlet) continue;
-        if (MODE == 0) {
-          *y = out.x[(int64_t)k * nn + nc.n] - (k < 3 ? out.vD[(int64_t)k * nn + nc.n] : 0.0);
-        } else if (MODE == 1) {
+        if (MODE == 1) {
           *y = out.dx ? out.dx[(int64_t)k * nn + nc.n] : (double)out.dx32[(int64_t)k * nn + nc.n];
         } else {
           *y = 1.0;
@@ -354,7 +317,7 @@ struct CoefArrays {
   int64_t nxyp;  // nxp * ny
 };
 
-// Coefficient build: fields as NSOp MODE 0 (v(3), p, dv/dt(3), rho, mu, then alpha^s,
+// Coefficient build: fields as NSOp MODE 2 (v(3), p, dv/dt(3), rho, mu, then alpha^s,
 // B^s(6) per solid of the pass).  Only the CTA that owns an element writes it.  Later
 // solid passes (fluid == 0) add their solids' sums into aB and aG.
 struct NSBuildOp {
@@ -545,7 +508,7 @@ struct CoefRef {
 
 
 // ----------------------------------------------------------------- AC block
-// fields: [dphi (JVP)], v(3), phi, dphi/dt
+// fields: [dphi (JVP)], v(3), phi
 template <typename TT, int MODE>
 struct ACOp {
   using T = TT;
@@ -586,15 +549,7 @@ struct ACOp {
       const T s_hat = gam * (T(3) * phi * phi - T(1));
       const T tau = T(1) / sqrt(dt2 + vGv + T(9) * k_hat * k_hat * T(P.GG) + s_hat * s_hat);
       const T W = T(this->W);
-      if (MODE == 0) {
-        cr.get(base + 4, u);
-        const T pdot = interp_v(u, w);
-        const T Fp = phi * phi * phi - phi;
-        const T sF = T(0.5) * fabs(phi * phi - T(1));
-        const T R = pdot + v[0] * ph.gx + v[1] * ph.gy + v[2] * ph.gz + gam * (Fp - bet * sF);
-        scatter_vg(c[0], w, W * R, W * (k_hat * ph.gx + tau * v[0] * R), W * (k_hat * ph.gy + tau * v[1] * R),
-                   W * (k_hat * ph.gz + tau * v[2] * R), rhx, rhy, rhz);
-      } else {
+      {
         const T p2 = phi * phi - T(1);
         const T dsF = p2 > T(0) ? phi : (p2 < T(0) ? -phi : T(0));
         const T rp = gam * (T(3) * phi * phi - T(1) - bet * dsF);
@@ -708,7 +663,7 @@ struct ACEBuildOp {
 
 
 // ----------------------------------------------------------------- B block
-// fields: [dB(6) (JVP)], v(3), alpha^s, B(6), dB/dt(6)
+// fields: [dB(6) (JVP)], v(3), alpha^s
 template <typename TT, int MODE>
 struct BOp {
   using T = TT;
@@ -766,24 +721,14 @@ struct BOp {
         }
         continue;
       }
-      // B (residual: state; JVP: alpha dB) with gradient, and its rate
+      // alpha dB with gradient, and the rate of the increment
       T B[6], cv[6];
-      const int fb = MODE == 1 ? 0 : base + 4;
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) {
-        cr.get(fb + cc, u);
+        cr.get(cc, u);
         const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
-        const T sc = MODE == 1 ? alpha : T(1);
-        B[cc] = sc * r.v;
-        cv[cc] = sc * (v[0] * r.gx + v[1] * r.gy + v[2] * r.gz);
-        if (MODE == 1) cv[cc] += cm * r.v;  // rate of the increment
-      }
-      if (MODE == 0) {
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) {
-          cr.get(base + 10 + cc, u);
-          cv[cc] += interp_v(u, w);
-        }
+        B[cc] = alpha * r.v;
+        cv[cc] = alpha * (v[0] * r.gx + v[1] * r.gy + v[2] * r.gz) + cm * r.v;
       }
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) {
@@ -791,8 +736,7 @@ struct BOp {
         T st = T(0);
 #pragma unroll
         for (int m = 0; m < 3; ++m) st += L[k][m] * B[sym_idx(m, l)] + B[sym_idx(k, m)] * L[l][m];
-        const T rec = B[cc] - ((MODE == 0 && cc < 3) ? T(1) : T(0));
-        const T R = al * (cv[cc] - st) + (T(1) - al) * rec;
+        const T R = al * (cv[cc] - st) + (T(1) - al) * B[cc];
         const T tr = W * tau * R;
         scatter_vg(c[cc], w, W * R, tr * v[0], tr * v[1], tr * v[2], rhx, rhy, rhz);
       }

@@ -152,38 +152,6 @@ __global__ void __launch_bounds__(128) be_elem_kernel(const double* __restrict__
     for (int a = 0; a < 8; ++a) E[(8 * cc + a) * I.es + I.e] = c[cc][a];
 }
 
-template <int NC>
-__global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__ E, int nx, int ny, int nz, int nxp,
-                                                      int64_t nxyp, int64_t nn, double* __restrict__ y) {
-  int i;
-  const int64_t jk = row_index(nx + 1, &i);
-  if (i > nx || jk >= (int64_t)(ny + 1) * (nz + 1)) return;
-  const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
-  const int64_t n = i + (int64_t)(nx + 1) * (j + (int64_t)(ny + 1) * k);
-  const int64_t es = (int64_t)nz * nxyp;
-  double s[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) s[c] = 0.0;
-  for (int az = 1; az >= 0; --az) {
-    const int ez = k - az;
-    if (ez < 0 || ez >= nz) continue;
-    for (int ay = 1; ay >= 0; --ay) {
-      const int ey = j - ay;
-      if (ey < 0 || ey >= ny) continue;
-      for (int ax = 1; ax >= 0; --ax) {
-        const int ex = i - ax;
-        if (ex < 0 || ex >= nx) continue;
-        const int64_t e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
-        const int a = ax + 2 * ay + 4 * az;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] += E[(8 * c + a) * es + e];
-      }
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < NC; ++c) y[c * nn + n] = s[c];
-}
-
 // E[slots][nz * nxyp] scratch of the element-centric products (NS, AC and B in turn)
 int ensure_elem_scratch(fsi_mesh* m, int slots, int64_t nxyp) {
   const int64_t elen = (int64_t)slots * m->g.nz * nxyp;

@@ -107,8 +107,7 @@ constexpr int jvp_class(int kind) {
 template <typename T, int MODE>
 constexpr int op_class(int kind) {
   return MODE == 1 ? jvp_class<T>(kind)
-                   : (MODE == 0 ? (kind == 0 ? P_NS_RES : (kind == 1 ? P_AC_RES : P_B_RES))
-                                : (kind == 0 ? P_NS_DIAG : (kind == 1 ? P_AC_DIAG : P_B_DIAG)));
+                   : (kind == 0 ? P_NS_DIAG : (kind == 1 ? P_AC_DIAG : P_B_DIAG));
 }
 
 // The increment of a product: float64 kernels read dx itself, float32 kernels the
@@ -161,9 +160,7 @@ int ns_pass(fsi_mesh* m, const double* dx, double* y, unsigned flags, int s0, in
   op.out.y = y;
   op.out.dx = dx;
   op.out.dx32 = sizeof(T) == 4 ? m->dx32 : nullptr;
-  op.out.x = m->staged_x;
   op.out.mask = m->mask;
-  op.out.vD = m->vD;
   op.out.accumulate = first ? 0 : 1;
   op.out.dirichlet = first ? 1 : 0;
   op.out.pin = m->pin_active;
@@ -173,8 +170,7 @@ int ns_pass(fsi_mesh* m, const double* dx, double* y, unsigned flags, int s0, in
 
 template <typename T>
 int launch_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
-  const bool need_solids = (mode == 0) || (flags & FSI_ELASTIC_AUG);
-  const int ns = need_solids ? m->ns : 0;
+  const int ns = (flags & FSI_ELASTIC_AUG) ? m->ns : 0;
   const int fixed = (mode == 1 ? 4 : 0) + 9;
   // bounded by shared memory and by the MAXF staged-field slots of Fields
   const int per = std::min(solids_per_pass<T>(fixed), (MAXF - fixed) / 7);
@@ -184,8 +180,7 @@ int launch_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags
   do {
     const int s1 = ns == 0 ? 0 : std::min(ns, s0 + per);
     int rc;
-    if (mode == 0) rc = ns_pass<T, 0>(m, dx, y, flags, s0, s1, first);
-    else if (mode == 1) rc = ns_pass<T, 1>(m, dx, y, flags, s0, s1, first);
+    if (mode == 1) rc = ns_pass<T, 1>(m, dx, y, flags, s0, s1, first);
     else rc = ns_pass<T, 2>(m, dx, y, flags, s0, s1, first);
     if (rc) return rc;
     first = false;
@@ -245,12 +240,14 @@ inline RowLaunch elem_launch(const Geom& g) { return row_launch(g.nx, (int64_t)g
 inline RowLaunch node_launch(const Geom& g) { return row_launch(g.nx + 1, (int64_t)(g.ny + 1) * (g.nz + 1)); }
 
 // NS node sums: y = W * sum of the element slots, the Dirichlet rows (velocity; pressure
-// at the pin node when pinned) take the increment itself (dx, or its float32 copy dx32)
+// at the pin node when pinned) take the increment itself (dx, or its float32 copy dx32), less
+// the prescribed velocity vD when that is given (a residual: dx is x^{n+1})
 template <typename T>
 __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, int nx, int ny, int nz, int nxp,
                                                       int64_t nxyp, int64_t nn, double W, const uint8_t* __restrict__ mask,
                                                       int pin, const double* __restrict__ dx,
-                                                      const float* __restrict__ dx32, double* __restrict__ y) {
+                                                      const float* __restrict__ dx32, const double* __restrict__ vD,
+                                                      double* __restrict__ y) {
   int i;
   const int64_t jk = row_index(nx + 1, &i);
   if (i > nx || jk >= (int64_t)(ny + 1) * (nz + 1)) return;
@@ -278,8 +275,46 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
     const bool dir = ((mk >> f) & 1) && (f < 3 || pin);
-    y[f * nn + n] = dir ? (dx ? dx[f * nn + n] : (double)dx32[f * nn + n]) : W * (double)s[f];
+    double v = W * (double)s[f];
+    if (dir) {
+      v = dx ? dx[f * nn + n] : (double)dx32[f * nn + n];
+      if (vD && f < 3) v -= vD[f * nn + n];
+    }
+    y[f * nn + n] = v;
   }
+}
+
+// the same sums of NC components without Dirichlet rows or weight
+template <int NC>
+__global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__ E, int nx, int ny, int nz, int nxp,
+                                                      int64_t nxyp, int64_t nn, double* __restrict__ y) {
+  int i;
+  const int64_t jk = row_index(nx + 1, &i);
+  if (i > nx || jk >= (int64_t)(ny + 1) * (nz + 1)) return;
+  const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
+  const int64_t n = i + (int64_t)(nx + 1) * (j + (int64_t)(ny + 1) * k);
+  const int64_t es = (int64_t)nz * nxyp;
+  double s[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) s[c] = 0.0;
+  for (int az = 1; az >= 0; --az) {
+    const int ez = k - az;
+    if (ez < 0 || ez >= nz) continue;
+    for (int ay = 1; ay >= 0; --ay) {
+      const int ey = j - ay;
+      if (ey < 0 || ey >= ny) continue;
+      for (int ax = 1; ax >= 0; --ax) {
+        const int ex = i - ax;
+        if (ex < 0 || ex >= nx) continue;
+        const int64_t e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
+        const int a = ax + 2 * ay + 4 * az;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c] += E[(8 * c + a) * es + e];
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) y[c * nn + n] = s[c];
 }
 
 // NS product from the quadrature-point coefficients (see nsq_point) of element (ex, ey, ez)
@@ -382,7 +417,7 @@ int launch_nsq(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   FSI_LAUNCH(m, P_NODE_SUM,
              ns_node_kernel<T><<<nl.grid, nl.block, 0, m->stream>>>(
                  E, g.nx, g.ny, g.nz, nxp, nxyp, nn, g.hx * g.hy * g.hz / 8.0, m->mask, m->pin_active,
-                 dx, sizeof(T) == 4 ? m->dx32 : nullptr, y));
+                 dx, sizeof(T) == 4 ? m->dx32 : nullptr, nullptr, y));
   return FSI_OK;
 }
 
@@ -391,13 +426,11 @@ int ac_run(fsi_mesh* m, int i, const double* dx, double* y) {
   ACOp<T, MODE> op;
   memset(&op, 0, sizeof(op));
   const T* xa = Staged<T>::xa(m);
-  const T* xd = Staged<T>::xd(m);
   const int64_t nn = m->nn;
   int f = 0;
   if (MODE == 1) put_dx<T>(op.F, f++, m, dx, 0);
   for (int k = 0; k < 3; ++k) put<T>(op.F, f++, xa + k * nn);
   put<T>(op.F, f++, xa + (4 + i) * nn);
-  if (MODE == 0) put<T>(op.F, f++, xd + (4 + i) * nn);
   op.nf = f;
   op.P = m->P;
   fill_common(m, op.rh, &op.W);
@@ -426,7 +459,6 @@ int launch_ac(fsi_mesh* m, int mode, int i, const double* dx, double* y) {
       if (++m->ake_count > ACE_AFTER) return launch_ace(m, i, dx, y);
     }
   }
-  if (mode == 0) return ac_run<T, 0>(m, i, dx, y);
   if (mode == 1) return ac_run<T, 1>(m, i, dx, y);
   return ac_run<T, 2>(m, i, dx, y);
 }
@@ -436,19 +468,13 @@ int b_run(fsi_mesh* m, int s, const double* dx, double* y) {
   BOp<T, MODE> op;
   memset(&op, 0, sizeof(op));
   const T* xa = Staged<T>::xa(m);
-  const T* xd = Staged<T>::xd(m);
   const T* mat = Staged<T>::mat(m);
   const int64_t nn = m->nn;
-  const int c0 = 4 + m->N + 6 * s;
   int f = 0;
   if (MODE == 1)
     for (int c = 0; c < 6; ++c) put_dx<T>(op.F, f++, m, dx, c * nn);
   for (int k = 0; k < 3; ++k) put<T>(op.F, f++, xa + k * nn);
   put<T>(op.F, f++, mat + (2 + s) * nn);
-  if (MODE == 0) {
-    for (int c = 0; c < 6; ++c) put<T>(op.F, f++, xa + (c0 + c) * nn);
-    for (int c = 0; c < 6; ++c) put<T>(op.F, f++, xd + (c0 + c) * nn);
-  }
   op.nf = f;
   op.P = m->P;
   fill_common(m, op.rh, &op.W);
@@ -472,7 +498,6 @@ int launch_b(fsi_mesh* m, int mode, int s, const double* dx, double* y) {
       if (++m->bke_count > BE_AFTER) return launch_be(m, s, dx, y);
     }
   }
-  if (mode == 0) return b_run<T, 0>(m, s, dx, y);
   if (mode == 1) return b_run<T, 1>(m, s, dx, y);
   return b_run<T, 2>(m, s, dx, y);
 }
