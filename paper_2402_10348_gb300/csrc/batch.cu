@@ -991,7 +991,7 @@ int inner_solve(fsi_batch* b, std::vector<int> live, double rtol, int max_iter, 
 
 int stage_all(fsi_batch* b, const fsi_state* states, bool f32) {
   for (int i = 0; i < b->n; ++i) {
-    int rc = stage(b->meshes[i], &states[i], f32);
+    int rc = stage(b->meshes[i], &states[i], f32, nullptr);
     if (rc) return rc;
   }
   return FSI_OK;
@@ -1445,7 +1445,7 @@ int batch_rhs(fsi_batch* b, const std::vector<int>& inst, const std::vector<int>
       FSI_CUDA(cudaMemsetAsync(r, 0, sizeof(double) * bi.n, m->stream));
       continue;
     }
-    if (i != last && (rc = stage(m, &states[i], f32))) return rc;
+    if (i != last && (rc = stage(m, &states[i], f32, nullptr))) return rc;
     last = i;
     if (bi.kind == 1) {
       double gb[2];

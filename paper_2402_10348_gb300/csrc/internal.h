@@ -145,9 +145,6 @@ int cuda_check(cudaError_t e, const char* what);
     if (_e != cudaSuccess) return fsi::cuda_check(_e, #call); \
   } while (0)
 
-// staging of x^{n+alpha}, dx/dt^{n+alpha_m} and materials (api.cu)
-int stage(fsi_mesh* m, const fsi_state* st, bool fp32);
-
 // block bookkeeping
 struct BlockInfo {
   int kind;   // 0 NS, 1 AC, 2 B
@@ -157,6 +154,10 @@ struct BlockInfo {
   int64_t n;  // vector length
 };
 int block_info(const fsi_mesh* m, int32_t block, BlockInfo* bi);
+
+// staging of x^{n+alpha}, dx/dt^{n+alpha_m} and materials (api.cu): the planes that block b reads,
+// or all of them (b null: several blocks use one staging)
+int stage(fsi_mesh* m, const fsi_state* st, bool fp32, const BlockInfo* b);
 
 // operator launches on staged state (ops_f64.cu / ops_f32.cu)
 int op_residual(fsi_mesh* m, const BlockInfo& b, double* r);

@@ -1374,7 +1374,7 @@ int fsi_pc_apply(fsi_pc* pc, const fsi_state* st, const double* r, double* z) {
   if (!pc || !st || !r || !z) return set_error(FSI_EINVAL, "fsi_pc_apply: null argument");
   fsi_mesh* m = pc->m;
   int rc;
-  if ((rc = stage(m, st, false))) return rc;
+  if ((rc = stage(m, st, false, nullptr))) return rc;
   BlockInfo b;
   if ((rc = block_info(m, FSI_BLOCK_NS, &b))) return rc;
   if ((rc = op_diag(m, b, pc->tmp, FSI_ELASTIC_AUG))) return rc;
@@ -1458,7 +1458,7 @@ int fsi_pc_add_smooth_pairs(fsi_pc* pc, const fsi_state* st, int32_t count, uint
   fsi_mesh* m = pc->m;
   if (m->tet) return set_error(FSI_EINVAL, "fsi_pc_add_smooth_pairs: structured meshes only");
   int rc;
-  if ((rc = stage(m, st, false))) return rc;
+  if ((rc = stage(m, st, false, nullptr))) return rc;
   BlockInfo b;
   if ((rc = block_info(m, FSI_BLOCK_NS, &b))) return rc;
   // the system of the step's NS solves: unpinned where the step shifts the pressure
@@ -1516,7 +1516,7 @@ int fsi_pc_add_pair(fsi_pc* pc, const fsi_state* st, const double* r, const doub
   if (pc->cap <= 0) return set_error(FSI_EINVAL, "fsi_pc_add_pair: the preconditioner holds no pair storage");
   fsi_mesh* m = pc->m;
   int rc;
-  if ((rc = stage(m, st, false))) return rc;
+  if ((rc = stage(m, st, false, nullptr))) return rc;
   BlockInfo b;
   if ((rc = block_info(m, FSI_BLOCK_NS, &b))) return rc;
   double* dinv = pc->tmp;

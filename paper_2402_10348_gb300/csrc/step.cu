@@ -82,7 +82,7 @@ int fsi_gmres(fsi_mesh* m, int32_t block, const fsi_state* st, const double* rhs
   BlockInfo b;
   int rc = block_info(m, block, &b);
   if (rc) return rc;
-  if ((rc = stage(m, st, o->precision == FSI_PREC_FP32_IR))) return rc;
+  if ((rc = stage(m, st, o->precision == FSI_PREC_FP32_IR, &b))) return rc;
   return gmres_solve(m, b, rhs, x, *o, info);
 }
 
@@ -111,7 +111,7 @@ int fsi_step(fsi_mesh* m, fsi_state* st, const fsi_step_opts* o, fsi_step_info* 
       const int32_t id = bi == 0 ? FSI_BLOCK_NS : (bi <= m->N ? FSI_BLOCK_AC(bi - 1) : FSI_BLOCK_B(bi - 1 - m->N));
       BlockInfo b;
       if ((rc = block_info(m, id, &b))) return rc;
-      if ((rc = stage(m, st, fp32))) return rc;
+      if ((rc = stage(m, st, fp32, &b))) return rc;
       if (b.kind == 1) {
         double gb[2];
         if ((rc = op_coeffs(m, b.index, gb))) return rc;
