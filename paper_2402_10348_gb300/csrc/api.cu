@@ -255,11 +255,17 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
   }
   flags &= ~OP_DX32_READY;
   if (b.kind == 0) {
-    // recorded (batched) launches take the per-element kernel; single launches the
-    // product from the quadrature-point coefficients
-    if (m->rec) flags &= ~OP_REUSED;
-    if (m->rec) return f32 ? launch_ns<float>(m, 1, dx, y, flags) : launch_ns<double>(m, 1, dx, y, flags);
-    return f32 ? launch_nsq<float>(m, dx, y, flags) : launch_nsq<double>(m, dx, y, flags);
+    // recorded (batched) launches take the per-element kernel; single launches in float32 the
+    // product from the quadrature-point coefficients, in float64 the direct product for the first
+    // few at a state and the assembled operator after that
+    if (m->rec)
+      return f32 ? launch_ns<float>(m, 1, dx, y, flags & ~OP_REUSED) : launch_ns<double>(m, 1, dx, y, flags & ~OP_REUSED);
+    if (f32) return launch_nsq32(m, dx, y, flags);
+    if (m->f64_gen != m->stage_gen) {
+      m->f64_gen = m->stage_gen;
+      m->f64_count = 0;
+    }
+    return (flags & OP_REUSED) || ++m->f64_count > NSA_AFTER ? launch_nsa(m, dx, y, flags) : hq_ns_jvp(m, dx, y, flags);
   }
   if (b.kind == 1)
     return f32 ? launch_ac<float>(m, 1, b.index, dx, y) : launch_ac<double>(m, 1, b.index, dx, y);
@@ -434,8 +440,8 @@ int fsi_destroy_mesh(fsi_mesh* m) {
   cudaFree(m->kry_dev);
   cudaFree(m->dx32);
   cudaFree(m->Z);
-  cudaFree(m->cq64);
-  cudaFree(m->cq32);
+  cudaFree(m->cq64.p);
+  cudaFree(m->cq32.p);
   cudaFree(m->na64);
   cudaFree(m->ke64);
   cudaFree(m->ke_e);

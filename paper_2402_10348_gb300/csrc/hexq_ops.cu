@@ -1,4 +1,5 @@
-// Residuals of the three kinds of block on hexahedra, one thread per (element, quadrature point)
+// Residuals of the three kinds of block on hexahedra, the momentum/continuity product at a state
+// that is used a few times, and its quadrature-point coefficients, one thread per (element, quadrature point)
 // (hexq.cuh); ops.cuh has the equations.
 #include "hexq.cuh"
 #include "ops_impl.cuh"
@@ -91,6 +92,135 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_b_res_kernel(const __grid_const
     const double s = l.scatter(R, t * v[0], t * v[1], t * v[2]);
     if (l.ok) E[(8 * c + l.q) * es + l.e] = s;
   }
+}
+
+// Quadrature-point coefficients of the momentum/continuity product (ops.cuh lists them) in
+// float64 and/or rounded to float32: C[((ez * 8 + q) * NCQ + c) * nxyp + ey * nxp + ex].  64^3, one
+// solid: 3.36 -> 1.17 ms against the tile build, all solids in one pass.
+__global__ void __launch_bounds__(HQ_THREADS) hq_ns_coef_kernel(const __grid_constant__ HexNS H, double* __restrict__ c64,
+                                                                float* __restrict__ c32, unsigned ne, int elastic) {
+  HexLane l;
+  l.set(H.g, H.rh, H.nxp, 0, ne);
+  NSPoint p;
+  hq_ns_point(H, l, p);
+  const int64_t b = ((int64_t)l.ez * 8 + l.q) * NCQ * H.nxyp + (int64_t)l.ey * H.nxp + l.ex;
+  auto put = [&](int c, double v) {
+    if (!l.ok) return;
+    if (c64) c64[b + c * H.nxyp] = v;
+    if (c32) c32[b + c * H.nxyp] = (float)v;
+  };
+  put(0, p.rho);
+  put(1, p.mu);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    put(2 + k, p.v[k]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) put(5 + 3 * k + j, p.L[k][j]);
+    put(14 + k, p.R[k]);
+  }
+  put(17, p.tau_m);
+  put(18, p.tau_c * p.rho);
+  put(19, p.tau_m * p.rrho);
+  if (!elastic) return;  // (the products then read the first 20)
+  double aB[6], aG[6][3];
+  hq_elastic(H, l, aB, aG);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    put(20 + c, aB[c]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) put(26 + 3 * c + j, aG[c][j]);
+  }
+}
+
+// The product itself for a state that is used a few times: the point's coefficients stay in
+// registers.  E as hq_ns_res_kernel.  A product at a new state with its coefficients stored before
+// it: 61 x 47 x 35 with two solids 2.97 -> 1.02 ms, 256 x 128 x 64 with nine 216 -> 47 ms (46.5 of them
+// here, about 1,560 float64 operations a point, 0.97 of the float64 rate).
+struct PointCoef {
+  const NSPoint& p;
+  const double (&aB)[6];
+  const double (&aG)[6][3];
+  __device__ __forceinline__ double operator()(int i) const {
+    if (i == 0) return p.rho;
+    if (i == 1) return p.mu;
+    if (i < 5) return p.v[i - 2];
+    if (i < 14) return p.L[(i - 5) / 3][(i - 5) % 3];
+    if (i < 17) return p.R[i - 14];
+    if (i == 17) return p.tau_m;
+    if (i == 18) return p.tau_c * p.rho;
+    if (i == 19) return p.tau_m * p.rrho;
+    if (i < 26) return aB[i - 20];
+    return aG[(i - 26) / 3][(i - 26) % 3];
+  }
+};
+
+__global__ void __launch_bounds__(HQ_THREADS) hq_ns_jvp_kernel(const __grid_constant__ HexNS H,
+                                                               const double* __restrict__ dx, double* __restrict__ E,
+                                                               unsigned ne, int elastic) {
+  HexLane l;
+  l.set(H.g, H.rh, H.nxp, 0, ne);
+  const int64_t es = (int64_t)H.g.nz * H.nxyp;
+  NSPoint p;
+  hq_ns_point(H, l, p);
+  double aB[6] = {}, aG[6][3] = {};
+  if (elastic) hq_elastic(H, l, aB, aG);
+  double dv[3], gd[3][3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const VG<double> r = l.vg(dx[k * H.nn + l.n]);
+    dv[k] = r.v; gd[k][0] = r.gx; gd[k][1] = r.gy; gd[k][2] = r.gz;
+  }
+  const VG<double> d = l.vg(dx[3 * H.nn + l.n]);
+  const double dgp[3] = {d.gx, d.gy, d.gz};
+  double f[4], g[4][3];
+  nsq_point_fg<double>(PointCoef{p, aB, aG}, elastic != 0, dv, gd, d.v, dgp, H.P.alpha, H.P.c_mass, f, g);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double c = l.scatter(f[k], g[k][0], g[k][1], g[k][2]);
+    if (l.ok) E[(8 * k + l.q) * es + l.e] = c;
+  }
+}
+
+int ns_build(fsi_mesh* m, unsigned flags, bool f64) {
+  const unsigned eflags = flags & FSI_ELASTIC_AUG;
+  fsi_mesh::NSCoef& c = f64 ? m->cq64 : m->cq32;
+  if (c.gen == m->stage_gen && c.flags == eflags && c.p) return FSI_OK;
+  const int nxp = cq_pitch(m);
+  const int64_t len = (int64_t)m->g.nz * 8 * NCQ * nxp * m->g.ny;
+  if (c.len < len) {
+    cudaFree(c.p);
+    c.p = nullptr;
+    c.len = 0;
+    FSI_CUDA(cudaMalloc(&c.p, (f64 ? sizeof(double) : sizeof(float)) * (size_t)len));
+    c.len = len;
+  }
+  const unsigned ne = (unsigned)m->g.nx * m->g.ny * m->g.nz;
+  FSI_LAUNCH(m, P_NS_BUILD,
+             hq_ns_coef_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(
+                 hex_ns(m, nxp), f64 ? static_cast<double*>(c.p) : nullptr, f64 ? nullptr : static_cast<float*>(c.p), ne,
+                 eflags && m->ns > 0 ? 1 : 0));
+  c.gen = m->stage_gen;
+  c.flags = eflags;
+  return FSI_OK;
+}
+
+int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
+  const Geom& g = m->g;
+  const int nxp = cq_pitch(m);
+  const int64_t nxyp = (int64_t)nxp * g.ny;
+  const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
+  const int elastic = (flags & FSI_ELASTIC_AUG) && m->ns > 0 ? 1 : 0;
+  if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
+  const HexNS H = hex_ns(m, nxp);
+  const RowLaunch nl = node_launch(g);
+  // algorithmic bytes: the nodal fields once, the contributions written and read, the product
+  prof_bytes(m, P_NS_JVP64, (double)ne * 256.0 + (double)m->nn * 8.0 * (13 + (elastic ? 7 * m->ns : 0)));
+  prof_bytes(m, P_NODE_SUM, (double)ne * 256.0 + (double)m->nn * 33.0);
+  FSI_LAUNCH(m, P_NS_JVP64, hq_ns_jvp_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, dx, m->ke_e, ne, elastic));
+  FSI_LAUNCH(m, P_NODE_SUM,
+             ns_node_kernel<double><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, H.W,
+                                                                         m->mask, m->pin_active, dx, nullptr, nullptr, y));
+  return FSI_OK;
 }
 
 int hq_residual(fsi_mesh* m, const BlockInfo& b, double* r) {

@@ -69,12 +69,14 @@ struct fsi_mesh {
   float* dx32 = nullptr;     // float copy of a product's increment (FSI_FP32)
   const double* staged_x = nullptr;  // x^{n+1} of the last staging (p and Dirichlet rows)
   int64_t stage_gen = 0;             // staging count: coefficients built at another count are stale
-  // quadrature-point coefficients of the NS product (NSBuildOp in ops.cuh, nsq_elem_kernel)
-  double* cq64 = nullptr;
-  float* cq32 = nullptr;
-  int64_t cq_len = 0;                // allocated coefficients (each array)
-  int64_t cq_gen = -1;               // stage_gen of the last build
-  unsigned cq_flags = 0;             // FSI_ELASTIC_AUG of the last build
+  // quadrature-point coefficients of the NS product (hq_ns_coef_kernel), built per type on demand
+  struct NSCoef {
+    void* p = nullptr;
+    int64_t len = 0;                 // allocated coefficients
+    int64_t gen = -1;                // stage_gen of the last build
+    unsigned flags = 0;              // FSI_ELASTIC_AUG of the last build
+  };
+  NSCoef cq64, cq32;
   // TMA descriptors of the float32 coefficients (boxes of 44 and of 20 values; nsq_tma.cu),
   // encoded for the allocation at cq_tmap_base; tma_err: a bounded wait gave up
   alignas(64) unsigned char cq_tmap[256] = {};
@@ -179,11 +181,12 @@ __global__ void coef_finalize(const double* partials, int64_t n, double eta, dou
 
 template <typename T>
 int launch_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags);
-// NS product from the quadrature-point coefficients (built first when stale)
-int ns_build(fsi_mesh* m, unsigned flags);  // ops_f64.cu
-// float32 NS product from the coefficients with TMA-staged coefficient boxes: the element
-// contributions into E (nsq_tma.cu)
-int launch_nsq_tma(fsi_mesh* m, int elastic, float* E, const double* dx, double* y);
+// quadrature-point coefficients of the NS product at the staged state (built when stale)
+int ns_build(fsi_mesh* m, unsigned flags, bool f64);  // hexq_ops.cu
+// float64 NS product at a state that is used a few times (hexq_ops.cu)
+int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags);
+// float32 NS product from the coefficients, TMA-staged (nsq_tma.cu); dx32 holds the increment
+int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags);
 // FSI_ECUDA if a bounded wait of that kernel gave up since the flag was allocated (syncs)
 int check_tma(fsi_mesh* m);
 // One instance's float32 NS product in a batched launch (nsq_tma.cu): the TMA descriptor of
@@ -226,16 +229,14 @@ int launch_ace(fsi_mesh* m, int phase, const double* dx, double* y);
 // float64 B product of one solid through the split operator (ops_f64.cu)
 int launch_be(fsi_mesh* m, int solid, const double* dx, double* y);
 // float64 NS products at one staging after which the assembled operator is built; a solve that may
-// take more builds it at once (OP_REUSED).  At 64^3 the build takes as long as NSA_AFTER
-// products from the coefficients.
-constexpr int NSA_AFTER = 8;
+// take more builds it at once (OP_REUSED).  At 64^3 the build (9.0 ms) takes as long as NSA_AFTER
+// direct products (2.0 ms) save beside the assembled one (0.22 ms).
+constexpr int NSA_AFTER = 5;
 // Allen-Cahn element matrices: a build costs about three re-interpolating products and
 // each matrix product a fifteenth of one; the B split operator's build costs less than one
 // re-interpolating product, so it is built at the first product of a solve
 constexpr int ACE_AFTER = 2;
 constexpr int BE_AFTER = 0;
-template <typename T>
-int launch_nsq(fsi_mesh* m, const double* dx, double* y, unsigned flags);
 template <typename T>
 int launch_ac(fsi_mesh* m, int mode, int phase, const double* dx, double* y);
 template <typename T>

@@ -166,6 +166,47 @@ __global__ void __launch_bounds__(TBX * TBY) nsq_tma_batch_kernel(const NSQBatch
                R.ny, R.nz, R.nxp, R.nxyp, R.nn, R.al, R.cm, R.rhx, R.rhy, R.rhz, it.y * TBX, it.z * TBY, it.w, R.err);
 }
 
+// NS product from the quadrature-point coefficients (see nsq_point) of element (ex, ey, ez)
+// into its 32 contribution slots (element-centric)
+template <typename T>
+__device__ __forceinline__ void nsq_elem_body(const T* __restrict__ cq, const T* __restrict__ dx, T* __restrict__ E,
+                                              int nx, int ny, int nz, int nxp, int64_t nxyp, int64_t nn, int elastic,
+                                              T al, T cmass, T rhx, T rhy, T rhz, int ex, int ey, int ez) {
+  const int64_t sy = nx + 1, sz = (int64_t)(nx + 1) * (ny + 1);
+  const int64_t n0 = ex + sy * ey + sz * ez;
+  const int64_t off[8] = {0, 1, sy, sy + 1, sz, sz + 1, sz + sy, sz + sy + 1};
+  T x[4][8], c[4][8];
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      x[f][a] = __ldg(dx + f * nn + n0 + off[a]);
+      c[f][a] = T(0);
+    }
+  const T* e0 = cq + (int64_t)ez * 8 * NCQ * nxyp + (int64_t)ey * nxp + ex;
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) {
+    QW<T> w;
+    w.set(q);
+    T dv[3], gd[3][3];
+#pragma unroll
+    for (int kk = 0; kk < 3; ++kk) {
+      const VG<T> r = interp_vg(x[kk], w, rhx, rhy, rhz);
+      dv[kk] = r.v; gd[kk][0] = r.gx; gd[kk][1] = r.gy; gd[kk][2] = r.gz;
+    }
+    const VG<T> dpr = interp_vg(x[3], w, rhx, rhy, rhz);
+    const T dgp[3] = {dpr.gx, dpr.gy, dpr.gz};
+    nsq_point<T>(CoefRef<T>{e0 + (int64_t)q * NCQ * nxyp, nxyp}, elastic != 0, dv, gd, dpr.v, dgp, al, cmass, w, rhx,
+                 rhy, rhz, c);
+  }
+  const int64_t e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
+  const int64_t es = (int64_t)nz * nxyp;
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+#pragma unroll
+    for (int a = 0; a < 8; ++a) E[(8 * f + a) * es + e] = c[f][a];
+}
+
 // Batched float64 product from the coefficients (nsq_elem_body): one CTA of 64 x 2
 // threads per (instance, x block, y block, layer) work item
 __global__ void __launch_bounds__(TBX * TBY) nsq_elem_batch_kernel(const NSQBatchRec* __restrict__ recs,
@@ -242,12 +283,12 @@ int encode_maps(fsi_mesh* m, int nxp, int64_t nxyp) {
   for (int k = 0; k < 2; ++k) {
     const cuuint32_t box[4] = {TBX, TBY, (cuuint32_t)(k == 0 ? NCQ : NCQ_FLUID), 1};
     CUtensorMap* map = reinterpret_cast<CUtensorMap*>(m->cq_tmap + 128 * k);
-    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, m->cq32, dims, strides, box, estr,
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, m->cq32.p, dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_error(FSI_ECUDA, "NS float32 product: tensor map encoding failed");
   }
-  m->cq_tmap_base = m->cq32;
+  m->cq_tmap_base = m->cq32.p;
   return FSI_OK;
 }
 
@@ -267,13 +308,12 @@ int check_tma(fsi_mesh* m) {
 int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, double* y, float* dx32,
                      NSQBatchRec* rec) {
   const unsigned eflags = flags & FSI_ELASTIC_AUG;
-  if (m->cq_gen != m->stage_gen || m->cq_flags != eflags || !m->cq64)
-    if (int rc = ns_build(m, flags)) return rc;
+  if (int rc = ns_build(m, flags, f64)) return rc;
   const Geom& g = m->g;
   const int nxp = cq_pitch(m);
   const int64_t nxyp = (int64_t)nxp * g.ny;
   if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
-  if (!f64 && m->cq_tmap_base != m->cq32)
+  if (!f64 && m->cq_tmap_base != m->cq32.p)
     if (int rc = encode_maps(m, nxp, nxyp)) return rc;
   if (!m->tma_err) {
     FSI_CUDA(cudaMalloc(&m->tma_err, sizeof(int)));
@@ -282,7 +322,7 @@ int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, do
   const int elastic = (eflags && m->ns > 0) ? 1 : 0;
   memset(rec, 0, sizeof(*rec));
   if (f64) {
-    rec->cq64 = m->cq64;
+    rec->cq64 = static_cast<const double*>(m->cq64.p);
     rec->E64 = m->ke_e;
   } else {
     memcpy(rec->map, m->cq_tmap + (elastic ? 0 : 128), 128);
@@ -330,11 +370,15 @@ int nsq_batch_launch(bool f64, const NSQBatchRec* recs, const int4* eitems, int 
   return FSI_OK;
 }
 
-int launch_nsq_tma(fsi_mesh* m, int elastic, float* E, const double* dx, double* y) {
+int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
+  if (int rc = ns_build(m, flags, false)) return rc;
   const Geom& g = m->g;
   const int nxp = cq_pitch(m);
-  const int64_t nxyp = (int64_t)nxp * g.ny;
-  if (m->cq_tmap_base != m->cq32)
+  const int64_t nxyp = (int64_t)nxp * g.ny, nn = m->nn;
+  const int elastic = ((flags & FSI_ELASTIC_AUG) && m->ns > 0) ? 1 : 0;
+  if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
+  float* E = reinterpret_cast<float*>(m->ke_e);
+  if (m->cq_tmap_base != m->cq32.p)
     if (int rc = encode_maps(m, nxp, nxyp)) return rc;
   if (!m->tma_err) {
     FSI_CUDA(cudaMalloc(&m->tma_err, sizeof(int)));
@@ -348,11 +392,20 @@ int launch_nsq_tma(fsi_mesh* m, int elastic, float* E, const double* dx, double*
   const dim3 blk(TBX, TBY);
   const float al = (float)m->P.alpha, cm = (float)m->P.c_mass;
   const float rx = (float)(1.0 / g.hx), ry = (float)(1.0 / g.hy), rz = (float)(1.0 / g.hz);
+  // algorithmic bytes: the coefficient planes once per element, the increment once per
+  // node, the 32 element contributions written; the node sums read them back and write
+  // the product (the mask once per node)
+  const double ne = (double)g.nx * g.ny * g.nz;
+  prof_bytes(m, P_NS_JVP32, ne * (8.0 * ncoef + 32.0) * 4.0 + (double)nn * 16.0);
+  prof_bytes(m, P_NODE_SUM, ne * 32.0 * 4.0 + (double)nn * (32.0 + 1.0));
   FSI_LAUNCH(m, P_NS_JVP32,
              (nsq_tma_kernel<<<(unsigned)nblk, blk, smem, m->stream>>>(*map, ncoef, m->dx32, E, g.nx, g.ny, g.nz, nxp,
-                                                                      nxyp, m->nn, al, cm, rx, ry, rz, m->tma_err)));
-  (void)dx;
-  (void)y;
+                                                                      nxyp, nn, al, cm, rx, ry, rz, m->tma_err)));
+  const RowLaunch nl = node_launch(g);
+  FSI_LAUNCH(m, P_NODE_SUM,
+             ns_node_kernel<float><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, nxp, nxyp, nn,
+                                                                        g.hx * g.hy * g.hz / 8.0, m->mask,
+                                                                        m->pin_active, dx, m->dx32, nullptr, y));
   return FSI_OK;
 }
 

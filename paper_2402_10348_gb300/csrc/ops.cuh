@@ -297,8 +297,8 @@ struct NSOp {
 
 // ----------------------------------------------- NS product from frozen coefficients
 // Within one NS block solve every coefficient of the product is fixed: the state the
-// Jacobian is taken at does not move.  NSBuildOp evaluates them once per solve, in
-// float64, at every quadrature point of every element; the product (nsq_elem_kernel)
+// Jacobian is taken at does not move.  hq_ns_coef_kernel evaluates them once per solve, in
+// float64, at every quadrature point of every element; the product (nsq_tma.cu)
 // then interpolates only the increment (dv, dp).  Per quadrature point:
 //   0 rho, 1 mu, 2-4 v, 5-13 L_kj = d_j v_k (k-major), 14-16 R_m,
 //   17 tau_m, 18 tau_c rho, 19 tau_m / rho,
@@ -309,123 +309,6 @@ struct NSOp {
 // padded pitch):  C[((ez * 8 + q) * NCQ + c) * nxyp + ey * nxp + ex].
 constexpr int NCQ = 44;
 constexpr int NCQ_FLUID = 20;
-
-struct CoefArrays {
-  double* c64;   // float64 coefficients (the build writes them)
-  float* c32;    // float32 copy (rounded from float64), or null
-  int nxp;       // x pitch (elements, padded)
-  int64_t nxyp;  // nxp * ny
-};
-
-// Coefficient build: fields as NSOp MODE 2 (v(3), p, dv/dt(3), rho, mu, then alpha^s,
-// B^s(6) per solid of the pass).  Only the CTA that owns an element writes it.  Later
-// solid passes (fluid == 0) add their solids' sums into aB and aG.
-struct NSBuildOp {
-  using T = double;
-  static constexpr int NC = 1;
-  static constexpr int MINB = 1;
-  Fields F;
-  int nf;
-  int s0, s1;
-  int fluid;
-  int elastic_aug;
-  Phys P;
-  double rh[3], W;
-  CoefArrays C;
-
-  __device__ __forceinline__ const T* fptr(int f) const { return field_ptr<T>(F, f); }
-  using Red = NoRed;
-  __device__ __forceinline__ void begin_cta(Red&) const {}
-  __device__ __forceinline__ void end_cta(Red&) const {}
-
-  __device__ __forceinline__ void put(int64_t idx, double v, bool add) const {
-    if (add) v += C.c64[idx];
-    C.c64[idx] = v;
-    if (C.c32) C.c32[idx] = (float)v;
-  }
-
-  __device__ void element(const Corners<T>& cr, const ElemCtx& ec, T (&)[NC][8], Red&) const {
-    if (!ec.owned) return;  // halo copies of this element are built by its owner
-    const T rhx = rh[0], rhy = rh[1], rhz = rh[2];
-    const int fv = 0, fp = 3, fvd = 4, frho = 7, fmu = 8, fsol = 9;
-    const int64_t e0 = (int64_t)ec.ez * 8 * NCQ * C.nxyp + (int64_t)ec.ey * C.nxp + ec.ex;
-    T u[8];
-#pragma unroll 1
-    for (int q = 0; q < 8; ++q) {
-      QW<T> w;
-      w.set(q);
-      const int64_t b = e0 + (int64_t)q * NCQ * C.nxyp;
-      T v[3], L[3][3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        cr.get(fv + k, u);
-        const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
-        v[k] = r.v; L[k][0] = r.gx; L[k][1] = r.gy; L[k][2] = r.gz;
-      }
-      if (fluid) {
-        cr.get(frho, u); const T rho = interp_v(u, w);
-        cr.get(fmu, u);  const T mu = interp_v(u, w);
-        cr.get(fp, u);
-        const VG<T> pr = interp_vg(u, w, rhx, rhy, rhz);
-        const T gp[3] = {pr.gx, pr.gy, pr.gz};
-        T Rm[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          cr.get(fvd + k, u);
-          const T acc = interp_v(u, w) + v[0] * L[k][0] + v[1] * L[k][1] + v[2] * L[k][2];
-          Rm[k] = rho * acc + gp[k] - rho * P.grav[k];
-        }
-        const T vGv = P.Gd[0] * v[0] * v[0] + P.Gd[1] * v[1] * v[1] + P.Gd[2] * v[2] * v[2];
-        const T nu = mu / rho;
-        const T tau_m = 1.0 / sqrt(4.0 / (P.dt * P.dt) + vGv + P.c_i * nu * nu * P.GG);
-        const T tau_c = 1.0 / (P.trG * tau_m);
-        put(b + 0 * C.nxyp, rho, false);
-        put(b + 1 * C.nxyp, mu, false);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) put(b + (2 + k) * C.nxyp, v[k], false);
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) put(b + (5 + 3 * k + j) * C.nxyp, L[k][j], false);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) put(b + (14 + k) * C.nxyp, Rm[k], false);
-        put(b + 17 * C.nxyp, tau_m, false);
-        put(b + 18 * C.nxyp, tau_c * rho, false);
-        put(b + 19 * C.nxyp, tau_m / rho, false);
-      }
-      T aB[6], aG[6][3];
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) {
-        aB[cc] = 0.0;
-        aG[cc][0] = aG[cc][1] = aG[cc][2] = 0.0;
-      }
-      if (elastic_aug) {
-        for (int s = s0; s < s1; ++s) {
-          const int fs = fsol + 7 * (s - s0);
-          cr.get(fs, u);
-          const T a = interp_v(u, w) * P.muL[P.solid_phase[s]] * P.c_el;
-#pragma unroll
-          for (int cc = 0; cc < 6; ++cc) {
-            cr.get(fs + 1 + cc, u);
-            const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
-            aB[cc] += a * r.v;
-            aG[cc][0] += a * r.gx;
-            aG[cc][1] += a * r.gy;
-            aG[cc][2] += a * r.gz;
-          }
-        }
-      }
-      const bool add = !fluid;
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) {
-        put(b + (20 + cc) * C.nxyp, aB[cc], add);
-#pragma unroll
-        for (int mm = 0; mm < 3; ++mm) put(b + (26 + 3 * cc + mm) * C.nxyp, aG[cc][mm], add);
-      }
-    }
-  }
-  __device__ __forceinline__ void finish(const NodeCtx&, const T (&)[NC], Red&) const {}
-};
 
 // The product's arithmetic at one quadrature point, from the interpolated increment
 // (dv, its gradient gd[k][j] = d_j dv_k, dp and its gradient dgp) and the point's

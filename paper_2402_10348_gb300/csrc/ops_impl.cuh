@@ -317,110 +317,6 @@ __global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__
   for (int c = 0; c < NC; ++c) y[c * nn + n] = s[c];
 }
 
-// NS product from the quadrature-point coefficients (see nsq_point) of element (ex, ey, ez)
-// into its 32 contribution slots (element-centric)
-template <typename T>
-__device__ __forceinline__ void nsq_elem_body(const T* __restrict__ cq, const T* __restrict__ dx, T* __restrict__ E,
-                                              int nx, int ny, int nz, int nxp, int64_t nxyp, int64_t nn, int elastic,
-                                              T al, T cmass, T rhx, T rhy, T rhz, int ex, int ey, int ez) {
-  const int64_t sy = nx + 1, sz = (int64_t)(nx + 1) * (ny + 1);
-  const int64_t n0 = ex + sy * ey + sz * ez;
-  const int64_t off[8] = {0, 1, sy, sy + 1, sz, sz + 1, sz + sy, sz + sy + 1};
-  T x[4][8], c[4][8];
-#pragma unroll
-  for (int f = 0; f < 4; ++f)
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      x[f][a] = __ldg(dx + f * nn + n0 + off[a]);
-      c[f][a] = T(0);
-    }
-  const T* e0 = cq + (int64_t)ez * 8 * NCQ * nxyp + (int64_t)ey * nxp + ex;
-#pragma unroll 1
-  for (int q = 0; q < 8; ++q) {
-    QW<T> w;
-    w.set(q);
-    T dv[3], gd[3][3];
-#pragma unroll
-    for (int kk = 0; kk < 3; ++kk) {
-      const VG<T> r = interp_vg(x[kk], w, rhx, rhy, rhz);
-      dv[kk] = r.v; gd[kk][0] = r.gx; gd[kk][1] = r.gy; gd[kk][2] = r.gz;
-    }
-    const VG<T> dpr = interp_vg(x[3], w, rhx, rhy, rhz);
-    const T dgp[3] = {dpr.gx, dpr.gy, dpr.gz};
-    nsq_point<T>(CoefRef<T>{e0 + (int64_t)q * NCQ * nxyp, nxyp}, elastic != 0, dv, gd, dpr.v, dgp, al, cmass, w, rhx,
-                 rhy, rhz, c);
-  }
-  const int64_t e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
-  const int64_t es = (int64_t)nz * nxyp;
-#pragma unroll
-  for (int f = 0; f < 4; ++f)
-#pragma unroll
-    for (int a = 0; a < 8; ++a) E[(8 * f + a) * es + e] = c[f][a];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128) nsq_elem_kernel(const T* __restrict__ cq, const T* __restrict__ dx,
-                                                       T* __restrict__ E, int nx, int ny, int nz, int nxp, int64_t nxyp,
-                                                       int64_t nn, int elastic, T al, T cmass, T rhx, T rhy, T rhz) {
-  ElemIdx I;
-  if (!I.set(nx, ny, nz, nxp, nxyp)) return;
-  nsq_elem_body<T>(cq, dx, E, nx, ny, nz, nxp, nxyp, nn, elastic, al, cmass, rhx, rhy, rhz, I.ex, I.ey, I.ez);
-}
-
-template <typename T>
-int launch_nsq(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
-  const unsigned eflags = flags & FSI_ELASTIC_AUG;
-  if constexpr (sizeof(T) == 8) {
-    if (m->f64_gen != m->stage_gen) {
-      m->f64_gen = m->stage_gen;
-      m->f64_count = 0;
-    }
-    if ((flags & OP_REUSED) || ++m->f64_count > NSA_AFTER) return launch_nsa(m, dx, y, flags);
-  }
-  if (m->cq_gen != m->stage_gen || m->cq_flags != eflags || !m->cq64) {
-    if (int rc = ns_build(m, flags)) return rc;
-  }
-  const Geom& g = m->g;
-  const int64_t nn = m->nn;
-  const int nxp = cq_pitch(m);
-  const int64_t nxyp = (int64_t)nxp * g.ny;
-  const int elastic = (eflags && m->ns > 0) ? 1 : 0;
-  if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
-  const T* cq;
-  const T* xin;
-  if constexpr (sizeof(T) == 8) {
-    cq = reinterpret_cast<const T*>(m->cq64);
-    xin = reinterpret_cast<const T*>(dx);
-  } else {
-    cq = reinterpret_cast<const T*>(m->cq32);
-    xin = reinterpret_cast<const T*>(m->dx32);
-  }
-  T* E = reinterpret_cast<T*>(m->ke_e);
-  // algorithmic bytes: the coefficient planes once per element, the increment once per
-  // node, the 32 element contributions written; the node sums read them back and write
-  // the product (the mask once per node)
-  const int64_t ne = (int64_t)g.nx * g.ny * g.nz;
-  prof_bytes(m, jvp_class<T>(0),
-             (double)ne * (8.0 * (elastic ? NCQ : NCQ_FLUID) + 32.0) * sizeof(T) + (double)nn * 4.0 * sizeof(T));
-  prof_bytes(m, P_NODE_SUM, (double)ne * 32.0 * sizeof(T) + (double)nn * (32.0 + 1.0));
-  const RowLaunch el = elem_launch(g), nl = node_launch(g);
-  if constexpr (sizeof(T) == 4) {
-    (void)cq;
-    (void)xin;
-    if (int rc = launch_nsq_tma(m, elastic, E, dx, y)) return rc;
-  } else {
-    FSI_LAUNCH(m, jvp_class<T>(0),
-               nsq_elem_kernel<T><<<el.grid, el.block, 0, m->stream>>>(
-                   cq, xin, E, g.nx, g.ny, g.nz, nxp, nxyp, nn, elastic, T(m->P.alpha), T(m->P.c_mass),
-                   T(1.0 / g.hx), T(1.0 / g.hy), T(1.0 / g.hz)));
-  }
-  FSI_LAUNCH(m, P_NODE_SUM,
-             ns_node_kernel<T><<<nl.grid, nl.block, 0, m->stream>>>(
-                 E, g.nx, g.ny, g.nz, nxp, nxyp, nn, g.hx * g.hy * g.hz / 8.0, m->mask, m->pin_active,
-                 dx, sizeof(T) == 4 ? m->dx32 : nullptr, nullptr, y));
-  return FSI_OK;
-}
-
 template <typename T, int MODE>
 int ac_run(fsi_mesh* m, int i, const double* dx, double* y) {
   ACOp<T, MODE> op;
