@@ -254,28 +254,33 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
       FSI_LAUNCH(m, P_KRY_CONV, to_float_kernel<<<vec_grid(b.n), 256, 0, m->stream>>>(dx, m->dx32, b.n));
   }
   flags &= ~OP_DX32_READY;
-  if (b.kind == 0) {
-    // recorded (batched) launches take the per-element kernel; single launches in float32 the
-    // product from the quadrature-point coefficients, in float64 the direct product for the first
-    // few at a state and the assembled operator after that
-    if (m->rec)
-      return f32 ? launch_ns<float>(m, 1, dx, y, flags & ~OP_REUSED) : launch_ns<double>(m, 1, dx, y, flags & ~OP_REUSED);
-    if (f32) return launch_nsq32(m, dx, y, flags);
-    if (m->f64_gen != m->stage_gen) {
-      m->f64_gen = m->stage_gen;
-      m->f64_count = 0;
-    }
-    return (flags & OP_REUSED) || ++m->f64_count > NSA_AFTER ? launch_nsa(m, dx, y, flags) : hq_ns_jvp(m, dx, y, flags);
+  if (m->rec) {  // recorded (batched) launches take the per-element kernels
+    flags &= ~OP_REUSED;
+    if (b.kind == 0) return f32 ? launch_ns<float>(m, 1, dx, y, flags) : launch_ns<double>(m, 1, dx, y, flags);
+    if (b.kind == 1) return f32 ? launch_ac<float>(m, 1, b.index, dx, y) : launch_ac<double>(m, 1, b.index, dx, y);
+    return f32 ? launch_b<float>(m, 1, b.index, dx, y) : launch_b<double>(m, 1, b.index, dx, y);
   }
-  if (b.kind == 1)
-    return f32 ? launch_ac<float>(m, 1, b.index, dx, y) : launch_ac<double>(m, 1, b.index, dx, y);
-  return f32 ? launch_b<float>(m, 1, b.index, dx, y) : launch_b<double>(m, 1, b.index, dx, y);
+  if (f32) {
+    if (b.kind == 0) return launch_nsq32(m, dx, y, flags);
+    return b.kind == 1 ? launch_ac<float>(m, 1, b.index, dx, y) : launch_b<float>(m, 1, b.index, dx, y);
+  }
+  // float64: direct products for the first few at a state, then the assembled operator
+  const int32_t id = (b.kind << 16) | b.index;
+  if (m->f64_gen != m->stage_gen || m->f64_block != id) {
+    m->f64_gen = m->stage_gen;
+    m->f64_block = id;
+    m->f64_count = 0;
+  }
+  ++m->f64_count;
+  if (b.kind == 0)
+    return (flags & OP_REUSED) || m->f64_count > NSA_AFTER ? launch_nsa(m, dx, y, flags) : hq_ns_jvp(m, dx, y, flags);
+  return (flags & OP_REUSED) || m->f64_count > STENCIL_AFTER ? stencil_jvp(m, b, dx, y) : hq_jvp(m, b, dx, y);
 }
 
 int op_diag(fsi_mesh* m, const BlockInfo& b, double* d, unsigned flags) {
   if (m->tet) return tet_op(m, b, 2, nullptr, d, flags & ~OP_REUSED);
   const bool f32 = flags & FSI_FP32;
-  if (b.kind == 0 && !f32 && !m->rec && (flags & OP_REUSED)) return nsa_diag(m, d, flags);
+  if (!f32 && !m->rec && (flags & OP_REUSED)) return b.kind == 0 ? nsa_diag(m, d, flags) : stencil_diag(m, b, d);
   flags &= ~OP_REUSED;
   if (b.kind == 0)
     return f32 ? launch_ns<float>(m, 2, nullptr, d, flags) : launch_ns<double>(m, 2, nullptr, d, flags);
@@ -446,8 +451,8 @@ int fsi_destroy_mesh(fsi_mesh* m) {
   cudaFree(m->ke64);
   cudaFree(m->ke_e);
   cudaFree(m->tma_err);
-  cudaFree(m->ake64);
-  cudaFree(m->bke64);
+  cudaFree(m->acst.A);
+  cudaFree(m->bst.A);
   tet_free(m->tet);
   if (m->kry_est) cudaFreeHost(m->kry_est);
   for (cudaEvent_t e : m->kry_ev) cudaEventDestroy(e);

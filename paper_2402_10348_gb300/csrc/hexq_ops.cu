@@ -1,5 +1,5 @@
-// Residuals of the three kinds of block on hexahedra, the momentum/continuity product at a state
-// that is used a few times, and its quadrature-point coefficients, one thread per (element, quadrature point)
+// Residuals of the three kinds of block on hexahedra, their float64 products at a state that is used
+// a few times, and the quadrature-point coefficients of the momentum block, one thread per (element, quadrature point)
 // (hexq.cuh); ops.cuh has the equations.
 #include "hexq.cuh"
 #include "ops_impl.cuh"
@@ -181,6 +181,66 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ns_jvp_kernel(const __grid_cons
   }
 }
 
+// Allen-Cahn and B products at a state that is used a few times
+__global__ void __launch_bounds__(HQ_THREADS) hq_ac_jvp_kernel(const __grid_constant__ HexNS H, int phase, double gam,
+                                                               double bet, const double* __restrict__ dx,
+                                                               double* __restrict__ E, unsigned ne) {
+  HexLane l;
+  l.set(H.g, H.rh, H.nxp, 0, ne);
+  const Phys& P = H.P;
+  double v[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = l.val(H.xa[k * H.nn + l.n]);
+  const double phi = l.val(H.xa[(4 + phase) * H.nn + l.n]);
+  const VG<double> d = l.vg(dx[l.n]);
+  const double k_hat = gam * P.eps * P.eps, s_hat = gam * (3.0 * phi * phi - 1.0);
+  const double vGv = P.Gd[0] * v[0] * v[0] + P.Gd[1] * v[1] * v[1] + P.Gd[2] * v[2] * v[2];
+  const double tau = rsqrt(H.dt2 + vGv + 9.0 * k_hat * k_hat * P.GG + s_hat * s_hat);
+  const double p2 = phi * phi - 1.0;
+  const double dsF = p2 > 0.0 ? phi : (p2 < 0.0 ? -phi : 0.0);
+  const double rp = gam * (3.0 * phi * phi - 1.0 - bet * dsF);
+  const double dR = P.c_mass * d.v + P.alpha * (v[0] * d.gx + v[1] * d.gy + v[2] * d.gz + rp * d.v);
+  const double t = tau * dR, ka = k_hat * P.alpha;
+  const double c = l.scatter(dR, ka * d.gx + t * v[0], ka * d.gy + t * v[1], ka * d.gz + t * v[2]);
+  if (l.ok) E[l.q * (int64_t)H.g.nz * H.nxyp + l.e] = H.W * c;
+}
+
+__global__ void __launch_bounds__(HQ_THREADS) hq_b_jvp_kernel(const __grid_constant__ HexNS H, int solid,
+                                                              const double* __restrict__ dx, double* __restrict__ E,
+                                                              unsigned ne) {
+  HexLane l;
+  l.set(H.g, H.rh, H.nxp, 0, ne);
+  const Phys& P = H.P;
+  const int64_t nn = H.nn, es = (int64_t)H.g.nz * H.nxyp;
+  double v[3], L[3][3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const VG<double> r = l.vg(H.xa[k * nn + l.n]);
+    v[k] = r.v; L[k][0] = r.gx; L[k][1] = r.gy; L[k][2] = r.gz;
+  }
+  const double al = l.val(H.mat[(2 + solid) * nn + l.n]);
+  const double vGv = P.Gd[0] * v[0] * v[0] + P.Gd[1] * v[1] * v[1] + P.Gd[2] * v[2] * v[2];
+  const double tau = rsqrt(H.dt2 + vGv);
+  double B[6], cv[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const VG<double> r = l.vg(dx[c * nn + l.n]);
+    B[c] = P.alpha * r.v;
+    cv[c] = P.alpha * (v[0] * r.gx + v[1] * r.gy + v[2] * r.gz) + P.c_mass * r.v;
+  }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int k = sym_k(c), m = sym_l(c);
+    double st = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) st += L[k][i] * B[sym_idx(i, m)] + B[sym_idx(k, i)] * L[m][i];
+    const double R = H.W * (al * (cv[c] - st) + (1.0 - al) * B[c]);
+    const double t = tau * R;
+    const double s = l.scatter(R, t * v[0], t * v[1], t * v[2]);
+    if (l.ok) E[(8 * c + l.q) * es + l.e] = s;
+  }
+}
+
 int ns_build(fsi_mesh* m, unsigned flags, bool f64) {
   const unsigned eflags = flags & FSI_ELASTIC_AUG;
   fsi_mesh::NSCoef& c = f64 ? m->cq64 : m->cq32;
@@ -223,12 +283,36 @@ int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   return FSI_OK;
 }
 
+int hq_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y) {
+  const Geom& g = m->g;
+  const int nxp = cq_pitch(m);
+  const int64_t nxyp = (int64_t)nxp * g.ny;
+  const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
+  if (int rc = ensure_elem_scratch(m, 8 * b.nc, nxyp)) return rc;
+  const HexNS H = hex_ns(m, nxp);
+  const RowLaunch nl = node_launch(g);
+  prof_bytes(m, P_NODE_SUM, (double)ne * 64 * b.nc + (double)m->nn * 8 * b.nc);
+  if (b.kind == 1) {
+    prof_bytes(m, P_AC_JVP64, (double)ne * 64.0 + (double)m->nn * 40.0);
+    FSI_LAUNCH(m, P_AC_JVP64, hq_ac_jvp_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(
+                                  H, b.index, m->gamma[b.index], m->beta[b.index], dx, m->ke_e, ne));
+    FSI_LAUNCH(m, P_NODE_SUM,
+               em_node_kernel<1><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, y));
+  } else {
+    prof_bytes(m, P_B_JVP64, (double)ne * 384.0 + (double)m->nn * 80.0);
+    FSI_LAUNCH(m, P_B_JVP64, hq_b_jvp_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, b.index, dx, m->ke_e, ne));
+    FSI_LAUNCH(m, P_NODE_SUM,
+               em_node_kernel<6><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, y));
+  }
+  return FSI_OK;
+}
+
 int hq_residual(fsi_mesh* m, const BlockInfo& b, double* r) {
   const Geom& g = m->g;
   const int nxp = cq_pitch(m);
   const int64_t nxyp = (int64_t)nxp * g.ny;
   const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
-  const int nc = b.kind == 0 ? 4 : b.kind == 1 ? 1 : 6;
+  const int nc = b.nc;
   if (int rc = ensure_elem_scratch(m, 8 * nc, nxyp)) return rc;
   const HexNS H = hex_ns(m, nxp);
   const RowLaunch nl = node_launch(g);

@@ -91,18 +91,17 @@ struct fsi_mesh {
   int64_t ke_len = 0;
   double* ke_e = nullptr;            // [slots][elements] corner contributions of the element-centric products
   int64_t ke_e_len = 0;
-  int64_t f64_gen = -1, f64_count = 0;  // float64 NS products applied at staging f64_gen
-  // float64 Allen-Cahn element matrices (ace_elem_kernel) of one phase at one staging
-  double* ake64 = nullptr;
-  int64_t ake_len = 0;
-  int64_t ake_gen = -1, ake_count = 0;  // staging the products were counted at / built for
-  int ake_phase = -1, ake_built = 0;
-  double ake_gamma = 0.0, ake_beta = 0.0;
-  // float64 B split operators (be_elem_kernel) of one solid at one staging
-  double* bke64 = nullptr;
-  int64_t bke_len = 0;
-  int64_t bke_gen = -1, bke_count = 0;
-  int bke_solid = -1, bke_built = 0;
+  int64_t f64_gen = -1, f64_count = 0;  // float64 products applied at staging f64_gen ...
+  int32_t f64_block = -1;               // ... on this kind and index of block
+  // assembled float64 Allen-Cahn and B operators (stencil.cu) of one indicator and one solid
+  struct Stencil {
+    double* A = nullptr;
+    int64_t len = 0;
+    int64_t gen = -1;                // stage_gen of the last build
+    int index = -1, built = 0;
+    double gamma = 0.0, beta = 0.0;
+  };
+  Stencil acst, bst;
   const double* staged_xa = nullptr; // the x^{n+alpha} array in use
   // coefficients
   double gamma[fsi::MAXP] = {0};
@@ -224,19 +223,18 @@ int ensure_elem_scratch(fsi_mesh* m, int slots, int64_t nxyp);
 int nsa_build(fsi_mesh* m, unsigned flags);
 int launch_nsa(fsi_mesh* m, const double* dx, double* y, unsigned flags);
 int nsa_diag(fsi_mesh* m, double* d, unsigned flags);
-// float64 Allen-Cahn product of one phase through element matrices (ops_f64.cu)
-int launch_ace(fsi_mesh* m, int phase, const double* dx, double* y);
-// float64 B product of one solid through the split operator (ops_f64.cu)
-int launch_be(fsi_mesh* m, int solid, const double* dx, double* y);
+// float64 Allen-Cahn and B products at a state that is used a few times (hexq_ops.cu), and the assembled
+// operators: build when stale, product and diagonal (stencil.cu)
+int hq_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y);
+int stencil_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y);
+int stencil_diag(fsi_mesh* m, const BlockInfo& b, double* d);
+int ensure_elem_matrices(fsi_mesh* m, int64_t len);  // nsa.cu
 // float64 NS products at one staging after which the assembled operator is built; a solve that may
 // take more builds it at once (OP_REUSED).  At 64^3 the build (9.0 ms) takes as long as NSA_AFTER
 // direct products (2.0 ms) save beside the assembled one (0.22 ms).
 constexpr int NSA_AFTER = 5;
-// Allen-Cahn element matrices: a build costs about three re-interpolating products and
-// each matrix product a fifteenth of one; the B split operator's build costs less than one
-// re-interpolating product, so it is built at the first product of a solve
-constexpr int ACE_AFTER = 2;
-constexpr int BE_AFTER = 0;
+// the same for Allen-Cahn and B products: an assembly costs two to three direct products
+constexpr int STENCIL_AFTER = 2;
 template <typename T>
 int launch_ac(fsi_mesh* m, int mode, int phase, const double* dx, double* y);
 template <typename T>

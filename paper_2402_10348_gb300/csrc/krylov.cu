@@ -1060,7 +1060,7 @@ int gmres_solve(fsi_mesh* m, const BlockInfo& blk, const double* rhs, double* x,
                                  OP_REUSED);
   // a float64 solve that may take many products assembles the operator before the first one (its
   // diagonal comes with it)
-  if (o.precision == FSI_PREC_FP64 && o.max_iter > NSA_AFTER) opflags |= OP_REUSED;
+  if (o.precision == FSI_PREC_FP64 && o.max_iter > (blk.kind == 0 ? NSA_AFTER : STENCIL_AFTER)) opflags |= OP_REUSED;
   // read by the solver loop only: network/Jacobi alternation, and no stop on stagnation
   const unsigned alt = o.flags & (FSI_PC_ALTERNATE | FSI_NO_STALL_STOP);
   const bool stall_stop = (o.flags & FSI_NO_STALL_STOP) == 0;

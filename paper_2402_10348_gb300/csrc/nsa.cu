@@ -358,6 +358,17 @@ __global__ void nsa_diag_kernel(const double* __restrict__ A, int64_t nn, const 
 // element matrices kept at a time (they are needed until the node planes on both sides are summed)
 constexpr int64_t NSA_SLAB_BYTES = (int64_t)1 << 30;
 
+// scratch of the element matrices (every block in turn)
+int ensure_elem_matrices(fsi_mesh* m, int64_t len) {
+  if (m->ke_len >= len) return FSI_OK;
+  cudaFree(m->ke64);
+  m->ke64 = nullptr;
+  m->ke_len = 0;
+  FSI_CUDA(cudaMalloc(&m->ke64, sizeof(double) * (size_t)len));
+  m->ke_len = len;
+  return FSI_OK;
+}
+
 int nsa_build(fsi_mesh* m, unsigned flags) {
   const unsigned eflags = flags & FSI_ELASTIC_AUG;
   if (m->na_gen == m->stage_gen && m->na_flags == eflags && m->na64) return FSI_OK;
@@ -373,13 +384,7 @@ int nsa_build(fsi_mesh* m, unsigned flags) {
     m->na_len = len;
   }
   const int slots = (int)std::min<int64_t>(g.nz, std::max<int64_t>(2, NSA_SLAB_BYTES / (8 * layer)));
-  if (m->ke_len < slots * layer) {
-    cudaFree(m->ke64);
-    m->ke64 = nullptr;
-    m->ke_len = 0;
-    FSI_CUDA(cudaMalloc(&m->ke64, sizeof(double) * (size_t)(slots * layer)));
-    m->ke_len = slots * layer;
-  }
+  if (int rc = ensure_elem_matrices(m, slots * layer)) return rc;
   const HexNS H = hex_ns(m, nxp);
   const int elastic = eflags && m->ns > 0 ? 1 : 0;
   const int64_t plane = (int64_t)(g.nx + 1) * (g.ny + 1);

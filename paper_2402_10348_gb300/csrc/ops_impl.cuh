@@ -206,25 +206,6 @@ __device__ __forceinline__ int64_t row_index(int len, int* x) {
   return byi * blockDim.y + threadIdx.y;
 }
 
-struct ElemIdx {
-  int ex, ey, ez;
-  int64_t n0, e, es;
-  int64_t off[8];
-  __device__ __forceinline__ bool set(int nx, int ny, int nz, int nxp, int64_t nxyp) {
-    const int64_t eyz = row_index(nx, &ex);
-    ey = (int)(eyz % ny);
-    if (ex >= nx || eyz >= (int64_t)ny * nz) return false;
-    ez = (int)(eyz / ny);
-    const int64_t sy = nx + 1, sz = (int64_t)(nx + 1) * (ny + 1);
-    n0 = ex + sy * ey + sz * ez;
-    off[0] = 0; off[1] = 1; off[2] = sy; off[3] = sy + 1;
-    off[4] = sz; off[5] = sz + 1; off[6] = sz + sy; off[7] = sz + sy + 1;
-    e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
-    es = (int64_t)nz * nxyp;
-    return true;
-  }
-};
-
 // Launch shape over rows of `len` items (elements or nodes along x), `rows` rows: CTAs of
 // bx x by threads (bx the row length rounded up to a warp, at most 128; by = 128 / bx
 // rows), numbered x-block fastest in a one-dimensional grid (no 65,535 limit on rows).
@@ -236,7 +217,6 @@ inline RowLaunch row_launch(int len, int64_t rows) {
   const int64_t nbx = (len + bx - 1) / bx, nby = (rows + by - 1) / by;
   return RowLaunch{dim3((unsigned)(nbx * nby)), dim3(bx, by)};
 }
-inline RowLaunch elem_launch(const Geom& g) { return row_launch(g.nx, (int64_t)g.ny * g.nz); }
 inline RowLaunch node_launch(const Geom& g) { return row_launch(g.nx + 1, (int64_t)(g.ny + 1) * (g.nz + 1)); }
 
 // NS node sums: y = W * sum of the element slots, the Dirichlet rows (velocity; pressure
@@ -339,22 +319,6 @@ int ac_run(fsi_mesh* m, int i, const double* dx, double* y) {
 
 template <typename T>
 int launch_ac(fsi_mesh* m, int mode, int i, const double* dx, double* y) {
-  if constexpr (sizeof(T) == 8) {
-    // a float64 solve of this phase at this staging: after ACE_AFTER products switch to the
-    // element matrices (not for recorded batched launches)
-    if (mode == 1 && !m->rec) {
-      if (m->ake_gen != m->stage_gen || m->ake_phase != i || m->ake_gamma != m->gamma[i] ||
-          m->ake_beta != m->beta[i]) {
-        m->ake_gen = m->stage_gen;
-        m->ake_phase = i;
-        m->ake_gamma = m->gamma[i];
-        m->ake_beta = m->beta[i];
-        m->ake_count = 0;
-        m->ake_built = 0;
-      }
-      if (++m->ake_count > ACE_AFTER) return launch_ace(m, i, dx, y);
-    }
-  }
   if (mode == 1) return ac_run<T, 1>(m, i, dx, y);
   return ac_run<T, 2>(m, i, dx, y);
 }
@@ -381,19 +345,6 @@ int b_run(fsi_mesh* m, int s, const double* dx, double* y) {
 
 template <typename T>
 int launch_b(fsi_mesh* m, int mode, int s, const double* dx, double* y) {
-  if constexpr (sizeof(T) == 8) {
-    // a float64 solve of this solid at this staging: after BE_AFTER products switch to the
-    // split operator (not for recorded batched launches)
-    if (mode == 1 && !m->rec) {
-      if (m->bke_gen != m->stage_gen || m->bke_solid != s) {
-        m->bke_gen = m->stage_gen;
-        m->bke_solid = s;
-        m->bke_count = 0;
-        m->bke_built = 0;
-      }
-      if (++m->bke_count > BE_AFTER) return launch_be(m, s, dx, y);
-    }
-  }
   if (mode == 1) return b_run<T, 1>(m, s, dx, y);
   return b_run<T, 2>(m, s, dx, y);
 }
