@@ -76,13 +76,6 @@ int prof_end(fsi_mesh* m, int cls) {
   return FSI_OK;
 }
 
-void tile_grid(const fsi_mesh* m, dim3* grid) {
-  const int ncx = (m->g.nx + 1 + OX - 1) / OX;
-  const int ncy = (m->g.ny + 1 + OY - 1) / OY;
-  const int planes = m->g.nz + 1;
-  const int chunks = (planes + m->g.zc - 1) / m->g.zc;
-  *grid = dim3(ncx, ncy, chunks);
-}
 
 // --------------------------------------------------------------- staging
 // x^{n+alpha} = x^n + alpha (x^{n+1} - x^n) (pressure plane: p^{n+1}),

@@ -34,7 +34,9 @@ struct HexLane {
   double sx, sy, sz;  // 1/h with the sign that turns partner - own into the derivative
   // elements [e0, e1) of the mesh (32-bit: a state of 2^31 elements exceeds the memory)
   __device__ __forceinline__ void set(const Geom& g, const double (&rh)[3], int nxp, unsigned e0, unsigned e1) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    set(g, rh, nxp, e0, e1, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  }
+  __device__ __forceinline__ void set(const Geom& g, const double (&rh)[3], int nxp, unsigned e0, unsigned e1, int64_t t) {
     q = (int)(t & 7);
     ok = e0 + (t >> 3) < e1;
     const unsigned f = ok ? e0 + (unsigned)(t >> 3) : e1 - 1;

@@ -336,4 +336,135 @@ int hq_residual(fsi_mesh* m, const BlockInfo& b, double* r) {
   return FSI_OK;
 }
 
+// ------------------------------------------------------------------ gamma, beta
+// Sections 2.2.1 and 2.2.2 as CoefOp (ops.cuh) has them: the corner contributions of the lumped
+// projection of q = grad phi^T grad v grad phi / |grad phi|^2, unweighted (its denominator is W times
+// the node's elements), and the CTA's partial integrals of F' and sqrt F over its elements.
+__global__ void __launch_bounds__(HQ_THREADS) hq_coef_kernel(const __grid_constant__ HexNS H, int phase,
+                                                             double* __restrict__ E, double* __restrict__ part, unsigned ne) {
+  const double* phi = H.xa + (int64_t)(4 + phase) * H.nn;
+  const int64_t es = (int64_t)H.g.nz * H.nxyp, nt = (int64_t)ne * 8;
+  double sF = 0.0, sS = 0.0;
+  // whole warps stay in the loop together (32 lanes: four elements)
+  for (int64_t t = (int64_t)blockIdx.x * HQ_THREADS + threadIdx.x; t - (threadIdx.x & 31) < nt;
+       t += (int64_t)gridDim.x * HQ_THREADS) {
+    HexLane l;
+    l.set(H.g, H.rh, H.nxp, 0, ne, t);
+    const VG<double> ph = l.vg(phi[l.n]);
+    const double g[3] = {ph.gx, ph.gy, ph.gz};
+    double num = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const VG<double> r = l.vg(H.xa[j * H.nn + l.n]);
+      num = fma(g[j], r.gx * g[0] + r.gy * g[1] + r.gz * g[2], num);
+    }
+    const double n2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
+    const double c = l.val(n2 < 1e-30 ? 0.0 : num / n2);
+    if (l.ok) {
+      E[l.q * es + l.e] = c;
+      sF += ph.v * ph.v * ph.v - ph.v;
+      sS += 0.5 * fabs(ph.v * ph.v - 1.0);
+    }
+  }
+  __shared__ double red[2][HQ_THREADS / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sF += __shfl_down_sync(0xffffffffu, sF, o);
+    sS += __shfl_down_sync(0xffffffffu, sS, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = sF;
+    red[1][threadIdx.x >> 5] = sS;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double s = 0.0;
+    for (int i = 0; i < HQ_THREADS / 32; ++i) s += red[threadIdx.x][i];
+    part[2 * blockIdx.x + threadIdx.x] = H.W * s;
+  }
+}
+
+// the CTA's partial sum of squared nodal values and count of nodes in the band |phi| <= 0.9
+__global__ void __launch_bounds__(NTHREADS) hq_coef_node_kernel(const double* __restrict__ E, int nx, int ny, int nz, int nxp,
+                                                                int64_t nxyp, int64_t nn, const double* __restrict__ phi,
+                                                                double* __restrict__ part) {
+  __shared__ double scratch[NTHREADS / 32];
+  const int64_t es = (int64_t)nz * nxyp;
+  double v2 = 0.0, cnt = 0.0;
+  for (int64_t n = (int64_t)blockIdx.x * NTHREADS + threadIdx.x; n < nn; n += (int64_t)gridDim.x * NTHREADS) {
+    if (!(fabs(phi[n]) <= 0.9)) continue;
+    const unsigned row = (unsigned)n / (unsigned)(nx + 1);
+    const int i = (int)((unsigned)n - row * (unsigned)(nx + 1)), k = (int)(row / (unsigned)(ny + 1));
+    const int j = (int)(row - (unsigned)k * (unsigned)(ny + 1));
+    double s = 0.0, elems = 0.0;
+    for (int az = 1; az >= 0; --az)
+      for (int ay = 1; ay >= 0; --ay)
+        for (int ax = 1; ax >= 0; --ax) {
+          const int ex = i - ax, ey = j - ay, ez = k - az;
+          if (ex < 0 || ex >= nx || ey < 0 || ey >= ny || ez < 0 || ez >= nz) continue;
+          s += E[(ax + 2 * ay + 4 * az) * es + (int64_t)ez * nxyp + (int64_t)ey * nxp + ex];
+          elems += 1.0;
+        }
+    const double v = fabs(s / elems);
+    v2 += v * v;
+    cnt += 1.0;
+  }
+  const double a = block_sum(v2, scratch);
+  const double b = block_sum(cnt, scratch);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = a;
+    part[2 * blockIdx.x + 1] = b;
+  }
+}
+
+// out = {gamma, beta} from the partials of ne element and nn node CTAs, summed in a fixed order
+__global__ void __launch_bounds__(NTHREADS) hq_coef_final_kernel(const double* __restrict__ pe, int ne,
+                                                                 const double* __restrict__ pn, int nn, double eta,
+                                                                 double* __restrict__ out) {
+  __shared__ double scratch[NTHREADS / 32];
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = threadIdx.x; i < nn; i += NTHREADS) {
+    a[0] += pn[2 * i];
+    a[1] += pn[2 * i + 1];
+  }
+  for (int i = threadIdx.x; i < ne; i += NTHREADS) {
+    a[2] += pe[2 * i];
+    a[3] += pe[2 * i + 1];
+  }
+  double s[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) s[c] = block_sum(a[c], scratch);
+  if (threadIdx.x == 0) {
+    out[0] = s[1] > 0.0 ? sqrt(s[0] / s[1]) / eta : 0.0;
+    out[1] = s[3] != 0.0 ? s[2] / s[3] : 0.0;
+  }
+}
+
+int op_coeffs(fsi_mesh* m, int phase, double* gb) {
+  if (m->tet) return tet_coeffs(m, phase, gb);
+  const Geom& g = m->g;
+  const int nxp = cq_pitch(m);
+  const int64_t nxyp = (int64_t)nxp * g.ny;
+  const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
+  if (int rc = ensure_elem_scratch(m, 8, nxyp)) return rc;
+  const int ge = (int)std::min<unsigned>(hq_blocks(ne), 152 * 8), gn = (int)std::min<int64_t>((m->nn + NTHREADS - 1) / NTHREADS, 152 * 4);
+  if (m->n_partials < ge + gn) {
+    cudaFree(m->partials);
+    m->partials = nullptr;
+    m->n_partials = 0;
+    FSI_CUDA(cudaMalloc(&m->partials, sizeof(double) * 4 * (ge + gn)));
+    m->n_partials = ge + gn;
+  }
+  double* pn = m->partials + 2 * ge;
+  const double* phi = m->staged_xa + (int64_t)(4 + phase) * m->nn;
+  FSI_LAUNCH(m, P_COEF, hq_coef_kernel<<<ge, HQ_THREADS, 0, m->stream>>>(hex_ns(m, nxp), phase, m->ke_e, m->partials, ne));
+  FSI_LAUNCH(m, P_COEF, hq_coef_node_kernel<<<gn, NTHREADS, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, phi, pn));
+  FSI_LAUNCH(m, P_COEF, hq_coef_final_kernel<<<1, NTHREADS, 0, m->stream>>>(m->partials, ge, pn, gn, m->P.eta, m->red));
+  FSI_CUDA(cudaMemcpyAsync(m->red_host, m->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+  FSI_CUDA(cudaStreamSynchronize(m->stream));
+  gb[0] = m->red_host[0];
+  gb[1] = m->red_host[1];
+  return FSI_OK;
+}
+
 }  // namespace fsi

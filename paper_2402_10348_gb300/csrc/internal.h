@@ -249,8 +249,6 @@ int vec_recip(fsi_mesh* m, const double* a, double* y, int64_t n);              
 int gmres_solve(fsi_mesh* m, const BlockInfo& b, const double* rhs, double* x, const fsi_solve_opts& o,
                 fsi_solve_info* info);
 
-// tile launch geometry
-void tile_grid(const fsi_mesh* m, dim3* grid);
 
 // linear tetrahedra (tet.cu): residual (mode 0), product (1), diagonal (2) of each block
 int tet_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags);

@@ -40,37 +40,4 @@ __global__ void coef_finalize(const double* partials, int64_t n, double eta, dou
   }
 }
 
-int op_coeffs(fsi_mesh* m, int i, double* gb) {
-  static_assert(CoefOp::MINB == 1, "the partial sums are sized for the mesh's own tile grid");
-  if (m->tet) return tet_coeffs(m, i, gb);
-  CoefOp op;
-  memset(&op, 0, sizeof(op));
-  const int64_t nn = m->nn;
-  for (int k = 0; k < 3; ++k) { op.F.d[k] = m->staged_xa + k * nn; op.F.f[k] = nullptr; }
-  op.F.d[3] = m->staged_xa + (4 + i) * nn;
-  op.nf = 4;
-  fill_common(m, op.rh, &op.W);
-  op.phi_node = m->staged_xa + (4 + i) * nn;
-  dim3 grid;
-  tile_grid(m, &grid);
-  op.ncta_xy[0] = grid.x;
-  op.ncta_xy[1] = grid.y;
-  const int64_t ncta = (int64_t)grid.x * grid.y * grid.z;
-  if (m->n_partials < ncta) {
-    if (m->partials) cudaFree(m->partials);
-    m->partials = nullptr;
-    FSI_CUDA(cudaMalloc(&m->partials, sizeof(double) * 4 * ncta));
-    m->n_partials = ncta;
-  }
-  op.partials = m->partials;
-  int rc = run_tile(m, op, P_COEF);
-  if (rc) return rc;
-  FSI_LAUNCH(m, P_COEF, coef_finalize<<<1, NTHREADS, 0, m->stream>>>(m->partials, ncta, m->P.eta, m->red));
-  FSI_CUDA(cudaMemcpyAsync(m->red_host, m->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-  FSI_CUDA(cudaStreamSynchronize(m->stream));
-  gb[0] = m->red_host[0];
-  gb[1] = m->red_host[1];
-  return FSI_OK;
-}
-
 }  // namespace fsi
