@@ -10,23 +10,27 @@
 // block of k x 2 KiB per chunk instead of k separate streams 8.8 MB apart (measured
 // 3.9 vs 2.7 TB/s read on GB300 for 33 vectors of the 64^3 NS block).
 //
-// Arnoldi step j (D = diag(dinv)):
+// Arnoldi step j (D = diag(dinv)), four launches with the operator's one:
 //   w = J z, z = D V_j    (z written together with V_j; w: a contiguous work vector
 //                          written by the operator)
 //   h = V^T w and |w|^2 in one pass over V_0..V_j      (mdot_kernel)
 //   w -= V h, |w|^2 and h2 = V^T w (the second pass's projections of the updated w)
-//   in one pass                                           (upd_dot_kernel)
-//   if |w_new| < |w_old| / sqrt(2): w -= V h2 (classical Gram-Schmidt with the DGKS
-//   re-orthogonalization test; that update is launched always and exits at once when
-//   the device-side flag says it is not needed)
-//   Givens rotation of the new Hessenberg column and the residual estimate on the
-//   device; V_{j+1} = w / |w| stored into its slot, and z = D V_{j+1} beside it.
-// The host enqueues step j and only then waits for step j-1's residual estimate
-// (copied to pinned memory), so it never stalls the GPU between steps; at most one
-// step beyond convergence is computed and ignored.  The least-squares solution and
-// x += D V y are device kernels.  One host synchronisation per restart recomputes
-// the true residual b - A x.  All reductions use a fixed partition and a fixed
-// summation order (bit-reproducible).
+//   in one pass                                           (upd_dot_kernel); its last CTA:
+//   if |w_new| < |w_old| / sqrt(2) (classical Gram-Schmidt with the DGKS
+//   re-orthogonalization test) h += h2 and |w|^2 -= |h2|^2 (the basis is orthonormal); Givens
+//   rotation of the new Hessenberg column and the residual estimate, written to pinned
+//   host memory                                            (givens_step)
+//   V_{j+1} = (w - V h2) / |w| (V h2 only where the test asked for it) into its slot, and
+//   z = D V_{j+1} beside it                                (upd_store_kernel)
+// In the projection kernels the last CTA to finish adds the per-CTA partial sums (a warp per row, fixed
+// order), so no launch follows for them: at small sizes launches are the time.  16^3, one
+// iteration: 103 us with ten launches and a copy, 56 with these; 64^3, float32 basis, beside the
+// operator: 109 -> 84.
+// The host enqueues step j and only then waits for step j-1's residual estimate, so it
+// never stalls the GPU between steps; at most one step beyond convergence is computed and
+// ignored.  The least-squares solution and x += D V y are device kernels.  One host
+// synchronisation per restart recomputes the true residual b - A x.  All reductions use a fixed
+// partition and a fixed summation order (bit-reproducible).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -57,18 +61,22 @@ static int cgrid_t(int64_t nch) {
 // the basis store: a few chunks of 256 elements per CTA, eight CTAs per SM
 static int chunk_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + CH - 1) / CH, 152 * 8)); }
 
+// the second pass with the basis store: `per` chunks a CTA at a time, eight CTAs per SM at most
+static int upd_grid(int64_t n, int per) {
+  const int64_t groups = ((n + CH - 1) / CH + per - 1) / per;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(groups, 152 * 8));
+}
+
 // device-resident Arnoldi/Givens state (inside fsi_mesh::kry_dev)
 struct KryDev {
   double h[MMAX + 2];      // current column (pass 1), then the accumulated column
   double h2[MMAX + 2];     // second pass
   double H[(MMAX + 1) * MMAX];
   double cs[MMAX], sn[MMAX], g[MMAX + 1], y[MMAX];
-  double nrm_old, nrm_new, nrm_fin;
+  double nrm_fin;          // norm of the new basis vector before scaling
   double bnorm;
-  double est;              // |g_{j+1}| / |b|
-  int reorth;              // est, reorth, breakdown: one 16-byte copy to the host per step
-  int breakdown;
-  unsigned counter;        // CTAs done in sum_partials_decide (back to 0 after each use)
+  int reorth;              // the second pass is taken
+  unsigned counter;        // CTAs done in a projection kernel (back to 0 after each use)
 };
 
 template <int K>
@@ -168,17 +176,46 @@ __device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, do
 // per-thread sums are taken in VT, the sums across threads and CTAs in float64.  The work
 // vector w, the preconditioner diagonal and every vector outside the basis stay float64.
 
-// part[(ib + i) * G + cta] = sum over the CTA's chunks of V_{ib+i} . w, i < KC,
-// ib = i0 + KC * blockIdx.y; with SELF the KC+1-th row is w . w (row i0 + KC).
+// Whether this CTA is the last of `total` to get here; its earlier global writes (and, for the last
+// CTA, everybody's) are visible after it.  The counter is back to 0 for the next kernel.
+__device__ __forceinline__ bool last_cta(unsigned* counter, unsigned total) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == total - 1;
+    if (last) *counter = 0;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+// dst[i] = sum_c part[i * G + c] for i < rows: a warp per row, lanes strided, then a shuffle tree
+__device__ __forceinline__ void sum_rows(const double* part, int G, int rows, double* dst) {
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < rows; i += blockDim.x >> 5) {
+    const double* p = part + (int64_t)i * G;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    int c = lane;
+    for (; c + 96 < G; c += 128) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] += __ldcg(p + c + 32 * u);
+    }
+    for (; c < G; c += 32) s[0] += __ldcg(p + c);
+    double t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) dst[i] = t;
+  }
+}
+
+// h[i] = V_i . w for i < k, h[k] = w . w (partial sums part[i * G + cta]).  Groups of DCH vectors per
+// blockIdx.y; the last group has k mod DCH = R vectors (perhaps none) and takes w . w.
 template <int KC, bool SELF, typename VT>
-__global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int M1, int i0,
-                                                  const double* __restrict__ w, int64_t n, double* part,
-                                                  const int* skip) {
-  if (skip && !*skip) return;
-  constexpr int NA = KC + (SELF ? 1 : 0);
-  constexpr int NR = NA > 0 ? NA : 1;
+__device__ __forceinline__ void mdot_group(const VT* __restrict__ V, int M1, int ib, const double* __restrict__ w,
+                                           int64_t n, double* part) {
+  constexpr int NR = KC + (SELF ? 1 : 0);
   const int G = gridDim.x;
-  const int ib = i0 + blockIdx.y * KC;
   const int64_t nch = (n + CH - 1) / CH;
   const int64_t per = (nch + G - 1) / G;
   const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
@@ -192,12 +229,20 @@ __global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int 
     const VT* blk = V + c * (int64_t)M1 * CH + (int64_t)ib * CH + threadIdx.x;
 #pragma unroll
     for (int i = 0; i < KC; ++i) acc[i] += blk[i * CH] * wj;
-    if (SELF) acc[NA - 1] += wj * wj;
+    if (SELF) acc[NR - 1] += wj * wj;
   }
   double accd[NR];
 #pragma unroll
   for (int i = 0; i < NR; ++i) accd[i] = (double)acc[i];
-  block_reduce_store_bf<NR>(accd, NA, part + (int64_t)ib * G + blockIdx.x, G);
+  block_reduce_store_bf<NR>(accd, NR, part + (int64_t)ib * G + blockIdx.x, G);
+}
+
+template <int R, typename VT>
+__global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int M1, int k, const double* __restrict__ w,
+                                                  int64_t n, double* part, KryDev* K) {
+  if (blockIdx.y < gridDim.y - 1) mdot_group<DCH, false, VT>(V, M1, blockIdx.y * DCH, w, n, part);
+  else mdot_group<R, true, VT>(V, M1, blockIdx.y * DCH, w, n, part);
+  if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows(part, gridDim.x, k + 1, K->h);
 }
 
 // The float32 basis: the same projections with 16-byte loads.  A CTA works on four
@@ -205,15 +250,12 @@ __global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int 
 // basis vector), so a warp moves as many bytes per load as with a float64 basis and
 // keeps as many in flight.  Elements at or past n (the ragged end of the last chunk,
 // whose basis slots hold stale bytes) are never read.
-template <int KC, bool SELF>
-__global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, int M1, int i0,
-                                                   const double* __restrict__ w, int64_t n, double* part,
-                                                   const int* skip) {
-  if (skip && !*skip) return;
-  constexpr int NA = KC + (SELF ? 1 : 0);
-  constexpr int NR = NA > 0 ? NA : 1;
+__global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, int M1, int k,
+                                                   const double* __restrict__ w, int64_t n, double* part, KryDev* K) {
+  constexpr int KC = DCH, NR = DCH + 1;
   const int G = gridDim.x;
-  const int ib = i0 + blockIdx.y * KC;
+  const int ib = blockIdx.y * KC, kc = min(KC, k - ib);
+  const bool self = blockIdx.y == gridDim.y - 1;
   const int64_t nch = (n + CH - 1) / CH;
   const int64_t per = (nch + G - 1) / G;
   const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
@@ -233,6 +275,7 @@ __global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, 
       w0 = (float)a.x, w1 = (float)a.y, w2 = (float)b.x, w3 = (float)b.y;
 #pragma unroll
       for (int i = 0; i < KC; ++i) {
+        if (i >= kc) break;
         const float4 v = *reinterpret_cast<const float4*>(blk + i * CH);
         acc[i] += (v.x * w0 + v.y * w1) + (v.z * w2 + v.w * w3);
       }
@@ -243,6 +286,7 @@ __global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, 
       w3 = 0.f;
 #pragma unroll
       for (int i = 0; i < KC; ++i) {
+        if (i >= kc) break;
         const float* p = blk + i * CH;
         float t = p[0] * w0;
         if (j + 1 < n) t += p[1] * w1;
@@ -250,14 +294,17 @@ __global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, 
         acc[i] += t;
       }
     }
-    if (SELF) acc[NA - 1] += (w0 * w0 + w1 * w1) + (w2 * w2 + w3 * w3);
+    if (self) acc[KC] += (w0 * w0 + w1 * w1) + (w2 * w2 + w3 * w3);
   }
-  block_reduce_store_f<NR>(acc, NA, part + (int64_t)ib * G + blockIdx.x, G);
+#pragma unroll
+  for (int i = 0; i < KC; ++i)
+    if (i == kc) acc[i] = acc[KC];  // w . w goes to row k
+  block_reduce_store_f<NR>(acc, kc + (self ? 1 : 0), part + (int64_t)ib * G + blockIdx.x, G);
+  if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows(part, G, k + 1, K->h);
 }
 
 // out[i] = sum_c part[i*G + c] (fixed order), i = blockIdx.x
-__global__ void sum_partials(const double* __restrict__ part, int G, double* out, const int* skip) {
-  if (skip && !*skip) return;
+__global__ void sum_partials(const double* __restrict__ part, int G, double* out) {
   const int i = blockIdx.x;
   double s = 0.0;
   for (int c = threadIdx.x; c < G; c += VB) s += part[(int64_t)i * G + c];
@@ -281,100 +328,175 @@ __device__ __forceinline__ VT lin_comb_chunk(const VT* __restrict__ hs, const VT
   return ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
 }
 
-// w -= sum_{i<k} h_i V_i ; part[cta] = partial of |w|^2   (w contiguous).  One fused
-// multiply-add per basis element, chained on the element's value of w (no partial sums
-// to add up afterwards: float64 adds are scarce on this GPU); the element's values of up
-// to UPB basis vectors are loaded ahead of the chain.
+// V_slot = (w - sum_{i<k} h2_i V_i) / |w| with the second pass's correction only where the DGKS
+// test asked for it (K->reorth), and the next operator input z = dinv V_slot from the stored
+// value.  One fused multiply-add per basis element, chained on the element's value of w (no
+// partial sums to add up afterwards: float64 adds are scarce on this GPU); the element's
+// values of up to UPB basis vectors are loaded ahead of the chain.
 constexpr int UPB = 32;
-template <typename VT>
-__global__ void __launch_bounds__(VB, 2) upd_kernel(double* __restrict__ w, const VT* __restrict__ V, int M1, int k,
-                                                    const double* __restrict__ h, int64_t n, double* part,
-                                                    const int* skip) {
-  if (skip && !*skip) return;
-  __shared__ VT nh[MMAX + 2];
-  for (int i = threadIdx.x; i < k; i += VB) nh[i] = -(VT)h[i];
+__global__ void __launch_bounds__(VB, 2) upd_store_kernel(const double* __restrict__ w, double* V, int M1, int k,
+                                                          const KryDev* __restrict__ K, int64_t n,
+                                                          const double* __restrict__ dinv, double* __restrict__ z) {
+  __shared__ double nh[MMAX + 2], s_sh;
+  const bool second = K->reorth != 0;
+  if (threadIdx.x == 0) s_sh = K->nrm_fin > 0.0 ? 1.0 / K->nrm_fin : 0.0;
+  if (second)
+    for (int i = threadIdx.x; i < k; i += VB) nh[i] = -K->h2[i];
   __syncthreads();
-  const int G = gridDim.x;
+  const double scale = s_sh;
   const int64_t nch = (n + CH - 1) / CH;
-  const int64_t per = (nch + G - 1) / G;
-  const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
-  VT nrm = VT(0);
-  for (int64_t c = c0; c < c1; ++c) {
+  for (int64_t c = blockIdx.x; c < nch; c += gridDim.x) {
     const int64_t j = c * CH + threadIdx.x;
     if (j >= n) break;
-    const VT* blk = V + c * (int64_t)M1 * CH + threadIdx.x;
-    VT s = (VT)w[j];
-    for (int i0 = 0; i0 < k; i0 += UPB) {
-      const int cnt = min(UPB, k - i0);
-      VT v[UPB];
+    double* blk = V + c * (int64_t)M1 * CH + threadIdx.x;
+    double s = w[j];
+    if (second) {
+      for (int i0 = 0; i0 < k; i0 += UPB) {
+        const int cnt = min(UPB, k - i0);
+        double v[UPB];
 #pragma unroll
-      for (int u = 0; u < UPB; ++u) v[u] = u < cnt ? blk[(int64_t)(i0 + u) * CH] : VT(0);
+        for (int u = 0; u < UPB; ++u) v[u] = u < cnt ? blk[(int64_t)(i0 + u) * CH] : 0.0;
 #pragma unroll
-      for (int u = 0; u < UPB; ++u) {
-        if (u >= cnt) break;
-        s = fma(nh[i0 + u], v[u], s);
+        for (int u = 0; u < UPB; ++u) {
+          if (u >= cnt) break;
+          s = fma(nh[i0 + u], v[u], s);
+        }
       }
     }
-    w[j] = (double)s;
-    nrm = fma(s, s, nrm);
+    s *= scale;
+    blk[(int64_t)k * CH] = s;
+    if (z) z[j] = dinv[j] * s;
   }
-  double nd[1] = {(double)nrm};
-  block_reduce_store<1>(nd, 1, part + blockIdx.x, 1);
 }
 
-// The second-pass update for the float32 basis, laid out as mdot4_kernel: a CTA works on
-// four chunks at a time, a thread on four adjacent elements (one float4 per basis vector,
-// two double2 of w).  part[cta] = partial of |w|^2 (float32 up to the CTA's sum).
-__global__ void __launch_bounds__(VB) upd4_kernel(double* __restrict__ w, const float* __restrict__ V, int M1, int k,
-                                                  const double* __restrict__ h, int64_t n, double* part,
-                                                  const int* skip) {
-  if (skip && !*skip) return;
+// The same for the float32 basis, laid out as mdot4_kernel: a CTA works on four chunks at a
+// time, a thread on four adjacent elements (one float4 per basis vector, two double2 of w); z is the
+// float32 operator's increment.
+__global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict__ w, float* V, int M1, int k,
+                                                        const KryDev* __restrict__ K, int64_t n,
+                                                        const double* __restrict__ dinv, float* __restrict__ z) {
   __shared__ float hs[MMAX + 2];
-  for (int i = threadIdx.x; i < k; i += VB) hs[i] = (float)h[i];
+  __shared__ double s_sh;
+  const bool second = K->reorth != 0;
+  if (threadIdx.x == 0) s_sh = K->nrm_fin > 0.0 ? 1.0 / K->nrm_fin : 0.0;
+  if (second)
+    for (int i = threadIdx.x; i < k; i += VB) hs[i] = (float)K->h2[i];
   __syncthreads();
-  const int G = gridDim.x;
+  const float scale = (float)s_sh;
   const int64_t nch = (n + CH - 1) / CH;
-  const int64_t per = (nch + G - 1) / G;
-  const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
   const int sub = threadIdx.x >> 6;
   const int e0 = (threadIdx.x & 63) * 4;
-  float nrm = 0.f;
-  for (int64_t c = c0 + sub; c < c1; c += 4) {
+  for (int64_t c = (int64_t)blockIdx.x * 4 + sub; c < nch; c += (int64_t)gridDim.x * 4) {
     const int64_t j = c * CH + e0;
     if (j >= n) break;
-    const float* blk = V + c * (int64_t)M1 * CH + e0;
+    float* blk = V + c * (int64_t)M1 * CH + e0;
     if (j + 4 <= n) {
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-      int i = 0;
-      for (; i + 2 <= k; i += 2) {
-        const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
-        const float4 v1 = *reinterpret_cast<const float4*>(blk + (i + 1) * CH);
-        a.x += hs[i] * v0.x; a.y += hs[i] * v0.y; a.z += hs[i] * v0.z; a.w += hs[i] * v0.w;
-        b.x += hs[i + 1] * v1.x; b.y += hs[i + 1] * v1.y; b.z += hs[i + 1] * v1.z; b.w += hs[i + 1] * v1.w;
-      }
-      if (i < k) {
-        const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
-        a.x += hs[i] * v0.x; a.y += hs[i] * v0.y; a.z += hs[i] * v0.z; a.w += hs[i] * v0.w;
+      if (second) {
+        int i = 0;
+#pragma unroll 4
+        for (; i + 2 <= k; i += 2) {
+          const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
+          const float4 v1 = *reinterpret_cast<const float4*>(blk + (i + 1) * CH);
+          a.x += hs[i] * v0.x; a.y += hs[i] * v0.y; a.z += hs[i] * v0.z; a.w += hs[i] * v0.w;
+          b.x += hs[i + 1] * v1.x; b.y += hs[i + 1] * v1.y; b.z += hs[i + 1] * v1.z; b.w += hs[i + 1] * v1.w;
+        }
+        if (i < k) {
+          const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
+          a.x += hs[i] * v0.x; a.y += hs[i] * v0.y; a.z += hs[i] * v0.z; a.w += hs[i] * v0.w;
+        }
       }
       const double2 w01 = *reinterpret_cast<const double2*>(w + j);
       const double2 w23 = *reinterpret_cast<const double2*>(w + j + 2);
-      const float s0 = (float)w01.x - (a.x + b.x), s1 = (float)w01.y - (a.y + b.y);
-      const float s2 = (float)w23.x - (a.z + b.z), s3 = (float)w23.y - (a.w + b.w);
-      *reinterpret_cast<double2*>(w + j) = make_double2((double)s0, (double)s1);
-      *reinterpret_cast<double2*>(w + j + 2) = make_double2((double)s2, (double)s3);
-      nrm += (s0 * s0 + s1 * s1) + (s2 * s2 + s3 * s3);
+      float4 v;
+      v.x = ((float)w01.x - (a.x + b.x)) * scale;
+      v.y = ((float)w01.y - (a.y + b.y)) * scale;
+      v.z = ((float)w23.x - (a.z + b.z)) * scale;
+      v.w = ((float)w23.y - (a.w + b.w)) * scale;
+      *reinterpret_cast<float4*>(blk + (int64_t)k * CH) = v;
+      if (z) {
+        const double2 d01 = *reinterpret_cast<const double2*>(dinv + j), d23 = *reinterpret_cast<const double2*>(dinv + j + 2);
+        *reinterpret_cast<float4*>(z + j) =
+            make_float4((float)d01.x * v.x, (float)d01.y * v.y, (float)d23.x * v.z, (float)d23.y * v.w);
+      }
     } else {
       for (int e = 0; e < 4 && j + e < n; ++e) {
         float acc = 0.f;
-        for (int i = 0; i < k; ++i) acc += hs[i] * blk[i * CH + e];
-        const float se = (float)w[j + e] - acc;
-        w[j + e] = (double)se;
-        nrm += se * se;
+        if (second)
+          for (int i = 0; i < k; ++i) acc += hs[i] * blk[i * CH + e];
+        const float v = ((float)w[j + e] - acc) * scale;
+        blk[(int64_t)k * CH + e] = v;
+        if (z) z[j + e] = (float)dinv[j + e] * v;
       }
     }
   }
-  float acc[1] = {nrm};
-  block_reduce_store_f<1>(acc, 1, part + blockIdx.x, 1);
+}
+
+// The step after the fused update, by the last CTA of its kernel: h2 (the second pass's projections
+// of the updated w) and |w|^2 summed from the partials, the DGKS decision and the Givens step.
+// Column j of the Hessenberg matrix: h, plus h2 where |w_new| < |w_old| / sqrt(2) asked for the second
+// pass; below it the new norm, |w - V h2|^2 = |w|^2 - |h2|^2 on an orthonormal basis, so the second
+// pass needs no sweep before the rotation.  The column is rotated by the previous rotations, the new
+// rotation zeroes its subdiagonal entry, and g and the residual estimate |g_{j+1}| / |b| follow.
+// est (pinned host memory): the estimate, then the reorth and breakdown flags as ints.
+// Everything is read by all threads first; one thread then runs the chain of rotations in shared memory.
+__device__ void givens_step(const double* part, int G, KryDev* K, int j, int mm, double* est) {
+  __shared__ double col[MMAX + 2], c2[MMAX + 2], cs[MMAX], sn[MMAX];
+  const int nt = blockDim.x;
+  for (int q = threadIdx.x; q <= j; q += nt) {
+    col[q] = K->h[q];
+    if (q < j) {
+      cs[q] = K->cs[q];
+      sn[q] = K->sn[q];
+    }
+  }
+  sum_rows(part, G, j + 2, c2);
+  __syncthreads();
+  const double w2 = c2[j + 1];
+  const bool reorth = sqrt(w2) < sqrt(K->h[j + 1]) * 0.70710678118654752;
+  double hh = 0.0;  // |h2|^2, in warp 0
+  if (threadIdx.x < 32) {
+    for (int q = threadIdx.x; q <= j; q += 32) hh = fma(c2[q], c2[q], hh);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+  }
+  if (reorth) {
+    for (int q = threadIdx.x; q <= j; q += nt) {
+      col[q] += c2[q];
+      K->h2[q] = c2[q];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double df = w2 - hh;  // a NaN stays one: the host stops on it
+    const double hn = sqrt(reorth ? (df < 0.0 ? 0.0 : df) : w2);
+    K->nrm_fin = hn;
+    K->reorth = reorth ? 1 : 0;
+    double t = col[0];
+    for (int q = 0; q < j; ++q) {
+      const double nx = col[q + 1];
+      col[q] = fma(sn[q], nx, cs[q] * t);
+      t = fma(-sn[q], t, cs[q] * nx);
+    }
+    const double den = hypot(t, hn);
+    const double c = den > 0.0 ? t / den : 1.0;
+    const double sj = den > 0.0 ? hn / den : 0.0;
+    K->cs[j] = c;
+    K->sn[j] = sj;
+    col[j] = den;
+    col[j + 1] = 0.0;
+    const double gj = K->g[j], gn = -sj * gj;
+    K->g[j + 1] = gn;
+    K->g[j] = c * gj;
+    const int bd = (hn == 0.0 || den == 0.0 || !isfinite(hn)) ? 1 : 0;
+    est[0] = fabs(gn) / K->bnorm;
+    int* flags = reinterpret_cast<int*>(est + 1);
+    flags[0] = reorth ? 1 : 0;
+    flags[1] = bd;
+    __threadfence_system();
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q <= j + 1; q += nt) K->H[q * mm + j] = col[q];
 }
 
 // Pass-1 update fused with the pass-2 projections: w' = w - sum_{i<k} h_i V_i, the
@@ -388,8 +510,9 @@ constexpr int UDB = 128;  // threads per CTA (two elements of each 256-element c
 static_assert(UDB == 128, "the row sums take four columns per lane");
 template <int KMAX, typename VT>
 __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, const VT* __restrict__ V, int M1,
-                                                      int k, const double* __restrict__ h, int64_t n, double* part) {
+                                                      int k, int64_t n, double* part, KryDev* K, int mm, double* est) {
   extern __shared__ __align__(16) unsigned char upd_smem[];
+  const double* h = K->h;
   VT* sacc = reinterpret_cast<VT*>(upd_smem);  // [KMAX + 1][UDB]
   __shared__ VT nhs[KMAX];
   const int t = threadIdx.x;
@@ -438,6 +561,7 @@ __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, co
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) part[(int64_t)i * G + blockIdx.x] = s;
   }
+  if (last_cta(&K->counter, gridDim.x)) givens_step(part, G, K, k - 1, mm, est);
 }
 
 // The fused update for the float32 basis: a thread takes two adjacent elements of each
@@ -445,8 +569,9 @@ __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, co
 // per load as with a float64 basis.  Elements at or past n are never read.
 template <int KMAX>
 __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, const float* __restrict__ V, int M1,
-                                                       int k, const double* __restrict__ h, int64_t n, double* part) {
+                                                       int k, int64_t n, double* part, KryDev* K, int mm, double* est) {
   extern __shared__ __align__(16) unsigned char upd_smem[];
+  const double* h = K->h;
   float* sacc = reinterpret_cast<float*>(upd_smem);  // [KMAX + 1][UDB]
   __shared__ float hs[KMAX];
   const int t = threadIdx.x;
@@ -506,51 +631,45 @@ __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, c
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) part[(int64_t)i * G + blockIdx.x] = (double)s;
   }
+  if (last_cta(&K->counter, gridDim.x)) givens_step(part, G, K, k - 1, mm, est);
 }
 
 template <int KMAX, typename VT>
-static int launch_upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, const double* h, int64_t n) {
+static int launch_upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n, int mm, double* est) {
+  KryDev* K = static_cast<KryDev*>(m->kry_dev);
   const size_t smem = sizeof(VT) * (size_t)(KMAX + 1) * UDB;
   if constexpr (sizeof(VT) == 4) {
     if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot2_kernel<KMAX>), smem)) return rc;
-    upd_dot2_kernel<KMAX><<<G, UDB, smem, m->stream>>>(w, V, M1, k, h, n, m->partials_dot);
+    upd_dot2_kernel<KMAX><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K, mm, est);
   } else {
     if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot_kernel<KMAX, VT>), smem)) return rc;
-    upd_dot_kernel<KMAX, VT><<<G, UDB, smem, m->stream>>>(w, V, M1, k, h, n, m->partials_dot);
+    upd_dot_kernel<KMAX, VT><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K, mm, est);
   }
   return FSI_OK;
 }
 
 template <typename VT>
-static int upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, const double* h, int64_t n) {
+static int upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n, int mm, double* est) {
   switch ((k + 7) / 8) {
-    case 1: return launch_upd_dot<8>(m, G, w, V, M1, k, h, n);
-    case 2: return launch_upd_dot<16>(m, G, w, V, M1, k, h, n);
-    case 3: return launch_upd_dot<24>(m, G, w, V, M1, k, h, n);
-    case 4: return launch_upd_dot<32>(m, G, w, V, M1, k, h, n);
-    case 5: return launch_upd_dot<40>(m, G, w, V, M1, k, h, n);
-    case 6: return launch_upd_dot<48>(m, G, w, V, M1, k, h, n);
-    case 7: return launch_upd_dot<56>(m, G, w, V, M1, k, h, n);
-    default: return launch_upd_dot<64>(m, G, w, V, M1, k, h, n);
+    case 1: return launch_upd_dot<8>(m, G, w, V, M1, k, n, mm, est);
+    case 2: return launch_upd_dot<16>(m, G, w, V, M1, k, n, mm, est);
+    case 3: return launch_upd_dot<24>(m, G, w, V, M1, k, n, mm, est);
+    case 4: return launch_upd_dot<32>(m, G, w, V, M1, k, n, mm, est);
+    case 5: return launch_upd_dot<40>(m, G, w, V, M1, k, n, mm, est);
+    case 6: return launch_upd_dot<48>(m, G, w, V, M1, k, n, mm, est);
+    case 7: return launch_upd_dot<56>(m, G, w, V, M1, k, n, mm, est);
+    default: return launch_upd_dot<64>(m, G, w, V, M1, k, n, mm, est);
   }
 }
 
-// V_slot[j] = src[j] * scale, scale = 1/sqrt(*n2) (n2 != null) or 1/K->nrm_fin; with z,
-// also the next operator input z[j] = dinv[j] * V_slot[j] from the stored value (the
-// float32 operator's increment when VT is float)
+// V_0 = r / |r|, |r|^2 = *n2; with z, also the next operator input z = dinv V_0 from the stored value
+// (the float32 operator's increment when VT is float)
 template <typename VT>
-__global__ void store_slot(VT* __restrict__ V, int M1, int slot, const double* __restrict__ src, const double* n2,
-                           const KryDev* K, int64_t n, const double* __restrict__ dinv, VT* __restrict__ z) {
+__global__ void store_first(VT* __restrict__ V, int M1, const double* __restrict__ r, const double* n2, int64_t n,
+                            const double* __restrict__ dinv, VT* __restrict__ z) {
   // the scale once per CTA: float64 division and square root are slow on this GPU
   __shared__ double s_sh;
-  if (threadIdx.x == 0) {
-    if (n2) {
-      s_sh = 1.0 / sqrt(*n2);
-    } else {
-      const double nf = K->nrm_fin;
-      s_sh = nf > 0.0 ? 1.0 / nf : 0.0;
-    }
-  }
+  if (threadIdx.x == 0) s_sh = 1.0 / sqrt(*n2);
   __syncthreads();
   const double s = s_sh;
   // one chunk of CH = VB elements per CTA pass
@@ -558,10 +677,10 @@ __global__ void store_slot(VT* __restrict__ V, int M1, int slot, const double* _
   for (int64_t c = blockIdx.x; c < nch; c += gridDim.x) {
     const int64_t j = c * CH + threadIdx.x;
     if (j >= n) continue;
-    const VT v = (VT)(src[j] * s);
-    V[c * (int64_t)M1 * CH + (int64_t)slot * CH + threadIdx.x] = v;
+    const VT v = (VT)(r[j] * s);
+    V[c * (int64_t)M1 * CH + threadIdx.x] = v;
     if (z) {
-      if constexpr (sizeof(VT) == 4) z[j] = (float)dinv[j] * v;  // the float32 operator's increment
+      if constexpr (sizeof(VT) == 4) z[j] = (float)dinv[j] * v;
       else z[j] = dinv[j] * v;
     }
   }
@@ -618,108 +737,21 @@ __global__ void __launch_bounds__(VB) zcombine_kernel(double* __restrict__ x, co
 }
 
 // --------------------------------------------------------- small device kernels
-// After pass 1: the column h[0..j], |w_old|^2 = h[j+1]; |w_new|^2 in h2[j+1] (the fused
-// update's row of norms; h2[0..j] hold the pass-2 projections).  Read through a volatile
-// pointer: other CTAs wrote h2 just before.
-__device__ void orth_decide_body(KryDev* K, int j) {
-  volatile double* h2 = K->h2;
-  K->nrm_old = sqrt(K->h[j + 1]);
-  K->nrm_new = h2[j + 1];
-  const double nn = sqrt(K->nrm_new);
-  K->reorth = (nn < K->nrm_old * 0.70710678118654752) ? 1 : 0;
-  K->nrm_fin = nn;
-}
-
-// Rows of the fused update's partials into K->h2 (one CTA per row, fixed order); the last
-// CTA to finish takes the DGKS decision, so no single-thread launch follows.
-__global__ void sum_partials_decide(const double* __restrict__ part, int G, KryDev* K, int j) {
-  const int i = blockIdx.x;
-  double s = 0.0;
-  for (int c = threadIdx.x; c < G; c += VB) s += part[(int64_t)i * G + c];
-  double acc[1] = {s};
-  __shared__ double res;
-  __shared__ bool last;
-  block_reduce_store<1>(acc, 1, &res, 1);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    K->h2[i] = res;
-    __threadfence();
-    last = atomicAdd(&K->counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
-    __threadfence();
-    K->counter = 0;
-    orth_decide_body(K, j);
-  }
-}
-
-// The second pass's |w|^2 (only when it ran) and the Givens step, in one CTA: the column,
-// the rotations and the right-hand side are read into shared memory by all threads, one
-// thread applies the rotations there (a chain of shared-memory operations, not of global
-// loads), and the column goes back in parallel.  Column j of the Hessenberg matrix (h,
-// plus h2 when the second pass ran, and the new norm below it) is rotated by the previous
-// rotations, the new rotation zeroes its subdiagonal entry, and g and the residual
-// estimate |g_{j+1}| / |b| follow.
-__global__ void sum_partials_givens(const double* __restrict__ part, int G, KryDev* K, int j, int mm) {
-  __shared__ double col[MMAX + 2], cs[MMAX], sn[MMAX];
-  __shared__ double res;
-  const int reorth = K->reorth;
-  if (reorth) {
-    double s = 0.0;
-    for (int c = threadIdx.x; c < G; c += VB) s += part[c];
-    double acc[1] = {s};
-    block_reduce_store<1>(acc, 1, &res, 1);
-  }
-  for (int i = threadIdx.x; i <= j; i += VB) {
-    double h = K->h[i];
-    if (reorth) {
-      h += K->h2[i];
-      K->h[i] = h;
-    }
-    col[i] = h;
-    if (i < j) {
-      cs[i] = K->cs[i];
-      sn[i] = K->sn[i];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (reorth) {
-      K->nrm_new = res;
-      K->nrm_fin = sqrt(res);
-    }
-    const double hn = K->nrm_fin;
-    col[j + 1] = hn;
-    for (int i = 0; i < j; ++i) {
-      const double a = cs[i] * col[i] + sn[i] * col[i + 1];
-      col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-      col[i] = a;
-    }
-    const double den = hypot(col[j], col[j + 1]);
-    const double c = den > 0.0 ? col[j] / den : 1.0;
-    const double sj = den > 0.0 ? col[j + 1] / den : 0.0;
-    K->cs[j] = c;
-    K->sn[j] = sj;
-    col[j] = den;
-    col[j + 1] = 0.0;
-    const double gj = K->g[j];
-    K->g[j + 1] = -sj * gj;
-    K->g[j] = c * gj;
-    K->est = fabs(K->g[j + 1]) / K->bnorm;
-    K->breakdown = (hn == 0.0 || den == 0.0 || !isfinite(hn)) ? 1 : 0;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i <= j + 1; i += VB) K->H[i * mm + j] = col[i];
-}
-
-// y = R^{-1} g for the first jend columns (back substitution).
+// y = R^{-1} g for the first jend columns: one warp, the entries above the current one updated by
+// column in shared memory
 __global__ void lsq_kernel(KryDev* K, int jend, int mm) {
+  __shared__ double R[MMAX * MMAX], g[MMAX];
+  for (int q = threadIdx.x; q < jend * jend; q += blockDim.x) R[q] = K->H[(q / jend) * mm + q % jend];
+  for (int q = threadIdx.x; q < jend; q += blockDim.x) g[q] = K->g[q];
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
   for (int i = jend - 1; i >= 0; --i) {
-    double s = K->g[i];
-    for (int k = i + 1; k < jend; ++k) s -= K->H[i * mm + k] * K->y[k];
-    const double d = K->H[i * mm + i];
-    K->y[i] = d != 0.0 ? s / d : 0.0;
+    const double d = R[i * jend + i];
+    const double y = d != 0.0 ? g[i] / d : 0.0;
+    if (threadIdx.x == 0) K->y[i] = y;
+    __syncwarp();
+    for (int q = threadIdx.x; q < i; q += 32) g[q] = fma(-R[q * jend + i], y, g[q]);
+    __syncwarp();
   }
 }
 
@@ -742,6 +774,20 @@ __global__ void __launch_bounds__(VB) dot_kernel(const double* __restrict__ a, c
   for (int64_t j = lo + threadIdx.x; j < hi; j += VB) acc[0] += a[j] * b[j];
   block_reduce_store<1>(acc, 1, part + blockIdx.x, 1);
 }
+// r = b - t and the partial |r|^2 (the same partition)
+__global__ void __launch_bounds__(VB) resid_kernel(const double* __restrict__ b, const double* __restrict__ t,
+                                                   double* __restrict__ r, int64_t n, double* part) {
+  const int G = gridDim.x;
+  const int64_t per = (n + G - 1) / G;
+  const int64_t lo = blockIdx.x * per, hi = min(n, lo + per);
+  double acc[1] = {0.0};
+  for (int64_t j = lo + threadIdx.x; j < hi; j += VB) {
+    const double v = b[j] - t[j];
+    r[j] = v;
+    acc[0] += v * v;
+  }
+  block_reduce_store<1>(acc, 1, part + blockIdx.x, 1);
+}
 __global__ void axpby_kernel(double a, const double* __restrict__ x, double b, double* __restrict__ y, int64_t n) {
   for (int64_t j = blockIdx.x * (int64_t)VB + threadIdx.x; j < n; j += (int64_t)gridDim.x * VB) y[j] = a * x[j] + b * y[j];
 }
@@ -759,54 +805,38 @@ __global__ void fill_kernel(double* y, double v, int64_t n) {
 }
 
 // ---------------------------------------------------------------- host helpers
-template <int R, bool SELF, typename VT>
-static void launch_mdot(fsi_mesh* m, dim3 grid, const VT* V, int M1, int i0, const double* w, int64_t n,
-                        const int* skip) {
-  if constexpr (sizeof(VT) == 4)
-    mdot4_kernel<R, SELF><<<grid, VB, 0, m->stream>>>(V, M1, i0, w, n, m->partials_dot, skip);
-  else
-    mdot_kernel<R, SELF, VT><<<grid, VB, 0, m->stream>>>(V, M1, i0, w, n, m->partials_dot, skip);
-}
-
-template <bool SELF, typename VT>
-static void launch_mdot_rem(fsi_mesh* m, int rem, dim3 g1, const VT* V, int M1, int i0, const double* w,
-                            int64_t n, const int* skip) {
-  switch (rem) {
-    case 0: launch_mdot<0, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 1: launch_mdot<1, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 2: launch_mdot<2, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 3: launch_mdot<3, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 4: launch_mdot<4, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 5: launch_mdot<5, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 6: launch_mdot<6, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 7: launch_mdot<7, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 8: launch_mdot<8, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 9: launch_mdot<9, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 10: launch_mdot<10, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 11: launch_mdot<11, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 12: launch_mdot<12, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 13: launch_mdot<13, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    case 14: launch_mdot<14, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-    default: launch_mdot<15, SELF>(m, g1, V, M1, i0, w, n, skip); break;
-  }
-}
-
-// out[0..k) = V_i . w for the basis slots i < k; with self, out[k] = w . w.
 template <typename VT>
-static int basis_dots(fsi_mesh* m, const VT* V, int M1, int k, const double* w, int64_t n, double* out, bool self,
-                      const int* skip = nullptr) {
-  const int G = cgrid_t<VT>((n + CH - 1) / CH);
-  const int nfull = k / DCH, rem = k % DCH;
-  if (nfull)
-    FSI_LAUNCH(m, P_KRY_DOT, (launch_mdot<DCH, false>(m, dim3(G, nfull), V, M1, 0, w, n, skip)));
-  if (rem || self) {
-    if (self)
-      FSI_LAUNCH(m, P_KRY_DOT, (launch_mdot_rem<true>(m, rem, dim3(G, 1), V, M1, nfull * DCH, w, n, skip)));
-    else
-      FSI_LAUNCH(m, P_KRY_DOT, (launch_mdot_rem<false>(m, rem, dim3(G, 1), V, M1, nfull * DCH, w, n, skip)));
+static void launch_mdot(fsi_mesh* m, dim3 grid, const VT* V, int M1, int k, const double* w, int64_t n, KryDev* K) {
+  switch (k % DCH) {
+    case 0: mdot_kernel<0, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 1: mdot_kernel<1, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 2: mdot_kernel<2, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 3: mdot_kernel<3, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 4: mdot_kernel<4, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 5: mdot_kernel<5, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 6: mdot_kernel<6, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 7: mdot_kernel<7, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 8: mdot_kernel<8, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 9: mdot_kernel<9, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 10: mdot_kernel<10, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 11: mdot_kernel<11, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 12: mdot_kernel<12, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 13: mdot_kernel<13, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 14: mdot_kernel<14, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    default: mdot_kernel<15, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
   }
-  const int rows = k + (self ? 1 : 0);
-  FSI_LAUNCH(m, P_KRY_DOT, sum_partials<<<rows, VB, 0, m->stream>>>(m->partials_dot, G, out, skip));
+}
+
+// K->h[0..k) = V_i . w for the basis slots i < k, K->h[k] = w . w
+template <typename VT>
+static int basis_dots(fsi_mesh* m, const VT* V, int M1, int k, const double* w, int64_t n, KryDev* K) {
+  const int G = cgrid_t<VT>((n + CH - 1) / CH);
+  // one group more than the full ones: it holds the rest, or only w . w
+  const dim3 grid(G, k / DCH + 1);
+  if constexpr (sizeof(VT) == 4)
+    FSI_LAUNCH(m, P_KRY_DOT, mdot4_kernel<<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K));
+  else
+    FSI_LAUNCH(m, P_KRY_DOT, launch_mdot<VT>(m, grid, V, M1, k, w, n, K));
   return FSI_OK;
 }
 
@@ -822,7 +852,7 @@ static int dot_dev(fsi_mesh* m, const double* a, const double* b, int64_t n, dou
   if (rc) return rc;
   const int G = vgrid(n);
   FSI_LAUNCH(m, P_KRY_DOT, dot_kernel<<<G, VB, 0, m->stream>>>(a, b, n, m->partials_dot));
-  FSI_LAUNCH(m, P_KRY_DOT, sum_partials<<<1, VB, 0, m->stream>>>(m->partials_dot, G, out, nullptr));
+  FSI_LAUNCH(m, P_KRY_DOT, sum_partials<<<1, VB, 0, m->stream>>>(m->partials_dot, G, out));
   return FSI_OK;
 }
 
@@ -913,9 +943,9 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
   double rel = 1.0, cycle_rel = 1.0;
   bool first_cycle = true;
   int n_arnoldi_pairs = 0;
+  if ((rc = dot_dev(m, r, r, n, m->red))) return rc;
   while (true) {
-    // |r| on the device; the host needs it for the stopping and stall tests
-    if ((rc = dot_dev(m, r, r, n, m->red))) return rc;
+    // |r|^2 on the device (m->red); the host needs it for the stopping and stall tests
     FSI_CUDA(cudaMemcpyAsync(m->red_host, m->red, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     FSI_CUDA(cudaStreamSynchronize(m->stream));
     const double beta2 = m->red_host[0];
@@ -931,7 +961,7 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
     FSI_LAUNCH(m, P_KRY_SMALL, cycle_start<<<1, 1, 0, m->stream>>>(K, m->red, mm));
     // the operator input of the plain (Jacobi) steps: z = dinv V_j, written with V_j
     VT* zn = pc ? nullptr : (F32 ? reinterpret_cast<VT*>(m->dx32) : reinterpret_cast<VT*>(z));
-    FSI_LAUNCH(m, P_KRYLOV, store_slot<VT><<<chunk_grid(n), VB, 0, m->stream>>>(V, M1, 0, r, m->red, K, n, m->dinv, zn));
+    FSI_LAUNCH(m, P_KRYLOV, store_first<VT><<<chunk_grid(n), VB, 0, m->stream>>>(V, M1, r, m->red, n, m->dinv, zn));
     int jend = 0, enq = 0;
     bool done = false;
     const int jmax = std::min(mm, max_iter - *iters);
@@ -965,31 +995,23 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
         }
       }
       // pass 1: h = V^T w and |w|^2 (slot j+1 of h)
-      if ((rc = basis_dots(m, V, M1, j + 1, w, n, K->h, true))) return rc;
-      // pass-1 update fused with the pass-2 projections of the updated vector
-      {
-        const int Gc = cgrid_t<VT>((n + CH - 1) / CH);
-        FSI_LAUNCH(m, P_KRY_UPD, rc = upd_dot<VT>(m, Gc, w, V, M1, j + 1, K->h, n));
-        if (rc) return rc;
-        FSI_LAUNCH(m, P_KRY_UPD, sum_partials_decide<<<j + 2, VB, 0, m->stream>>>(m->partials_dot, Gc, K, j));
-        prof_bytes(m, P_KRY_DOT, (j + 1) * vb + wb);      // j+1 basis vectors and w read once
-        prof_bytes(m, P_KRY_UPD, (j + 1) * vb + 2 * wb);  // j+1 basis vectors and w read, w written
-        // the pass-2 update only when the DGKS test asked for it (exits at once otherwise),
-        // then its norm and the Givens step
-        if constexpr (F32) {
-          FSI_LAUNCH(m, P_KRY_UPD, upd4_kernel<<<Gc, VB, 0, m->stream>>>(w, reinterpret_cast<const float*>(V), M1,
-                                                                        j + 1, K->h2, n, m->partials_dot, &K->reorth));
-        } else {
-          FSI_LAUNCH(m, P_KRY_UPD, upd_kernel<VT><<<Gc, VB, 0, m->stream>>>(w, V, M1, j + 1, K->h2, n,
-                                                                             m->partials_dot, &K->reorth));
-        }
-        FSI_LAUNCH(m, P_KRY_SMALL, sum_partials_givens<<<1, VB, 0, m->stream>>>(m->partials_dot, Gc, K, j, mm));
-      }
-      FSI_LAUNCH(m, P_KRYLOV, store_slot<VT><<<chunk_grid(n), VB, 0, m->stream>>>(V, M1, j + 1, w, nullptr, K, n, m->dinv, zn));
-      // estimate, reorth and breakdown flags: one copy (the fields are adjacent)
-      FSI_CUDA(cudaMemcpyAsync(est + 3 * j, &K->est, sizeof(double) + 2 * sizeof(int), cudaMemcpyDeviceToHost,
-                               m->stream));
+      if ((rc = basis_dots(m, V, M1, j + 1, w, n, K))) return rc;
+      // pass-1 update fused with the pass-2 projections of the updated vector, then the Givens step
+      const int Gc = cgrid_t<VT>((n + CH - 1) / CH);
+      FSI_LAUNCH(m, P_KRY_UPD, rc = upd_dot<VT>(m, Gc, w, V, M1, j + 1, n, mm, est + 3 * j));
+      if (rc) return rc;
+      prof_bytes(m, P_KRY_DOT, (j + 1) * vb + wb);      // j+1 basis vectors and w read once
+      prof_bytes(m, P_KRY_UPD, (j + 1) * vb + 2 * wb);  // j+1 basis vectors and w read, w written
       FSI_CUDA(cudaEventRecord(m->kry_ev[j], m->stream));
+      // the pass-2 update (only when the DGKS test asked for it), the new basis vector and the next input
+      if constexpr (F32) {
+        FSI_LAUNCH(m, P_KRY_UPD, upd_store4_kernel<<<upd_grid(n, 4), VB, 0, m->stream>>>(
+                                     w, reinterpret_cast<float*>(V), M1, j + 1, K, n, m->dinv, reinterpret_cast<float*>(zn)));
+      } else {
+        FSI_LAUNCH(m, P_KRY_UPD, upd_store_kernel<<<upd_grid(n, 1), VB, 0, m->stream>>>(
+                                     w, reinterpret_cast<double*>(V), M1, j + 1, K, n, m->dinv, reinterpret_cast<double*>(zn)));
+      }
+      prof_bytes(m, P_KRY_UPD, 2 * wb + 2 * vb);  // w and dinv read, V_{j+1} and z written
       ++*iters;
       jend = j + 1;
       enq = j + 1;
@@ -1011,9 +1033,9 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
     for (int j = 0; j < enq; ++j) {  // the second passes that ran
       int ro = 0;
       memcpy(&ro, reinterpret_cast<const char*>(est + 3 * j) + sizeof(double), sizeof(int));
-      if (ro) prof_bytes(m, P_KRY_UPD, (j + 1) * vb + 2 * wb);
+      if (ro) prof_bytes(m, P_KRY_UPD, (j + 1) * vb);
     }
-    FSI_LAUNCH(m, P_KRY_SMALL, lsq_kernel<<<1, 1, 0, m->stream>>>(K, jend, mm));
+    FSI_LAUNCH(m, P_KRY_SMALL, lsq_kernel<<<1, VB, 0, m->stream>>>(K, jend, mm));
     if (pc) {
       FSI_LAUNCH(m, P_KRYLOV, zcombine_kernel<<<G, VB, 0, m->stream>>>(x, m->Z, jend, K, n));
     } else {
@@ -1022,8 +1044,8 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
     }
     // true residual r = b - A x
     if ((rc = op_jvp(m, blk, x, t, flags))) return rc;
-    FSI_CUDA(cudaMemcpyAsync(r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, m->stream));
-    if ((rc = vec_axpy(m, -1.0, t, r, n))) return rc;
+    FSI_LAUNCH(m, P_KRYLOV, resid_kernel<<<G, VB, 0, m->stream>>>(b, t, r, n, m->partials_dot));
+    FSI_LAUNCH(m, P_KRY_DOT, sum_partials<<<1, VB, 0, m->stream>>>(m->partials_dot, G, m->red));
     ++*restarts;
   }
   *rel_out = rel;

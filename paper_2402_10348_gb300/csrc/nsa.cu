@@ -342,6 +342,48 @@ __global__ void __launch_bounds__(4 * NAT) nsa_apply_kernel(const T* __restrict_
   y[q] = dir ? (dx ? dx[q] : (double)x[q]) : (double)((acc[0] + acc[1]) + (acc[2] + acc[3]));
 }
 
+// The same with three threads per (node, row field), one per neighbour plane, summed through shared
+// memory: CTAs of 32 nodes.  For meshes whose 128-node CTAs leave SMs idle or with one CTA, where a
+// thread's 27 dependent rounds of loads are all of the time.
+__global__ void __launch_bounds__(384) nsa_apply_split_kernel(const double* __restrict__ A, const double* __restrict__ x,
+                                                              int nx, int ny, int nz, int64_t nn,
+                                                              const uint8_t* __restrict__ mask, int pin,
+                                                              double* __restrict__ y) {
+  __shared__ double part[2][4][32];
+  const int64_t n = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  const int r = threadIdx.y, dz = (int)threadIdx.z - 1;
+  double s = 0.0;
+  if (n < nn) {
+    const unsigned row = (unsigned)n / (unsigned)(nx + 1);
+    const int i = (int)((unsigned)n - row * (unsigned)(nx + 1)), k = (int)(row / (unsigned)(ny + 1));
+    const int j = (int)(row - (unsigned)k * (unsigned)(ny + 1));
+    const int64_t sy = nx + 1, sz = sy * (ny + 1);
+    const double* a = A + ((n / NAT * 27 + 9 * (dz + 1)) * 16 + 4 * r) * NAT + n % NAT;
+    const bool okz = k + dz >= 0 && k + dz <= nz;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+      const bool okyz = okz && j + dy >= 0 && j + dy <= ny;
+#pragma unroll
+      for (int dx = -1; dx <= 1; ++dx) {
+        const bool ok = okyz && i + dx >= 0 && i + dx <= nx;
+        const int64_t nb = ok ? n + dx + sy * dy + sz * dz : n;
+        const double* ao = a + 16 * ((dx + 1) + 3 * (dy + 1)) * NAT;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] += __ldg(ao + c * NAT) * __ldg(x + c * nn + nb);
+      }
+    }
+    s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  }
+  if (dz != 0) part[dz > 0][r][threadIdx.x] = s;
+  __syncthreads();
+  if (dz != 0 || n >= nn) return;
+  s = part[0][r][threadIdx.x] + s + part[1][r][threadIdx.x];
+  const bool dir = ((mask[n] >> r) & 1) && (r < 3 || pin);
+  const int64_t q = (int64_t)r * nn + n;
+  y[q] = dir ? x[q] : s;
+}
+
 // the diagonal of the assembled operator (1 on Dirichlet rows)
 __global__ void nsa_diag_kernel(const double* __restrict__ A, int64_t nn, const uint8_t* __restrict__ mask, int pin,
                                 double* __restrict__ d) {
@@ -406,11 +448,20 @@ int nsa_build(fsi_mesh* m, unsigned flags) {
   return FSI_OK;
 }
 
+// below this many nodes the split kernel is taken
+constexpr int64_t NSA_SPLIT_NODES = 152 * 256;
+
 int launch_nsa(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   if (int rc = nsa_build(m, flags)) return rc;
   const Geom& g = m->g;
   // algorithmic bytes: the blocks once, the increment in, the product out, the mask
   prof_bytes(m, P_NS_JVP64E, (double)m->nn * (27.0 * 16 * 8 + 32 + 32 + 1));
+  if (m->nn < NSA_SPLIT_NODES) {
+    FSI_LAUNCH(m, P_NS_JVP64E,
+               nsa_apply_split_kernel<<<(unsigned)((m->nn + 31) / 32), dim3(32, 4, 3), 0, m->stream>>>(
+                   m->na64, dx, g.nx, g.ny, g.nz, m->nn, m->mask, m->pin_active, y));
+    return FSI_OK;
+  }
   FSI_LAUNCH(m, P_NS_JVP64E,
              nsa_apply_kernel<double><<<(unsigned)((m->nn + NAT - 1) / NAT), dim3(NAT, 4), 0, m->stream>>>(
                  m->na64, dx, g.nx, g.ny, g.nz, m->nn, m->mask, m->pin_active, dx, y));
