@@ -239,7 +239,7 @@ int ensure_dx32(fsi_mesh* m) {
 int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigned flags) {
   m->applies++;
   m->dof_applied += b.n;
-  if (m->tet) return tet_op(m, b, 1, dx, y, flags & ~(OP_DX32_READY | OP_REUSED));
+  if (m->tet) return tet_op(m, b, 1, dx, y, flags & ~OP_DX32_READY);
   const bool f32 = flags & FSI_FP32;
   if (f32) {  // float copy of the increment for the float32 kernels (unless the caller wrote it)
     if (int rc = ensure_dx32(m)) return rc;
@@ -271,7 +271,7 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
 }
 
 int op_diag(fsi_mesh* m, const BlockInfo& b, double* d, unsigned flags) {
-  if (m->tet) return tet_op(m, b, 2, nullptr, d, flags & ~OP_REUSED);
+  if (m->tet) return tet_op(m, b, 2, nullptr, d, flags);
   const bool f32 = flags & FSI_FP32;
   if (!f32 && !m->rec && (flags & OP_REUSED)) return b.kind == 0 ? nsa_diag(m, d, flags) : stencil_diag(m, b, d);
   flags &= ~OP_REUSED;

@@ -28,11 +28,21 @@ struct TetData {
   int64_t* nptr = nullptr;  // [nn + 1]
   int32_t* nlist = nullptr; // 4 e + a of every (element, corner) at a node, by element
   double* E = nullptr;      // [24][ne] element contributions, slot (a * ncomp + eq)
-  // float64 NS element matrices [256][ne], row a * 4 + eq, column b * 4 + f, built once a
-  // solve has taken NSA_AFTER products on one staging (k_stage) with one elastic flag
+  // NS element matrices [256][ne] of the assembly, row a * 4 + eq, column b * 4 + f
   double* K = nullptr;
-  int64_t k_stage = -1;
-  int k_elastic = -1, k_count = 0, k_built = 0;
+  // assembled NS operator: the neighbours of the node (itself included, ascending) in slices of 32
+  // nodes as wide as their longest row; entry p of the slice at off: node col[off + p * 32 +
+  // lane], block A[((off / 32 + p) * 16 + 4 r + c) * 32 + lane].  -1: neighbour lists not built,
+  // 0: some node has more than TET_ROW neighbours (element matrices are kept), 1: built
+  int rows = -1;
+  int64_t n_blocks = 0;     // blocks with padding
+  int64_t* off = nullptr;   // [slices + 1]
+  int32_t* col = nullptr;
+  double* A = nullptr;
+  int64_t k_stage = -1;     // staging and elastic flag of the built matrices
+  int k_elastic = -1, k_built = 0;
+  int64_t c_stage = -1;     // products counted at a staging
+  int c_count = 0;
 };
 
 constexpr int TG = 19;
@@ -47,6 +57,9 @@ void tet_free(TetData* t) {
   cudaFree(t->nlist);
   cudaFree(t->E);
   cudaFree(t->K);
+  cudaFree(t->off);
+  cudaFree(t->col);
+  cudaFree(t->A);
   delete t;
 }
 
@@ -359,39 +372,220 @@ __global__ void __launch_bounds__(128) tet_nsk_apply(const int32_t* __restrict__
   }
 }
 
+// ------------------------------------------------------------------ assembled NS operator
+// Rows of 4 x 4 blocks over a node's neighbours: about 15 blocks (240 float64 FMAs) a node where the
+// element matrices of its 24 elements' share take 1,536, and no contributions to sum.  32^3 cells
+// (196,608 elements): 173 -> 25 us a product.
+constexpr int TET_ROW = 96;  // most neighbours of a node
+constexpr int TSL = 32;      // nodes per slice
+
+// the node's neighbours, ascending, into nb; more than TET_ROW: returns TET_ROW + 1
+__device__ int tet_neighbours(const int64_t* __restrict__ nptr, const int32_t* __restrict__ nlist,
+                              const int32_t* __restrict__ conn, int64_t ne, int64_t n, int32_t* nb) {
+  int cnt = 0;
+  for (int64_t i = nptr[n]; i < nptr[n + 1]; ++i) {
+    const int64_t e = nlist[i] >> 2;
+    for (int b = 0; b < 4; ++b) {
+      const int32_t v = conn[(int64_t)b * ne + e];
+      int p = cnt;
+      while (p > 0 && nb[p - 1] > v) --p;
+      if (p > 0 && nb[p - 1] == v) continue;
+      if (cnt == TET_ROW) return TET_ROW + 1;
+      for (int q = cnt; q > p; --q) nb[q] = nb[q - 1];
+      nb[p] = v;
+      ++cnt;
+    }
+  }
+  if (cnt == 0) nb[cnt++] = (int32_t)n;  // a node of no element: its own zero block
+  return cnt;
+}
+
+// width of every slice; fill: the columns too (padding and nodes past the last: the node itself or 0)
+__global__ void __launch_bounds__(TSL) tet_rows_kernel(const int64_t* __restrict__ nptr, const int32_t* __restrict__ nlist,
+                                                       const int32_t* __restrict__ conn, int64_t ne, int64_t nn,
+                                                       int32_t* __restrict__ width, const int64_t* __restrict__ off,
+                                                       int32_t* __restrict__ col) {
+  const int64_t n = (int64_t)blockIdx.x * TSL + threadIdx.x;
+  int32_t nb[TET_ROW];
+  const int cnt = n < nn ? tet_neighbours(nptr, nlist, conn, ne, n, nb) : 0;
+  if (!col) {
+    int w = cnt;
+    for (int o = 16; o > 0; o >>= 1) w = max(w, __shfl_xor_sync(0xffffffffu, w, o));
+    if (threadIdx.x == 0) width[blockIdx.x] = w;
+    return;
+  }
+  const int64_t o = off[blockIdx.x];
+  const int w = (int)((off[blockIdx.x + 1] - o) / TSL);
+  for (int p = 0; p < w; ++p) col[o + (int64_t)p * TSL + threadIdx.x] = p < cnt ? nb[p] : (int32_t)(n < nn ? n : 0);
+}
+
+// blocks from the element matrices, element order: blockDim (TSL, 4), thread (node, row field)
+__global__ void __launch_bounds__(4 * TSL) tet_rows_gather(const int64_t* __restrict__ nptr, const int32_t* __restrict__ nlist,
+                                                           const int32_t* __restrict__ conn, int64_t ne, int64_t nn,
+                                                           const int64_t* __restrict__ off, const int32_t* __restrict__ col,
+                                                           const double* __restrict__ K, double* __restrict__ A) {
+  const int64_t n = (int64_t)blockIdx.x * TSL + threadIdx.x;
+  const int r = threadIdx.y;
+  const int64_t o = off[blockIdx.x];
+  const int w = (int)((off[blockIdx.x + 1] - o) / TSL);
+  int32_t prev = -1;
+  for (int p = 0; p < w; ++p) {
+    const int32_t v = col[o + (int64_t)p * TSL + threadIdx.x];
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    if (n < nn && v > prev) {  // (padding repeats the node behind its larger neighbours)
+      for (int64_t i = nptr[n]; i < nptr[n + 1]; ++i) {
+        const int32_t t = nlist[i];
+        const int64_t e = t >> 2;
+        const int a = t & 3;
+        for (int b = 0; b < 4; ++b) {
+          if (conn[(int64_t)b * ne + e] != v) continue;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[c] += K[(int64_t)((a * 4 + r) * 16 + b * 4 + c) * ne + e];
+        }
+      }
+      prev = v;
+    } else {
+      prev = 0x7fffffff;
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) A[((o / TSL + p) * 16 + 4 * r + c) * TSL + threadIdx.x] = acc[c];
+  }
+}
+
+// y = A x with the Dirichlet rows: blockDim (TSL, 4), one slice per CTA
+__global__ void __launch_bounds__(4 * TSL) tet_rows_apply(const double* __restrict__ A, const int64_t* __restrict__ off,
+                                                          const int32_t* __restrict__ col, const double* __restrict__ dx,
+                                                          int64_t nn, const uint8_t* __restrict__ mask, int pin,
+                                                          double* __restrict__ y) {
+  const int64_t n = (int64_t)blockIdx.x * TSL + threadIdx.x;
+  if (n >= nn) return;
+  const int r = threadIdx.y;
+  const int64_t o = off[blockIdx.x];
+  const int w = (int)((off[blockIdx.x + 1] - o) / TSL);
+  const int32_t* cp = col + o + threadIdx.x;
+  const double* a = A + (o / TSL * 16 + 4 * r) * TSL + threadIdx.x;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int p = 0; p < w; ++p) {
+    const int32_t v = cp[p * TSL];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] += a[(int64_t)(16 * p + c) * TSL] * __ldg(dx + (int64_t)c * nn + v);
+  }
+  const bool dir = ((mask[n] >> r) & 1) && (r < 3 || pin);
+  y[(int64_t)r * nn + n] = dir ? dx[(int64_t)r * nn + n] : (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+
+__global__ void tet_rows_diag(const double* __restrict__ A, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
+                              int64_t nn, const uint8_t* __restrict__ mask, int pin, double* __restrict__ d) {
+  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= nn) return;
+  const int lane = (int)(n % TSL);
+  const int64_t o = off[n / TSL];
+  int p = 0;
+  while (col[o + (int64_t)p * TSL + lane] != (int32_t)n) ++p;  // every list holds its node
+  for (int r = 0; r < 4; ++r) {
+    const bool dir = ((mask[n] >> r) & 1) && (r < 3 || pin);
+    d[(int64_t)r * nn + n] = dir ? 1.0 : A[((o / TSL + p) * 16 + 5 * r) * TSL + lane];
+  }
+}
+
+// the neighbour lists, once per mesh (synchronises)
+static int tet_rows_init(fsi_mesh* m) {
+  TetData* t = m->tet;
+  const int64_t ns = (m->nn + TSL - 1) / TSL;
+  int32_t* width = nullptr;
+  FSI_CUDA(cudaMalloc(&width, sizeof(int32_t) * (size_t)ns));
+  std::vector<int32_t> w(ns);
+  std::vector<int64_t> off(ns + 1, 0);
+  cudaError_t e = cudaSuccess;
+  tet_rows_kernel<<<(unsigned)ns, TSL, 0, m->stream>>>(t->nptr, t->nlist, t->conn, t->ne, m->nn, width, nullptr, nullptr);
+  if ((e = cudaGetLastError()) == cudaSuccess)
+    e = cudaMemcpyAsync(w.data(), width, sizeof(int32_t) * (size_t)ns, cudaMemcpyDeviceToHost, m->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+  cudaFree(width);
+  FSI_CUDA(e);
+  for (int64_t i = 0; i < ns; ++i) {
+    if (w[i] > TET_ROW) {
+      t->rows = 0;
+      return FSI_OK;
+    }
+    off[i + 1] = off[i] + (int64_t)w[i] * TSL;
+  }
+  cudaFree(t->off);
+  cudaFree(t->col);
+  t->off = nullptr;
+  t->col = nullptr;
+  FSI_CUDA(cudaMalloc(&t->off, sizeof(int64_t) * (size_t)(ns + 1)));
+  FSI_CUDA(cudaMalloc(&t->col, sizeof(int32_t) * (size_t)off[ns]));
+  FSI_CUDA(cudaMemcpyAsync(t->off, off.data(), sizeof(int64_t) * (size_t)(ns + 1), cudaMemcpyHostToDevice, m->stream));
+  FSI_CUDA(cudaStreamSynchronize(m->stream));  // the host array ends here
+  tet_rows_kernel<<<(unsigned)ns, TSL, 0, m->stream>>>(t->nptr, t->nlist, t->conn, t->ne, m->nn, nullptr, t->off, t->col);
+  FSI_CUDA(cudaGetLastError());
+  t->n_blocks = off[ns];
+  t->rows = 1;
+  return FSI_OK;
+}
+
+// element matrices, and the rows where every node's list fits, at the staged state
+static int tet_ns_build(fsi_mesh* m, int elastic) {
+  TetData* t = m->tet;
+  if (t->k_built && t->k_stage == m->stage_gen && t->k_elastic == elastic) return FSI_OK;
+  t->k_built = 0;
+  if (t->rows < 0)
+    if (int rc = tet_rows_init(m)) return rc;
+  if (!t->K) FSI_CUDA(cudaMalloc(&t->K, sizeof(double) * 256 * (size_t)t->ne));
+  if (t->rows && !t->A) FSI_CUDA(cudaMalloc(&t->A, sizeof(double) * 16 * (size_t)t->n_blocks));
+  TetArgs A;
+  A.conn = t->conn;
+  A.geo = t->geo;
+  A.ne = t->ne;
+  A.xa = m->staged_xa;
+  A.xd = m->xd;
+  A.mat = m->mat;
+  A.dx = nullptr;
+  A.E = t->E;
+  A.nn = m->nn;
+  A.elastic = elastic;
+  A.P = m->P;
+  FSI_LAUNCH(m, P_NS_BUILD, tet_nsk_build<<<(unsigned)((t->ne + 127) / 128), 128, 0, m->stream>>>(A, t->K));
+  if (t->rows)
+    FSI_LAUNCH(m, P_NS_BUILD, tet_rows_gather<<<(unsigned)((m->nn + TSL - 1) / TSL), dim3(TSL, 4), 0, m->stream>>>(
+                                  t->nptr, t->nlist, t->conn, t->ne, m->nn, t->off, t->col, t->K, t->A));
+  t->k_stage = m->stage_gen;
+  t->k_elastic = elastic;
+  t->k_built = 1;
+  return FSI_OK;
+}
+
 int tet_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
   if (flags & FSI_FP32) return set_error(FSI_EINVAL, "tetrahedral meshes: float64 operators only");
-  if (mode == 1 && !m->rec) {
-    // a float64 solve on one staging: after NSA_AFTER products switch to element matrices
-    TetData* t = m->tet;
-    const int elastic = ((flags & FSI_ELASTIC_AUG) && m->ns > 0) ? 1 : 0;
-    if (t->k_stage != m->stage_gen || t->k_elastic != elastic) {
-      t->k_stage = m->stage_gen;
-      t->k_elastic = elastic;
-      t->k_count = 0;
-      t->k_built = 0;
+  TetData* t = m->tet;
+  const int elastic = ((flags & FSI_ELASTIC_AUG) && m->ns > 0) ? 1 : 0;
+  if (mode == 2 && (flags & OP_REUSED)) {
+    if (int rc = tet_ns_build(m, elastic)) return rc;
+    if (t->rows) {
+      FSI_LAUNCH(m, P_NS_DIAG, tet_rows_diag<<<(unsigned)((m->nn + 255) / 256), 256, 0, m->stream>>>(
+                                   t->A, t->off, t->col, m->nn, m->mask, m->pin_active, y));
+      return FSI_OK;
     }
-    if (++t->k_count > NSA_AFTER) {
-      const unsigned grid = (unsigned)((t->ne + 127) / 128);
-      if (!t->k_built) {
-        if (!t->K) FSI_CUDA(cudaMalloc(&t->K, sizeof(double) * 256 * (size_t)t->ne));
-        TetArgs A;
-        A.conn = t->conn;
-        A.geo = t->geo;
-        A.ne = t->ne;
-        A.xa = m->staged_xa;
-        A.xd = m->xd;
-        A.mat = m->mat;
-        A.dx = nullptr;
-        A.E = t->E;
-        A.nn = m->nn;
-        A.elastic = elastic;
-        A.P = m->P;
-        FSI_LAUNCH(m, P_NS_BUILD, tet_nsk_build<<<grid, 128, 0, m->stream>>>(A, t->K));
-        t->k_built = 1;
+  }
+  if (mode == 1 && !m->rec) {
+    // direct products for the first few at a state, as on hexahedra
+    if (t->c_stage != m->stage_gen) {
+      t->c_stage = m->stage_gen;
+      t->c_count = 0;
+    }
+    if (++t->c_count > NSA_AFTER || (flags & OP_REUSED)) {
+      if (int rc = tet_ns_build(m, elastic)) return rc;
+      if (t->rows) {
+        prof_bytes(m, P_NS_JVP64E, (double)t->n_blocks * (128.0 + 4.0) + (double)m->nn * 65.0);
+        FSI_LAUNCH(m, P_NS_JVP64E, tet_rows_apply<<<(unsigned)((m->nn + TSL - 1) / TSL), dim3(TSL, 4), 0, m->stream>>>(
+                                       t->A, t->off, t->col, dx, m->nn, m->mask, m->pin_active, y));
+        return FSI_OK;
       }
       prof_bytes(m, P_NS_JVP64E, (double)t->ne * (256 * 8.0 + 16 * 4.0 + 16 * 8.0) + (double)m->nn * 32.0);
-      FSI_LAUNCH(m, P_NS_JVP64E, tet_nsk_apply<<<grid, 128, 0, m->stream>>>(t->conn, t->K, dx, t->E, t->ne, m->nn));
+      FSI_LAUNCH(m, P_NS_JVP64E, tet_nsk_apply<<<(unsigned)((t->ne + 127) / 128), 128, 0, m->stream>>>(t->conn, t->K, dx,
+                                                                                                      t->E, t->ne, m->nn));
       FSI_LAUNCH(m, P_NODE_SUM, tet_ns_node<1><<<(unsigned)((m->nn + 255) / 256), 256, 0, m->stream>>>(
                                     t->nptr, t->nlist, t->E, t->ne, m->nn, m->mask, m->pin_active, m->staged_x, m->vD,
                                     dx, y));
