@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_b_res_kernel(const __grid_const
 // Quadrature-point coefficients of the momentum/continuity product (ops.cuh lists them) in
 // float64 and/or rounded to float32: C[((ez * 8 + q) * NCQ + c) * nxyp + ey * nxp + ex].  64^3, one
 // solid: 3.36 -> 1.17 ms against the tile build, all solids in one pass.
+template <bool MANY>
 __global__ void __launch_bounds__(HQ_THREADS) hq_ns_coef_kernel(const __grid_constant__ HexNS H, double* __restrict__ c64,
                                                                 float* __restrict__ c32, unsigned ne, int elastic) {
   HexLane l;
@@ -123,7 +124,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ns_coef_kernel(const __grid_con
   put(19, p.tau_m * p.rrho);
   if (!elastic) return;  // (the products then read the first 20)
   double aB[6], aG[6][3];
-  hq_elastic(H, l, aB, aG);
+  hq_elastic<MANY>(H, l, aB, aG);
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
     put(20 + c, aB[c]);
@@ -134,8 +135,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ns_coef_kernel(const __grid_con
 
 // The product itself for a state that is used a few times: the point's coefficients stay in
 // registers.  E as hq_ns_res_kernel.  A product at a new state with its coefficients stored before
-// it: 61 x 47 x 35 with two solids 2.97 -> 1.02 ms, 256 x 128 x 64 with nine 216 -> 47 ms (46.5 of them
-// here, about 1,560 float64 operations a point, 0.97 of the float64 rate).
+// it: 61 x 47 x 35 with two solids 2.97 -> 1.02 ms, 256 x 128 x 64 with nine 216 -> 33 ms.
 struct PointCoef {
   const NSPoint& p;
   const double (&aB)[6];
@@ -154,6 +154,7 @@ struct PointCoef {
   }
 };
 
+template <bool MANY>
 __global__ void __launch_bounds__(HQ_THREADS) hq_ns_jvp_kernel(const __grid_constant__ HexNS H,
                                                                const double* __restrict__ dx, double* __restrict__ E,
                                                                unsigned ne, int elastic) {
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ns_jvp_kernel(const __grid_cons
   NSPoint p;
   hq_ns_point(H, l, p);
   double aB[6] = {}, aG[6][3] = {};
-  if (elastic) hq_elastic(H, l, aB, aG);
+  if (elastic) hq_elastic<MANY>(H, l, aB, aG);
   double dv[3], gd[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -255,8 +256,9 @@ int ns_build(fsi_mesh* m, unsigned flags, bool f64) {
     c.len = len;
   }
   const unsigned ne = (unsigned)m->g.nx * m->g.ny * m->g.nz;
+  auto* kernel = m->ns >= HQ_MANY ? &hq_ns_coef_kernel<true> : &hq_ns_coef_kernel<false>;
   FSI_LAUNCH(m, P_NS_BUILD,
-             hq_ns_coef_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(
+             kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(
                  hex_ns(m, nxp), f64 ? static_cast<double*>(c.p) : nullptr, f64 ? nullptr : static_cast<float*>(c.p), ne,
                  eflags && m->ns > 0 ? 1 : 0));
   c.gen = m->stage_gen;
@@ -276,7 +278,8 @@ int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   // algorithmic bytes: the nodal fields once, the contributions written and read, the product
   prof_bytes(m, P_NS_JVP64, (double)ne * 256.0 + (double)m->nn * 8.0 * (13 + (elastic ? 7 * m->ns : 0)));
   prof_bytes(m, P_NODE_SUM, (double)ne * 256.0 + (double)m->nn * 33.0);
-  FSI_LAUNCH(m, P_NS_JVP64, hq_ns_jvp_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, dx, m->ke_e, ne, elastic));
+  auto* kernel = m->ns >= HQ_MANY ? &hq_ns_jvp_kernel<true> : &hq_ns_jvp_kernel<false>;
+  FSI_LAUNCH(m, P_NS_JVP64, kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, dx, m->ke_e, ne, elastic));
   FSI_LAUNCH(m, P_NODE_SUM,
              ns_node_kernel<double><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, H.W,
                                                                          m->mask, m->pin_active, dx, nullptr, nullptr, y));

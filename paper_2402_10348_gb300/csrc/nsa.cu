@@ -109,6 +109,7 @@ struct Walsh {
 // columns, N_a d_c N_b al + d_j N_a (N_b tau_m (al L_jc + delta_jc cm) + delta_jc tau_m al v.grad N_b)
 // for the continuity rows and tau_m / rho grad N_a . grad N_b in their corner (the product's
 // linearization at one point, nsq_point_fg, read off by field).
+template <bool MANY>
 __global__ void __launch_bounds__(HQ_THREADS) nsa_elem_kernel(const __grid_constant__ HexNS H, double* __restrict__ K,
                                                               unsigned e0, unsigned e1, int slots, int elastic) {
   HexLane l;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(HQ_THREADS) nsa_elem_kernel(const __grid_const
   hq_ns_point(H, l, p);
   double aB[6], aG[6][3];
   if (elastic) {
-    hq_elastic(H, l, aB, aG);
+    hq_elastic<MANY>(H, l, aB, aG);
   } else {
 #pragma unroll
     for (int c = 0; c < 6; ++c) aB[c] = aG[c][0] = aG[c][1] = aG[c][2] = 0.0;
@@ -428,6 +429,7 @@ int nsa_build(fsi_mesh* m, unsigned flags) {
   const int slots = (int)std::min<int64_t>(g.nz, std::max<int64_t>(2, NSA_SLAB_BYTES / (8 * layer)));
   if (int rc = ensure_elem_matrices(m, slots * layer)) return rc;
   const HexNS H = hex_ns(m, nxp);
+  auto* kernel = m->ns >= HQ_MANY ? &nsa_elem_kernel<true> : &nsa_elem_kernel<false>;
   const int elastic = eflags && m->ns > 0 ? 1 : 0;
   const int64_t plane = (int64_t)(g.nx + 1) * (g.ny + 1);
   // a ring of layer slots: after the layers [z0, z1), the planes [z0, z1) are complete, and layer
@@ -437,7 +439,7 @@ int nsa_build(fsi_mesh* m, unsigned flags) {
     const int z1 = std::min(g.nz, z0 + step);
     const unsigned e0 = (unsigned)z0 * g.ny * g.nx, e1 = (unsigned)z1 * g.ny * g.nx;
     FSI_LAUNCH(m, P_NS_BUILD,
-               nsa_elem_kernel<<<hq_blocks(e1 - e0), HQ_THREADS, 0, m->stream>>>(H, m->ke64, e0, e1, slots, elastic));
+               kernel<<<hq_blocks(e1 - e0), HQ_THREADS, 0, m->stream>>>(H, m->ke64, e0, e1, slots, elastic));
     const int64_t n0 = z0 * plane, n1 = (z1 == g.nz ? z1 + 1 : z1) * plane;
     FSI_LAUNCH(m, P_NS_BUILD,
                nsa_gather_kernel<<<(unsigned)((n1 - n0 + NAT - 1) / NAT), dim3(NAT, 4), 0, m->stream>>>(
