@@ -4,8 +4,8 @@
 // summed into node rows once per solve: 27 FMAs a node for an indicator (64 an element before, in
 // element matrices) and 648 for a solid's six components (1,440 an element before).  One product:
 // Allen-Cahn 96 x 96 x 192 102 us (0.93 of the float64 FMA rate) against 517 with the node sums, B 64^3
-// 323 us (1.06 of it) against 929.  Builds: Allen-Cahn 7.7 ms against 19.3 (and 9.2 for the
-// diagonal, 15 for the two products before it), B 3.6 ms against 2.0 (and 2.5 for the diagonal).
+// 323 us (1.06 of it) against 929.  Builds: Allen-Cahn 5.0 ms against 19.3 (and 9.2 for the
+// diagonal, 15 for the two products before it), B 3.5 ms against 2.0 (and 2.5 for the diagonal).
 //
 // Allen-Cahn (Eq. PPV_AC's linearization, gamma, beta and tau_phi frozen): with
 //   T_a = N_a + tau v.grad N_a,  R_b = (c_m + alpha gamma (3 phi^2 - 1 - beta dsqrtF)) N_b + alpha v.grad N_b
@@ -26,12 +26,44 @@ namespace fsi {
 
 constexpr int ST = 128;
 
-// Element matrices of the layers from e0: K[((ez % slots) * 64 + 8 a + b) * nxyp + ey * nxp + ex].
-// Lane q evaluates T and R at its point for all corners; lane b then sums column b over the points,
-// T_a(q) and its own R_b(q) by shuffles.  The diffusion part is the same for every element.
+// T and R of the lane's point q for its corners in the order x = corner ^ q: the weights are then constants
+// of x and the gradients' signs the lane's own (vr_j = v_j / h_j, signed for the lane's side), and what
+// another lane needs of them sits in a register known at compile time.
+//   T = W (N + tau v.grad N),   R = mass N + conv v.grad N
+__device__ __forceinline__ void test_trial(const HexLane& l, const double (&v)[3], double W, double tau, double mass,
+                                           double conv, double (&T)[8], double (&R)[8]) {
+  // the lane's own corner lies on the side of its sign: d_j N at the corner q is -sx rhx ... in HexLane's
+  // signs (sx turns partner - own into the derivative)
+  const double vx = -l.sx * v[0], vy = -l.sy * v[1], vz = -l.sz * v[2];
+  const double Wt = W * tau;
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const double wx = (x & 1) ? FSI_G1 : FSI_G0, wy = (x & 2) ? FSI_G1 : FSI_G0, wz = (x & 4) ? FSI_G1 : FSI_G0;
+    const double vg = fma((x & 1) ? -wy * wz : wy * wz, vx,
+                          fma((x & 2) ? -wx * wz : wx * wz, vy, ((x & 4) ? -wx * wy : wx * wy) * vz));
+    T[x] = fma(Wt, vg, W * (wx * wy * wz));
+    R[x] = fma(conv, vg, mass * (wx * wy * wz));
+  }
+}
+
+// M[z] += sum_q T_a(q) R_b(q) for column b = lane and row a = lane ^ z, from all eight points q = lane ^ y
+__device__ __forceinline__ void outer_sum(const double (&T)[8], const double (&R)[8], double (&M)[8]) {
+#pragma unroll
+  for (int y = 0; y < 8; ++y) {
+    const double r = hq_shx(R[y], y);
+#pragma unroll
+    for (int z = 0; z < 8; ++z) M[z] = fma(hq_shx(T[z ^ y], y), r, M[z]);
+  }
+}
+
+// Element matrices of the layers from e0: K[((ez % slots) * 64 + 8 a + b) * nxyp + ey * nxp + ex].  The
+// diffusion part depends on a ^ b alone and is the same for every element (D, from the host).
+struct Diffusion {
+  double d[8];
+};
 __global__ void __launch_bounds__(HQ_THREADS) ac_elem_kernel(const __grid_constant__ HexNS H, int phase, double gam,
-                                                             double bet, double* __restrict__ K, unsigned e0, unsigned e1,
-                                                             int slots) {
+                                                             double bet, const __grid_constant__ Diffusion D,
+                                                             double* __restrict__ K, unsigned e0, unsigned e1, int slots) {
   HexLane l;
   l.set(H.g, H.rh, H.nxp, e0, e1);
   const Phys& P = H.P;
@@ -45,42 +77,15 @@ __global__ void __launch_bounds__(HQ_THREADS) ac_elem_kernel(const __grid_consta
   const double p2 = phi * phi - 1.0;
   const double dsF = p2 > 0.0 ? phi : (p2 < 0.0 ? -phi : 0.0);
   const double mass = P.c_mass + P.alpha * gam * (3.0 * phi * phi - 1.0 - bet * dsF);
-  double Ta[8], Rb[8];
+  double T[8], R[8], M[8];
+  test_trial(l, v, H.W, tau, mass, P.alpha, T, R);
 #pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const double wx = ((a ^ l.q) & 1) ? FSI_G1 : FSI_G0, wy = ((a ^ l.q) & 2) ? FSI_G1 : FSI_G0,
-                 wz = ((a ^ l.q) & 4) ? FSI_G1 : FSI_G0;
-    const double yz = wy * wz, N = wx * yz;
-    const double vgN = v[0] * ((a & 1) ? H.rh[0] : -H.rh[0]) * yz + wx * (v[1] * ((a & 2) ? H.rh[1] : -H.rh[1]) * wz +
-                                                                         v[2] * ((a & 4) ? H.rh[2] : -H.rh[2]) * wy);
-    Ta[a] = H.W * fma(tau, vgN, N);
-    Rb[a] = fma(P.alpha, vgN, mass * N);
-  }
-  double M[8];  // column b = lane
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    // grad N_a . grad N_b over the element: the 1D mass factors are 1/3 (same corner) and 1/6
-    const double mx = ((a ^ l.q) & 1) ? 1.0 / 6.0 : 1.0 / 3.0, my = ((a ^ l.q) & 2) ? 1.0 / 6.0 : 1.0 / 3.0,
-                 mz = ((a ^ l.q) & 4) ? 1.0 / 6.0 : 1.0 / 3.0;
-    const double gx = ((a ^ l.q) & 1) ? -1.0 : 1.0, gy = ((a ^ l.q) & 2) ? -1.0 : 1.0, gz = ((a ^ l.q) & 4) ? -1.0 : 1.0;
-    M[a] = 8.0 * H.W * k_hat * P.alpha *
-           (gx * H.rh[0] * H.rh[0] * my * mz + gy * H.rh[1] * H.rh[1] * mx * mz + gz * H.rh[2] * H.rh[2] * mx * my);
-  }
-  // exchange: after x steps lane b holds R_b of point b ^ x
-#pragma unroll
-  for (int x = 0; x < 8; ++x) {
-    // R_b(q), q = lane ^ x: lane q sends its R of corner q ^ x
-    double send = 0.0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) send = (l.q ^ x) == c ? Rb[c] : send;
-    const double r = hq_shx(send, x);
-#pragma unroll
-    for (int a = 0; a < 8; ++a) M[a] = fma(hq_shx(Ta[a], x), r, M[a]);
-  }
+  for (int z = 0; z < 8; ++z) M[z] = D.d[z];
+  outer_sum(T, R, M);
   if (!l.ok) return;
   double* out = K + ((int64_t)(l.ez % slots) * 64 + l.q) * H.nxyp + (int64_t)l.ey * H.nxp + l.ex;
 #pragma unroll
-  for (int a = 0; a < 8; ++a) out[(int64_t)(8 * a) * H.nxyp] = M[a];
+  for (int z = 0; z < 8; ++z) out[(int64_t)(8 * (l.q ^ z)) * H.nxyp] = M[z];
 }
 
 // Ten element matrices of a solid (S, then R_km row-major): layer slots of 640 planes.
@@ -99,43 +104,39 @@ __global__ void __launch_bounds__(HQ_THREADS) b_elem_kernel(const __grid_constan
   const double al = l.val(H.mat[(2 + solid) * nn + l.n]);
   const double vGv = P.Gd[0] * v[0] * v[0] + P.Gd[1] * v[1] * v[1] + P.Gd[2] * v[2] * v[2];
   const double tau = rsqrt(H.dt2 + vGv);
-  const double mass = al * P.c_mass + (1.0 - al) * P.alpha, conv = al * P.alpha;
-  double Ta[8], Rb[8];
+  const double conv = al * P.alpha;
+  double T[8], M[8];
+  {
+    double R[8];
+    test_trial(l, v, H.W, tau, al * P.c_mass + (1.0 - al) * P.alpha, conv, T, R);
 #pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const double wx = ((a ^ l.q) & 1) ? FSI_G1 : FSI_G0, wy = ((a ^ l.q) & 2) ? FSI_G1 : FSI_G0,
-                 wz = ((a ^ l.q) & 4) ? FSI_G1 : FSI_G0;
-    const double yz = wy * wz, N = wx * yz;
-    const double vgN = v[0] * ((a & 1) ? H.rh[0] : -H.rh[0]) * yz + wx * (v[1] * ((a & 2) ? H.rh[1] : -H.rh[1]) * wz +
-                                                                         v[2] * ((a & 4) ? H.rh[2] : -H.rh[2]) * wy);
-    Ta[a] = H.W * fma(tau, vgN, N);
-    Rb[a] = fma(conv, vgN, mass * N);
+    for (int z = 0; z < 8; ++z) M[z] = 0.0;
+    outer_sum(T, R, M);
   }
   double* out = K + ((int64_t)(l.ez % slots) * 640 + l.q) * H.nxyp + (int64_t)l.ey * H.nxp + l.ex;
-  double M[8];
-#pragma unroll
-  for (int a = 0; a < 8; ++a) M[a] = 0.0;
-#pragma unroll
-  for (int x = 0; x < 8; ++x) {
-    double send = 0.0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) send = (l.q ^ x) == c ? Rb[c] : send;
-    const double r = hq_shx(send, x);
-#pragma unroll
-    for (int a = 0; a < 8; ++a) M[a] = fma(hq_shx(Ta[a], x), r, M[a]);
-  }
   if (l.ok) {
 #pragma unroll
-    for (int a = 0; a < 8; ++a) out[(int64_t)(8 * a) * H.nxyp] = M[a];
+    for (int z = 0; z < 8; ++z) out[(int64_t)(8 * (l.q ^ z)) * H.nxyp] = M[z];
   }
-  // R_km: the trial side is N_b alone, an interpolation's transpose over the lanes
+  // R_km: the trial side is N_b alone, so the sum over the points is the transposed interpolation: per
+  // axis G0 own + G1 of the lane across it, whose row a sits one register bit away
 #pragma unroll
   for (int km = 0; km < 9; ++km) {
     const double c = conv * L[km / 3][km % 3];
+    double f[8];
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const double r = l.val(Ta[a] * c);  // sum_q N_lane(q) ...: the 2 x 2 weights are symmetric
-      if (l.ok) out[(int64_t)(64 * (km + 1) + 8 * a) * H.nxyp] = r;
+    for (int x = 0; x < 8; ++x) f[x] = T[x] * c;
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) {
+      double p[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) p[x] = hq_shx(f[x ^ d], d);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) f[x] = fma(FSI_G1, p[x] - f[x], f[x]);
+    }
+    if (l.ok) {
+#pragma unroll
+      for (int z = 0; z < 8; ++z) out[(int64_t)(64 * (km + 1) + 8 * (l.q ^ z)) * H.nxyp] = f[z];
     }
   }
 }
@@ -307,6 +308,18 @@ int stencil_build(fsi_mesh* m, const BlockInfo& b) {
   const HexNS H = hex_ns(m, nxp);
   const int64_t plane = (int64_t)(g.nx + 1) * (g.ny + 1);
   const int step = slots == g.nz ? g.nz : slots - 1;
+  // alpha gamma eps^2 grad N_a . grad N_b over an element, by a ^ b: 1D factors 1/3 (same side) and 1/6
+  Diffusion D;
+  for (int x = 0; x < 8; ++x) {
+    double s = 0.0;
+    for (int j = 0; j < 3; ++j) {
+      double t = ((x >> j) & 1) ? -H.rh[j] * H.rh[j] : H.rh[j] * H.rh[j];
+      for (int i = 0; i < 3; ++i)
+        if (i != j) t *= ((x >> i) & 1) ? 1.0 / 6.0 : 1.0 / 3.0;
+      s += t;
+    }
+    D.d[x] = 8.0 * H.W * gam * m->P.eps * m->P.eps * m->P.alpha * s;
+  }
   for (int z0 = 0; z0 < g.nz; z0 += step) {
     const int z1 = std::min(g.nz, z0 + step);
     const unsigned e0 = (unsigned)z0 * g.ny * g.nx, e1 = (unsigned)z1 * g.ny * g.nx;
@@ -319,7 +332,7 @@ int stencil_build(fsi_mesh* m, const BlockInfo& b) {
                                     m->ke64, g.nx, g.ny, g.nz, nxp, nxyp, slots, n0, n1, S.A));
     } else {
       FSI_LAUNCH(m, P_NS_BUILD, ac_elem_kernel<<<hq_blocks(e1 - e0), HQ_THREADS, 0, m->stream>>>(
-                                    H, b.index, gam, bet, m->ke64, e0, e1, slots));
+                                    H, b.index, gam, bet, D, m->ke64, e0, e1, slots));
       FSI_LAUNCH(m, P_NS_BUILD, stencil_gather_kernel<false><<<grid, ST, 0, m->stream>>>(
                                     m->ke64, g.nx, g.ny, g.nz, nxp, nxyp, slots, n0, n1, S.A));
     }
