@@ -17,11 +17,11 @@
 //   w -= V h, |w|^2 and h2 = V^T w (the second pass's projections of the updated w)
 //   in one pass                                           (upd_dot_kernel); its last CTA:
 //   if |w_new| < |w_old| / sqrt(2) (classical Gram-Schmidt with the DGKS
-//   re-orthogonalization test) h += h2 and |w|^2 -= |h2|^2 (the basis is orthonormal); Givens
-//   rotation of the new Hessenberg column and the residual estimate, written to pinned
-//   host memory                                            (givens_step)
+//   re-orthogonalization test) h += h2 and |w|^2 -= |h2|^2 (the basis is orthonormal)
 //   V_{j+1} = (w - V h2) / |w| (V h2 only where the test asked for it) into its slot, and
-//   z = D V_{j+1} beside it                                (upd_store_kernel)
+//   z = D V_{j+1} beside it                                (upd_store_kernel); one more CTA: the
+//   Givens rotation of the new Hessenberg column and the residual estimate, written to pinned
+//   host memory
 // In the projection kernels the last CTA to finish adds the per-CTA partial sums (a warp per row, fixed
 // order), so no launch follows for them: at small sizes launches are the time.  16^3, one
 // iteration: 103 us with ten launches and a copy, 56 with these; 64^3, float32 basis, beside the
@@ -190,22 +190,29 @@ __device__ __forceinline__ bool last_cta(unsigned* counter, unsigned total) {
   if (last) __threadfence();
   return last;
 }
-// dst[i] = sum_c part[i * G + c] for i < rows: a warp per row, lanes strided, then a shuffle tree
+// dst[i] = sum_c part[i * G + c] for i < rows: a warp takes U rows at a time (their loads in flight
+// together: this runs in one CTA while the GPU waits), lanes strided, then shuffle trees
+template <int U>
 __device__ __forceinline__ void sum_rows(const double* part, int G, int rows, double* dst) {
-  const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x >> 5; i < rows; i += blockDim.x >> 5) {
-    const double* p = part + (int64_t)i * G;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    int c = lane;
-    for (; c + 96 < G; c += 128) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int i0 = (threadIdx.x >> 5) * U; i0 < rows; i0 += U * nw) {
+    const int cnt = min(U, rows - i0);
+    const double* p = part + (int64_t)i0 * G;
+    double s[U];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) s[u] += __ldcg(p + c + 32 * u);
+    for (int u = 0; u < U; ++u) s[u] = 0.0;
+#pragma unroll 4
+    for (int c = lane; c < G; c += 32) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (u < cnt) s[u] += __ldcg(p + (int64_t)u * G + c);
     }
-    for (; c < G; c += 32) s[0] += __ldcg(p + c);
-    double t = (s[0] + s[1]) + (s[2] + s[3]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) dst[i] = t;
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+      if (lane == 0 && u < cnt) dst[i0 + u] = s[u];
+    }
   }
 }
 
@@ -242,7 +249,7 @@ __global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int 
                                                   int64_t n, double* part, KryDev* K) {
   if (blockIdx.y < gridDim.y - 1) mdot_group<DCH, false, VT>(V, M1, blockIdx.y * DCH, w, n, part);
   else mdot_group<R, true, VT>(V, M1, blockIdx.y * DCH, w, n, part);
-  if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows(part, gridDim.x, k + 1, K->h);
+  if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows<4>(part, gridDim.x, k + 1, K->h);
 }
 
 // The float32 basis: the same projections with 16-byte loads.  A CTA works on four
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, 
   for (int i = 0; i < KC; ++i)
     if (i == kc) acc[i] = acc[KC];  // w . w goes to row k
   block_reduce_store_f<NR>(acc, kc + (self ? 1 : 0), part + (int64_t)ib * G + blockIdx.x, G);
-  if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows(part, G, k + 1, K->h);
+  if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows<4>(part, G, k + 1, K->h);
 }
 
 // out[i] = sum_c part[i*G + c] (fixed order), i = blockIdx.x
@@ -328,15 +335,90 @@ __device__ __forceinline__ VT lin_comb_chunk(const VT* __restrict__ hs, const VT
   return ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
 }
 
+// After the fused update, by the last CTA of its kernel: h2 (the second pass's projections of the
+// updated w) and |w|^2 summed from the partials, and the DGKS decision.  K->h becomes column j of the
+// Hessenberg matrix: h, plus h2 where |w_new| < |w_old| / sqrt(2) asked for the second pass, and
+// K->nrm_fin the new norm below it: |w - V h2|^2 = |w|^2 - |h2|^2 on an orthonormal basis, so the
+// second pass needs no sweep before its norm is known.
+__device__ __forceinline__ void orth_step(const double* part, int G, KryDev* K, int j) {
+  __shared__ double c2[MMAX + 2];
+  sum_rows<8>(part, G, j + 2, c2);
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const double w2 = c2[j + 1];
+  const bool reorth = sqrt(w2) < sqrt(K->h[j + 1]) * 0.70710678118654752;
+  double hh = 0.0;  // |h2|^2
+  for (int q = threadIdx.x; q <= j; q += 32) {
+    hh = fma(c2[q], c2[q], hh);
+    if (reorth) {
+      K->h[q] += c2[q];
+      K->h2[q] = c2[q];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+  if (threadIdx.x == 0) {
+    const double df = w2 - hh;  // a NaN stays one: the host stops on it
+    K->nrm_fin = sqrt(reorth ? (df < 0.0 ? 0.0 : df) : w2);
+    K->reorth = reorth ? 1 : 0;
+  }
+}
+
+// The Givens step by one CTA, beside the basis store: column j is rotated by the previous rotations
+// (one thread, in shared memory), the new rotation zeroes its subdiagonal entry, and g and the
+// residual estimate |g_{j+1}| / |b| follow.  est (pinned host memory): the estimate, then the
+// reorth and breakdown flags as ints.
+__device__ __forceinline__ void givens_step(KryDev* K, int j, int mm, double* est) {
+  __shared__ double col[MMAX + 2], cs[MMAX], sn[MMAX];
+  for (int q = threadIdx.x; q <= j; q += blockDim.x) {
+    col[q] = K->h[q];
+    if (q < j) {
+      cs[q] = K->cs[q];
+      sn[q] = K->sn[q];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double hn = K->nrm_fin;
+    double t = col[0];
+    for (int q = 0; q < j; ++q) {
+      const double nx = col[q + 1];
+      col[q] = fma(sn[q], nx, cs[q] * t);
+      t = fma(-sn[q], t, cs[q] * nx);
+    }
+    const double den = hypot(t, hn);
+    const double c = den > 0.0 ? t / den : 1.0;
+    const double sj = den > 0.0 ? hn / den : 0.0;
+    K->cs[j] = c;
+    K->sn[j] = sj;
+    col[j] = den;
+    col[j + 1] = 0.0;
+    const double gj = K->g[j], gn = -sj * gj;
+    K->g[j + 1] = gn;
+    K->g[j] = c * gj;
+    est[0] = fabs(gn) / K->bnorm;
+    int* flags = reinterpret_cast<int*>(est + 1);
+    flags[0] = K->reorth;
+    flags[1] = (hn == 0.0 || den == 0.0 || !isfinite(hn)) ? 1 : 0;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q <= j + 1; q += blockDim.x) K->H[q * mm + j] = col[q];
+}
+
 // V_slot = (w - sum_{i<k} h2_i V_i) / |w| with the second pass's correction only where the DGKS
 // test asked for it (K->reorth), and the next operator input z = dinv V_slot from the stored
 // value.  One fused multiply-add per basis element, chained on the element's value of w (no
 // partial sums to add up afterwards: float64 adds are scarce on this GPU); the element's
 // values of up to UPB basis vectors are loaded ahead of the chain.
 constexpr int UPB = 32;
-__global__ void __launch_bounds__(VB, 2) upd_store_kernel(const double* __restrict__ w, double* V, int M1, int k,
-                                                          const KryDev* __restrict__ K, int64_t n,
-                                                          const double* __restrict__ dinv, double* __restrict__ z) {
+// The last CTA takes the Givens step instead (column k - 1).
+__global__ void __launch_bounds__(VB, 2) upd_store_kernel(const double* __restrict__ w, double* V, int M1, int k, KryDev* K,
+                                                          int64_t n, const double* __restrict__ dinv,
+                                                          double* __restrict__ z, int mm, double* est) {
+  if (blockIdx.x == gridDim.x - 1) {
+    givens_step(K, k - 1, mm, est);
+    return;
+  }
   __shared__ double nh[MMAX + 2], s_sh;
   const bool second = K->reorth != 0;
   if (threadIdx.x == 0) s_sh = K->nrm_fin > 0.0 ? 1.0 / K->nrm_fin : 0.0;
@@ -345,7 +427,7 @@ __global__ void __launch_bounds__(VB, 2) upd_store_kernel(const double* __restri
   __syncthreads();
   const double scale = s_sh;
   const int64_t nch = (n + CH - 1) / CH;
-  for (int64_t c = blockIdx.x; c < nch; c += gridDim.x) {
+  for (int64_t c = blockIdx.x; c < nch; c += gridDim.x - 1) {
     const int64_t j = c * CH + threadIdx.x;
     if (j >= n) break;
     double* blk = V + c * (int64_t)M1 * CH + threadIdx.x;
@@ -372,9 +454,13 @@ __global__ void __launch_bounds__(VB, 2) upd_store_kernel(const double* __restri
 // The same for the float32 basis, laid out as mdot4_kernel: a CTA works on four chunks at a
 // time, a thread on four adjacent elements (one float4 per basis vector, two double2 of w); z is the
 // float32 operator's increment.
-__global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict__ w, float* V, int M1, int k,
-                                                        const KryDev* __restrict__ K, int64_t n,
-                                                        const double* __restrict__ dinv, float* __restrict__ z) {
+__global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict__ w, float* V, int M1, int k, KryDev* K,
+                                                        int64_t n, const double* __restrict__ dinv,
+                                                        float* __restrict__ z, int mm, double* est) {
+  if (blockIdx.x == gridDim.x - 1) {
+    givens_step(K, k - 1, mm, est);
+    return;
+  }
   __shared__ float hs[MMAX + 2];
   __shared__ double s_sh;
   const bool second = K->reorth != 0;
@@ -386,7 +472,7 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
   const int64_t nch = (n + CH - 1) / CH;
   const int sub = threadIdx.x >> 6;
   const int e0 = (threadIdx.x & 63) * 4;
-  for (int64_t c = (int64_t)blockIdx.x * 4 + sub; c < nch; c += (int64_t)gridDim.x * 4) {
+  for (int64_t c = (int64_t)blockIdx.x * 4 + sub; c < nch; c += (int64_t)(gridDim.x - 1) * 4) {
     const int64_t j = c * CH + e0;
     if (j >= n) break;
     float* blk = V + c * (int64_t)M1 * CH + e0;
@@ -432,73 +518,6 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
   }
 }
 
-// The step after the fused update, by the last CTA of its kernel: h2 (the second pass's projections
-// of the updated w) and |w|^2 summed from the partials, the DGKS decision and the Givens step.
-// Column j of the Hessenberg matrix: h, plus h2 where |w_new| < |w_old| / sqrt(2) asked for the second
-// pass; below it the new norm, |w - V h2|^2 = |w|^2 - |h2|^2 on an orthonormal basis, so the second
-// pass needs no sweep before the rotation.  The column is rotated by the previous rotations, the new
-// rotation zeroes its subdiagonal entry, and g and the residual estimate |g_{j+1}| / |b| follow.
-// est (pinned host memory): the estimate, then the reorth and breakdown flags as ints.
-// Everything is read by all threads first; one thread then runs the chain of rotations in shared memory.
-__device__ void givens_step(const double* part, int G, KryDev* K, int j, int mm, double* est) {
-  __shared__ double col[MMAX + 2], c2[MMAX + 2], cs[MMAX], sn[MMAX];
-  const int nt = blockDim.x;
-  for (int q = threadIdx.x; q <= j; q += nt) {
-    col[q] = K->h[q];
-    if (q < j) {
-      cs[q] = K->cs[q];
-      sn[q] = K->sn[q];
-    }
-  }
-  sum_rows(part, G, j + 2, c2);
-  __syncthreads();
-  const double w2 = c2[j + 1];
-  const bool reorth = sqrt(w2) < sqrt(K->h[j + 1]) * 0.70710678118654752;
-  double hh = 0.0;  // |h2|^2, in warp 0
-  if (threadIdx.x < 32) {
-    for (int q = threadIdx.x; q <= j; q += 32) hh = fma(c2[q], c2[q], hh);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
-  }
-  if (reorth) {
-    for (int q = threadIdx.x; q <= j; q += nt) {
-      col[q] += c2[q];
-      K->h2[q] = c2[q];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const double df = w2 - hh;  // a NaN stays one: the host stops on it
-    const double hn = sqrt(reorth ? (df < 0.0 ? 0.0 : df) : w2);
-    K->nrm_fin = hn;
-    K->reorth = reorth ? 1 : 0;
-    double t = col[0];
-    for (int q = 0; q < j; ++q) {
-      const double nx = col[q + 1];
-      col[q] = fma(sn[q], nx, cs[q] * t);
-      t = fma(-sn[q], t, cs[q] * nx);
-    }
-    const double den = hypot(t, hn);
-    const double c = den > 0.0 ? t / den : 1.0;
-    const double sj = den > 0.0 ? hn / den : 0.0;
-    K->cs[j] = c;
-    K->sn[j] = sj;
-    col[j] = den;
-    col[j + 1] = 0.0;
-    const double gj = K->g[j], gn = -sj * gj;
-    K->g[j + 1] = gn;
-    K->g[j] = c * gj;
-    const int bd = (hn == 0.0 || den == 0.0 || !isfinite(hn)) ? 1 : 0;
-    est[0] = fabs(gn) / K->bnorm;
-    int* flags = reinterpret_cast<int*>(est + 1);
-    flags[0] = reorth ? 1 : 0;
-    flags[1] = bd;
-    __threadfence_system();
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q <= j + 1; q += nt) K->H[q * mm + j] = col[q];
-}
-
 // Pass-1 update fused with the pass-2 projections: w' = w - sum_{i<k} h_i V_i, the
 // partial |w'|^2 and the partial V_i . w' (i < k) of the updated vector, from one read
 // of the basis: a thread keeps the k basis values of its element in registers, uses
@@ -510,7 +529,7 @@ constexpr int UDB = 128;  // threads per CTA (two elements of each 256-element c
 static_assert(UDB == 128, "the row sums take four columns per lane");
 template <int KMAX, typename VT>
 __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, const VT* __restrict__ V, int M1,
-                                                      int k, int64_t n, double* part, KryDev* K, int mm, double* est) {
+                                                      int k, int64_t n, double* part, KryDev* K) {
   extern __shared__ __align__(16) unsigned char upd_smem[];
   const double* h = K->h;
   VT* sacc = reinterpret_cast<VT*>(upd_smem);  // [KMAX + 1][UDB]
@@ -561,7 +580,7 @@ __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, co
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) part[(int64_t)i * G + blockIdx.x] = s;
   }
-  if (last_cta(&K->counter, gridDim.x)) givens_step(part, G, K, k - 1, mm, est);
+  if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1);
 }
 
 // The fused update for the float32 basis: a thread takes two adjacent elements of each
@@ -569,7 +588,7 @@ __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, co
 // per load as with a float64 basis.  Elements at or past n are never read.
 template <int KMAX>
 __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, const float* __restrict__ V, int M1,
-                                                       int k, int64_t n, double* part, KryDev* K, int mm, double* est) {
+                                                       int k, int64_t n, double* part, KryDev* K) {
   extern __shared__ __align__(16) unsigned char upd_smem[];
   const double* h = K->h;
   float* sacc = reinterpret_cast<float*>(upd_smem);  // [KMAX + 1][UDB]
@@ -631,34 +650,34 @@ __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, c
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) part[(int64_t)i * G + blockIdx.x] = (double)s;
   }
-  if (last_cta(&K->counter, gridDim.x)) givens_step(part, G, K, k - 1, mm, est);
+  if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1);
 }
 
 template <int KMAX, typename VT>
-static int launch_upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n, int mm, double* est) {
+static int launch_upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n) {
   KryDev* K = static_cast<KryDev*>(m->kry_dev);
   const size_t smem = sizeof(VT) * (size_t)(KMAX + 1) * UDB;
   if constexpr (sizeof(VT) == 4) {
     if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot2_kernel<KMAX>), smem)) return rc;
-    upd_dot2_kernel<KMAX><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K, mm, est);
+    upd_dot2_kernel<KMAX><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
   } else {
     if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot_kernel<KMAX, VT>), smem)) return rc;
-    upd_dot_kernel<KMAX, VT><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K, mm, est);
+    upd_dot_kernel<KMAX, VT><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
   }
   return FSI_OK;
 }
 
 template <typename VT>
-static int upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n, int mm, double* est) {
+static int upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n) {
   switch ((k + 7) / 8) {
-    case 1: return launch_upd_dot<8>(m, G, w, V, M1, k, n, mm, est);
-    case 2: return launch_upd_dot<16>(m, G, w, V, M1, k, n, mm, est);
-    case 3: return launch_upd_dot<24>(m, G, w, V, M1, k, n, mm, est);
-    case 4: return launch_upd_dot<32>(m, G, w, V, M1, k, n, mm, est);
-    case 5: return launch_upd_dot<40>(m, G, w, V, M1, k, n, mm, est);
-    case 6: return launch_upd_dot<48>(m, G, w, V, M1, k, n, mm, est);
-    case 7: return launch_upd_dot<56>(m, G, w, V, M1, k, n, mm, est);
-    default: return launch_upd_dot<64>(m, G, w, V, M1, k, n, mm, est);
+    case 1: return launch_upd_dot<8>(m, G, w, V, M1, k, n);
+    case 2: return launch_upd_dot<16>(m, G, w, V, M1, k, n);
+    case 3: return launch_upd_dot<24>(m, G, w, V, M1, k, n);
+    case 4: return launch_upd_dot<32>(m, G, w, V, M1, k, n);
+    case 5: return launch_upd_dot<40>(m, G, w, V, M1, k, n);
+    case 6: return launch_upd_dot<48>(m, G, w, V, M1, k, n);
+    case 7: return launch_upd_dot<56>(m, G, w, V, M1, k, n);
+    default: return launch_upd_dot<64>(m, G, w, V, M1, k, n);
   }
 }
 
@@ -737,17 +756,21 @@ __global__ void __launch_bounds__(VB) zcombine_kernel(double* __restrict__ x, co
 }
 
 // --------------------------------------------------------- small device kernels
-// y = R^{-1} g for the first jend columns: one warp, the entries above the current one updated by
-// column in shared memory
+// y = R^{-1} g for the first jend columns: the diagonal's reciprocals by all threads (a float64
+// division takes most of a microsecond here), then one warp, the entries above the current one
+// updated by column in shared memory
 __global__ void lsq_kernel(KryDev* K, int jend, int mm) {
-  __shared__ double R[MMAX * MMAX], g[MMAX];
+  __shared__ double R[MMAX * MMAX], g[MMAX], inv[MMAX];
   for (int q = threadIdx.x; q < jend * jend; q += blockDim.x) R[q] = K->H[(q / jend) * mm + q % jend];
-  for (int q = threadIdx.x; q < jend; q += blockDim.x) g[q] = K->g[q];
+  for (int q = threadIdx.x; q < jend; q += blockDim.x) {
+    g[q] = K->g[q];
+    const double d = K->H[q * mm + q];
+    inv[q] = d != 0.0 ? 1.0 / d : 0.0;
+  }
   __syncthreads();
   if (threadIdx.x >= 32) return;
   for (int i = jend - 1; i >= 0; --i) {
-    const double d = R[i * jend + i];
-    const double y = d != 0.0 ? g[i] / d : 0.0;
+    const double y = g[i] * inv[i];
     if (threadIdx.x == 0) K->y[i] = y;
     __syncwarp();
     for (int q = threadIdx.x; q < i; q += 32) g[q] = fma(-R[q * jend + i], y, g[q]);
@@ -996,21 +1019,24 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
       }
       // pass 1: h = V^T w and |w|^2 (slot j+1 of h)
       if ((rc = basis_dots(m, V, M1, j + 1, w, n, K))) return rc;
-      // pass-1 update fused with the pass-2 projections of the updated vector, then the Givens step
+      // pass-1 update fused with the pass-2 projections of the updated vector, then the DGKS test
       const int Gc = cgrid_t<VT>((n + CH - 1) / CH);
-      FSI_LAUNCH(m, P_KRY_UPD, rc = upd_dot<VT>(m, Gc, w, V, M1, j + 1, n, mm, est + 3 * j));
+      FSI_LAUNCH(m, P_KRY_UPD, rc = upd_dot<VT>(m, Gc, w, V, M1, j + 1, n));
       if (rc) return rc;
       prof_bytes(m, P_KRY_DOT, (j + 1) * vb + wb);      // j+1 basis vectors and w read once
       prof_bytes(m, P_KRY_UPD, (j + 1) * vb + 2 * wb);  // j+1 basis vectors and w read, w written
-      FSI_CUDA(cudaEventRecord(m->kry_ev[j], m->stream));
-      // the pass-2 update (only when the DGKS test asked for it), the new basis vector and the next input
+      // the pass-2 update (only when the DGKS test asked for it), the new basis vector and the next
+      // input; in its last CTA the Givens step and the estimate
       if constexpr (F32) {
-        FSI_LAUNCH(m, P_KRY_UPD, upd_store4_kernel<<<upd_grid(n, 4), VB, 0, m->stream>>>(
-                                     w, reinterpret_cast<float*>(V), M1, j + 1, K, n, m->dinv, reinterpret_cast<float*>(zn)));
+        FSI_LAUNCH(m, P_KRY_UPD, upd_store4_kernel<<<upd_grid(n, 4) + 1, VB, 0, m->stream>>>(
+                                     w, reinterpret_cast<float*>(V), M1, j + 1, K, n, m->dinv,
+                                     reinterpret_cast<float*>(zn), mm, est + 3 * j));
       } else {
-        FSI_LAUNCH(m, P_KRY_UPD, upd_store_kernel<<<upd_grid(n, 1), VB, 0, m->stream>>>(
-                                     w, reinterpret_cast<double*>(V), M1, j + 1, K, n, m->dinv, reinterpret_cast<double*>(zn)));
+        FSI_LAUNCH(m, P_KRY_UPD, upd_store_kernel<<<upd_grid(n, 1) + 1, VB, 0, m->stream>>>(
+                                     w, reinterpret_cast<double*>(V), M1, j + 1, K, n, m->dinv,
+                                     reinterpret_cast<double*>(zn), mm, est + 3 * j));
       }
+      FSI_CUDA(cudaEventRecord(m->kry_ev[j], m->stream));
       prof_bytes(m, P_KRY_UPD, 2 * wb + 2 * vb);  // w and dinv read, V_{j+1} and z written
       ++*iters;
       jend = j + 1;
