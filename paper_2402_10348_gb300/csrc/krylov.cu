@@ -146,25 +146,50 @@ __device__ __forceinline__ void block_reduce_store_bf(double (&acc)[K], int kc, 
   }
 }
 
-// The same in float32 up to the CTA's sums, which are stored as float64: this GPU
-// issues float64 adds at 1/64 of the float32 rate, so a float64 tree over every
-// thread's sums costs more than the float32 basis kernel's streaming.
-template <int K>
-__device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, double* out, int stride) {
-  __shared__ float smf[K][VB / 32];
+// The same in float32 up to the CTA's sums, which are stored as float64: this GPU issues float64
+// adds at 1/64 of the float32 rate, so a float64 tree over every thread's sums costs more than
+// the float32 basis kernel's streaming.  Values in groups of 8 by the transposing butterfly (9
+// shuffles a group against 40 for plain trees: with a few basis chunks a thread, the trees took as
+// long as the streaming), the last ones by plain trees.  NT threads.  out[i * stride], i < kc; with
+// tail the row kc - 1 is the last value's sum.
+template <int K, int NT>
+__device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, bool tail, double* out, int stride) {
+  __shared__ float smf[K][NT / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int KG = K / 8 * 8;
 #pragma unroll
-  for (int i = 0; i < K; ++i) {
+  for (int i0 = 0; i0 < KG; i0 += 8) {
+    float a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = acc[i0 + q];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const int o = 16 >> l, half = 4 >> l;
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int q = 0; q < half; ++q) {
+        const float send = up ? a[q] : a[q + half], keep = up ? a[q + half] : a[q];
+        a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    float v = a[0];
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if ((lane & 3) == 0) smf[i0 + (lane >> 2)][warp] = v;
+  }
+#pragma unroll
+  for (int i = KG; i < K; ++i) {
     float v = acc[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if (lane == 0) smf[i][warp] = v;
   }
   __syncthreads();
-  if (threadIdx.x < kc) {
+  for (int i = threadIdx.x; i < kc; i += NT) {
     float s = 0.f;
-    for (int wi = 0; wi < VB / 32; ++wi) s += smf[threadIdx.x][wi];
-    out[threadIdx.x * stride] = (double)s;
+#pragma unroll
+    for (int wi = 0; wi < NT / 32; ++wi) s += smf[tail && i == kc - 1 ? K - 1 : i][wi];
+    out[i * stride] = (double)s;
   }
 }
 
@@ -257,7 +282,7 @@ __global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int 
 // basis vector), so a warp moves as many bytes per load as with a float64 basis and
 // keeps as many in flight.  Elements at or past n (the ragged end of the last chunk,
 // whose basis slots hold stale bytes) are never read.
-__global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, int M1, int k,
+__global__ void __launch_bounds__(VB, 4) mdot4_kernel(const float* __restrict__ V, int M1, int k,
                                                    const double* __restrict__ w, int64_t n, double* part, KryDev* K) {
   constexpr int KC = DCH, NR = DCH + 1;
   const int G = gridDim.x;
@@ -303,10 +328,7 @@ __global__ void __launch_bounds__(VB) mdot4_kernel(const float* __restrict__ V, 
     }
     if (self) acc[KC] += (w0 * w0 + w1 * w1) + (w2 * w2 + w3 * w3);
   }
-#pragma unroll
-  for (int i = 0; i < KC; ++i)
-    if (i == kc) acc[i] = acc[KC];  // w . w goes to row k
-  block_reduce_store_f<NR>(acc, kc + (self ? 1 : 0), part + (int64_t)ib * G + blockIdx.x, G);
+  block_reduce_store_f<NR, VB>(acc, kc + (self ? 1 : 0), self, part + (int64_t)ib * G + blockIdx.x, G);
   if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows<4>(part, G, k + 1, K->h);
 }
 
@@ -585,24 +607,23 @@ __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, co
 
 // The fused update for the float32 basis: a thread takes two adjacent elements of each
 // chunk (one float2 per basis vector, one double2 of w), so a warp moves as many bytes
-// per load as with a float64 basis.  Elements at or past n are never read.
+// per load as with a float64 basis, and keeps the projections in registers.  Elements at or past n
+// are never read.
 template <int KMAX>
 __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, const float* __restrict__ V, int M1,
                                                        int k, int64_t n, double* part, KryDev* K) {
-  extern __shared__ __align__(16) unsigned char upd_smem[];
-  const double* h = K->h;
-  float* sacc = reinterpret_cast<float*>(upd_smem);  // [KMAX + 1][UDB]
-  __shared__ float hs[KMAX];
+  __shared__ float nhs[KMAX];
   const int t = threadIdx.x;
-  for (int i = t; i < KMAX; i += UDB) hs[i] = i < k ? (float)h[i] : 0.f;
-  for (int i = 0; i <= KMAX; ++i) sacc[i * UDB + t] = 0.f;
+  for (int i = t; i < KMAX; i += UDB) nhs[i] = i < k ? -(float)K->h[i] : 0.f;
   __syncthreads();
   const int G = gridDim.x;
   const int64_t nch = (n + CH - 1) / CH;
   const int64_t per = (nch + G - 1) / G;
   const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
   const int e0 = 2 * t;
-  float nrm = 0.f;
+  float acc[KMAX + 1];
+#pragma unroll
+  for (int i = 0; i <= KMAX; ++i) acc[i] = 0.f;
   for (int64_t c = c0; c < c1; ++c) {
     const int64_t j = c * CH + e0;
     if (j >= n) break;
@@ -619,48 +640,37 @@ __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, c
     float sx0 = 0.f, sx1 = 0.f, sy0 = 0.f, sy1 = 0.f;
 #pragma unroll
     for (int i = 0; i < KMAX; i += 2) {
-      sx0 += hs[i] * v[i].x;
-      sx1 += hs[i + 1] * v[i + 1].x;
-      sy0 += hs[i] * v[i].y;
-      sy1 += hs[i + 1] * v[i + 1].y;
+      sx0 = fmaf(nhs[i], v[i].x, sx0);
+      sx1 = fmaf(nhs[i + 1], v[i + 1].x, sx1);
+      sy0 = fmaf(nhs[i], v[i].y, sy0);
+      sy1 = fmaf(nhs[i + 1], v[i + 1].y, sy1);
     }
-    float wx, wy;
+    float wx, wy = 0.f;
     if (pair) {
       const double2 wd = *reinterpret_cast<const double2*>(w + j);
-      wx = (float)wd.x - (sx0 + sx1);
-      wy = (float)wd.y - (sy0 + sy1);
+      wx = (float)wd.x + (sx0 + sx1);
+      wy = (float)wd.y + (sy0 + sy1);
       *reinterpret_cast<double2*>(w + j) = make_double2((double)wx, (double)wy);
     } else {
-      wx = (float)w[j] - (sx0 + sx1);
-      wy = 0.f;
+      wx = (float)w[j] + (sx0 + sx1);
       w[j] = (double)wx;
     }
-    nrm += wx * wx + wy * wy;
+    acc[KMAX] += wx * wx + wy * wy;
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) sacc[i * UDB + t] += v[i].x * wx + v[i].y * wy;
+    for (int i = 0; i < KMAX; ++i) acc[i] += v[i].x * wx + v[i].y * wy;
   }
-  sacc[KMAX * UDB + t] = nrm;
-  __syncthreads();
-  // one warp per row, lanes on consecutive columns (no bank conflicts), float32 sums
-  const int lane = t & 31;
-  for (int i = t >> 5; i <= k; i += UDB / 32) {
-    const float* rp = sacc + (i < k ? i : KMAX) * UDB;
-    float s = (rp[lane] + rp[lane + 32]) + (rp[lane + 64] + rp[lane + 96]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) part[(int64_t)i * G + blockIdx.x] = (double)s;
-  }
+  // rows i < k the projections, row k the norm
+  block_reduce_store_f<KMAX + 1, UDB>(acc, k + 1, true, part + blockIdx.x, G);
   if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1);
 }
 
 template <int KMAX, typename VT>
 static int launch_upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n) {
   KryDev* K = static_cast<KryDev*>(m->kry_dev);
-  const size_t smem = sizeof(VT) * (size_t)(KMAX + 1) * UDB;
   if constexpr (sizeof(VT) == 4) {
-    if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot2_kernel<KMAX>), smem)) return rc;
-    upd_dot2_kernel<KMAX><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
+    upd_dot2_kernel<KMAX><<<G, UDB, 0, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
   } else {
+    const size_t smem = sizeof(VT) * (size_t)(KMAX + 1) * UDB;
     if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot_kernel<KMAX, VT>), smem)) return rc;
     upd_dot_kernel<KMAX, VT><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
   }
@@ -717,18 +727,58 @@ __global__ void precond_kernel(const VT* __restrict__ V, int M1, int slot, const
 }
 
 // x += dinv * sum_i y_i V_i
-template <typename VT>
 __global__ void __launch_bounds__(VB) combine_kernel(double* __restrict__ x, const double* __restrict__ dinv,
-                                                     const VT* __restrict__ V, int M1, int k, const KryDev* K,
-                                                     int64_t n) {
-  __shared__ VT ys[MMAX];
-  for (int i = threadIdx.x; i < k; i += VB) ys[i] = (VT)K->y[i];
+                                                     const double* __restrict__ V, int M1, int k,
+                                                     const KryDev* __restrict__ K, int64_t n) {
+  __shared__ double ys[MMAX];
+  for (int i = threadIdx.x; i < k; i += VB) ys[i] = K->y[i];
   __syncthreads();
   const int64_t nch = (n + CH - 1) / CH;
   for (int64_t c = blockIdx.x; c < nch; c += gridDim.x) {
     const int64_t j = c * CH + threadIdx.x;
     if (j >= n) continue;
-    x[j] += dinv[j] * (double)lin_comb_chunk<VT>(ys, V + c * (int64_t)M1 * CH + threadIdx.x, k);
+    x[j] += dinv[j] * lin_comb_chunk<double>(ys, V + c * (int64_t)M1 * CH + threadIdx.x, k);
+  }
+}
+
+// the same from the float32 basis, four adjacent elements a thread (upd_store4_kernel's layout)
+__global__ void __launch_bounds__(VB) combine4_kernel(double* __restrict__ x, const double* __restrict__ dinv,
+                                                      const float* __restrict__ V, int M1, int k,
+                                                      const KryDev* __restrict__ K, int64_t n) {
+  __shared__ float ys[MMAX];
+  for (int i = threadIdx.x; i < k; i += VB) ys[i] = (float)K->y[i];
+  __syncthreads();
+  const int64_t nch = (n + CH - 1) / CH;
+  const int sub = threadIdx.x >> 6, e0 = (threadIdx.x & 63) * 4;
+  for (int64_t c = (int64_t)blockIdx.x * 4 + sub; c < nch; c += (int64_t)gridDim.x * 4) {
+    const int64_t j = c * CH + e0;
+    if (j >= n) break;
+    const float* blk = V + c * (int64_t)M1 * CH + e0;
+    if (j + 4 <= n) {
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+      int i = 0;
+#pragma unroll 4
+      for (; i + 2 <= k; i += 2) {
+        const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
+        const float4 v1 = *reinterpret_cast<const float4*>(blk + (i + 1) * CH);
+        a.x += ys[i] * v0.x; a.y += ys[i] * v0.y; a.z += ys[i] * v0.z; a.w += ys[i] * v0.w;
+        b.x += ys[i + 1] * v1.x; b.y += ys[i + 1] * v1.y; b.z += ys[i + 1] * v1.z; b.w += ys[i + 1] * v1.w;
+      }
+      if (i < k) {
+        const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
+        a.x += ys[i] * v0.x; a.y += ys[i] * v0.y; a.z += ys[i] * v0.z; a.w += ys[i] * v0.w;
+      }
+      x[j] += dinv[j] * (double)(a.x + b.x);
+      x[j + 1] += dinv[j + 1] * (double)(a.y + b.y);
+      x[j + 2] += dinv[j + 2] * (double)(a.z + b.z);
+      x[j + 3] += dinv[j + 3] * (double)(a.w + b.w);
+    } else {
+      for (int e = 0; e < 4 && j + e < n; ++e) {
+        float s = 0.f;
+        for (int i = 0; i < k; ++i) s += ys[i] * blk[i * CH + e];
+        x[j + e] += dinv[j + e] * (double)s;
+      }
+    }
   }
 }
 
@@ -1064,9 +1114,10 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
     FSI_LAUNCH(m, P_KRY_SMALL, lsq_kernel<<<1, VB, 0, m->stream>>>(K, jend, mm));
     if (pc) {
       FSI_LAUNCH(m, P_KRYLOV, zcombine_kernel<<<G, VB, 0, m->stream>>>(x, m->Z, jend, K, n));
+    } else if constexpr (F32) {
+      FSI_LAUNCH(m, P_KRYLOV, combine4_kernel<<<upd_grid(n, 4), VB, 0, m->stream>>>(x, m->dinv, V, M1, jend, K, n));
     } else {
-      FSI_LAUNCH(m, P_KRYLOV, combine_kernel<VT><<<cgrid((n + CH - 1) / CH), VB, 0, m->stream>>>(x, m->dinv, V, M1,
-                                                                                                jend, K, n));
+      FSI_LAUNCH(m, P_KRYLOV, combine_kernel<<<upd_grid(n, 1), VB, 0, m->stream>>>(x, m->dinv, V, M1, jend, K, n));
     }
     // true residual r = b - A x
     if ((rc = op_jvp(m, blk, x, t, flags))) return rc;
