@@ -18,9 +18,10 @@ import torch  # noqa: E402
 
 from oracle import ac, cgt, ns  # noqa: E402
 from oracle.fields import Problem, State  # noqa: E402
+from oracle.tet import TetProblem  # noqa: E402
 from paper_2402_10348_gb300 import fsi  # noqa: E402
 from tests.helpers import desc_small  # noqa: E402
-from workloads import random_state  # noqa: E402
+from workloads import random_state, tet_box_mesh  # noqa: E402
 
 TOL64 = 1e-10
 GAMMA, BETA = 0.37, -0.21
@@ -69,3 +70,43 @@ def test_assembly_in_several_slabs_of_layers():
         y = torch.zeros_like(x)
         fsi.fsi_jvp(g.mesh, block, *g.st(), x, y)
         _agree(rel, rhs.cpu().numpy(), y.cpu().numpy())
+
+
+def _tet_solve(d, coords, conn, st, aug=True):
+    mesh = fsi.fsi_create_tet_mesh(d, coords, conn)
+    fsi.fsi_set_stream(mesh)
+    dst = [T(a) for a in st]
+    rhs = T(np.random.default_rng(3).normal(size=4 * d.nn))
+    x = torch.zeros_like(rhs)
+    o = fsi.solve_opts(m=8, max_iter=16, rtol=1e-14, flags=fsi.FSI_ELASTIC_AUG if aug else 0)
+    info = fsi.fsi_gmres(mesh, fsi.FSI_BLOCK_NS, *dst, rhs, x, o, allow_noconv=True)
+    return mesh, dst, x, rhs.cpu().numpy(), info.rel_res
+
+
+# nodes below, at and above slices of 32 (8; 4 x 4 x 2 = 32; 60; 420)
+@pytest.mark.parametrize("n,kw", [((1, 1, 1), {}), ((3, 3, 1), dict(n_solid=2)), ((4, 3, 2), dict(rho_inf=0.5)),
+                                  ((9, 5, 6), dict(n_solid=2, rho_inf=0.5))])
+def test_assembled_tetrahedra_match_the_oracle(n, kw):
+    d = desc_small(n=n, **kw)
+    st = random_state(d, 4)
+    pb, os = TetProblem(d, jitter=0.25, seed=3), State(*st)
+    for aug in (True, False):
+        _, _, x, rhs, rel = _tet_solve(d, pb.mesh.X, pb.mesh.conn, st, aug)
+        _agree(rel, rhs, ns.ns_jvp(pb, os, x.cpu().numpy().reshape(4, -1), elastic_aug=aug).ravel())
+
+
+def test_tetrahedra_with_a_row_too_long_for_the_slices():
+    """Node 0 shares elements with more nodes than a row holds: the element matrices are applied."""
+    d = desc_small(n=(6, 6, 6))
+    X, conn = tet_box_mesh(d, 0.1, 5)
+    others = np.random.default_rng(0).permutation(np.arange(1, d.nn))[: (d.nn - 1) // 3 * 3].reshape(-1, 3)
+    extra = np.concatenate([np.zeros((len(others), 1), dtype=conn.dtype), others], axis=1)
+    e = [X[:, extra[:, a]] - X[:, extra[:, 0]] for a in (1, 2, 3)]
+    vol = np.einsum("ie,ie->e", e[0], np.cross(e[1].T, e[2].T).T)
+    extra[vol < 0] = extra[vol < 0][:, [0, 2, 1, 3]]
+    extra = extra[np.abs(vol) > 1e-6]
+    assert 3 * len(extra) > 100
+    mesh, dst, x, rhs, rel = _tet_solve(d, X, np.concatenate([conn, extra]), random_state(d, 4))
+    y = torch.zeros_like(x)
+    fsi.fsi_jvp(mesh, fsi.FSI_BLOCK_NS, *dst, x, y)
+    _agree(rel, rhs, y.cpu().numpy())
