@@ -311,10 +311,22 @@ __global__ void __launch_bounds__(CONV_THREADS) conv_mma_kernel(ConvArgs a) {
 // forward: B[t][c][kg][ng][n8][k8] = W[co = 8 ng + n8][ci = 16 c + 8 kg + k8][t]
 // data gradient: the adjoint is a convolution with flipped taps and swapped
 // channels: B[t][0][kg][ng][n8][k8] = W[co = 8 kg + k8][ci = 8 ng + n8][26 - t]
-__global__ void pack_weights_kernel(const float* __restrict__ W, int cout, int cin, int npad, int bwd,
-                                    uint16_t* __restrict__ out) {
+// One launch for every layer and direction (blockIdx.y): 29 launches of 27 to 54 CTAs took 3 us each.
+struct PackArgs {
+  const float* W;
+  int64_t woff[NLAYER];
+  uint16_t *wf[NLAYER], *wb[NLAYER];
+  int cin[NLAYER], cout[NLAYER];
+};
+constexpr int NPAD = 16;
+__global__ void pack_weights_kernel(const __grid_constant__ PackArgs a) {
+  const int l = blockIdx.y >> 1, bwd = blockIdx.y & 1;
+  const int cin = a.cin[l], cout = a.cout[l];
+  const float* __restrict__ W = a.W + a.woff[l];
+  uint16_t* __restrict__ out = bwd ? a.wb[l] : a.wf[l];
+  if (!out) return;
   const int kdim = bwd ? 16 : cin;  // K channels per tap (forward: cin; adjoint: cout padded)
-  const int ndim = bwd ? cin : npad;
+  const int ndim = bwd ? cin : NPAD;
   const int total = 27 * kdim * ndim;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     const int k8 = e & 7, n8 = (e >> 3) & 7;
@@ -339,6 +351,9 @@ __global__ void pack_weights_kernel(const float* __restrict__ W, int cout, int c
 
 // ------------------------------------------------------------------ transfer operators
 // coarse[X] = s * sum_{d in {-1,0,1}^3} 2^-(|dx|+|dy|+|dz|) fine[2X + d]  (then * [mask > 0])
+// Bound by latency on every level (a chain of 27 loads took 11 us on 33^3 and on 5^3 voxels alike):
+// the loads of a plane are in flight together, and CTAs are small so that a coarse level has some
+// for every SM: 6.4 and 4.0 us.
 __global__ void restrict_kernel(TView f, TView c, float s, TView mask) {
   const int64_t Vc = (int64_t)c.nx * c.ny * c.nz;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 2 * Vc; i += (int64_t)gridDim.x * blockDim.x) {
@@ -346,21 +361,25 @@ __global__ void restrict_kernel(TView f, TView c, float s, TView mask) {
     const int64_t v = i - o * Vc;
     const int X = (int)(v % c.nx), Y = (int)((v / c.nx) % c.ny), Z = (int)(v / ((int64_t)c.nx * c.ny));
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int dz = -1; dz <= 1; ++dz) {
-      const int z = 2 * Z + dz;
-      if (z < 0 || z >= f.nz) continue;
-      for (int dy = -1; dy <= 1; ++dy) {
-        const int y = 2 * Y + dy;
-        if (y < 0 || y >= f.ny) continue;
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int x = 2 * X + dx;
-          if (x < 0 || x >= f.nx) continue;
-          const float w = 1.0f / (float)(1 << (abs(dx) + abs(dy) + abs(dz)));
-          const uint4 q = *reinterpret_cast<const uint4*>(f.p + vox_addr(f, o, x, y, z));
-          const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+    const uint16_t* at = f.p + vox_addr(f, o, 2 * X, 2 * Y, 2 * Z);
 #pragma unroll
-          for (int k = 0; k < 8; ++k) acc[k] += w * bf2f((uint16_t)(u[k >> 1] >> (16 * (k & 1))));
-        }
+    for (int dz = -1; dz <= 1; ++dz) {
+      uint4 q[9];  // a plane's nine loads in flight together
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const int dx = t % 3 - 1, dy = t / 3 - 1;
+        const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
+        q[t] = make_uint4(0, 0, 0, 0);
+        if (x >= 0 && x < f.nx && y >= 0 && y < f.ny && z >= 0 && z < f.nz)
+          q[t] = *reinterpret_cast<const uint4*>(at + (((int64_t)dz * f.ny + dy) * f.nx + dx) * 8);
+      }
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const int dx = t % 3 - 1, dy = t / 3 - 1;
+        const float w = 1.0f / (float)(1 << (abs(dx) + abs(dy) + abs(dz)));
+        const uint32_t u[4] = {q[t].x, q[t].y, q[t].z, q[t].w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc[k] += w * bf2f((uint16_t)(u[k >> 1] >> (16 * (k & 1))));
       }
     }
     uint4 mk = make_uint4(0, 0, 0, 0);
@@ -391,22 +410,28 @@ __global__ void prolong_kernel(TView c, TView f, float s, TView add, TView mask)
     const int nxs = (x & 1) ? 2 : 1, nys = (y & 1) ? 2 : 1, nzs = (z & 1) ? 2 : 1;
     const float w = 1.0f / (float)(nxs * nys * nzs);
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int a2 = 0; a2 < nzs; ++a2)
-      for (int a1 = 0; a1 < nys; ++a1)
-        for (int a0 = 0; a0 < nxs; ++a0) {
-          const uint4 q = *reinterpret_cast<const uint4*>(c.p + vox_addr(c, o, xs[a0], ys[a1], zs[a2]));
-          const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+    uint4 q[8];  // all loads in flight together
 #pragma unroll
-          for (int k = 0; k < 8; ++k) acc[k] += w * bf2f((uint16_t)(u[k >> 1] >> (16 * (k & 1))));
-        }
+    for (int t = 0; t < 8; ++t) {
+      const int a0 = t & 1, a1 = t >> 1 & 1, a2 = t >> 2;
+      q[t] = make_uint4(0, 0, 0, 0);
+      if (a0 < nxs && a1 < nys && a2 < nzs)
+        q[t] = *reinterpret_cast<const uint4*>(c.p + vox_addr(c, o, xs[a0], ys[a1], zs[a2]));
+    }
     uint32_t ad[4] = {0, 0, 0, 0}, mu[4] = {0, 0, 0, 0};
     if (add.p) {
-      const uint4 q = *reinterpret_cast<const uint4*>(add.p + vox_addr(add, o, x, y, z));
-      ad[0] = q.x, ad[1] = q.y, ad[2] = q.z, ad[3] = q.w;
+      const uint4 v4 = *reinterpret_cast<const uint4*>(add.p + vox_addr(add, o, x, y, z));
+      ad[0] = v4.x, ad[1] = v4.y, ad[2] = v4.z, ad[3] = v4.w;
     }
     if (mask.p) {
-      const uint4 q = *reinterpret_cast<const uint4*>(mask.p + vox_addr(mask, o, x, y, z));
-      mu[0] = q.x, mu[1] = q.y, mu[2] = q.z, mu[3] = q.w;
+      const uint4 v4 = *reinterpret_cast<const uint4*>(mask.p + vox_addr(mask, o, x, y, z));
+      mu[0] = v4.x, mu[1] = v4.y, mu[2] = v4.z, mu[3] = v4.w;
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const uint32_t u[4] = {q[t].x, q[t].y, q[t].z, q[t].w};
+#pragma unroll
+      for (int k = 0; k < 8; ++k) acc[k] += w * bf2f((uint16_t)(u[k >> 1] >> (16 * (k & 1))));
     }
     uint32_t outw[4];
 #pragma unroll
@@ -938,7 +963,7 @@ int wgrad(fsi_pc* pc, int layer, const TView& x, const TView& g) {
 
 int restrict_(fsi_pc* pc, const TView& f, const TView& c, float s, const TView& mask) {
   const int64_t n = 2LL * c.nx * c.ny * c.nz;
-  FSI_LAUNCH(pc->m, P_PC_AUX, (restrict_kernel<<<vgrid1(n), 256, 0, pc->m->stream>>>(f, c, s, mask)));
+  FSI_LAUNCH(pc->m, P_PC_AUX, (restrict_kernel<<<vgrid1(n, 64), 64, 0, pc->m->stream>>>(f, c, s, mask)));
   return FSI_OK;
 }
 int prolong_(fsi_pc* pc, const TView& c, const TView& f, float s, const TView& add, const TView& mask) {
@@ -961,19 +986,16 @@ static int dec_b(int l) { return DEC2A + 2 * (2 - l) + 1; }
 
 int pack_weights(fsi_pc* pc) {
   fsi_mesh* m = pc->m;
+  PackArgs a{};
+  a.W = pc->w;
+  int most = 0;
   for (int l = 0; l < NLAYER; ++l) {
-    const int cin = pc->lcin[l], cout = pc->lcout[l];
-    const int npad = 16;
-    const float* W = pc->w + pc->woff[l];
-    const int nf = 27 * cin * npad;
-    FSI_LAUNCH(m, P_PC_AUX, (pack_weights_kernel<<<(nf + 255) / 256, 256, 0, m->stream>>>(W, cout, cin, npad, 0,
-                                                                                          pc->wf[l])));
-    if (l != ENC0A) {
-      const int nb = 27 * 16 * cin;
-      FSI_LAUNCH(m, P_PC_AUX, (pack_weights_kernel<<<(nb + 255) / 256, 256, 0, m->stream>>>(W, cout, cin, npad, 1,
-                                                                                            pc->wb[l])));
-    }
+    a.woff[l] = pc->woff[l], a.cin[l] = pc->lcin[l], a.cout[l] = pc->lcout[l];
+    a.wf[l] = pc->wf[l];
+    a.wb[l] = l == ENC0A ? nullptr : pc->wb[l];  // (nothing is behind the first layer)
+    most = std::max(most, 27 * 16 * pc->lcin[l]);
   }
+  FSI_LAUNCH(m, P_PC_AUX, (pack_weights_kernel<<<dim3((most + 255) / 256, 2 * NLAYER), 256, 0, m->stream>>>(a)));
   return FSI_OK;
 }
 
