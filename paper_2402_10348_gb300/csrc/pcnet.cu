@@ -493,192 +493,175 @@ __global__ void prolong_f32_kernel(const float* __restrict__ c, Grid3 gc, float*
 }
 
 // ------------------------------------------------------------------ weight gradient
-// g[(co cin + ci) 27 + t] = sum_b part[b][co][ci][t] for co < cout, in a fixed order: a CTA takes 32
-// weights, its warps every WGR-th block, and warp 0 adds the warps' sums (one thread per weight over
-// all blocks ran 57 us on 912 blocks, a chain of loads in 27 CTAs; now 8)
+// g[(co cin + ci) 27 + t] = sum_b part[b][a][co][dz cin + ci] for co < cout (a = the (dy, dx) tap), in a
+// fixed order: a CTA takes 32 sums, its warps every WGR-th block, and warp 0 adds the warps' sums (one
+// thread per weight over all blocks ran 57 us on 912 blocks, a chain of loads in 27 CTAs)
 constexpr int WGR = 32;
 __global__ void __launch_bounds__(32 * WGR) wgrad_reduce_kernel(const float* __restrict__ part, int nblk, int cin, int cout,
                                                                 float* __restrict__ g) {
   __shared__ float sm[WGR][32];
-  const int n = cout * cin * 27, stride = 16 * cin * 27;
+  const int stride = 16 * cin * 27;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
+  const int m = e % (3 * cin), co = e / (3 * cin) % 16, a = e / (3 * cin * 16);
+  const bool in = e < stride && co < cout;
   float s = 0.0f;
-  if (e < n) {
+  if (in) {
 #pragma unroll 8
     for (int b = w; b < nblk; b += WGR) s += part[(int64_t)b * stride + e];
   }
   sm[w][lane] = s;
   __syncthreads();
-  if (w == 0 && e < n) {
+  if (w == 0 && in) {
     float t = 0.0f;
 #pragma unroll
     for (int q = 0; q < WGR; ++q) t += sm[q][lane];
-    g[e] = t;
+    g[((int64_t)co * cin + m % cin) * 27 + m / cin * 9 + a] = t;
   }
 }
 
 // ------------------------------------------------------------------ weight gradient on tensor cores
-// dW[co][ci][t] = sum_v dY[v][co] X[v + delta_t][ci] as implicit GEMMs, one per group of
-// MT = 128 / CIN taps: D[(t_local, ci)][co] (M = 128, N = 16) accumulates over K = voxels,
-// 16 voxels per tcgen05.mma.  Both operands are staged K-major without swizzle (core
-// matrix = 8 rows x 8 voxels, the layout the convolution's B operand uses):
-// A[m][k] = X[v_k + delta_t(m)][ci(m)], B[co][k] = dY[v_k][co].  Each CTA walks a
-// contiguous range of voxels with double-buffered staging; its TMEM accumulators (16
-// columns per tap group) become per-CTA partials in the [co][ci][27] layout that
-// wgrad_reduce_kernel sums in a fixed order.
-//
-// The MMAs are a small part; staging is what takes the time.  A thread keeps one voxel of the stage (its
-// index divisions once a stage), loads its taps' channel octets for the next stage while the current
-// one is stored, and eight lanes transpose 8 voxels x 8 channels among themselves (6 shuffles) into one
-// 16-byte store a lane, where each octet used to be eight 2-byte stores on the same banks.  64^3, 16
-// channels: 61 -> 35 us, 32: 176 -> 85 us.
-constexpr int WGM_THREADS = 128;
-constexpr int WGM_KS = 16;  // voxels per stage: one MMA K-step
+// dW[co][ci][t] = sum_v dY[v][co] X[v + delta_t][ci] as implicit GEMMs over voxels (K), one per tap
+// (dy, dx): D[(dz, ci)][co], M = 128, N = 16, 16 voxels (8 along x, 2 rows) per tcgen05.mma.
+// Both operands lie in shared memory as they lie in global memory, 16 bytes = 8 channels of a
+// voxel, and are read M/N-major: a core matrix is 8 voxels x 8 channels, K groups are rows apart
+// (LBO), M groups octet planes apart (SBO).  A tap's shift by dx and dy moves the start address; the
+// octet planes of consecutive z planes are M groups of one matrix, so the three dz of a tap are one
+// MMA (M rows past 3 CIN read whatever follows inside the allocation and are not stored).
+// A work unit is 8 x 16 voxels of 4 z planes: its 6 input planes with their halo (180 x 16 bytes
+// an octet) and the gradient's 4 are copied by cp.async into one of two stages while the other's 288
+// MMAs run; warp 0 issues those, the other eight copy.  Each CTA walks a contiguous range of units with
+// the nine accumulators in TMEM (144 columns) and writes them once, as rows of consecutive M
+// that wgrad_reduce_kernel sums in a fixed order.
+// Staging the 27 shifted copies of every voxel, transposed by shuffles, took 72 us on 64^3 (16
+// channels) and 177 (32); now 44 and 61.
+constexpr int WGM_LOADERS = 256;
+constexpr int WGM_THREADS = 32 + WGM_LOADERS;
+constexpr int WGM_P = 4;  // z planes of a unit
 
 template <int CIN>
 struct WgmCfg {
-  static constexpr int MT = 128 / CIN;             // taps per group
-  static constexpr int NG = (27 + MT - 1) / MT;    // tap groups
-  static constexpr int ABYTES = 128 * WGM_KS * 2;  // one group's A tile
-  static constexpr int BBYTES = 16 * WGM_KS * 2;
-  static constexpr int STAGE = NG * ABYTES + BBYTES;
+  static constexpr int NO = CIN / 8;
+  static constexpr int SLOT = NO * OCT_BYTES;                  // one staged input plane
+  static constexpr int XBYTES = (WGM_P + 2) * SLOT;
+  static constexpr int GOCT = TILE_X * TILE_Y * 16;            // one octet of a gradient plane
+  static constexpr int STAGE = XBYTES + WGM_P * 2 * GOCT;
   static constexpr int HEAD = 128;
-  static constexpr int SMEM = HEAD + 2 * STAGE;
-  static constexpr int NCOLS = NG * 16 <= 32 ? 32 : (NG * 16 <= 64 ? 64 : 128);
+  // the last plane's matrix spans 16 octet planes from its start, past the stage's end for CIN = 16
+  static constexpr int SPAN = (WGM_P - 1) * SLOT + 16 * OCT_BYTES;
+  static constexpr int SMEM = HEAD + STAGE + (SPAN > STAGE ? SPAN : STAGE);
+  static constexpr int NCOLS = 256;                            // nine accumulators of 16
 };
 
-// 8 x 8 transposition of 16-bit values over 8 adjacent lanes: lane l holds column l (channels 0..7 of
-// voxel l) and gets row l (channel l of voxels 0..7)
-__device__ __forceinline__ uint4 transpose8(uint4 q, int l) {
-  const bool b2 = l & 4, b1 = l & 2, b0 = l & 1;
-  // distance 4: channels 0-3 stay with the lower lanes, 4-7 with the upper
-  const uint32_t p0 = __shfl_xor_sync(0xffffffffu, b2 ? q.x : q.z, 4), p1 = __shfl_xor_sync(0xffffffffu, b2 ? q.y : q.w, 4);
-  const uint32_t x00 = b2 ? p0 : q.x, x01 = b2 ? p1 : q.y, x10 = b2 ? q.z : p0, x11 = b2 ? q.w : p1;
-  // distance 2: one pair of channels
-  const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b1 ? x00 : x01, 2), r1 = __shfl_xor_sync(0xffffffffu, b1 ? x10 : x11, 2);
-  const uint32_t z00 = b1 ? r0 : x00, z01 = b1 ? x01 : r0, z10 = b1 ? r1 : x10, z11 = b1 ? x11 : r1;
-  // distance 1: one channel
-  const uint32_t ss = b0 ? 0x5410u : 0x7632u;
-  const uint32_t t0 = __shfl_xor_sync(0xffffffffu, __byte_perm(z00, z01, ss), 1);
-  const uint32_t t1 = __shfl_xor_sync(0xffffffffu, __byte_perm(z10, z11, ss), 1);
-  const uint32_t s0 = b0 ? 0x3254u : 0x5410u, s1 = b0 ? 0x3276u : 0x7610u;
-  return make_uint4(__byte_perm(z00, t0, s0), __byte_perm(z01, t0, s1), __byte_perm(z10, t1, s0), __byte_perm(z11, t1, s1));
+struct WgmGrid {
+  int tx, ty, units;
+};
+__host__ __device__ inline WgmGrid wgm_grid(const TView& g) {
+  WgmGrid w;
+  w.tx = (g.nx + TILE_X - 1) / TILE_X, w.ty = (g.ny + TILE_Y - 1) / TILE_Y;
+  w.units = w.tx * w.ty * ((g.nz + WGM_P - 1) / WGM_P);
+  return w;
+}
+
+// unit u = ((ty * tiles_x) + tx) * panels + panel
+template <int CIN>
+__device__ __forceinline__ void wgm_load(const TView& x, const TView& g, const WgmGrid& w, int u, uint32_t stage, int t0) {
+  using C = WgmCfg<CIN>;
+  const int panels = w.units / (w.tx * w.ty);
+  const int pz = u % panels, col = u / panels;
+  const int x0 = col % w.tx * TILE_X, y0 = col / w.tx * TILE_Y, z0 = pz * WGM_P;
+  for (int i = t0; i < (WGM_P + 2) * C::NO * SY * SX; i += WGM_LOADERS) {
+    const int pl = i / (SY * SX), rem = i - pl * (SY * SX), yy = rem / SX, xx = rem - yy * SX;
+    const int z = z0 - 1 + pl / C::NO, gx = x0 - 1 + xx, gy = y0 - 1 + yy;
+    const bool in = z >= 0 && z < x.nz && gx >= 0 && gx < x.nx && gy >= 0 && gy < x.ny;
+    cp_async16(stage + 16 * i, in ? x.p + vox_addr(x, pl % C::NO, gx, gy, z) : x.p, in);
+  }
+  for (int i = t0; i < WGM_P * 2 * TILE_X * TILE_Y; i += WGM_LOADERS) {
+    const int gx = x0 + (i & 7), gy = y0 + (i >> 3 & 15), o = i >> 7 & 1, z = z0 + (i >> 8);
+    const bool in = gx < g.nx && gy < g.ny && z < g.nz;
+    cp_async16(stage + C::XBYTES + 16 * i, in ? g.p + vox_addr(g, o, gx, gy, z) : g.p, in);
+  }
 }
 
 template <int CIN>
-__global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g, int spc, int64_t nstages,
-                                                              float* __restrict__ part, int* err) {
+__global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g, float* __restrict__ part, int* err) {
   using C = WgmCfg<CIN>;
   extern __shared__ __align__(1024) uint8_t sm[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm);
   uint32_t* holder = reinterpret_cast<uint32_t*>(sm + 16);
-  uint8_t* stage_base = sm + C::HEAD;
+  const uint32_t base = smem_u32(sm + C::HEAD);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t V = (int64_t)g.nx * g.ny * g.nz;
-  const int64_t s0 = (int64_t)blockIdx.x * spc, s1 = min(nstages, s0 + spc);
+  const WgmGrid w = wgm_grid(g);
+  const int u0 = (int)((int64_t)w.units * blockIdx.x / gridDim.x);
+  const int nu = (int)((int64_t)w.units * (blockIdx.x + 1) / gridDim.x) - u0;
+  if (nu <= 0) return;  // (not with at most one CTA per unit) uniform, before any barrier or allocation
   if (tid == 0) {
     mbar_init(smem_u32(&bars[0]), 1);
     mbar_init(smem_u32(&bars[1]), 1);
     fence_mbar_init();
   }
   if (warp == 0) tmem_alloc(smem_u32(holder), C::NCOLS);
-  // both buffers start at zero: the rows of the taps past 26 stay zero
-  for (int i = tid; i < 2 * C::STAGE / 16; i += WGM_THREADS)
-    reinterpret_cast<uint4*>(stage_base)[i] = make_uint4(0, 0, 0, 0);
+  if (warp > 0) wgm_load<CIN>(x, g, w, u0, base, tid - 32);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *holder;
-  constexpr uint32_t IDESC = idesc_bf16(16, 128);
+  // M/N-major A and B
+  constexpr uint32_t IDESC = idesc_bf16(16, 128) | (1u << 15) | (1u << 16);
   bool bad = false;
-  // items of a thread: voxel k of the stage, taps and octets r = tid / 16 + 8 j (tap r % 27)
-  constexpr int NR = 27 * (CIN / 8), NJ = (NR + 7) / 8;
-  const int k = tid & 15, r0 = tid >> 4;
-  const uint32_t nx = g.nx, ny = g.ny;
-  uint4 q[NJ], qg;
-  auto load = [&](int64_t st) {
-    const int64_t v = st * WGM_KS + k;
-    const bool in = v < V;
-    const uint32_t u = in ? (uint32_t)v : 0u, row = u / nx;
-    const int vx = (int)(u - row * nx), vz = (int)(row / ny), vy = (int)(row - (uint32_t)vz * ny);
-    const uint16_t* at = x.p + vox_addr(x, 0, vx, vy, vz);
-    const int64_t octs = (int64_t)x.nx * x.ny * x.nz * 8;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int r = r0 + 8 * j;
-      const int o = r / 27, t = r - 27 * o;
-      const int dx = t % 3 - 1, dy = t / 3 % 3 - 1, dz = t / 9 - 1;
-      const int xx = vx + dx, yy = vy + dy, zz = vz + dz;
-      q[j] = make_uint4(0, 0, 0, 0);
-      if (in && r < NR && xx >= 0 && xx < x.nx && yy >= 0 && yy < x.ny && zz >= 0 && zz < x.nz)
-        q[j] = *reinterpret_cast<const uint4*>(at + o * octs + (((int64_t)dz * x.ny + dy) * x.nx + dx) * 8);
-    }
-    qg = make_uint4(0, 0, 0, 0);
-    if (warp == 0 && in) qg = *reinterpret_cast<const uint4*>(g.p + vox_addr(g, lane >> 4, vx, vy, vz));
-  };
-  if (s0 < s1) load(s0);
-  for (int64_t st = s0; st < s1; ++st) {
-    const int it = (int)(st - s0), b = it & 1;
-    if (it >= 2) {  // the MMAs that read this buffer two stages ago are done
-      const bool ok = mbar_wait(smem_u32(&bars[b]), (uint32_t)(((it - 2) >> 1) & 1));
-      if (__syncthreads_or(!ok)) {
-        bad = true;
-        break;
-      }
-    }
-    uint16_t* A = reinterpret_cast<uint16_t*>(stage_base + b * C::STAGE);
-    uint16_t* B = reinterpret_cast<uint16_t*>(stage_base + b * C::STAGE + C::NG * C::ABYTES);
-    // A: row m = (tap in its group) CIN + channel, the octet's eight rows are one core-matrix group
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int r = r0 + 8 * j;
-      const int o = r / 27, t = r - 27 * o;
-      const uint4 w = transpose8(q[j], lane & 7);
-      if (r < NR) {
-        const int m = (t % C::MT) * CIN + o * 8 + (lane & 7);
-        *reinterpret_cast<uint4*>(A + (t / C::MT) * (C::ABYTES / 2) + ((k >> 3) * 16 + (m >> 3)) * 64 + (m & 7) * 8) = w;
-      }
-    }
-    if (warp == 0) {  // B: gradient octet lane / 16
-      const uint4 w = transpose8(qg, lane & 7);
-      *reinterpret_cast<uint4*>(B + ((k >> 3) * 2 + (lane >> 4)) * 64 + (lane & 7) * 8) = w;
-    }
-    if (st + 1 < s1) load(st + 1);
+  for (int i = 0; i < nu; ++i) {
+    const int s = i & 1;
+    cp_async_commit();
+    cp_async_wait_all();
     fence_proxy_async();
     tc_fence_before();
-    __syncthreads();
-    if (tid == 0) {
-      tc_fence_after();
-      const uint32_t abase = smem_u32(A), bbase = smem_u32(B);
-#pragma unroll 1
-      for (int gi = 0; gi < C::NG; ++gi)
-        mma_bf16(tmem + (uint32_t)(gi * 16), sdesc(abase + gi * C::ABYTES, 16 * 128, 128), sdesc(bbase, 2 * 128, 128),
-                 IDESC, it > 0 ? 1u : 0u);
-      mma_commit(smem_u32(&bars[b]));
+    if (__syncthreads_or(bad)) {
+      bad = true;
+      break;
     }
-    __syncwarp();
+    tc_fence_after();
+    if (warp == 0) {
+      if (lane == 0) {
+        const uint32_t xb = base + s * C::STAGE, gb = xb + C::XBYTES;
+        const int panels = w.units / (w.tx * w.ty);
+        const int planes = min(WGM_P, g.nz - (u0 + i) % panels * WGM_P);
+#pragma unroll 1
+        for (int z = 0; z < planes; ++z)
+#pragma unroll 1
+          for (int kk = 0; kk < TILE_Y / 2; ++kk) {
+            const uint64_t db = sdesc(gb + (z * 2) * C::GOCT + kk * 2 * TILE_X * 16, TILE_X * 16, C::GOCT);
+            const uint64_t da = sdesc(xb + z * C::SLOT + 2 * kk * SX * 16, SX * 16, OCT_BYTES);
+            const uint32_t acc = i > 0 || z > 0 || kk > 0 ? 1u : 0u;
+#pragma unroll
+            for (int a = 0; a < 9; ++a)  // (the start address is the descriptor's lowest field, in 16 bytes)
+              mma_bf16(tmem + 16 * a, da + (uint64_t)(a / 3 * SX + a % 3), db, IDESC, acc);
+          }
+        mma_commit(smem_u32(&bars[s]));
+      }
+      __syncwarp();
+    } else if (i + 1 < nu) {
+      // the other stage is free once the MMAs of unit i - 1 are done
+      if (i >= 1 && !mbar_wait(smem_u32(&bars[s ^ 1]), (uint32_t)(((i - 1) >> 1) & 1))) bad = true;
+      if (!bad) wgm_load<CIN>(x, g, w, u0 + i + 1, base + (s ^ 1) * C::STAGE, tid - 32);
+    }
   }
-  const int nst = (int)(s1 - s0);
-  if (!bad && nst > 0) {
-    const int last = nst - 1;
-    const bool ok = mbar_wait(smem_u32(&bars[last & 1]), (uint32_t)((last >> 1) & 1));
+  if (!bad) {
+    const bool ok = mbar_wait(smem_u32(&bars[(nu - 1) & 1]), (uint32_t)(((nu - 1) >> 1) & 1));
     if (__syncthreads_or(!ok)) bad = true;
   }
   if (!bad) {
     tc_fence_after();
-    const int m = warp * 32 + lane;
-    const int t_local = m / CIN, ci = m % CIN;
-    float* dst = part + (int64_t)blockIdx.x * (16 * CIN * 27);
+    if (warp < 4) {
+      const int m = warp * 32 + lane;
+      float* dst = part + (int64_t)blockIdx.x * (16 * CIN * 27) + m;
 #pragma unroll 1
-    for (int gi = 0; gi < C::NG; ++gi) {
-      uint32_t r[16];
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(gi * 16), r);
-      const int t = gi * C::MT + t_local;
-      if (t < 27) {
+      for (int a = 0; a < 9; ++a) {
+        uint32_t r[16];
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * 16), r);
+        if (m < 3 * CIN) {
 #pragma unroll
-        for (int co = 0; co < 16; ++co)
-          dst[((int64_t)co * CIN + ci) * 27 + t] = nst > 0 ? __uint_as_float(r[co]) : 0.0f;
+          for (int co = 0; co < 16; ++co) dst[(a * 16 + co) * 3 * CIN] = __uint_as_float(r[co]);
+        }
       }
     }
   } else if (tid == 0) {
@@ -934,15 +917,11 @@ int launch_wgrad_mma(fsi_pc* pc, const TView& x, const TView& g, int* nblk_out) 
   using C = WgmCfg<CIN>;
   fsi_mesh* m = pc->m;
   if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&wgrad_mma_kernel<CIN>), C::SMEM)) return rc;
-  const int64_t V = (int64_t)g.nx * g.ny * g.nz;
-  const int64_t nst = (V + WGM_KS - 1) / WGM_KS;
-  const int per_sm = std::max(1, std::min(std::min(8, 512 / C::NCOLS), (227 * 1024) / (C::SMEM + 1024)));
-  const int64_t target = (int64_t)per_sm * 152;
-  const int spc = (int)std::max<int64_t>(1, (nst + target - 1) / target);
-  const int nblk = (int)((nst + spc - 1) / spc);
+  // shared memory and 256 of 512 TMEM columns: two CTAs per SM for 16 channels, one for 32
+  const int per_sm = std::max(1, std::min(512 / C::NCOLS, (228 * 1024) / (C::SMEM + 1024)));
+  const int nblk = std::min(wgm_grid(g).units, per_sm * 152);
   if ((int64_t)nblk * 16 * CIN * 27 > pc->wpart_n) return set_error(FSI_EINVAL, "pc: weight-gradient scratch too small");
-  FSI_LAUNCH(m, P_PC_WGRAD, (wgrad_mma_kernel<CIN><<<nblk, WGM_THREADS, C::SMEM, m->stream>>>(x, g, spc, nst,
-                                                                                              pc->wpart, pc->err)));
+  FSI_LAUNCH(m, P_PC_WGRAD, (wgrad_mma_kernel<CIN><<<nblk, WGM_THREADS, C::SMEM, m->stream>>>(x, g, pc->wpart, pc->err)));
   *nblk_out = nblk;
   return FSI_OK;
 }
@@ -954,7 +933,7 @@ int wgrad(fsi_pc* pc, int layer, const TView& x, const TView& g) {
   if (cin == 16) rc = launch_wgrad_mma<16>(pc, x, g, &nblk);
   else rc = launch_wgrad_mma<32>(pc, x, g, &nblk);
   if (rc) return rc;
-  const int n = cout * cin * 27;
+  const int n = 16 * cin * 27;
   FSI_LAUNCH(m, P_PC_WGRAD, (wgrad_reduce_kernel<<<(n + 31) / 32, 32 * WGR, 0, m->stream>>>(pc->wpart, nblk, cin, cout,
                                                                                           pc->grad + pc->woff[layer])));
   pc->flops += 2.0 * (double)g.nx * g.ny * g.nz * 27.0 * cin * 16;
@@ -1318,16 +1297,9 @@ int fsi_pc_create(fsi_mesh* m, const fsi_pc_desc* d, fsi_pc** out) {
       (rc = dalloc(&pc->ys1, (int64_t)pc->cout * pc->lv[1].nv())) ||
       (rc = dalloc(&pc->loss_dev, 1 << 16)) || (rc = dalloc(&pc->err, 1)))
     return fail(rc);
-  // weight-gradient partials: room for the launch with the most CTAs over all levels
+  // weight-gradient partials: one CTA per SM with 32 input channels or two with 16
   {
-    int64_t nblk = 0;
-    for (int l = 0; l < NLEVEL; ++l) {
-      const Grid3& g = pc->lv[l];
-      const int gx = (g.nx + TILE_X - 1) / TILE_X, gy = (g.ny + TILE_Y - 1) / TILE_Y;
-      const int zc = std::max(1, (int)((int64_t)g.nz * gx * gy / (2 * 152)));
-      nblk = std::max(nblk, (int64_t)gx * gy * ((g.nz + zc - 1) / zc));
-    }
-    pc->wpart_n = std::max<int64_t>(nblk, 8 * 152) * 16 * 32 * 27;
+    pc->wpart_n = (int64_t)152 * 16 * 32 * 27;
     if ((rc = dalloc(&pc->wpart, pc->wpart_n))) return fail(rc);
   }
   pc->dmask = m->mask;
