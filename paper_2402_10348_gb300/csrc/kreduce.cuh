@@ -1,0 +1,106 @@
+// Sums across a CTA for the Krylov kernels (krylov.cu, batch.cu).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace fsi {
+
+// Sums over a CTA of several values a thread, out[i * stride] for i < kc.  Float64 values with few
+// float64 adds (this GPU issues them at a small fraction of the float32 rate; a plain shuffle tree
+// costs 5 adds a lane per value).
+// Inside a warp a transposing butterfly takes the first P values (P the largest power of
+// two <= K, at most 32): at shuffle distance 16 a lane keeps half of its values and adds
+// its partner's copy of that half, at distance 8 half of that half, and so on; after
+// log2 P levels the lane holds value number lane >> (5 - log2 P) summed over the lanes
+// that differ from it in the top log2 P bits, and plain shuffles over the remaining bits
+// finish the warp's sum (P - 1 + 5 - log2 P adds a lane).  Values past P take plain trees.
+// NT: most threads of the CTA; with tail the row kc - 1 is the last value's sum.
+template <int K, int NT>
+__device__ __forceinline__ void block_reduce_store_bf(double (&acc)[K], int kc, bool tail, double* out, int stride) {
+  constexpr int P = K >= 32 ? 32 : K >= 16 ? 16 : K >= 8 ? 8 : K >= 4 ? 4 : K >= 2 ? 2 : 1;
+  constexpr int L = P == 32 ? 5 : P == 16 ? 4 : P == 8 ? 3 : P == 4 ? 2 : P == 2 ? 1 : 0;
+  __shared__ double smb[K][NT / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double a[P];
+#pragma unroll
+  for (int q = 0; q < P; ++q) a[q] = acc[q];
+#pragma unroll
+  for (int l = 0; l < L; ++l) {
+    const int o = 16 >> l;
+    const int half = P >> (l + 1);
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int q = 0; q < half; ++q) {
+      const double send = up ? a[q] : a[q + half];  // the half the partner keeps
+      const double keep = up ? a[q + half] : a[q];
+      a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double s = a[0];
+#pragma unroll
+  for (int o = 16 >> L; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((lane & ((32 >> L) - 1)) == 0) smb[lane >> (5 - L)][warp] = s;
+#pragma unroll
+  for (int i = P; i < K; ++i) {
+    double v = acc[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) smb[i][warp] = v;
+  }
+  __syncthreads();
+  const int nw = blockDim.x >> 5;
+  for (int i = threadIdx.x; i < kc; i += blockDim.x) {
+    double t = 0.0;
+#pragma unroll
+    for (int wi = 0; wi < NT / 32; ++wi)
+      if (wi < nw) t += smb[tail && i == kc - 1 ? K - 1 : i][wi];
+    out[i * stride] = t;
+  }
+}
+
+// The same in float32 up to the CTA's sums, which are stored as float64: this GPU issues float64
+// adds at 1/64 of the float32 rate, so a float64 tree over every thread's sums costs more than
+// the float32 basis kernel's streaming.  Values in groups of 8 by the transposing butterfly (9
+// shuffles a group against 40 for plain trees: with a few basis chunks a thread, the trees took as
+// long as the streaming), the last ones by plain trees.
+template <int K, int NT>
+__device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, bool tail, double* out, int stride) {
+  __shared__ float smf[K][NT / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int KG = K / 8 * 8;
+#pragma unroll
+  for (int i0 = 0; i0 < KG; i0 += 8) {
+    float a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = acc[i0 + q];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const int o = 16 >> l, half = 4 >> l;
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int q = 0; q < half; ++q) {
+        const float send = up ? a[q] : a[q + half], keep = up ? a[q + half] : a[q];
+        a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    float v = a[0];
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if ((lane & 3) == 0) smf[i0 + (lane >> 2)][warp] = v;
+  }
+#pragma unroll
+  for (int i = KG; i < K; ++i) {
+    float v = acc[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) smf[i][warp] = v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kc; i += NT) {
+    float s = 0.f;
+#pragma unroll
+    for (int wi = 0; wi < NT / 32; ++wi) s += smf[tail && i == kc - 1 ? K - 1 : i][wi];
+    out[i * stride] = (double)s;
+  }
+}
+
+}  // namespace fsi

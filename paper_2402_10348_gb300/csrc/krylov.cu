@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "kreduce.cuh"
 #include "pcnet.h"
 
 namespace fsi {
@@ -49,15 +50,31 @@ constexpr int MMAX = 64;  // largest restart length
 static int vgrid(int64_t n) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + VB * 4 - 1) / (VB * 4), 152 * 4));
 }
-// two CTAs per SM: each streams enough chunks to amortise its end-of-kernel
+// The fused update (float64: upd_dot_kernel, float32: upd_dot2_kernel): one large CTA per SM, whose groups
+// of threads take half chunks (float32: chunks) in turn.  What follows the streaming (the CTA's
+// reduction, the last CTA's sums over all of them) costs by the CTA: with two CTAs of 128 threads per SM
+// (float32: four) it took 10-20 us of a kernel on the 64^3 NS block, more than the streaming at small k.
+// 64^3, float64 solve: 111.4 -> 108.5 ms; float32 basis: 1.018 x a solve.  The projections of
+// mdot_kernel did not gain from the same grid.  A vector of fewer half chunks gets only the
+// groups and CTAs that it fills: an idle group's zeros would be reduced like any other's sums (16^3: 4 % of
+// a solve).
+constexpr int KG = 152;
+constexpr int HCH = 128;         // elements of half a chunk
+constexpr int NHG = 3;           // groups of a full CTA (19 elements a thread at 64^3: 1 % of the time is rounding)
+constexpr int UDT = NHG * HCH;   // most threads
+struct ProjGrid {
+  int ctas, threads;
+};
+static ProjGrid pgrid(int64_t n) {
+  const int64_t units = std::max<int64_t>(1, (n + HCH - 1) / HCH);
+  const int64_t groups = std::min<int64_t>(NHG, (units + KG - 1) / KG);
+  return {(int)std::min<int64_t>(KG, (units + groups - 1) / groups), (int)groups * HCH};
+}
+// mdot_kernel: two CTAs per SM: each streams enough chunks to amortise its end-of-kernel
 // reduction of up to 16 sums (the reduction dominated at four CTAs per SM)
 static int cgrid(int64_t nch) { return (int)std::max<int64_t>(1, std::min<int64_t>(nch, 152 * 2)); }
-// the float32-basis kernels reduce in float32 up to the CTA (cheap): four CTAs per SM
-// keep more loads in flight
-template <typename VT>
-static int cgrid_t(int64_t nch) {
-  return sizeof(VT) == 4 ? (int)std::max<int64_t>(1, std::min<int64_t>(nch, 152 * 4)) : cgrid(nch);
-}
+// mdot4_kernel reduces in float32 up to the CTA (cheap): four CTAs per SM keep more loads in flight
+static int cgrid4(int64_t nch) { return (int)std::max<int64_t>(1, std::min<int64_t>(nch, 152 * 4)); }
 // the basis store: a few chunks of 256 elements per CTA, eight CTAs per SM
 static int chunk_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + CH - 1) / CH, 152 * 8)); }
 
@@ -95,101 +112,6 @@ __device__ __forceinline__ void block_reduce_store(double (&acc)[K], int kc, dou
     double s = 0.0;
     for (int wi = 0; wi < VB / 32; ++wi) s += sm[threadIdx.x][wi];
     out[threadIdx.x * stride] = s;
-  }
-}
-
-// The same for many float64 values with fewer float64 adds (this GPU issues them at a
-// small fraction of the float32 rate; a plain shuffle tree costs 5 adds a lane per value).
-// Inside a warp a transposing butterfly takes the first P values (P the largest power of
-// two <= K, at most 32): at shuffle distance 16 a lane keeps half of its values and adds
-// its partner's copy of that half, at distance 8 half of that half, and so on; after
-// log2 P levels the lane holds value number lane >> (5 - log2 P) summed over the lanes
-// that differ from it in the top log2 P bits, and plain shuffles over the remaining bits
-// finish the warp's sum (P - 1 + 5 - log2 P adds a lane).  Values past P take plain trees.
-template <int K>
-__device__ __forceinline__ void block_reduce_store_bf(double (&acc)[K], int kc, double* out, int stride) {
-  constexpr int P = K >= 32 ? 32 : K >= 16 ? 16 : K >= 8 ? 8 : K >= 4 ? 4 : K >= 2 ? 2 : 1;
-  constexpr int L = P == 32 ? 5 : P == 16 ? 4 : P == 8 ? 3 : P == 4 ? 2 : P == 2 ? 1 : 0;
-  __shared__ double smb[K][VB / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double a[P];
-#pragma unroll
-  for (int q = 0; q < P; ++q) a[q] = acc[q];
-#pragma unroll
-  for (int l = 0; l < L; ++l) {
-    const int o = 16 >> l;
-    const int half = P >> (l + 1);
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int q = 0; q < half; ++q) {
-      const double send = up ? a[q] : a[q + half];  // the half the partner keeps
-      const double keep = up ? a[q + half] : a[q];
-      a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  double s = a[0];
-#pragma unroll
-  for (int o = 16 >> L; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((lane & ((32 >> L) - 1)) == 0) smb[lane >> (5 - L)][warp] = s;
-#pragma unroll
-  for (int i = P; i < K; ++i) {
-    double v = acc[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) smb[i][warp] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kc) {
-    double t = 0.0;
-    for (int wi = 0; wi < VB / 32; ++wi) t += smb[threadIdx.x][wi];
-    out[threadIdx.x * stride] = t;
-  }
-}
-
-// The same in float32 up to the CTA's sums, which are stored as float64: this GPU issues float64
-// adds at 1/64 of the float32 rate, so a float64 tree over every thread's sums costs more than
-// the float32 basis kernel's streaming.  Values in groups of 8 by the transposing butterfly (9
-// shuffles a group against 40 for plain trees: with a few basis chunks a thread, the trees took as
-// long as the streaming), the last ones by plain trees.  NT threads.  out[i * stride], i < kc; with
-// tail the row kc - 1 is the last value's sum.
-template <int K, int NT>
-__device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, bool tail, double* out, int stride) {
-  __shared__ float smf[K][NT / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int KG = K / 8 * 8;
-#pragma unroll
-  for (int i0 = 0; i0 < KG; i0 += 8) {
-    float a[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) a[q] = acc[i0 + q];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      const int o = 16 >> l, half = 4 >> l;
-      const bool up = (lane & o) != 0;
-#pragma unroll
-      for (int q = 0; q < half; ++q) {
-        const float send = up ? a[q] : a[q + half], keep = up ? a[q + half] : a[q];
-        a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    }
-    float v = a[0];
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    if ((lane & 3) == 0) smf[i0 + (lane >> 2)][warp] = v;
-  }
-#pragma unroll
-  for (int i = KG; i < K; ++i) {
-    float v = acc[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) smf[i][warp] = v;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kc; i += NT) {
-    float s = 0.f;
-#pragma unroll
-    for (int wi = 0; wi < NT / 32; ++wi) s += smf[tail && i == kc - 1 ? K - 1 : i][wi];
-    out[i * stride] = (double)s;
   }
 }
 
@@ -243,37 +165,34 @@ __device__ __forceinline__ void sum_rows(const double* part, int G, int rows, do
 
 // h[i] = V_i . w for i < k, h[k] = w . w (partial sums part[i * G + cta]).  Groups of DCH vectors per
 // blockIdx.y; the last group has k mod DCH = R vectors (perhaps none) and takes w . w.
-template <int KC, bool SELF, typename VT>
-__device__ __forceinline__ void mdot_group(const VT* __restrict__ V, int M1, int ib, const double* __restrict__ w,
+template <int KC, bool SELF>
+__device__ __forceinline__ void mdot_group(const double* __restrict__ V, int M1, int ib, const double* __restrict__ w,
                                            int64_t n, double* part) {
   constexpr int NR = KC + (SELF ? 1 : 0);
   const int G = gridDim.x;
   const int64_t nch = (n + CH - 1) / CH;
   const int64_t per = (nch + G - 1) / G;
   const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
-  VT acc[NR];
+  double acc[NR];
 #pragma unroll
-  for (int i = 0; i < NR; ++i) acc[i] = VT(0);
+  for (int i = 0; i < NR; ++i) acc[i] = 0.0;
   for (int64_t c = c0; c < c1; ++c) {
     const int64_t j = c * CH + threadIdx.x;
     if (j >= n) break;
-    const VT wj = (VT)w[j];
-    const VT* blk = V + c * (int64_t)M1 * CH + (int64_t)ib * CH + threadIdx.x;
+    const double wj = w[j];
+    const double* blk = V + c * (int64_t)M1 * CH + (int64_t)ib * CH + threadIdx.x;
 #pragma unroll
     for (int i = 0; i < KC; ++i) acc[i] += blk[i * CH] * wj;
     if (SELF) acc[NR - 1] += wj * wj;
   }
-  double accd[NR];
-#pragma unroll
-  for (int i = 0; i < NR; ++i) accd[i] = (double)acc[i];
-  block_reduce_store_bf<NR>(accd, NR, part + (int64_t)ib * G + blockIdx.x, G);
+  block_reduce_store_bf<NR, VB>(acc, NR, false, part + (int64_t)ib * G + blockIdx.x, G);
 }
 
-template <int R, typename VT>
-__global__ void __launch_bounds__(VB) mdot_kernel(const VT* __restrict__ V, int M1, int k, const double* __restrict__ w,
+template <int R>
+__global__ void __launch_bounds__(VB) mdot_kernel(const double* __restrict__ V, int M1, int k, const double* __restrict__ w,
                                                   int64_t n, double* part, KryDev* K) {
-  if (blockIdx.y < gridDim.y - 1) mdot_group<DCH, false, VT>(V, M1, blockIdx.y * DCH, w, n, part);
-  else mdot_group<R, true, VT>(V, M1, blockIdx.y * DCH, w, n, part);
+  if (blockIdx.y < gridDim.y - 1) mdot_group<DCH, false>(V, M1, blockIdx.y * DCH, w, n, part);
+  else mdot_group<R, true>(V, M1, blockIdx.y * DCH, w, n, part);
   if (last_cta(&K->counter, gridDim.x * gridDim.y)) sum_rows<4>(part, gridDim.x, k + 1, K->h);
 }
 
@@ -547,57 +466,51 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
 // in its own shared-memory column; the columns are added once at the end (float64).
 // KMAX: k rounded up to a multiple of 8.  Rows of part: i < k the projections, row k
 // the norm; part[row * G + cta].
-constexpr int UDB = 128;  // threads per CTA (two elements of each 256-element chunk)
-static_assert(UDB == 128, "the row sums take four columns per lane");
-template <int KMAX, typename VT>
-__global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, const VT* __restrict__ V, int M1,
-                                                      int k, int64_t n, double* part, KryDev* K) {
+template <int KMAX>
+__global__ void __launch_bounds__(UDT) upd_dot_kernel(double* __restrict__ w, const double* __restrict__ V, int M1, int k,
+                                                      int64_t n, double* part, KryDev* K) {
   extern __shared__ __align__(16) unsigned char upd_smem[];
-  const double* h = K->h;
-  VT* sacc = reinterpret_cast<VT*>(upd_smem);  // [KMAX + 1][UDB]
-  __shared__ VT nhs[KMAX];
-  const int t = threadIdx.x;
-  for (int i = t; i < KMAX; i += UDB) nhs[i] = i < k ? -(VT)h[i] : VT(0);
-  for (int i = 0; i <= KMAX; ++i) sacc[i * UDB + t] = VT(0);
+  double* sacc = reinterpret_cast<double*>(upd_smem);  // [KMAX + 1][UDT]
+  __shared__ double nhs[KMAX];
+  const int t = threadIdx.x, NT = blockDim.x;
+  for (int i = t; i < KMAX; i += NT) nhs[i] = i < k ? -K->h[i] : 0.0;
+  for (int i = 0; i <= KMAX; ++i) sacc[i * UDT + t] = 0.0;
   __syncthreads();
   const int G = gridDim.x;
-  const int64_t nch = (n + CH - 1) / CH;
-  const int64_t per = (nch + G - 1) / G;
-  const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
-  VT nrm = VT(0);
-  for (int64_t c = c0; c < c1; ++c) {
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-      const int64_t j = c * CH + half * UDB + t;
-      if (j >= n) continue;
-      const VT* blk = V + c * (int64_t)M1 * CH + half * UDB + t;
-      VT v[KMAX];
+  const int64_t nu = (n + HCH - 1) / HCH;
+  double nrm = 0.0;
+  for (int64_t u = blockIdx.x + (int64_t)G * (t / HCH); u < nu; u += (int64_t)G * (blockDim.x / HCH)) {
+    const int64_t j = u * HCH + t % HCH;
+    if (j >= n) break;
+    const double* blk = V + (u >> 1) * (int64_t)M1 * CH + (u & 1) * HCH + t % HCH;
+    double v[KMAX];
 #pragma unroll
-      for (int i = 0; i < KMAX; ++i) v[i] = i < k ? blk[i * CH] : VT(0);
-      // one fused multiply-add per basis value, chained on w's value, and none for the
-      // padding past k (float64 operations are what this kernel is bound by)
-      VT ww = (VT)w[j];
+    for (int i = 0; i < KMAX; ++i) v[i] = i < k ? blk[i * CH] : 0.0;
+    // one fused multiply-add per basis value, chained on w's value, and none for the
+    // padding past k (float64 operations are what this kernel is bound by)
+    double ww = w[j];
 #pragma unroll
-      for (int i = 0; i < KMAX; ++i) {
-        if (i >= k) break;
-        ww = fma(nhs[i], v[i], ww);
-      }
-      w[j] = (double)ww;
-      nrm = fma(ww, ww, nrm);
+    for (int i = 0; i < KMAX; ++i) {
+      if (i >= k) break;
+      ww = fma(nhs[i], v[i], ww);
+    }
+    w[j] = ww;
+    nrm = fma(ww, ww, nrm);
 #pragma unroll
-      for (int i = 0; i < KMAX; ++i) {
-        if (i >= k) break;
-        sacc[i * UDB + t] = fma(v[i], ww, sacc[i * UDB + t]);
-      }
+    for (int i = 0; i < KMAX; ++i) {
+      if (i >= k) break;
+      sacc[i * UDT + t] = fma(v[i], ww, sacc[i * UDT + t]);
     }
   }
-  sacc[KMAX * UDB + t] = nrm;
+  sacc[KMAX * UDT + t] = nrm;
   __syncthreads();
   // one warp per row, lanes on consecutive columns, then a shuffle tree
   const int lane = t & 31;
-  for (int i = t >> 5; i <= k; i += UDB / 32) {
-    const VT* rp = sacc + (i < k ? i : KMAX) * UDB;
-    double s = ((double)rp[lane] + (double)rp[lane + 32]) + ((double)rp[lane + 64] + (double)rp[lane + 96]);
+  for (int i = t >> 5; i <= k; i += NT >> 5) {
+    const double* rp = sacc + (i < k ? i : KMAX) * UDT;
+    double s = 0.0;
+#pragma unroll 4
+    for (int c = 0; c < NT >> 5; ++c) s += rp[lane + 32 * c];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) part[(int64_t)i * G + blockIdx.x] = s;
@@ -610,21 +523,22 @@ __global__ void __launch_bounds__(UDB) upd_dot_kernel(double* __restrict__ w, co
 // per load as with a float64 basis, and keeps the projections in registers.  Elements at or past n
 // are never read.
 template <int KMAX>
-__global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, const float* __restrict__ V, int M1,
-                                                       int k, int64_t n, double* part, KryDev* K) {
+constexpr int ud2_threads() { return KMAX <= 32 ? 384 : 256; }
+template <int KMAX>
+__global__ void __launch_bounds__(ud2_threads<KMAX>()) upd_dot2_kernel(double* __restrict__ w, const float* __restrict__ V,
+                                                                       int M1, int k, int64_t n, double* part, KryDev* K) {
+  constexpr int NT = ud2_threads<KMAX>();
   __shared__ float nhs[KMAX];
   const int t = threadIdx.x;
-  for (int i = t; i < KMAX; i += UDB) nhs[i] = i < k ? -(float)K->h[i] : 0.f;
+  for (int i = t; i < KMAX; i += NT) nhs[i] = i < k ? -(float)K->h[i] : 0.f;
   __syncthreads();
   const int G = gridDim.x;
   const int64_t nch = (n + CH - 1) / CH;
-  const int64_t per = (nch + G - 1) / G;
-  const int64_t c0 = blockIdx.x * per, c1 = min(nch, c0 + per);
-  const int e0 = 2 * t;
+  const int e0 = 2 * (t & 127);
   float acc[KMAX + 1];
 #pragma unroll
   for (int i = 0; i <= KMAX; ++i) acc[i] = 0.f;
-  for (int64_t c = c0; c < c1; ++c) {
+  for (int64_t c = blockIdx.x + (int64_t)G * (t >> 7); c < nch; c += (int64_t)G * (NT / 128)) {
     const int64_t j = c * CH + e0;
     if (j >= n) break;
     const bool pair = j + 2 <= n;
@@ -660,34 +574,36 @@ __global__ void __launch_bounds__(UDB) upd_dot2_kernel(double* __restrict__ w, c
     for (int i = 0; i < KMAX; ++i) acc[i] += v[i].x * wx + v[i].y * wy;
   }
   // rows i < k the projections, row k the norm
-  block_reduce_store_f<KMAX + 1, UDB>(acc, k + 1, true, part + blockIdx.x, G);
+  block_reduce_store_f<KMAX + 1, NT>(acc, k + 1, true, part + blockIdx.x, G);
   if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1);
 }
 
 template <int KMAX, typename VT>
-static int launch_upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n) {
+static int launch_upd_dot(fsi_mesh* m, double* w, const VT* V, int M1, int k, int64_t n) {
   KryDev* K = static_cast<KryDev*>(m->kry_dev);
   if constexpr (sizeof(VT) == 4) {
-    upd_dot2_kernel<KMAX><<<G, UDB, 0, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
+    const int G = (int)std::max<int64_t>(1, std::min<int64_t>((n + CH - 1) / CH, KG));
+    upd_dot2_kernel<KMAX><<<G, ud2_threads<KMAX>(), 0, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
   } else {
-    const size_t smem = sizeof(VT) * (size_t)(KMAX + 1) * UDB;
-    if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot_kernel<KMAX, VT>), smem)) return rc;
-    upd_dot_kernel<KMAX, VT><<<G, UDB, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
+    const ProjGrid g = pgrid(n);
+    const size_t smem = sizeof(double) * (size_t)(KMAX + 1) * UDT;
+    if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&upd_dot_kernel<KMAX>), smem)) return rc;
+    upd_dot_kernel<KMAX><<<g.ctas, g.threads, smem, m->stream>>>(w, V, M1, k, n, m->partials_dot, K);
   }
   return FSI_OK;
 }
 
 template <typename VT>
-static int upd_dot(fsi_mesh* m, int G, double* w, const VT* V, int M1, int k, int64_t n) {
+static int upd_dot(fsi_mesh* m, double* w, const VT* V, int M1, int k, int64_t n) {
   switch ((k + 7) / 8) {
-    case 1: return launch_upd_dot<8>(m, G, w, V, M1, k, n);
-    case 2: return launch_upd_dot<16>(m, G, w, V, M1, k, n);
-    case 3: return launch_upd_dot<24>(m, G, w, V, M1, k, n);
-    case 4: return launch_upd_dot<32>(m, G, w, V, M1, k, n);
-    case 5: return launch_upd_dot<40>(m, G, w, V, M1, k, n);
-    case 6: return launch_upd_dot<48>(m, G, w, V, M1, k, n);
-    case 7: return launch_upd_dot<56>(m, G, w, V, M1, k, n);
-    default: return launch_upd_dot<64>(m, G, w, V, M1, k, n);
+    case 1: return launch_upd_dot<8>(m, w, V, M1, k, n);
+    case 2: return launch_upd_dot<16>(m, w, V, M1, k, n);
+    case 3: return launch_upd_dot<24>(m, w, V, M1, k, n);
+    case 4: return launch_upd_dot<32>(m, w, V, M1, k, n);
+    case 5: return launch_upd_dot<40>(m, w, V, M1, k, n);
+    case 6: return launch_upd_dot<48>(m, w, V, M1, k, n);
+    case 7: return launch_upd_dot<56>(m, w, V, M1, k, n);
+    default: return launch_upd_dot<64>(m, w, V, M1, k, n);
   }
 }
 
@@ -878,38 +794,37 @@ __global__ void fill_kernel(double* y, double v, int64_t n) {
 }
 
 // ---------------------------------------------------------------- host helpers
-template <typename VT>
-static void launch_mdot(fsi_mesh* m, dim3 grid, const VT* V, int M1, int k, const double* w, int64_t n, KryDev* K) {
+static void launch_mdot(fsi_mesh* m, const double* V, int M1, int k, const double* w, int64_t n, KryDev* K) {
+  // one group more than the full ones: it holds the rest, or only w . w
+  const dim3 grid(cgrid((n + CH - 1) / CH), k / DCH + 1);
   switch (k % DCH) {
-    case 0: mdot_kernel<0, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 1: mdot_kernel<1, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 2: mdot_kernel<2, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 3: mdot_kernel<3, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 4: mdot_kernel<4, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 5: mdot_kernel<5, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 6: mdot_kernel<6, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 7: mdot_kernel<7, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 8: mdot_kernel<8, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 9: mdot_kernel<9, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 10: mdot_kernel<10, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 11: mdot_kernel<11, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 12: mdot_kernel<12, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 13: mdot_kernel<13, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    case 14: mdot_kernel<14, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
-    default: mdot_kernel<15, VT><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 0: mdot_kernel<0><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 1: mdot_kernel<1><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 2: mdot_kernel<2><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 3: mdot_kernel<3><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 4: mdot_kernel<4><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 5: mdot_kernel<5><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 6: mdot_kernel<6><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 7: mdot_kernel<7><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 8: mdot_kernel<8><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 9: mdot_kernel<9><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 10: mdot_kernel<10><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 11: mdot_kernel<11><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 12: mdot_kernel<12><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 13: mdot_kernel<13><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    case 14: mdot_kernel<14><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
+    default: mdot_kernel<15><<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K); break;
   }
+}
+static void launch_mdot(fsi_mesh* m, const float* V, int M1, int k, const double* w, int64_t n, KryDev* K) {
+  const dim3 grid(cgrid4((n + CH - 1) / CH), k / DCH + 1);
+  mdot4_kernel<<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K);
 }
 
 // K->h[0..k) = V_i . w for the basis slots i < k, K->h[k] = w . w
 template <typename VT>
 static int basis_dots(fsi_mesh* m, const VT* V, int M1, int k, const double* w, int64_t n, KryDev* K) {
-  const int G = cgrid_t<VT>((n + CH - 1) / CH);
-  // one group more than the full ones: it holds the rest, or only w . w
-  const dim3 grid(G, k / DCH + 1);
-  if constexpr (sizeof(VT) == 4)
-    FSI_LAUNCH(m, P_KRY_DOT, mdot4_kernel<<<grid, VB, 0, m->stream>>>(V, M1, k, w, n, m->partials_dot, K));
-  else
-    FSI_LAUNCH(m, P_KRY_DOT, launch_mdot<VT>(m, grid, V, M1, k, w, n, K));
+  FSI_LAUNCH(m, P_KRY_DOT, launch_mdot(m, V, M1, k, w, n, K));
   return FSI_OK;
 }
 
@@ -1070,8 +985,7 @@ static int gmres_core_t(fsi_mesh* m, const BlockInfo& blk, const double* b, doub
       // pass 1: h = V^T w and |w|^2 (slot j+1 of h)
       if ((rc = basis_dots(m, V, M1, j + 1, w, n, K))) return rc;
       // pass-1 update fused with the pass-2 projections of the updated vector, then the DGKS test
-      const int Gc = cgrid_t<VT>((n + CH - 1) / CH);
-      FSI_LAUNCH(m, P_KRY_UPD, rc = upd_dot<VT>(m, Gc, w, V, M1, j + 1, n));
+      FSI_LAUNCH(m, P_KRY_UPD, rc = upd_dot<VT>(m, w, V, M1, j + 1, n));
       if (rc) return rc;
       prof_bytes(m, P_KRY_DOT, (j + 1) * vb + wb);      // j+1 basis vectors and w read once
       prof_bytes(m, P_KRY_UPD, (j + 1) * vb + 2 * wb);  // j+1 basis vectors and w read, w written
