@@ -440,7 +440,7 @@ int fsi_batch_layout(const fsi_batch* batch, int64_t* offsets, int32_t* target_m
 /* y = J_i(states[i]) dx for every instance (flags as in fsi_jvp).  NS batches: each
  * instance's quadrature-point coefficients are built at its state (Section 2.4's
  * linearization frozen), then one element launch over all instances' tiles (float32: the
- * coefficients TMA-staged) and one node launch; AC and B batches: one persistent launch of
+ * coefficients staged by bulk copies) and one node launch; AC and B batches: one persistent launch of
  * the re-interpolating element operators. */
 int fsi_batch_jvp(fsi_batch* batch, const fsi_state* states, const double* dx, double* y, uint32_t flags);
 /* fsi_gmres for every instance (FSI_PREC_FP64 or FSI_PREC_FP32_IR; opts.m must be the

@@ -135,7 +135,7 @@ struct fsi_batch {
   cudaGraphExec_t net_graph = nullptr;
   int net_warm = 0;
   // work lists of the batched float32 NS coefficient product (built on first use)
-  int4* nsq_eitems = nullptr;     // (instance, x block, y block, layer)
+  int4* nsq_eitems = nullptr;     // (instance, tile, 0, layer)
   int nsq_ne = 0;
   int4* nsq_nitems = nullptr;     // (instance, 128-node block, 0, 0)
   int nsq_nn = 0;
@@ -764,10 +764,8 @@ int ensure_nsq_items(fsi_batch* b) {
     std::vector<int4> ei, ni;
     for (int i = 0; i < b->n; ++i) {
       const Geom& g = b->meshes[i]->g;
-      const int nbx = (g.nx + NSQ_TBX - 1) / NSQ_TBX, nby = (g.ny + NSQ_TBY - 1) / NSQ_TBY;
       for (int ez = 0; ez < g.nz; ++ez)
-        for (int by = 0; by < nby; ++by)
-          for (int bx = 0; bx < nbx; ++bx) ei.push_back(make_int4(i, bx, by, ez));
+        for (int t = 0; t < nsq_tiles(g); ++t) ei.push_back(make_int4(i, t, 0, ez));
       const int64_t nblk = (b->meshes[i]->nn + 127) / 128;
       for (int64_t k = 0; k < nblk; ++k) ni.push_back(make_int4(i, (int)k, 0, 0));
     }
@@ -823,7 +821,7 @@ int record_set(fsi_batch* b, OpSet* set, unsigned flags, const double* dx_base, 
   for (int i = 0; i < b->n; ++i) all_ns = all_ns && b->blocks[i] == FSI_BLOCK_NS;
   if (all_ns) {
     // NS products from each instance's frozen coefficients (built here, on the staged
-    // states) in one element and one node launch: float32 TMA-staged, float64 read directly
+    // states) in one element and one node launch: float32 staged by bulk copies, float64 read directly
     std::vector<NSQBatchRec> recs(b->n);
     for (int i = 0; i < b->n; ++i) {
       int rc = nsq_batch_record(b->meshes[i], flags, !f32, dx_base + b->off[i], y_base + b->off[i],

@@ -77,10 +77,7 @@ struct fsi_mesh {
     unsigned flags = 0;              // FSI_ELASTIC_AUG of the last build
   };
   NSCoef cq64, cq32;
-  // TMA descriptors of the float32 coefficients (boxes of 44 and of 20 values; nsq_tma.cu),
-  // encoded for the allocation at cq_tmap_base; tma_err: a bounded wait gave up
-  alignas(64) unsigned char cq_tmap[256] = {};
-  const void* cq_tmap_base = nullptr;
+  // a bounded wait of the float32 product gave up (nsq_tma.cu)
   int* tma_err = nullptr;
   // assembled float64 NS operator (nsa.cu), and the element matrices it is summed from
   double* na64 = nullptr;
@@ -184,16 +181,15 @@ int launch_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags
 int ns_build(fsi_mesh* m, unsigned flags, bool f64);  // hexq_ops.cu
 // float64 NS product at a state that is used a few times (hexq_ops.cu)
 int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags);
-// float32 NS product from the coefficients, TMA-staged (nsq_tma.cu); dx32 holds the increment
+// float32 NS product from the coefficients, staged by bulk copies (nsq_tma.cu); dx32 holds the increment
 int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags);
 // FSI_ECUDA if a bounded wait of that kernel gave up since the flag was allocated (syncs)
 int check_tma(fsi_mesh* m);
-// One instance's float32 NS product in a batched launch (nsq_tma.cu): the TMA descriptor of
-// its coefficients, its increment (float copy and float64 for the Dirichlet rows), its
-// contribution scratch and output, its geometry.  64-byte aligned (the descriptor's rule).
-struct alignas(64) NSQBatchRec {
-  unsigned char map[128];
-  const double* cq64;  // float64 products: the coefficients, read directly
+// One instance's NS product in a batched launch (nsq_tma.cu): its coefficients, its increment (float
+// copy and float64 for the Dirichlet rows), its contribution scratch and output, its geometry.
+struct NSQBatchRec {
+  const float* cq32;
+  const double* cq64;  // float64 products
   double* E64;         // float64 products: the contribution scratch
   const float* dx32;
   const double* dx;
@@ -207,15 +203,16 @@ struct alignas(64) NSQBatchRec {
   int nx, ny, nz, nxp, pin, elastic;
   float al, cm, rhx, rhy, rhz;
 };
-// builds the instance's coefficients (if stale), scratch and descriptor and fills rec;
-// f64: a float64 product (coefficients read directly, no descriptor)
+// builds the instance's coefficients (if stale) and scratch and fills rec; f64: a float64 product
 int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, double* y, float* dx32,
                      NSQBatchRec* rec);
-// element and node launches of a batch (recs in device memory; items: (instance, x block,
-// y block, layer) and (instance, 128-node block)); active gates instances (nullable)
+// element and node launches of a batch (recs in device memory; items: (instance, tile, 0,
+// layer) and (instance, 128-node block)); active gates instances (nullable)
 int nsq_batch_launch(bool f64, const NSQBatchRec* recs, const int4* eitems, int neitems, const int4* nitems,
                      int nnitems, const int* active, cudaStream_t s);
-constexpr int NSQ_TBX = 64, NSQ_TBY = 2;  // element tile of the TMA product
+// The coefficient products take NSQ_TILE consecutive elements (x fastest) of a layer per CTA
+constexpr int NSQ_TILE = 128;
+__host__ __device__ inline int nsq_tiles(const Geom& g) { return (int)(((int64_t)g.nx * g.ny + NSQ_TILE - 1) / NSQ_TILE); }
 // [slots][elements] scratch of the element-centric products, grown on demand (ops_f64.cu)
 int ensure_elem_scratch(fsi_mesh* m, int slots, int64_t nxyp);
 // assembled float64 NS operator of the staged state (built when stale): build, product and

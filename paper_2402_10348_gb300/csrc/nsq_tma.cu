@@ -1,28 +1,26 @@
-// Float32 NS product from the quadrature-point coefficients, staged by the Tensor
-// Memory Accelerator (the FSI_FP32 product of the NS block inside mixed-precision
-// iterative refinement).
+// Float32 NS product from the quadrature-point coefficients, staged by bulk copies (the FSI_FP32
+// product of the NS block inside mixed-precision iterative refinement).
 //
-// The product is bound by streaming the coefficient planes (8 points x 44 or 20 float32
-// values per element, Section 2.4's linearization frozen per solve): one thread per
-// element reading 352 scattered planes keeps too few loads in flight.  Here a CTA owns a
-// tile of 64 x 2 elements of one element layer and receives, per quadrature point, one
-// four-dimensional TMA box (x 64, y 2, coefficient 44 or 20, layer-point 1) of the
-// coefficient array C[((ez * 8 + q) * 44 + c) * nxyp + ey * nxp + ex] into shared memory
-// (22.5 KB), double-buffered on two mbarriers: the copy of point q + 2 runs while point
-// q is evaluated.  Thread (tx, ty) evaluates element (x0 + tx, y0 + ty) exactly as the
-// element-centric kernel (nsq_point on the interpolated increment) and writes its 32
-// corner contributions into E[8 * field + corner][element]; ns_node_kernel sums them.
+// The product is bound by streaming the coefficients (8 points x 44 or 20 float32 values per
+// element, Section 2.4's linearization frozen per solve): one thread per element reading 352
+// scattered planes keeps too few loads in flight.  Here a CTA owns 128 consecutive elements (x
+// fastest) of one layer, whose coefficients lie together, C[(((ez * tiles + tile) * 8 + q) * 44 + c) *
+// 128 + element], and receives a point's 44 (or first 20) values of all 128 by one cp.async.bulk
+// (22.5 KB) into shared memory, double-buffered on two mbarriers: the copy of point q + 2 runs while
+// point q is evaluated.  Thread t evaluates element 128 tile + t (nsq_point on the interpolated
+// increment) and writes its 32 corner contributions into E[8 * field + corner][element];
+// ns_node_kernel sums them.  With 64 x 2 boxes of a plane layout instead, three quarters of the
+// threads and of the bytes in flight were idle on a 16^3 mesh: the product of twelve 16^3-48^3
+// cavities took 140 us, now 133; 64^3 62.5 either way.
 //
 // Every mbarrier wait is bounded; a wait that gives up sets *err, the CTA stops issuing
 // copies, waits (bounded) for the copies it has in flight and writes NaN contributions.
-#include <cuda.h>
-
 #include "ops_impl.cuh"
 
 namespace fsi {
 namespace {
 
-constexpr int TBX = NSQ_TBX, TBY = NSQ_TBY;  // CTA tile of elements (x, y), one thread each
+constexpr int TBE = NSQ_TILE;  // elements of a CTA's tile, one thread each
 constexpr int TSTAGES = 2;
 constexpr long long TWAIT = 1LL << 22;
 
@@ -43,35 +41,31 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-// one box of coefficients of layer-point zq into dst; completion counted on bar
-__device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, uint32_t bytes, int x0,
-                                         int y0, int zq) {
+// one point's coefficients into dst (both 16-byte aligned, bytes a multiple of 512); completion on bar
+__device__ __forceinline__ void load_point(uint32_t dst, const float* src, uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-      "%5}], [%6];\n" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x0), "r"(y0), "r"(0), "r"(zq), "r"(bar)
-      : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
 }
 
 // coefficient accessor over one element's column of a staged box
 struct SmemCoef {
   const float* p;
-  __device__ __forceinline__ float operator()(int i) const { return p[i * (TBX * TBY)]; }
+  __device__ __forceinline__ float operator()(int i) const { return p[i * TBE]; }
 };
 
-// One CTA's tile: elements (x0 .. x0 + 63, y0 .. y0 + 1) of layer ez, ncoef coefficients per
-// point staged from the tensor map `map` (in kernel parameter or global memory) into
-// `stage` ([TSTAGES][ncoef][TBY][TBX]); contributions into E (element plane pitch nxyp).
-__device__ __forceinline__ void nsq_tma_tile(float* stage, const CUtensorMap* map, int ncoef,
+// One CTA's tile: elements 128 tile .. of layer ez, ncoef coefficients per point staged from the tile's
+// coefficients C into `stage` ([TSTAGES][ncoef][TBE]); contributions into E (element plane pitch nxyp).
+__device__ __forceinline__ void nsq_tma_tile(float* stage, const float* __restrict__ C, int ncoef,
                                              const float* __restrict__ dx, float* __restrict__ E, int nx, int ny,
                                              int nz, int nxp, int64_t nxyp, int64_t nn, float al, float cmass,
-                                             float rhx, float rhy, float rhz, int x0, int y0, int ez, int* err) {
+                                             float rhx, float rhy, float rhz, int tile, int ez, int* err) {
   __shared__ __align__(8) uint64_t bar[TSTAGES];
   __shared__ int failed;
-  const int SF = ncoef * TBX * TBY;  // floats per stage
+  const int SF = ncoef * TBE;  // floats per stage
   const uint32_t SBYTES = (uint32_t)SF * sizeof(float);
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TBX + tx;
+  const int tid = threadIdx.x;
   if (tid == 0) {
     failed = 0;
     for (int s = 0; s < TSTAGES; ++s)
@@ -80,10 +74,11 @@ __device__ __forceinline__ void nsq_tma_tile(float* stage, const CUtensorMap* ma
   }
   __syncthreads();
   if (tid == 0)
-    for (int s = 0; s < TSTAGES; ++s) load_box(sptr(stage + s * SF), map, sptr(&bar[s]), SBYTES, x0, y0, ez * 8 + s);
+    for (int s = 0; s < TSTAGES; ++s) load_point(sptr(stage + s * SF), C + s * NCQ * TBE, sptr(&bar[s]), SBYTES);
   // the increment at the element's corners (while the first boxes arrive)
-  const int ex = x0 + tx, ey = y0 + ty;
-  const bool valid = ex < nx && ey < ny;
+  const unsigned f0 = (unsigned)tile * TBE + (unsigned)tid;
+  const int ey = (int)(f0 / (unsigned)nx), ex = (int)(f0 - (unsigned)ey * (unsigned)nx);
+  const bool valid = ey < ny;
   float x[4][8], c[4][8];
   const int64_t sy = nx + 1, sz = (int64_t)(nx + 1) * (ny + 1);
   const int64_t n0 = ex + sy * ey + sz * ez;
@@ -116,7 +111,8 @@ __device__ __forceinline__ void nsq_tma_tile(float* stage, const CUtensorMap* ma
                        c);
     }
     __syncthreads();  // every thread is done with stage s
-    if (tid == 0 && q + TSTAGES < 8) load_box(sptr(stage + s * SF), map, sptr(&bar[s]), SBYTES, x0, y0, ez * 8 + q + TSTAGES);
+    if (tid == 0 && q + TSTAGES < 8)
+      load_point(sptr(stage + s * SF), C + (q + TSTAGES) * NCQ * TBE, sptr(&bar[s]), SBYTES);
   }
   if (failed) {
     // copies issued for points q .. min(q + TSTAGES, 8) - 1 may still be in flight; the
@@ -139,31 +135,27 @@ __device__ __forceinline__ void nsq_tma_tile(float* stage, const CUtensorMap* ma
     for (int a = 0; a < 8; ++a) E[(8 * f + a) * es + e] = c[f][a];
 }
 
-__global__ void __launch_bounds__(TBX * TBY) nsq_tma_kernel(const __grid_constant__ CUtensorMap map, int ncoef,
-                                                            const float* __restrict__ dx, float* __restrict__ E, int nx,
-                                                            int ny, int nz, int nxp, int64_t nxyp, int64_t nn, float al,
-                                                            float cmass, float rhx, float rhy, float rhz, int* err) {
+__global__ void __launch_bounds__(TBE) nsq_tma_kernel(const float* __restrict__ C, int ncoef, int tiles,
+                                                      const float* __restrict__ dx, float* __restrict__ E, int nx, int ny,
+                                                      int nz, int nxp, int64_t nxyp, int64_t nn, float al, float cmass,
+                                                      float rhx, float rhy, float rhz, int* err) {
   extern __shared__ __align__(128) float stage[];
-  const int nbx = (nx + TBX - 1) / TBX, nby = (ny + TBY - 1) / TBY;
-  int64_t b = blockIdx.x;
-  const int bx = (int)(b % nbx);
-  b /= nbx;
-  const int by = (int)(b % nby);
-  const int ez = (int)(b / nby);
-  nsq_tma_tile(stage, &map, ncoef, dx, E, nx, ny, nz, nxp, nxyp, nn, al, cmass, rhx, rhy, rhz, bx * TBX, by * TBY, ez,
-               err);
+  const int ez = blockIdx.x / tiles, tile = blockIdx.x - ez * tiles;
+  nsq_tma_tile(stage, C + (int64_t)blockIdx.x * 8 * NCQ * TBE, ncoef, dx, E, nx, ny, nz, nxp, nxyp, nn, al, cmass, rhx, rhy,
+               rhz, tile, ez, err);
 }
 
-// Batched: one CTA per work item (instance, x block, y block, layer); the instance's
-// parameters and tensor map come from its record in global memory.
-__global__ void __launch_bounds__(TBX * TBY) nsq_tma_batch_kernel(const NSQBatchRec* __restrict__ recs,
-                                                                  const int4* __restrict__ items, const int* active) {
+// Batched: one CTA per work item (instance, tile, 0, layer); the instance's parameters come from
+// its record in global memory.
+__global__ void __launch_bounds__(TBE) nsq_tma_batch_kernel(const NSQBatchRec* __restrict__ recs,
+                                                            const int4* __restrict__ items, const int* active) {
   extern __shared__ __align__(128) float stage[];
   const int4 it = items[blockIdx.x];
   if (active && !active[it.x]) return;
   const NSQBatchRec& R = recs[it.x];
-  nsq_tma_tile(stage, reinterpret_cast<const CUtensorMap*>(R.map), R.elastic ? NCQ : NCQ_FLUID, R.dx32, R.E, R.nx,
-               R.ny, R.nz, R.nxp, R.nxyp, R.nn, R.al, R.cm, R.rhx, R.rhy, R.rhz, it.y * TBX, it.z * TBY, it.w, R.err);
+  const int tiles = (int)(((int64_t)R.nx * R.ny + TBE - 1) / TBE);
+  nsq_tma_tile(stage, R.cq32 + ((int64_t)it.w * tiles + it.y) * 8 * NCQ * TBE, R.elastic ? NCQ : NCQ_FLUID, R.dx32, R.E,
+               R.nx, R.ny, R.nz, R.nxp, R.nxyp, R.nn, R.al, R.cm, R.rhx, R.rhy, R.rhz, it.y, it.w, R.err);
 }
 
 // NS product from the quadrature-point coefficients (see nsq_point) of element (ex, ey, ez)
@@ -207,15 +199,16 @@ __device__ __forceinline__ void nsq_elem_body(const T* __restrict__ cq, const T*
     for (int a = 0; a < 8; ++a) E[(8 * f + a) * es + e] = c[f][a];
 }
 
-// Batched float64 product from the coefficients (nsq_elem_body): one CTA of 64 x 2
-// threads per (instance, x block, y block, layer) work item
-__global__ void __launch_bounds__(TBX * TBY) nsq_elem_batch_kernel(const NSQBatchRec* __restrict__ recs,
+// Batched float64 product from the coefficients (nsq_elem_body): one CTA per (instance, tile, 0,
+// layer) work item
+__global__ void __launch_bounds__(TBE) nsq_elem_batch_kernel(const NSQBatchRec* __restrict__ recs,
                                                                    const int4* __restrict__ items, const int* active) {
   const int4 it = items[blockIdx.x];
   if (active && !active[it.x]) return;
   const NSQBatchRec& R = recs[it.x];
-  const int ex = it.y * TBX + threadIdx.x, ey = it.z * TBY + threadIdx.y;
-  if (ex >= R.nx || ey >= R.ny) return;
+  const unsigned f = (unsigned)it.y * TBE + threadIdx.x;
+  const int ey = (int)(f / (unsigned)R.nx), ex = (int)(f - (unsigned)ey * (unsigned)R.nx);
+  if (ey >= R.ny) return;
   nsq_elem_body<double>(R.cq64, R.dx, R.E64, R.nx, R.ny, R.nz, R.nxp, R.nxyp, R.nn, R.elastic, R.al64, R.cm64,
                         R.rh64[0], R.rh64[1], R.rh64[2], ex, ey, it.w);
 }
@@ -256,41 +249,7 @@ __global__ void __launch_bounds__(128) ns_node_batch_kernel(const NSQBatchRec* _
   }
 }
 
-using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiled lookup_encode() {
-  void* fn = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess)
-    return nullptr;
-  return reinterpret_cast<EncodeTiled>(fn);
-}
-
-int encode_maps(fsi_mesh* m, int nxp, int64_t nxyp) {
-  static const EncodeTiled enc = lookup_encode();  // thread-safe one-time lookup
-  if (!enc) return set_error(FSI_ECUDA, "NS float32 product: cuTensorMapEncodeTiled not available");
-  const Geom& g = m->g;
-  const cuuint64_t dims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)NCQ, (cuuint64_t)g.nz * 8};
-  const cuuint64_t strides[3] = {(cuuint64_t)nxp * 4, (cuuint64_t)nxyp * 4, (cuuint64_t)NCQ * nxyp * 4};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  for (int k = 0; k < 2; ++k) {
-    const cuuint32_t box[4] = {TBX, TBY, (cuuint32_t)(k == 0 ? NCQ : NCQ_FLUID), 1};
-    CUtensorMap* map = reinterpret_cast<CUtensorMap*>(m->cq_tmap + 128 * k);
-    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, m->cq32.p, dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return set_error(FSI_ECUDA, "NS float32 product: tensor map encoding failed");
-  }
-  m->cq_tmap_base = m->cq32.p;
-  return FSI_OK;
-}
-
 }  // namespace
-
-static_assert(sizeof(CUtensorMap) == 128, "tensor map storage");
 
 int check_tma(fsi_mesh* m) {
   if (!m->tma_err) return FSI_OK;
@@ -309,8 +268,6 @@ int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, do
   const int nxp = cq_pitch(m);
   const int64_t nxyp = (int64_t)nxp * g.ny;
   if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
-  if (!f64 && m->cq_tmap_base != m->cq32.p)
-    if (int rc = encode_maps(m, nxp, nxyp)) return rc;
   if (!m->tma_err) {
     FSI_CUDA(cudaMalloc(&m->tma_err, sizeof(int)));
     FSI_CUDA(cudaMemsetAsync(m->tma_err, 0, sizeof(int), m->stream));
@@ -321,7 +278,7 @@ int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, do
     rec->cq64 = static_cast<const double*>(m->cq64.p);
     rec->E64 = m->ke_e;
   } else {
-    memcpy(rec->map, m->cq_tmap + (elastic ? 0 : 128), 128);
+    rec->cq32 = static_cast<const float*>(m->cq32.p);
   }
   rec->al64 = m->P.alpha;
   rec->cm64 = m->P.c_mass;
@@ -354,13 +311,13 @@ int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, do
 int nsq_batch_launch(bool f64, const NSQBatchRec* recs, const int4* eitems, int neitems, const int4* nitems,
                      int nnitems, const int* active, cudaStream_t s) {
   if (f64) {
-    if (neitems > 0) nsq_elem_batch_kernel<<<neitems, dim3(TBX, TBY), 0, s>>>(recs, eitems, active);
+    if (neitems > 0) nsq_elem_batch_kernel<<<neitems, TBE, 0, s>>>(recs, eitems, active);
     if (nnitems > 0) ns_node_batch_kernel<double><<<nnitems, 128, 0, s>>>(recs, nitems, active);
     FSI_CUDA(cudaGetLastError());
     return FSI_OK;
   }
-  const size_t smem = sizeof(float) * (size_t)TSTAGES * NCQ * TBX * TBY;
-  if (neitems > 0) nsq_tma_batch_kernel<<<neitems, dim3(TBX, TBY), smem, s>>>(recs, eitems, active);
+  const size_t smem = sizeof(float) * (size_t)TSTAGES * NCQ * TBE;
+  if (neitems > 0) nsq_tma_batch_kernel<<<neitems, TBE, smem, s>>>(recs, eitems, active);
   if (nnitems > 0) ns_node_batch_kernel<float><<<nnitems, 128, 0, s>>>(recs, nitems, active);
   FSI_CUDA(cudaGetLastError());
   return FSI_OK;
@@ -374,18 +331,15 @@ int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   const int elastic = ((flags & FSI_ELASTIC_AUG) && m->ns > 0) ? 1 : 0;
   if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
   float* E = reinterpret_cast<float*>(m->ke_e);
-  if (m->cq_tmap_base != m->cq32.p)
-    if (int rc = encode_maps(m, nxp, nxyp)) return rc;
   if (!m->tma_err) {
     FSI_CUDA(cudaMalloc(&m->tma_err, sizeof(int)));
     FSI_CUDA(cudaMemsetAsync(m->tma_err, 0, sizeof(int), m->stream));
   }
-  const int64_t nblk = (int64_t)((g.nx + TBX - 1) / TBX) * ((g.ny + TBY - 1) / TBY) * g.nz;
+  const int tiles = nsq_tiles(g);
+  const int64_t nblk = (int64_t)tiles * g.nz;
   if (nblk > INT32_MAX) return set_error(FSI_EINVAL, "NS float32 product: mesh too large for one launch");
-  const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(m->cq_tmap + (elastic ? 0 : 128));
   const int ncoef = elastic ? NCQ : NCQ_FLUID;
-  const size_t smem = sizeof(float) * (size_t)TSTAGES * ncoef * TBX * TBY;
-  const dim3 blk(TBX, TBY);
+  const size_t smem = sizeof(float) * (size_t)TSTAGES * ncoef * TBE;
   const float al = (float)m->P.alpha, cm = (float)m->P.c_mass;
   const float rx = (float)(1.0 / g.hx), ry = (float)(1.0 / g.hy), rz = (float)(1.0 / g.hz);
   // algorithmic bytes: the coefficient planes once per element, the increment once per
@@ -395,8 +349,9 @@ int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   prof_bytes(m, P_NS_JVP32, ne * (8.0 * ncoef + 32.0) * 4.0 + (double)nn * 16.0);
   prof_bytes(m, P_NODE_SUM, ne * 32.0 * 4.0 + (double)nn * (32.0 + 1.0));
   FSI_LAUNCH(m, P_NS_JVP32,
-             (nsq_tma_kernel<<<(unsigned)nblk, blk, smem, m->stream>>>(*map, ncoef, m->dx32, E, g.nx, g.ny, g.nz, nxp,
-                                                                      nxyp, nn, al, cm, rx, ry, rz, m->tma_err)));
+             (nsq_tma_kernel<<<(unsigned)nblk, TBE, smem, m->stream>>>(static_cast<const float*>(m->cq32.p), ncoef, tiles,
+                                                                       m->dx32, E, g.nx, g.ny, g.nz, nxp, nxyp, nn, al, cm,
+                                                                       rx, ry, rz, m->tma_err)));
   const RowLaunch nl = node_launch(g);
   FSI_LAUNCH(m, P_NODE_SUM,
              ns_node_kernel<float><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, nxp, nxyp, nn,
