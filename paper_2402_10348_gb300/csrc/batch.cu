@@ -39,6 +39,7 @@
 #include <sys/stat.h>
 
 #include "internal.h"
+#include "kreduce.cuh"
 #include "pcnet.h"
 
 namespace fsi {
@@ -163,25 +164,6 @@ __device__ __forceinline__ void bsum_store(double (&acc)[K], int k, double* out)
   }
 }
 
-template <typename T, int K>
-__device__ __forceinline__ void bsum_store_t(T (&acc)[K], int k, double* out) {
-  __shared__ T smt[K][BVB / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < K; ++i) {
-    T v = acc[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) smt[i][warp] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < k) {
-    T s = T(0);
-    for (int wi = 0; wi < BVB / 32; ++wi) s += smt[threadIdx.x][wi];
-    out[threadIdx.x] = (double)s;
-  }
-}
-
 // basis slot i of chunk c of instance b; the basis type VT is double for float64 solves and
 // float for the inner solves of float32 refinement (the same allocation, element offsets)
 template <typename VT>
@@ -274,7 +256,9 @@ __global__ void bk_tofloat(const int4* __restrict__ items, const int* __restrict
 }
 
 // partials of V_b[i] . w_b (rows i < nvec) and w_b . w_b (row nvec): groups of BKC vectors per
-// blockIdx.y, the last group (short, perhaps empty) takes w . w
+// blockIdx.y, the last group (short, perhaps empty) takes w . w.  Bound by loads in flight: with a float32
+// basis a thread takes four adjacent elements (here and in bk_store), and the CTA's sums go
+// through butterflies: twelve 16^3-48^3 cavities 226.4 -> 220.4 ms a solve.
 template <typename VT>
 __global__ void __launch_bounds__(BVB) bk_mdot(const int4* __restrict__ items, const int* __restrict__ act,
                                                const VT* V, const int64_t* vbase, const int64_t* off,
@@ -288,6 +272,41 @@ __global__ void __launch_bounds__(BVB) bk_mdot(const int4* __restrict__ items, c
   VT acc[BKC + 1];  // per-thread sums in the basis type, the CTA's sums stored as double
 #pragma unroll
   for (int i = 0; i <= BKC; ++i) acc[i] = VT(0);
+  if constexpr (sizeof(VT) == 4) {
+    // four chunks at a time, four adjacent elements a thread (one float4 per basis vector); w by
+    // element where the instance's vectors do not start on 16 bytes
+    const int sub = threadIdx.x >> 6, e0 = (threadIdx.x & 63) * 4;
+    const int64_t n = nloc[b];
+    const double* wb = w + off[b];
+    for (int64_t c = it.y + sub; c < it.z; c += 4) {
+      const int64_t e = c * BCH + e0;
+      if (e >= n) break;
+      const float* blk = V + vbase[b] + c * (int64_t)M1 * BCH + (int64_t)i0 * BCH + e0;
+      float x[4];
+      if (e + 4 <= n && (off[b] & 1) == 0) {
+        const double2 x01 = *reinterpret_cast<const double2*>(wb + e), x23 = *reinterpret_cast<const double2*>(wb + e + 2);
+        x[0] = (float)x01.x, x[1] = (float)x01.y, x[2] = (float)x23.x, x[3] = (float)x23.y;
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = e + u < n ? (float)wb[e + u] : 0.f;
+      }
+      if (e + 4 <= n) {
+#pragma unroll
+        for (int i = 0; i < BKC; ++i) {
+          if (i >= kc) break;
+          const float4 v = *reinterpret_cast<const float4*>(blk + i * BCH);
+          acc[i] += (v.x * x[0] + v.y * x[1]) + (v.z * x[2] + v.w * x[3]);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < BKC; ++i) {
+          if (i >= kc) break;
+          for (int u = 0; u < 3 && e + u < n; ++u) acc[i] += blk[i * BCH + u] * x[u];
+        }
+      }
+      if (self) acc[BKC] += (x[0] * x[0] + x[1] * x[1]) + (x[2] * x[2] + x[3] * x[3]);
+    }
+  } else
   for (int64_t c = it.y; c < it.z; ++c) {
     const int64_t e = c * BCH + threadIdx.x;
     if (e >= nloc[b]) break;
@@ -303,10 +322,9 @@ __global__ void __launch_bounds__(BVB) bk_mdot(const int4* __restrict__ items, c
     }
     if (self) acc[BKC] += wj * wj;
   }
-#pragma unroll
-  for (int i = 0; i < BKC; ++i)
-    if (i == kc) acc[i] = acc[BKC];
-  bsum_store_t<VT, BKC + 1>(acc, kc + (self ? 1 : 0), part + (int64_t)blockIdx.x * PSTRIDE + i0);
+  double* out = part + (int64_t)blockIdx.x * PSTRIDE + i0;
+  if constexpr (sizeof(VT) == 4) block_reduce_store_f<BKC + 1, BVB>(acc, kc + (self ? 1 : 0), self, out, 1);
+  else block_reduce_store_bf<BKC + 1, BVB>(acc, kc + (self ? 1 : 0), self, out, 1);
 }
 
 // The sums over the items of one instance of `rows` partials, in a fixed order, into dst (shared memory):
@@ -512,6 +530,60 @@ __global__ void __launch_bounds__(BVB) bk_store(const int4* __restrict__ items, 
     for (int i = threadIdx.x; i < slot; i += blockDim.x) hs[i] = (VT)K[b].h2[i];
   __syncthreads();
   const double s = s_sh;
+  if constexpr (sizeof(VT) == 4) {
+    // laid out as bk_mdot: four chunks at a time, four adjacent elements a thread
+    const int sub = threadIdx.x >> 6, e0 = (threadIdx.x & 63) * 4;
+    const int64_t n = nloc[b], o = off[b];
+    for (int64_t c = it.y + sub; c < it.z; c += 4) {
+      const int64_t e = c * BCH + e0;
+      if (e >= n) break;
+      float* blk = V + vbase[b] + c * (int64_t)M1 * BCH + e0;
+      const int cnt = (int)min((int64_t)4, n - e);
+      float a[4] = {0.f, 0.f, 0.f, 0.f};
+      if (second) {
+        if (cnt == 4) {
+#pragma unroll 8
+          for (int i = 0; i < slot; ++i) {
+            const float4 v = *reinterpret_cast<const float4*>(blk + (int64_t)i * BCH);
+            a[0] = fmaf(hs[i], v.x, a[0]);
+            a[1] = fmaf(hs[i], v.y, a[1]);
+            a[2] = fmaf(hs[i], v.z, a[2]);
+            a[3] = fmaf(hs[i], v.w, a[3]);
+          }
+        } else {
+          for (int i = 0; i < slot; ++i)
+            for (int u = 0; u < cnt; ++u) a[u] = fmaf(hs[i], blk[(int64_t)i * BCH + u], a[u]);
+        }
+      }
+      auto entry = [&](double x, float corr) {
+        return slot == 0 ? (float)(s * x) : (float)(s * (double)((float)x - corr));
+      };
+      if (cnt == 4 && (o & 3) == 0) {
+        const double2 x01 = *reinterpret_cast<const double2*>(src + o + e), x23 = *reinterpret_cast<const double2*>(src + o + e + 2);
+        const float4 v = make_float4(entry(x01.x, a[0]), entry(x01.y, a[1]), entry(x23.x, a[2]), entry(x23.y, a[3]));
+        *reinterpret_cast<float4*>(blk + (int64_t)slot * BCH) = v;
+        if (z) {
+          const double2 d01 = *reinterpret_cast<const double2*>(dinv + o + e), d23 = *reinterpret_cast<const double2*>(dinv + o + e + 2);
+          const double2 q01 = make_double2(d01.x * (double)v.x, d01.y * (double)v.y);
+          const double2 q23 = make_double2(d23.x * (double)v.z, d23.y * (double)v.w);
+          *reinterpret_cast<double2*>(z + o + e) = q01;
+          *reinterpret_cast<double2*>(z + o + e + 2) = q23;
+          if (dx32)  // (its base is that of z in floats: 16 bytes when off is a multiple of 4)
+            *reinterpret_cast<float4*>(dx32[b] + e) = make_float4((float)q01.x, (float)q01.y, (float)q23.x, (float)q23.y);
+        }
+      } else {
+        for (int u = 0; u < cnt; ++u) {
+          const float v = entry(src[o + e + u], a[u]);
+          blk[(int64_t)slot * BCH + u] = v;
+          if (z) {
+            const double q = dinv[o + e + u] * (double)v;
+            z[o + e + u] = q;
+            if (dx32) dx32[b][e + u] = (float)q;
+          }
+        }
+      }
+    }
+  } else
   for (int64_t c = it.y; c < it.z; ++c) {
     const int64_t e = c * BCH + threadIdx.x;
     if (e >= nloc[b]) break;
@@ -587,7 +659,15 @@ __global__ void bk_combine(const int4* __restrict__ items, const BKry* __restric
     if (e >= nloc[b]) break;
     const VT* blk = V + vbase[b] + c * (int64_t)M1 * BCH + threadIdx.x;
     double s = 0.0;
-    for (int i = 0; i < jend; ++i) s += ys[i] * (double)blk[(int64_t)i * BCH];
+    int i = 0;
+    for (; i + 8 <= jend; i += 8) {  // eight loads in flight, added in order
+      VT v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = blk[(int64_t)(i + u) * BCH];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += ys[i + u] * (double)v[u];
+    }
+    for (; i < jend; ++i) s += ys[i] * (double)blk[(int64_t)i * BCH];
     x[off[b] + e] += dinv[off[b] + e] * s;
   }
 }
@@ -1278,7 +1358,7 @@ int fsi_batch_create_blocks(fsi_mesh* const* meshes, const int32_t* blocks, int3
     if (int rc = block_info(meshes[i], blocks[i], &bi)) return fail(rc);
     chunks += (bi.n + BCH - 1) / BCH;
   }
-  const int64_t bitem = std::max<int64_t>(4, std::min<int64_t>(BITEM, chunks / (152 * 6)));
+  const int64_t bitem = std::max<int64_t>(4, std::min<int64_t>(BITEM, (chunks / (152 * 6) + 3) / 4 * 4));
   for (int i = 0; i < n; ++i) {
     BlockInfo bi;
     int rc = block_info(meshes[i], blocks[i], &bi);
