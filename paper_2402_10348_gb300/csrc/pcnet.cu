@@ -354,12 +354,12 @@ __global__ void pack_weights_kernel(const __grid_constant__ PackArgs a) {
 // Bound by latency on every level (a chain of 27 loads took 11 us on 33^3 and on 5^3 voxels alike):
 // the loads of a plane are in flight together, and CTAs are small so that a coarse level has some
 // for every SM: 6.4 and 4.0 us.
+// Threads over (x, y) of a plane, blockIdx.y the plane, blockIdx.z the octet.
 __global__ void restrict_kernel(TView f, TView c, float s, TView mask) {
-  const int64_t Vc = (int64_t)c.nx * c.ny * c.nz;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 2 * Vc; i += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(i / Vc);
-    const int64_t v = i - o * Vc;
-    const int X = (int)(v % c.nx), Y = (int)((v / c.nx) % c.ny), Z = (int)(v / ((int64_t)c.nx * c.ny));
+  const int v = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.z;
+  if (v >= c.nx * c.ny) return;
+  const int X = v % c.nx, Y = v / c.nx;
+  for (int Z = blockIdx.y; Z < c.nz; Z += gridDim.y) {
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const uint16_t* at = f.p + vox_addr(f, o, 2 * X, 2 * Y, 2 * Z);
 #pragma unroll
@@ -401,11 +401,10 @@ __global__ void restrict_kernel(TView f, TView c, float s, TView mask) {
 
 // fine[x] = (s * sum_X P[x, X] coarse[X] + add[x]) * [mask[x] > 0]   (add, mask optional)
 __global__ void prolong_kernel(TView c, TView f, float s, TView add, TView mask) {
-  const int64_t Vf = (int64_t)f.nx * f.ny * f.nz;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 2 * Vf; i += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(i / Vf);
-    const int64_t v = i - o * Vf;
-    const int x = (int)(v % f.nx), y = (int)((v / f.nx) % f.ny), z = (int)(v / ((int64_t)f.nx * f.ny));
+  const int v = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.z;
+  if (v >= f.nx * f.ny) return;
+  const int x = v % f.nx, y = v / f.nx;
+  for (int z = blockIdx.y; z < f.nz; z += gridDim.y) {
     const int xs[2] = {x >> 1, (x + 1) >> 1}, ys[2] = {y >> 1, (y + 1) >> 1}, zs[2] = {z >> 1, (z + 1) >> 1};
     const int nxs = (x & 1) ? 2 : 1, nys = (y & 1) ? 2 : 1, nzs = (z & 1) ? 2 : 1;
     const float w = 1.0f / (float)(nxs * nys * nzs);
@@ -528,38 +527,44 @@ __global__ void __launch_bounds__(32 * WGR) wgrad_reduce_kernel(const float* __r
 // (LBO), M groups octet planes apart (SBO).  A tap's shift by dx and dy moves the start address; the
 // octet planes of consecutive z planes are M groups of one matrix, so the three dz of a tap are one
 // MMA (M rows past 3 CIN read whatever follows inside the allocation and are not stored).
-// A work unit is 8 x 16 voxels of 4 z planes: its 6 input planes with their halo (180 x 16 bytes
-// an octet) and the gradient's 4 are copied by cp.async into one of two stages while the other's 288
-// MMAs run; warp 0 issues those, the other eight copy.  Each CTA walks a contiguous range of units with
-// the nine accumulators in TMEM (144 columns) and writes them once, as rows of consecutive M
-// that wgrad_reduce_kernel sums in a fixed order.
+// A work unit is 8 x 16 voxels of 1 to 4 z planes: its input planes and one on either side, with their
+// halo (180 x 16 bytes an octet), and the gradient's are copied by cp.async into one of two stages while
+// the other's MMAs (72 a plane) run; warp 0 issues those, the other eight copy.  Each CTA walks a
+// contiguous range of units with the nine accumulators in TMEM (144 columns) and writes them once, as
+// rows of consecutive M that wgrad_reduce_kernel sums in a fixed order.  Bound by the MMAs: the two
+// CTAs of an SM issue one every 48 cycles, 3 CIN of whose 128 rows are used.
 // Staging the 27 shifted copies of every voxel, transposed by shuffles, took 72 us on 64^3 (16
-// channels) and 177 (32); now 44 and 61.
+// channels) and 177 (32); now 44 and 41 (61 with one CTA per SM and 4-plane units).
 constexpr int WGM_LOADERS = 256;
 constexpr int WGM_THREADS = 32 + WGM_LOADERS;
-constexpr int WGM_P = 4;  // z planes of a unit
 
 template <int CIN>
 struct WgmCfg {
+  static constexpr int P = CIN == 16 ? 4 : 2;                  // most z planes of a unit: two CTAs fit an SM
   static constexpr int NO = CIN / 8;
   static constexpr int SLOT = NO * OCT_BYTES;                  // one staged input plane
-  static constexpr int XBYTES = (WGM_P + 2) * SLOT;
+  static constexpr int XBYTES = (P + 2) * SLOT;
   static constexpr int GOCT = TILE_X * TILE_Y * 16;            // one octet of a gradient plane
-  static constexpr int STAGE = XBYTES + WGM_P * 2 * GOCT;
+  static constexpr int STAGE = XBYTES + P * 2 * GOCT;
   static constexpr int HEAD = 128;
-  // the last plane's matrix spans 16 octet planes from its start, past the stage's end for CIN = 16
-  static constexpr int SPAN = (WGM_P - 1) * SLOT + 16 * OCT_BYTES;
+  // the last plane's matrix spans 16 octet planes from its start, past the stage's end
+  static constexpr int SPAN = (P - 1) * SLOT + 16 * OCT_BYTES;
   static constexpr int SMEM = HEAD + STAGE + (SPAN > STAGE ? SPAN : STAGE);
   static constexpr int NCOLS = 256;                            // nine accumulators of 16
 };
 
 struct WgmGrid {
-  int tx, ty, units;
+  int tx, ty, p, panels, units;  // tiles, z planes of a unit, units of a tile and in all
 };
-__host__ __device__ inline WgmGrid wgm_grid(const TView& g) {
+// p: the fewest z planes (1, 2, 4) with which a grid of `slots` CTAs takes all units at once, a CTA's MMAs
+// being a chain of 72 a plane (5^3 to 33^3 voxels: 15 us a kernel with 4 planes, 9 to 13 so); else the most
+static WgmGrid wgm_grid(const TView& g, int most, int slots) {
   WgmGrid w;
   w.tx = (g.nx + TILE_X - 1) / TILE_X, w.ty = (g.ny + TILE_Y - 1) / TILE_Y;
-  w.units = w.tx * w.ty * ((g.nz + WGM_P - 1) / WGM_P);
+  w.p = 1;
+  while (w.p < most && (int64_t)w.tx * w.ty * ((g.nz + w.p - 1) / w.p) > slots) w.p *= 2;
+  w.panels = (g.nz + w.p - 1) / w.p;
+  w.units = w.tx * w.ty * w.panels;
   return w;
 }
 
@@ -567,16 +572,15 @@ __host__ __device__ inline WgmGrid wgm_grid(const TView& g) {
 template <int CIN>
 __device__ __forceinline__ void wgm_load(const TView& x, const TView& g, const WgmGrid& w, int u, uint32_t stage, int t0) {
   using C = WgmCfg<CIN>;
-  const int panels = w.units / (w.tx * w.ty);
-  const int pz = u % panels, col = u / panels;
-  const int x0 = col % w.tx * TILE_X, y0 = col / w.tx * TILE_Y, z0 = pz * WGM_P;
-  for (int i = t0; i < (WGM_P + 2) * C::NO * SY * SX; i += WGM_LOADERS) {
+  const int pz = u % w.panels, col = u / w.panels;
+  const int x0 = col % w.tx * TILE_X, y0 = col / w.tx * TILE_Y, z0 = pz * w.p;
+  for (int i = t0; i < (w.p + 2) * C::NO * SY * SX; i += WGM_LOADERS) {
     const int pl = i / (SY * SX), rem = i - pl * (SY * SX), yy = rem / SX, xx = rem - yy * SX;
     const int z = z0 - 1 + pl / C::NO, gx = x0 - 1 + xx, gy = y0 - 1 + yy;
     const bool in = z >= 0 && z < x.nz && gx >= 0 && gx < x.nx && gy >= 0 && gy < x.ny;
     cp_async16(stage + 16 * i, in ? x.p + vox_addr(x, pl % C::NO, gx, gy, z) : x.p, in);
   }
-  for (int i = t0; i < WGM_P * 2 * TILE_X * TILE_Y; i += WGM_LOADERS) {
+  for (int i = t0; i < w.p * 2 * TILE_X * TILE_Y; i += WGM_LOADERS) {
     const int gx = x0 + (i & 7), gy = y0 + (i >> 3 & 15), o = i >> 7 & 1, z = z0 + (i >> 8);
     const bool in = gx < g.nx && gy < g.ny && z < g.nz;
     cp_async16(stage + C::XBYTES + 16 * i, in ? g.p + vox_addr(g, o, gx, gy, z) : g.p, in);
@@ -584,14 +588,14 @@ __device__ __forceinline__ void wgm_load(const TView& x, const TView& g, const W
 }
 
 template <int CIN>
-__global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g, float* __restrict__ part, int* err) {
+__global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g, WgmGrid w, float* __restrict__ part,
+                                                                int* err) {
   using C = WgmCfg<CIN>;
   extern __shared__ __align__(1024) uint8_t sm[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm);
   uint32_t* holder = reinterpret_cast<uint32_t*>(sm + 16);
   const uint32_t base = smem_u32(sm + C::HEAD);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const WgmGrid w = wgm_grid(g);
   const int u0 = (int)((int64_t)w.units * blockIdx.x / gridDim.x);
   const int nu = (int)((int64_t)w.units * (blockIdx.x + 1) / gridDim.x) - u0;
   if (nu <= 0) return;  // (not with at most one CTA per unit) uniform, before any barrier or allocation
@@ -623,8 +627,7 @@ __global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g
     if (warp == 0) {
       if (lane == 0) {
         const uint32_t xb = base + s * C::STAGE, gb = xb + C::XBYTES;
-        const int panels = w.units / (w.tx * w.ty);
-        const int planes = min(WGM_P, g.nz - (u0 + i) % panels * WGM_P);
+        const int planes = min(w.p, g.nz - (u0 + i) % w.panels * w.p);
 #pragma unroll 1
         for (int z = 0; z < planes; ++z)
 #pragma unroll 1
@@ -917,11 +920,11 @@ int launch_wgrad_mma(fsi_pc* pc, const TView& x, const TView& g, int* nblk_out) 
   using C = WgmCfg<CIN>;
   fsi_mesh* m = pc->m;
   if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&wgrad_mma_kernel<CIN>), C::SMEM)) return rc;
-  // shared memory and 256 of 512 TMEM columns: two CTAs per SM for 16 channels, one for 32
-  const int per_sm = std::max(1, std::min(512 / C::NCOLS, (228 * 1024) / (C::SMEM + 1024)));
-  const int nblk = std::min(wgm_grid(g).units, per_sm * 152);
+  static_assert(2 * (C::SMEM + 1024) <= 228 * 1024 && 2 * C::NCOLS <= 512, "two CTAs per SM");
+  const WgmGrid w = wgm_grid(g, C::P, 2 * 152);
+  const int nblk = std::min(w.units, 2 * 152);
   if ((int64_t)nblk * 16 * CIN * 27 > pc->wpart_n) return set_error(FSI_EINVAL, "pc: weight-gradient scratch too small");
-  FSI_LAUNCH(m, P_PC_WGRAD, (wgrad_mma_kernel<CIN><<<nblk, WGM_THREADS, C::SMEM, m->stream>>>(x, g, pc->wpart, pc->err)));
+  FSI_LAUNCH(m, P_PC_WGRAD, (wgrad_mma_kernel<CIN><<<nblk, WGM_THREADS, C::SMEM, m->stream>>>(x, g, w, pc->wpart, pc->err)));
   *nblk_out = nblk;
   return FSI_OK;
 }
@@ -940,14 +943,16 @@ int wgrad(fsi_pc* pc, int layer, const TView& x, const TView& g) {
   return FSI_OK;
 }
 
+dim3 plane_grid(const TView& t, int tb) {
+  return dim3((unsigned)((t.nx * t.ny + tb - 1) / tb), (unsigned)std::min(t.nz, 65535), 2);
+}
+
 int restrict_(fsi_pc* pc, const TView& f, const TView& c, float s, const TView& mask) {
-  const int64_t n = 2LL * c.nx * c.ny * c.nz;
-  FSI_LAUNCH(pc->m, P_PC_AUX, (restrict_kernel<<<vgrid1(n, 64), 64, 0, pc->m->stream>>>(f, c, s, mask)));
+  FSI_LAUNCH(pc->m, P_PC_AUX, (restrict_kernel<<<plane_grid(c, 64), 64, 0, pc->m->stream>>>(f, c, s, mask)));
   return FSI_OK;
 }
 int prolong_(fsi_pc* pc, const TView& c, const TView& f, float s, const TView& add, const TView& mask) {
-  const int64_t n = 2LL * f.nx * f.ny * f.nz;
-  FSI_LAUNCH(pc->m, P_PC_AUX, (prolong_kernel<<<vgrid1(n), 256, 0, pc->m->stream>>>(c, f, s, add, mask)));
+  FSI_LAUNCH(pc->m, P_PC_AUX, (prolong_kernel<<<plane_grid(f, 128), 128, 0, pc->m->stream>>>(c, f, s, add, mask)));
   return FSI_OK;
 }
 
@@ -1297,9 +1302,9 @@ int fsi_pc_create(fsi_mesh* m, const fsi_pc_desc* d, fsi_pc** out) {
       (rc = dalloc(&pc->ys1, (int64_t)pc->cout * pc->lv[1].nv())) ||
       (rc = dalloc(&pc->loss_dev, 1 << 16)) || (rc = dalloc(&pc->err, 1)))
     return fail(rc);
-  // weight-gradient partials: one CTA per SM with 32 input channels or two with 16
+  // weight-gradient partials of two CTAs per SM
   {
-    pc->wpart_n = (int64_t)152 * 16 * 32 * 27;
+    pc->wpart_n = (int64_t)2 * 152 * 16 * 32 * 27;
     if ((rc = dalloc(&pc->wpart, pc->wpart_n))) return fail(rc);
   }
   pc->dmask = m->mask;
