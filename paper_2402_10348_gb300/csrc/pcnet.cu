@@ -685,12 +685,13 @@ __global__ void loss_kernel(const float* __restrict__ y, const uint16_t* __restr
   double s = 0.0;
   const float ki[4] = {kinv.x, kinv.y, kinv.z, kinv.w};
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(v % dy.nx), yy = (int)((v / dy.nx) % dy.ny), z = (int)(v / ((int64_t)dy.nx * dy.ny));
     float gch[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) gch[c] = 0.0f;
     const uint8_t mk = dmask ? dmask[v] : 0;
-    for (int c = 0; c < cout; ++c) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (c >= cout) break;
       const bool valid = !((mk >> c) & 1);
       const float d = valid ? y[(int64_t)c * V + v] - bf2f(t[(int64_t)c * V + v]) * ki[c] : 0.0f;
       s += (double)wgt * d * d;
@@ -703,7 +704,7 @@ __global__ void loss_kernel(const float* __restrict__ y, const uint16_t* __restr
       o.y = (uint32_t)f2bf(gch[8 * q + 2]) | ((uint32_t)f2bf(gch[8 * q + 3]) << 16);
       o.z = (uint32_t)f2bf(gch[8 * q + 4]) | ((uint32_t)f2bf(gch[8 * q + 5]) << 16);
       o.w = (uint32_t)f2bf(gch[8 * q + 6]) | ((uint32_t)f2bf(gch[8 * q + 7]) << 16);
-      *reinterpret_cast<uint4*>(dy.p + vox_addr(dy, q, x, yy, z)) = o;
+      *reinterpret_cast<uint4*>(dy.p + ((int64_t)(dy.oct0 + q) * V + v) * 8) = o;
     }
   }
   __shared__ double sh[256];
@@ -894,9 +895,13 @@ int launch_conv(fsi_pc* pc, const TView& in, const TView& out, const TView& mask
   if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&conv_mma_kernel<CIN, N>), C::SMEM)) return rc;
   const int gx = (out.nx + TILE_X - 1) / TILE_X, gy = (out.ny + TILE_Y - 1) / TILE_Y;
   const int cols = gx * gy;
-  // CTAs resident per SM (shared memory bound) x 152 SMs: enough z-chunks to fill them
-  const int per_sm = std::max(1, std::min(8, (227 * 1024) / (C::SMEM + 1024)));
-  const int zc = std::max(1, (int)((int64_t)out.nz * cols / (per_sm * 152)));
+  // CTAs resident per SM (shared memory bound) x 152 SMs: as many z-chunks as fit at once.  (Rounded
+  // down, the chunk length gave a second wave of a few CTAs: 64^3, 990 CTAs of 3 planes on 912 slots, 22.0
+  // -> 19.7 us; 32 -> 16 channels 44.5 -> 37.4, 16 -> 32 26.4 -> 20.5.  What binds then is the MMAs: 128 x 16
+  // of A read from shared memory for 16 columns, one per 75 cycles and SM.)
+  const int slots = std::max(1, std::min(8, (227 * 1024) / (C::SMEM + 1024))) * 152;
+  const int most = std::max(1, slots / cols);  // z-chunks
+  const int zc = (out.nz + most - 1) / most;
   const int gz = (out.nz + zc - 1) / zc;
   ConvArgs a{in, out, mask, out32, nreal, wpk, zc, relu, pc->err};
   FSI_LAUNCH(m, P_PC_CONV, (conv_mma_kernel<CIN, N><<<dim3(gx, gy, gz), CONV_THREADS, C::SMEM, m->stream>>>(a)));
