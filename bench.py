@@ -71,8 +71,7 @@ def parse():
 def run_solve_case(precision: str = "fp32ir", block: str = "ns"):
     """Forty Arnoldi steps of one block of the 64^3 cavity (ns, ac: phase 0, b: the solid),
     float32 operator inside float64 refinement (fp32ir: the NS coefficient product in
-    float32) or float64 (NS: the first 8 products from the coefficients, the rest through
-    element matrices; AC: element matrices from the third product; B: the split operator):
+    float32) or float64 (assembled rows: NS and B from the first product, AC from the third):
     the launch sequences the profiles under profiles/ were captured on."""
     import torch
     from paper_2402_10348_gb300 import fsi
@@ -495,8 +494,8 @@ def run_tet_case(reps: int = 5):
     cell, interior nodes jittered by 0.2 h): the 64^3 cavity's box (1.57 M elements) and
     the falling sphere's 96x96x192 box (10.6 M elements), on seeded random states.  Each
     apply is an element kernel plus a node-sum kernel; time per apply = class time / calls.
-    Inside a 40-iteration NS GMRES the products after the eighth run through the element
-    matrices (`ns_jvp_f64_element_matrix`, with the one build's time)."""
+    Inside a 40-iteration NS GMRES the products run through the assembled rows
+    (`ns_jvp_f64_assembled`, with the one build's time)."""
     import torch
     from paper_2402_10348_gb300 import fsi
     from workloads import cavity64, falling, random_state, tet_box_mesh
@@ -539,7 +538,7 @@ def run_tet_case(reps: int = 5):
         prof = fsi.fsi_profile_read(mesh)
         fsi.fsi_profile(mesh, False)
         res["gamma_beta"] = {"ms_per_call": round(prof.get("gamma_beta", (0, 0.0))[1] / reps, 3)}
-        # inside a solve: after 8 products the NS product runs through element matrices
+        # inside a solve the NS product runs through assembled rows
         rhs = torch.randn(4 * nn, dtype=torch.float64, device=dev, generator=g)
         sol = torch.zeros_like(rhs)
         o = fsi.solve_opts(m=30, rtol=1e-30, max_iter=40)
@@ -552,7 +551,7 @@ def run_tet_case(reps: int = 5):
         em, nd, bld = (prof.get(k, (0, 0.0)) for k in ("ns_jvp_f64_em", "node_sums", "op_builds"))
         if em[0] > 0:
             per = (em[1] + nd[1]) / em[0]
-            res["ns_jvp_f64_element_matrix"] = {"ms_per_apply": round(per, 3), "gdofs": round(4 * nn / (per / 1e3) / 1e9, 3),
+            res["ns_jvp_f64_assembled"] = {"ms_per_apply": round(per, 3), "gdofs": round(4 * nn / (per / 1e3) / 1e9, 3),
                                                 "applies": em[0], "build_ms": round(bld[1], 3)}
         out[wl.name] = {"elements": int(conn.shape[0]), "nodes": nn, "operators": res}
         if wl.name == "cavity64":
@@ -748,14 +747,17 @@ class Clocks:
 # recomputation), counted from the arithmetic of the kernels' element functions;
 # multiply by the elements of one launch.
 def flops_per_element(kernel: str, n_solid: int) -> float:
-    """The float64 NS product through element matrices: 2 x 32 x 32 per element.  Per
-    quadrature point: the NS product from frozen coefficients 486 + 114 with solids
-    (interpolation of dv, dp: 172; convective and mass terms 54; stresses 92; the
-    elastic linearization 114; test-function scatter 166), its coefficient build
-    635 + 167 per solid, NS residual 635 + 167 per solid, AC JVP 247, B JVP 892; 8
-    points per element."""
-    if kernel == "ns_jvp_f64_em":
-        return 2.0 * 32 * 32  # the element matrix applied: 1024 FMAs per element
+    """Assembled float64 products, one FMA per stored entry: 27 blocks of 4 x 4 a node (NS), 27
+    entries (AC, from a solve's third product), 27 x 24 (B, from its first: 12 values, the
+    couplings used twice); taken per
+    element here (a mesh has a few percent more nodes).  Per quadrature point: the NS
+    product from frozen coefficients 486 + 114 with solids (interpolation of dv, dp: 172;
+    convective and mass terms 54; stresses 92; the elastic linearization 114;
+    test-function scatter 166), NS residual 635 + 167 per solid, AC JVP 247, B JVP 892
+    (float32); 8 points per element."""
+    assembled = {"ns_jvp_f64_em": 27 * 16, "ac_jvp_f64": 27, "b_jvp_f64": 27 * 24}
+    if kernel in assembled:
+        return 2.0 * assembled[kernel]
     per_qp = {"ns_jvp": 486 + (114 if n_solid > 0 else 0), "op_builds": 0,
               "ns_residual": 635 + 167 * n_solid, "ac_jvp": 247, "b_jvp": 892}
     for k, v in per_qp.items():
