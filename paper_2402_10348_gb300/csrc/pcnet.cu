@@ -527,20 +527,21 @@ __global__ void __launch_bounds__(32 * WGR) wgrad_reduce_kernel(const float* __r
 // (LBO), M groups octet planes apart (SBO).  A tap's shift by dx and dy moves the start address; the
 // octet planes of consecutive z planes are M groups of one matrix, so the three dz of a tap are one
 // MMA (M rows past 3 CIN read whatever follows inside the allocation and are not stored).
-// A work unit is 8 x 16 voxels of 1 to 4 z planes: its input planes and one on either side, with their
+// A work unit is 8 x 16 voxels of 1 or 2 z planes: its input planes and one on either side, with their
 // halo (180 x 16 bytes an octet), and the gradient's are copied by cp.async into one of two stages while
 // the other's MMAs (72 a plane) run; warp 0 issues those, the other eight copy.  Each CTA walks a
 // contiguous range of units with the nine accumulators in TMEM (144 columns) and writes them once, as
 // rows of consecutive M that wgrad_reduce_kernel sums in a fixed order.  Bound by the MMAs: the two
 // CTAs of an SM issue one every 48 cycles, 3 CIN of whose 128 rows are used.
 // Staging the 27 shifted copies of every voxel, transposed by shuffles, took 72 us on 64^3 (16
-// channels) and 177 (32); now 44 and 41 (61 with one CTA per SM and 4-plane units).
+// channels) and 177 (32); now 38 and 41.  (Units of 4 planes: 44, three units on the
+// busiest CTA against 2.5 on average, and 61, one CTA per SM.)
 constexpr int WGM_LOADERS = 256;
 constexpr int WGM_THREADS = 32 + WGM_LOADERS;
 
 template <int CIN>
 struct WgmCfg {
-  static constexpr int P = CIN == 16 ? 4 : 2;                  // most z planes of a unit: two CTAs fit an SM
+  static constexpr int P = 2;                                  // most z planes of a unit
   static constexpr int NO = CIN / 8;
   static constexpr int SLOT = NO * OCT_BYTES;                  // one staged input plane
   static constexpr int XBYTES = (P + 2) * SLOT;
@@ -556,7 +557,7 @@ struct WgmCfg {
 struct WgmGrid {
   int tx, ty, p, panels, units;  // tiles, z planes of a unit, units of a tile and in all
 };
-// p: the fewest z planes (1, 2, 4) with which a grid of `slots` CTAs takes all units at once, a CTA's MMAs
+// p: the fewest z planes (1, 2) with which a grid of `slots` CTAs takes all units at once, a CTA's MMAs
 // being a chain of 72 a plane (5^3 to 33^3 voxels: 15 us a kernel with 4 planes, 9 to 13 so); else the most
 static WgmGrid wgm_grid(const TView& g, int most, int slots) {
   WgmGrid w;

@@ -1,10 +1,10 @@
-"""The weight-gradient kernel where its work units (8 x 16 x 4 voxels) are ragged and where a CTA walks
-several of them (612 units on 152 or 304 CTAs), on inputs that are known exactly: with centre-tap
+"""The weight-gradient kernel where its work units (8 x 16 voxels of one or two planes) are ragged and
+where a CTA walks several of them (1,188 units on 304 CTAs), on inputs that are known exactly: with centre-tap
 identities on the finest level and zeros below, every activation there is the network's input x and
 every activation gradient the loss's gradient g, so dW[co][ci][t] = sum_v g[co][v] x[ci][v + t].
 
-Bound: bfloat16 products are exact in float32; a CTA adds at most 5 units x 32 of them in turn to
-an accumulator and up to 40 such sums follow, each addition off by at most 2^-22 of the sum of
+Bound: bfloat16 products are exact in float32; a CTA adds at most 160 sixteens of them in turn
+to an accumulator and up to 40 such sums follow, each addition off by at most 2^-22 of the sum of
 magnitudes: 200 x 2^-22 = 4.8e-5 of sum |g| |x|."""
 import numpy as np
 import pytest
