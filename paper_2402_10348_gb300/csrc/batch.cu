@@ -44,7 +44,7 @@
 
 namespace fsi {
 
-constexpr int BCH = 256;      // elements per basis chunk
+constexpr int BCH = KCH;      // elements per basis chunk
 constexpr int BMMAX = 64;     // largest restart length
 constexpr int BITEM = 32;     // most chunks per vector work item
 constexpr int BVB = 256;      // threads per CTA of the vector kernels
@@ -448,10 +448,13 @@ __global__ void __launch_bounds__(BUD) bk_upd_dot(const int4* __restrict__ items
   }
 }
 
-// Sums of those, the DGKS decision and the Givens step (givens_step in krylov.cu), one CTA per
+// Sums of those, the DGKS decision and the Givens step (orth_step and givens_step in krylov.cu), one CTA per
 // instance: the column and the rotations are read by all threads, one runs the chain in shared memory.
+template <typename VT>
 __global__ void __launch_bounds__(BROW * BRG) bk_givens(const int* __restrict__ first, const double* __restrict__ part,
-                                                        BKry* K, int* act, int j, int mm, double rtol) {
+                                                        BKry* K, int* act, int j, int mm, double rtol,
+                                                        const double* w, const VT* V, const int64_t* vbase,
+                                                        const int64_t* off, const int64_t* nloc, int M1) {
   __shared__ double sm[BRG][BROW];
   __shared__ double c2[BROW], col[BMMAX + 2], cs[BMMAX], sn[BMMAX];
   const int b = blockIdx.x;
@@ -467,11 +470,13 @@ __global__ void __launch_bounds__(BROW * BRG) bk_givens(const int* __restrict__ 
   item_sums(first, part, b, j + 2, sm, c2);
   const double w2 = c2[j + 1];
   const bool reorth = sqrt(w2) < sqrt(k.h[j + 1]) * 0.70710678118654752;
-  double hh = 0.0;  // |h2|^2, in warp 0
+  __shared__ double hh_sh;  // |h2|^2
   if (threadIdx.x < 32) {
+    double hh = 0.0;
     for (int i = threadIdx.x; i <= j; i += 32) hh = fma(c2[i], c2[i], hh);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+    if (threadIdx.x == 0) hh_sh = hh;
   }
   if (reorth)
     for (int i = threadIdx.x; i <= j; i += blockDim.x) {
@@ -479,9 +484,11 @@ __global__ void __launch_bounds__(BROW * BRG) bk_givens(const int* __restrict__ 
       k.h2[i] = c2[i];
     }
   __syncthreads();
+  double w2n = reorth ? w2 - hh_sh : w2;  // |w - V h2|^2; a NaN stays one and deactivates the instance below
+  if (reorth && hh_sh > PYTHAGORAS * w2)
+    w2n = corrected_norm2<VT, false>(w + off[b], V + vbase[b], M1, j + 1, c2, nloc[b]);
   if (threadIdx.x == 0) {
-    const double df = w2 - hh;  // |w - V h2|^2; a NaN stays one and deactivates the instance below
-    const double hn = sqrt(reorth ? (df < 0.0 ? 0.0 : df) : w2);
+    const double hn = sqrt(w2n);
     k.nrm_fin = hn;
     k.reorth = reorth ? 1 : 0;
     double t = col[0];
@@ -1079,7 +1086,8 @@ int enqueue_step_t(fsi_batch* b, int j, double rtol, bool f32) {
   BK_LAUNCH(b, P_KRY_DOT, bk_reduce<<<nb, BROW * BRG, 0, s>>>(b->item_first_dev, b->part, b->K, b->act, nvec));
   BK_LAUNCH(b, P_KRY_UPD, rc = launch_upd_dot<VT>(b, V, nvec));
   if (rc) return rc;
-  BK_LAUNCH(b, P_KRY_SMALL, bk_givens<<<nb, BROW * BRG, 0, s>>>(b->item_first_dev, b->part, b->K, b->act, j, b->mm, rtol));
+  BK_LAUNCH(b, P_KRY_SMALL, bk_givens<VT><<<nb, BROW * BRG, 0, s>>>(b->item_first_dev, b->part, b->K, b->act, j, b->mm, rtol,
+                                                                     b->w, V, b->vbase_dev, b->off_dev, b->nloc_dev, M1));
   BK_LAUNCH(b, P_KRY_UPD, bk_store<VT><<<NI, BVB, 0, s>>>(b->items_dev, b->K, b->act, V, b->vbase_dev, b->off_dev,
                                                        b->nloc_dev, M1, j + 1, b->w, b->dinv,
                                                        b->use_pc ? nullptr : b->z, f32 ? b->dx32_dev : nullptr));

@@ -103,4 +103,59 @@ __device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, bo
   }
 }
 
+// |w - V h2|^2 after the second Gram-Schmidt pass.  On an orthonormal basis it is |w|^2 - |h2|^2, which is
+// free, but wrong by delta |h2|^2 where V is orthonormal to delta (the basis type's rounding), and all
+// rounding where |h2| nears |w|: in an exhausted Krylov space the difference made vectors of length 7e-4 of
+// what is left, or 0, a breakdown that is none.  So it is taken up to PYTHAGORAS of |w|^2 only (an
+// error of 1e-4 of the basis type's rounding; the solves of the 16^3 to 64^3 cavities stay below); past it
+// corrected_norm2 sums the corrected vector itself.
+constexpr double PYTHAGORAS = 1e-4;
+constexpr int KCH = 256;  // elements of a basis chunk
+
+// By one CTA, for the whole vector (all threads take part; valid in thread 0): the entries that the basis
+// store makes, in its order of operations (what is left may be rounding alone), squares in float64.  PAIRS:
+// float basis, even and odd vectors in two sums where a group of four elements is whole (upd_store4_kernel),
+// else one chain.  w was written by other CTAs of the same launch.
+template <typename VT, bool PAIRS>
+__device__ __noinline__ double corrected_norm2(const double* w, const VT* __restrict__ V, int M1, int k, const double* h2,
+                                               int64_t n) {
+  __shared__ VT hs[96];
+  __shared__ double sw[32];
+  for (int i = threadIdx.x; i < k; i += blockDim.x) hs[i] = (VT)h2[i];
+  __syncthreads();
+  double s = 0.0;
+  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+    const VT* blk = V + j / KCH * (int64_t)M1 * KCH + j % KCH;
+    VT x = (VT)__ldcg(w + j);
+    if constexpr (sizeof(VT) == 8) {
+#pragma unroll 8
+      for (int i = 0; i < k; ++i) x = fma(-hs[i], blk[(int64_t)i * KCH], x);
+    } else {
+      VT a = 0, b = 0;
+      if (PAIRS && (j & ~(int64_t)3) + 4 <= n) {
+        int i = 0;
+#pragma unroll 4
+        for (; i + 2 <= k; i += 2) {
+          a = fmaf(hs[i], blk[(int64_t)i * KCH], a);
+          b = fmaf(hs[i + 1], blk[(int64_t)(i + 1) * KCH], b);
+        }
+        if (i < k) a = fmaf(hs[i], blk[(int64_t)i * KCH], a);
+      } else {
+#pragma unroll 8
+        for (int i = 0; i < k; ++i) a = fmaf(hs[i], blk[(int64_t)i * KCH], a);
+      }
+      x -= a + b;
+    }
+    s = fma((double)x, (double)x, s);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int q = 0; q < (int)blockDim.x >> 5; ++q) t += sw[q];
+  return t;
+}
+
 }  // namespace fsi

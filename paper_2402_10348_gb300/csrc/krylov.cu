@@ -17,7 +17,7 @@
 //   w -= V h, |w|^2 and h2 = V^T w (the second pass's projections of the updated w)
 //   in one pass                                           (upd_dot_kernel); its last CTA:
 //   if |w_new| < |w_old| / sqrt(2) (classical Gram-Schmidt with the DGKS
-//   re-orthogonalization test) h += h2 and |w|^2 -= |h2|^2 (the basis is orthonormal)
+//   re-orthogonalization test) h += h2 and |w|^2 -= |h2|^2 (summed anew where |h2| is near |w|)
 //   V_{j+1} = (w - V h2) / |w| (V h2 only where the test asked for it) into its slot, and
 //   z = D V_{j+1} beside it                                (upd_store_kernel); one more CTA: the
 //   Givens rotation of the new Hessenberg column and the residual estimate, written to pinned
@@ -43,7 +43,7 @@
 namespace fsi {
 
 constexpr int VB = 256;   // threads per CTA of the vector kernels
-constexpr int CH = 256;   // elements per basis chunk (one per thread)
+constexpr int CH = KCH;   // elements per basis chunk (one per thread)
 constexpr int DCH = 16;   // dot products per CTA pass
 constexpr int MMAX = 64;  // largest restart length
 
@@ -279,30 +279,37 @@ __device__ __forceinline__ VT lin_comb_chunk(const VT* __restrict__ hs, const VT
 // After the fused update, by the last CTA of its kernel: h2 (the second pass's projections of the
 // updated w) and |w|^2 summed from the partials, and the DGKS decision.  K->h becomes column j of the
 // Hessenberg matrix: h, plus h2 where |w_new| < |w_old| / sqrt(2) asked for the second pass, and
-// K->nrm_fin the new norm below it: |w - V h2|^2 = |w|^2 - |h2|^2 on an orthonormal basis, so the
-// second pass needs no sweep before its norm is known.
-__device__ __forceinline__ void orth_step(const double* part, int G, KryDev* K, int j) {
+// K->nrm_fin the new norm below it, without a sweep where |h2| is small beside |w| (PYTHAGORAS).
+template <typename VT>
+__device__ __forceinline__ void orth_step(const double* part, int G, KryDev* K, int j, const double* w, const VT* V, int M1,
+                                          int64_t n) {
   __shared__ double c2[MMAX + 2];
+  __shared__ bool measure;
   sum_rows<8>(part, G, j + 2, c2);
   __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const double w2 = c2[j + 1];
-  const bool reorth = sqrt(w2) < sqrt(K->h[j + 1]) * 0.70710678118654752;
-  double hh = 0.0;  // |h2|^2
-  for (int q = threadIdx.x; q <= j; q += 32) {
-    hh = fma(c2[q], c2[q], hh);
-    if (reorth) {
-      K->h[q] += c2[q];
-      K->h2[q] = c2[q];
+  if (threadIdx.x < 32) {
+    const double w2 = c2[j + 1];
+    const bool reorth = sqrt(w2) < sqrt(K->h[j + 1]) * 0.70710678118654752;
+    double hh = 0.0;  // |h2|^2
+    for (int q = threadIdx.x; q <= j; q += 32) {
+      hh = fma(c2[q], c2[q], hh);
+      if (reorth) {
+        K->h[q] += c2[q];
+        K->h2[q] = c2[q];
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+    if (threadIdx.x == 0) {
+      measure = reorth && hh > PYTHAGORAS * w2;
+      K->nrm_fin = sqrt(reorth && !measure ? w2 - hh : w2);  // a NaN stays one: the host stops on it
+      K->reorth = reorth ? 1 : 0;
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
-  if (threadIdx.x == 0) {
-    const double df = w2 - hh;  // a NaN stays one: the host stops on it
-    K->nrm_fin = sqrt(reorth ? (df < 0.0 ? 0.0 : df) : w2);
-    K->reorth = reorth ? 1 : 0;
-  }
+  __syncthreads();
+  if (!measure) return;
+  const double s = corrected_norm2<VT, sizeof(VT) == 4>(w, V, M1, j + 1, c2, n);
+  if (threadIdx.x == 0) K->nrm_fin = sqrt(s);
 }
 
 // The Givens step by one CTA, beside the basis store: column j is rotated by the previous rotations
@@ -515,7 +522,7 @@ __global__ void __launch_bounds__(UDT) upd_dot_kernel(double* __restrict__ w, co
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) part[(int64_t)i * G + blockIdx.x] = s;
   }
-  if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1);
+  if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1, w, V, M1, n);
 }
 
 // The fused update for the float32 basis: a thread takes two adjacent elements of each
@@ -575,7 +582,7 @@ __global__ void __launch_bounds__(ud2_threads<KMAX>()) upd_dot2_kernel(double* _
   }
   // rows i < k the projections, row k the norm
   block_reduce_store_f<KMAX + 1, NT>(acc, k + 1, true, part + blockIdx.x, G);
-  if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1);
+  if (last_cta(&K->counter, gridDim.x)) orth_step(part, G, K, k - 1, w, V, M1, n);
 }
 
 template <int KMAX, typename VT>
