@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
   if (second)
     for (int i = threadIdx.x; i < k; i += VB) hs[i] = (float)K->h2[i];
   __syncthreads();
-  const float scale = (float)s_sh;
+  const double scale = s_sh;  // (its rounding would be one error of 6e-8 common to all of V_k)
   const int64_t nch = (n + CH - 1) / CH;
   const int sub = threadIdx.x >> 6;
   const int e0 = (threadIdx.x & 63) * 4;
@@ -443,10 +443,10 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
       const double2 w01 = *reinterpret_cast<const double2*>(w + j);
       const double2 w23 = *reinterpret_cast<const double2*>(w + j + 2);
       float4 v;
-      v.x = ((float)w01.x - (a.x + b.x)) * scale;
-      v.y = ((float)w01.y - (a.y + b.y)) * scale;
-      v.z = ((float)w23.x - (a.z + b.z)) * scale;
-      v.w = ((float)w23.y - (a.w + b.w)) * scale;
+      v.x = (float)((double)((float)w01.x - (a.x + b.x)) * scale);
+      v.y = (float)((double)((float)w01.y - (a.y + b.y)) * scale);
+      v.z = (float)((double)((float)w23.x - (a.z + b.z)) * scale);
+      v.w = (float)((double)((float)w23.y - (a.w + b.w)) * scale);
       *reinterpret_cast<float4*>(blk + (int64_t)k * CH) = v;
       if (z) {
         const double2 d01 = *reinterpret_cast<const double2*>(dinv + j), d23 = *reinterpret_cast<const double2*>(dinv + j + 2);
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
         float acc = 0.f;
         if (second)
           for (int i = 0; i < k; ++i) acc += hs[i] * blk[i * CH + e];
-        const float v = ((float)w[j + e] - acc) * scale;
+        const float v = (float)((double)((float)w[j + e] - acc) * scale);
         blk[(int64_t)k * CH + e] = v;
         if (z) z[j + e] = (float)dinv[j + e] * v;
       }
