@@ -416,7 +416,9 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
   if (second)
     for (int i = threadIdx.x; i < k; i += VB) hs[i] = (float)K->h2[i];
   __syncthreads();
-  const double scale = s_sh;  // (its rounding would be one error of 6e-8 common to all of V_k)
+  // 1 / |w| in two floats: rounded to one, its error would be common to all of V_k
+  const float sh = (float)s_sh, sl = (float)(s_sh - (double)sh);
+  auto scaled = [&](float x) { return fmaf(x, sh, x * sl); };
   const int64_t nch = (n + CH - 1) / CH;
   const int sub = threadIdx.x >> 6;
   const int e0 = (threadIdx.x & 63) * 4;
@@ -443,10 +445,10 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
       const double2 w01 = *reinterpret_cast<const double2*>(w + j);
       const double2 w23 = *reinterpret_cast<const double2*>(w + j + 2);
       float4 v;
-      v.x = (float)((double)((float)w01.x - (a.x + b.x)) * scale);
-      v.y = (float)((double)((float)w01.y - (a.y + b.y)) * scale);
-      v.z = (float)((double)((float)w23.x - (a.z + b.z)) * scale);
-      v.w = (float)((double)((float)w23.y - (a.w + b.w)) * scale);
+      v.x = scaled((float)w01.x - (a.x + b.x));
+      v.y = scaled((float)w01.y - (a.y + b.y));
+      v.z = scaled((float)w23.x - (a.z + b.z));
+      v.w = scaled((float)w23.y - (a.w + b.w));
       *reinterpret_cast<float4*>(blk + (int64_t)k * CH) = v;
       if (z) {
         const double2 d01 = *reinterpret_cast<const double2*>(dinv + j), d23 = *reinterpret_cast<const double2*>(dinv + j + 2);
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(VB) upd_store4_kernel(const double* __restrict
         float acc = 0.f;
         if (second)
           for (int i = 0; i < k; ++i) acc += hs[i] * blk[i * CH + e];
-        const float v = (float)((double)((float)w[j + e] - acc) * scale);
+        const float v = scaled((float)w[j + e] - acc);
         blk[(int64_t)k * CH + e] = v;
         if (z) z[j + e] = (float)dinv[j + e] * v;
       }
