@@ -119,9 +119,9 @@ __device__ __forceinline__ void block_reduce_store(double (&acc)[K], int kc, dou
 // The basis type VT is double for float64 solves and float for the inner solves of
 // iterative refinement (a float32 operator inside float64 refinement: the inner solve
 // only has to reduce its residual by ir_inner_rtol, far above float32 rounding, and the
-// refinement's float64 residual removes what the inner solve leaves).  Products and
-// per-thread sums are taken in VT, the sums across threads and CTAs in float64.  The work
-// vector w, the preconditioner diagonal and every vector outside the basis stay float64.
+// refinement's float64 residual removes what the inner solve leaves).  Products, per-thread sums and,
+// with a float basis, the sums of a warp are taken in VT, those across warps and CTAs in float64.  The
+// work vector w, the preconditioner diagonal and every vector outside the basis stay float64.
 
 // Whether this CTA is the last of `total` to get here; its earlier global writes (and, for the last
 // CTA, everybody's) are visible after it.  The counter is back to 0 for the next kernel.
