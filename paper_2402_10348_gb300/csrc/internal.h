@@ -84,7 +84,7 @@ struct fsi_mesh {
   int64_t na_len = 0;
   int64_t na_gen = -1;               // stage_gen of the last build
   unsigned na_flags = 0;             // FSI_ELASTIC_AUG of the last build
-  double* ke64 = nullptr;            // some layers of element matrices
+  double* ke64 = nullptr;            // element matrices: some layers, on tetrahedra a slab (or all)
   int64_t ke_len = 0;
   double* ke_e = nullptr;            // [slots][elements] corner contributions of the element-centric products
   int64_t ke_e_len = 0;

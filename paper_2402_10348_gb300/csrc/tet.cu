@@ -28,12 +28,11 @@ struct TetData {
   int64_t* nptr = nullptr;  // [nn + 1]
   int32_t* nlist = nullptr; // 4 e + a of every (element, corner) at a node, by element
   double* E = nullptr;      // [24][ne] element contributions, slot (a * ncomp + eq)
-  // NS element matrices [256][ne] of the assembly, row a * 4 + eq, column b * 4 + f
-  double* K = nullptr;
   // assembled NS operator: the neighbours of the node (itself included, ascending) in slices of 32
   // nodes as wide as their longest row; entry p of the slice at off: node col[off + p * 32 +
   // lane], block A[((off / 32 + p) * 16 + 4 r + c) * 32 + lane].  -1: neighbour lists not built,
-  // 0: some node has more than TET_ROW neighbours (element matrices are kept), 1: built
+  // 0: some node has more than TET_ROW neighbours (element matrices are kept), 1: built.  The element
+  // matrices (row a * 4 + eq, column b * 4 + f) lie in the mesh's scratch ke64
   int rows = -1;
   int64_t n_blocks = 0;     // blocks with padding
   int64_t* off = nullptr;   // [slices + 1]
@@ -56,7 +55,6 @@ void tet_free(TetData* t) {
   cudaFree(t->nptr);
   cudaFree(t->nlist);
   cudaFree(t->E);
-  cudaFree(t->K);
   cudaFree(t->off);
   cudaFree(t->col);
   cudaFree(t->A);
@@ -321,11 +319,14 @@ int tet_ns_run(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
 // terms reduce to N_a N_b (one field, rho) and d_j N_a T_j with T_j taken once per column: about
 // 900 float64 operations a lane.  Lane b writes column b, rows in the order x = a ^ b.
 // 196,608 elements: 5.67 ms with the point arithmetic of 16 unit increments a thread, 1.2 ms now.
-__global__ void __launch_bounds__(128) tet_nsk_build(const __grid_constant__ TetArgs A, double* __restrict__ K) {
+// Elements [e0, e1) into K[256][ks].
+__global__ void __launch_bounds__(128) tet_nsk_build(const __grid_constant__ TetArgs A, double* __restrict__ K, int64_t e0,
+                                                     int64_t e1, int64_t ks) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int q = (int)(t & 3);
-  const bool ok = (t >> 2) < A.ne;
-  const int64_t e = ok ? t >> 2 : A.ne - 1;  // (whole warps take part in the shuffles)
+  const bool ok = e0 + (t >> 2) < e1;
+  const int64_t e = ok ? e0 + (t >> 2) : e1 - 1;  // (whole warps take part in the shuffles)
+  K += e - e0;
   const Phys& P = A.P;
   const int64_t nn = A.nn, n = A.conn[q * A.ne + e];
   auto shx = [](double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); };
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(128) tet_nsk_build(const __grid_constant__ Tet
   auto store = [&](int r, int c, const double (&en)[4]) {
     if (!ok) return;
 #pragma unroll
-    for (int x = 0; x < 4; ++x) K[(int64_t)(((q ^ x) * 4 + r) * 16 + q * 4 + c) * A.ne + e] = en[x];
+    for (int x = 0; x < 4; ++x) K[(int64_t)(((q ^ x) * 4 + r) * 16 + q * 4 + c) * ks] = en[x];
   };
   double en[4];
 #pragma unroll
@@ -540,28 +541,41 @@ __global__ void __launch_bounds__(TSL) tet_rows_kernel(const int64_t* __restrict
   for (int p = 0; p < w; ++p) col[o + (int64_t)p * TSL + threadIdx.x] = p < cnt ? nb[p] : (int32_t)(n < nn ? n : 0);
 }
 
-// blocks from the element matrices, element order: blockDim (TSL, 4), thread (node, row field)
+// blocks from the element matrices of [e0, e1), element order: blockDim (TSL, 4), thread (node, row field).
+// The first slab of elements writes every block, the later ones add to those of their nodes.
 __global__ void __launch_bounds__(4 * TSL) tet_rows_gather(const int64_t* __restrict__ nptr, const int32_t* __restrict__ nlist,
                                                            const int32_t* __restrict__ conn, int64_t ne, int64_t nn,
                                                            const int64_t* __restrict__ off, const int32_t* __restrict__ col,
-                                                           const double* __restrict__ K, double* __restrict__ A) {
+                                                           const double* __restrict__ K, double* __restrict__ A,
+                                                           int64_t e0, int64_t e1, int64_t ks) {
   const int64_t n = (int64_t)blockIdx.x * TSL + threadIdx.x;
   const int r = threadIdx.y;
   const int64_t o = off[blockIdx.x];
   const int w = (int)((off[blockIdx.x + 1] - o) / TSL);
+  // the node's elements of the slab
+  int64_t i0 = n < nn ? nptr[n] : 0, i1 = n < nn ? nptr[n + 1] : 0;
+  while (i0 < i1 && (nlist[i0] >> 2) < e0) ++i0;
+  while (i0 < i1 && (nlist[i1 - 1] >> 2) >= e1) --i1;
+  if (e0 > 0 && i0 == i1) return;
+  K -= e0;
   int32_t prev = -1;
   for (int p = 0; p < w; ++p) {
     const int32_t v = col[o + (int64_t)p * TSL + threadIdx.x];
+    double* at = A + ((o / TSL + p) * 16 + 4 * r) * TSL + threadIdx.x;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     if (n < nn && v > prev) {  // (padding repeats the node behind its larger neighbours)
-      for (int64_t i = nptr[n]; i < nptr[n + 1]; ++i) {
+      if (e0 > 0) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] = at[c * TSL];
+      }
+      for (int64_t i = i0; i < i1; ++i) {
         const int32_t t = nlist[i];
         const int64_t e = t >> 2;
         const int a = t & 3;
         for (int b = 0; b < 4; ++b) {
           if (conn[(int64_t)b * ne + e] != v) continue;
 #pragma unroll
-          for (int c = 0; c < 4; ++c) acc[c] += K[(int64_t)((a * 4 + r) * 16 + b * 4 + c) * ne + e];
+          for (int c = 0; c < 4; ++c) acc[c] += K[(int64_t)((a * 4 + r) * 16 + b * 4 + c) * ks + e];
         }
       }
       prev = v;
@@ -569,7 +583,7 @@ __global__ void __launch_bounds__(4 * TSL) tet_rows_gather(const int64_t* __rest
       prev = 0x7fffffff;
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) A[((o / TSL + p) * 16 + 4 * r + c) * TSL + threadIdx.x] = acc[c];
+    for (int c = 0; c < 4; ++c) at[c * TSL] = acc[c];
   }
 }
 
@@ -647,14 +661,18 @@ static int tet_rows_init(fsi_mesh* m) {
   return FSI_OK;
 }
 
-// element matrices, and the rows where every node's list fits, at the staged state
+// Element matrices, and the rows where every node's list fits, at the staged state.  Rows are summed a
+// slab of elements at a time: the matrices take 2 KB an element (22 GB on the falling sphere's 10.6 M),
+// which only the build reads.  Meshes of up to TET_SLAB elements are one slab.
+constexpr int64_t TET_SLAB = (int64_t)1 << 19;  // 1 GB of element matrices
 static int tet_ns_build(fsi_mesh* m, int elastic) {
   TetData* t = m->tet;
   if (t->k_built && t->k_stage == m->stage_gen && t->k_elastic == elastic) return FSI_OK;
   t->k_built = 0;
   if (t->rows < 0)
     if (int rc = tet_rows_init(m)) return rc;
-  if (!t->K) FSI_CUDA(cudaMalloc(&t->K, sizeof(double) * 256 * (size_t)t->ne));
+  const int64_t ks = t->rows ? std::min(t->ne, TET_SLAB) : t->ne;
+  if (int rc = ensure_elem_matrices(m, 256 * ks)) return rc;
   if (t->rows && !t->A) FSI_CUDA(cudaMalloc(&t->A, sizeof(double) * 16 * (size_t)t->n_blocks));
   TetArgs A;
   A.conn = t->conn;
@@ -668,10 +686,14 @@ static int tet_ns_build(fsi_mesh* m, int elastic) {
   A.nn = m->nn;
   A.elastic = elastic;
   A.P = m->P;
-  FSI_LAUNCH(m, P_NS_BUILD, tet_nsk_build<<<(unsigned)((t->ne * 4 + 127) / 128), 128, 0, m->stream>>>(A, t->K));
-  if (t->rows)
-    FSI_LAUNCH(m, P_NS_BUILD, tet_rows_gather<<<(unsigned)((m->nn + TSL - 1) / TSL), dim3(TSL, 4), 0, m->stream>>>(
-                                  t->nptr, t->nlist, t->conn, t->ne, m->nn, t->off, t->col, t->K, t->A));
+  for (int64_t e0 = 0; e0 < t->ne; e0 += ks) {
+    const int64_t e1 = std::min(t->ne, e0 + ks);
+    FSI_LAUNCH(m, P_NS_BUILD,
+               tet_nsk_build<<<(unsigned)(((e1 - e0) * 4 + 127) / 128), 128, 0, m->stream>>>(A, m->ke64, e0, e1, ks));
+    if (t->rows)
+      FSI_LAUNCH(m, P_NS_BUILD, tet_rows_gather<<<(unsigned)((m->nn + TSL - 1) / TSL), dim3(TSL, 4), 0, m->stream>>>(
+                                    t->nptr, t->nlist, t->conn, t->ne, m->nn, t->off, t->col, m->ke64, t->A, e0, e1, ks));
+  }
   t->k_stage = m->stage_gen;
   t->k_elastic = elastic;
   t->k_built = 1;
@@ -705,8 +727,8 @@ int tet_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
         return FSI_OK;
       }
       prof_bytes(m, P_NS_JVP64E, (double)t->ne * (256 * 8.0 + 16 * 4.0 + 16 * 8.0) + (double)m->nn * 32.0);
-      FSI_LAUNCH(m, P_NS_JVP64E, tet_nsk_apply<<<(unsigned)((t->ne + 127) / 128), 128, 0, m->stream>>>(t->conn, t->K, dx,
-                                                                                                      t->E, t->ne, m->nn));
+      FSI_LAUNCH(m, P_NS_JVP64E, tet_nsk_apply<<<(unsigned)((t->ne + 127) / 128), 128, 0, m->stream>>>(t->conn, m->ke64,
+                                                                                                      dx, t->E, t->ne, m->nn));
       FSI_LAUNCH(m, P_NODE_SUM, tet_ns_node<1><<<(unsigned)((m->nn + 255) / 256), 256, 0, m->stream>>>(
                                     t->nptr, t->nlist, t->E, t->ne, m->nn, m->mask, m->pin_active, m->staged_x, m->vD,
                                     dx, y));
