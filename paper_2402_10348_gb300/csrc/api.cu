@@ -443,6 +443,7 @@ int fsi_destroy_mesh(fsi_mesh* m) {
   cudaFree(m->na64);
   cudaFree(m->ke64);
   cudaFree(m->ke_e);
+  cudaFree(m->ke_s);
   cudaFree(m->tma_err);
   cudaFree(m->acst.A);
   cudaFree(m->bst.A);

@@ -10,7 +10,8 @@
 // thread interpolates the 8 corners for each point by itself, the transposed scatter 18
 // instead of 45, and a mesh has 8 times as many threads, which is what small meshes lack.
 // Corner contributions leave as E[8 x equation + corner][element]: four adjacent elements
-// of a warp fill one 32-byte sector of a plane.  A node kernel sums them in a fixed order.
+// of a warp fill one 32-byte sector of a plane.  A node kernel sums them in a fixed order; a mesh too
+// large for the scratch goes slab by slab of layers.
 //
 // Against the z-marching tiles (q1_tile.cuh), which evaluate a halo ring twice and give a small
 // mesh a handful of CTAs: momentum residual at 64^3 3.88 -> 1.18 ms, at 8^3 444 -> 18 us.
@@ -29,14 +30,13 @@ struct HexLane {
   int q;              // corner and quadrature point of the lane
   bool ok;
   int ex, ey, ez;
-  int64_t e;          // element index in the padded planes
   int64_t n;          // the lane's corner node
   double sx, sy, sz;  // 1/h with the sign that turns partner - own into the derivative
   // elements [e0, e1) of the mesh (32-bit: a state of 2^31 elements exceeds the memory)
-  __device__ __forceinline__ void set(const Geom& g, const double (&rh)[3], int nxp, unsigned e0, unsigned e1) {
-    set(g, rh, nxp, e0, e1, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  __device__ __forceinline__ void set(const Geom& g, const double (&rh)[3], unsigned e0, unsigned e1) {
+    set(g, rh, e0, e1, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   }
-  __device__ __forceinline__ void set(const Geom& g, const double (&rh)[3], int nxp, unsigned e0, unsigned e1, int64_t t) {
+  __device__ __forceinline__ void set(const Geom& g, const double (&rh)[3], unsigned e0, unsigned e1, int64_t t) {
     q = (int)(t & 7);
     ok = e0 + (t >> 3) < e1;
     const unsigned f = ok ? e0 + (unsigned)(t >> 3) : e1 - 1;
@@ -44,7 +44,6 @@ struct HexLane {
     ex = (int)(f - row * (unsigned)g.nx);
     ez = (int)(row / (unsigned)g.ny);
     ey = (int)(row - (unsigned)ez * (unsigned)g.ny);
-    e = ((int64_t)ez * g.ny + ey) * nxp + ex;
     n = (int64_t)(ex + (q & 1)) + (int64_t)(g.nx + 1) * ((ey + ((q >> 1) & 1)) + (int64_t)(g.ny + 1) * (ez + (q >> 2)));
     sx = (q & 1) ? -rh[0] : rh[0];
     sy = (q & 2) ? -rh[1] : rh[1];
@@ -95,6 +94,11 @@ struct HexNS {
   double rh[3];       // 1/h
   double dt2, rtrG;   // 4 / dt^2, 1 / tr G (a float64 division costs tens of instructions)
   double W;           // quadrature weight x |det J|
+  int layers;         // layers of elements that the contributions' scratch holds
+  __device__ __forceinline__ int64_t stride() const { return (int64_t)layers * nxyp; }  // of its slots
+  __device__ __forceinline__ int64_t at(const HexLane& l) const {                       // the lane's element in a slot
+    return (int64_t)(l.ez < layers ? l.ez : l.ez % layers) * nxyp + (int64_t)l.ey * nxp + l.ex;
+  }
 };
 
 // State of the equations at the lane's quadrature point (ops.cuh for the notation)
@@ -206,6 +210,7 @@ inline HexNS hex_ns(const fsi_mesh* m, int nxp) {
   H.dt2 = 4.0 / (m->P.dt * m->P.dt);
   H.rtrG = 1.0 / m->P.trG;
   H.W = m->g.hx * m->g.hy * m->g.hz / 8.0;
+  H.layers = m->g.nz;
   return H;
 }
 

@@ -8,10 +8,10 @@ namespace fsi {
 
 // R_m, tau and the stresses at a point, tested: E[8 x equation + corner][element], unweighted
 __global__ void __launch_bounds__(HQ_THREADS) hq_ns_res_kernel(const __grid_constant__ HexNS H, double* __restrict__ E,
-                                                               unsigned ne) {
+                                                               unsigned e0, unsigned e1) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
-  const int64_t es = (int64_t)H.g.nz * H.nxyp;
+  l.set(H.g, H.rh, e0, e1);
+  const int64_t es = H.stride(), at = H.at(l);
   NSPoint p;
   hq_ns_point(H, l, p);
   double S[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -31,17 +31,17 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ns_res_kernel(const __grid_cons
     for (int j = 0; j < 3; ++j)
       g[j] = fma(p.v[j], tR, fma(p.mu, p.L[k][j] + p.L[j][k], S[sym_idx(k, j)])) + (j == k ? iso : 0.0);
     const double c = l.scatter(p.R[k] - p.gp[k], g[0], g[1], g[2]);  // rho (acc_k - g_k)
-    if (l.ok) E[(8 * k + l.q) * es + l.e] = c;
+    if (l.ok) E[(8 * k + l.q) * es + at] = c;
   }
   const double r = p.tau_m * p.rrho;
   const double c = l.scatter(Rc, r * p.R[0], r * p.R[1], r * p.R[2]);
-  if (l.ok) E[(24 + l.q) * es + l.e] = c;
+  if (l.ok) E[(24 + l.q) * es + at] = c;
 }
 
 __global__ void __launch_bounds__(HQ_THREADS) hq_ac_res_kernel(const __grid_constant__ HexNS H, int phase, double gam,
-                                                               double bet, double* __restrict__ E, unsigned ne) {
+                                                               double bet, double* __restrict__ E, unsigned e0, unsigned e1) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
+  l.set(H.g, H.rh, e0, e1);
   const Phys& P = H.P;
   double v[3];
 #pragma unroll
@@ -55,15 +55,15 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ac_res_kernel(const __grid_cons
                    gam * (phi * phi * phi - phi - bet * (0.5 * fabs(phi * phi - 1.0)));
   const double t = tau * R;
   const double c = l.scatter(R, k_hat * ph.gx + t * v[0], k_hat * ph.gy + t * v[1], k_hat * ph.gz + t * v[2]);
-  if (l.ok) E[l.q * (int64_t)H.g.nz * H.nxyp + l.e] = H.W * c;
+  if (l.ok) E[l.q * H.stride() + H.at(l)] = H.W * c;
 }
 
 __global__ void __launch_bounds__(HQ_THREADS) hq_b_res_kernel(const __grid_constant__ HexNS H, int solid,
-                                                              double* __restrict__ E, unsigned ne) {
+                                                              double* __restrict__ E, unsigned e0, unsigned e1) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
+  l.set(H.g, H.rh, e0, e1);
   const Phys& P = H.P;
-  const int64_t nn = H.nn, es = (int64_t)H.g.nz * H.nxyp;
+  const int64_t nn = H.nn, es = H.stride(), at = H.at(l);
   double v[3], L[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_b_res_kernel(const __grid_const
     const double R = H.W * (al * (cv[c] - st) + (1.0 - al) * (B[c] - (c < 3 ? 1.0 : 0.0)));
     const double t = tau * R;
     const double s = l.scatter(R, t * v[0], t * v[1], t * v[2]);
-    if (l.ok) E[(8 * c + l.q) * es + l.e] = s;
+    if (l.ok) E[(8 * c + l.q) * es + at] = s;
   }
 }
 
@@ -102,7 +102,7 @@ template <bool MANY>
 __global__ void __launch_bounds__(HQ_THREADS) hq_ns_coef_kernel(const __grid_constant__ HexNS H, double* __restrict__ c64,
                                                                 float* __restrict__ c32, unsigned ne, int elastic) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
+  l.set(H.g, H.rh, 0, ne);
   NSPoint p;
   hq_ns_point(H, l, p);
   const int64_t b = ((int64_t)l.ez * 8 + l.q) * NCQ * H.nxyp + (int64_t)l.ey * H.nxp + l.ex;
@@ -160,10 +160,10 @@ struct PointCoef {
 template <bool MANY>
 __global__ void __launch_bounds__(HQ_THREADS) hq_ns_jvp_kernel(const __grid_constant__ HexNS H,
                                                                const double* __restrict__ dx, double* __restrict__ E,
-                                                               unsigned ne, int elastic) {
+                                                               unsigned e0, unsigned e1, int elastic) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
-  const int64_t es = (int64_t)H.g.nz * H.nxyp;
+  l.set(H.g, H.rh, e0, e1);
+  const int64_t es = H.stride(), at = H.at(l);
   NSPoint p;
   hq_ns_point(H, l, p);
   double aB[6] = {}, aG[6][3] = {};
@@ -181,16 +181,16 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ns_jvp_kernel(const __grid_cons
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const double c = l.scatter(f[k], g[k][0], g[k][1], g[k][2]);
-    if (l.ok) E[(8 * k + l.q) * es + l.e] = c;
+    if (l.ok) E[(8 * k + l.q) * es + at] = c;
   }
 }
 
 // Allen-Cahn and B products at a state that is used a few times
 __global__ void __launch_bounds__(HQ_THREADS) hq_ac_jvp_kernel(const __grid_constant__ HexNS H, int phase, double gam,
                                                                double bet, const double* __restrict__ dx,
-                                                               double* __restrict__ E, unsigned ne) {
+                                                               double* __restrict__ E, unsigned e0, unsigned e1) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
+  l.set(H.g, H.rh, e0, e1);
   const Phys& P = H.P;
   double v[3];
 #pragma unroll
@@ -206,16 +206,16 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_ac_jvp_kernel(const __grid_cons
   const double dR = P.c_mass * d.v + P.alpha * (v[0] * d.gx + v[1] * d.gy + v[2] * d.gz + rp * d.v);
   const double t = tau * dR, ka = k_hat * P.alpha;
   const double c = l.scatter(dR, ka * d.gx + t * v[0], ka * d.gy + t * v[1], ka * d.gz + t * v[2]);
-  if (l.ok) E[l.q * (int64_t)H.g.nz * H.nxyp + l.e] = H.W * c;
+  if (l.ok) E[l.q * H.stride() + H.at(l)] = H.W * c;
 }
 
 __global__ void __launch_bounds__(HQ_THREADS) hq_b_jvp_kernel(const __grid_constant__ HexNS H, int solid,
                                                               const double* __restrict__ dx, double* __restrict__ E,
-                                                              unsigned ne) {
+                                                              unsigned e0, unsigned e1) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, 0, ne);
+  l.set(H.g, H.rh, e0, e1);
   const Phys& P = H.P;
-  const int64_t nn = H.nn, es = (int64_t)H.g.nz * H.nxyp;
+  const int64_t nn = H.nn, es = H.stride(), at = H.at(l);
   double v[3], L[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_b_jvp_kernel(const __grid_const
     const double R = H.W * (al * (cv[c] - st) + (1.0 - al) * B[c]);
     const double t = tau * R;
     const double s = l.scatter(R, t * v[0], t * v[1], t * v[2]);
-    if (l.ok) E[(8 * c + l.q) * es + l.e] = s;
+    if (l.ok) E[(8 * c + l.q) * es + at] = s;
   }
 }
 
@@ -269,93 +269,109 @@ int ns_build(fsi_mesh* m, unsigned flags, bool f64) {
   return FSI_OK;
 }
 
-int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
+// Runs launch(E, H, e0, e1, k0, k1) for every slab of layers: the contributions of the elements [e0, e1) into E, then
+// the node planes [k0, k1) that they complete.  E is a ring of layers: the last one before a slab stays for
+// the slab's first plane.
+template <class F>
+static int hq_slabs(fsi_mesh* m, F launch) {
   const Geom& g = m->g;
   const int nxp = cq_pitch(m);
-  const int64_t nxyp = (int64_t)nxp * g.ny;
-  const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
-  const int elastic = (flags & FSI_ELASTIC_AUG) && m->ns > 0 ? 1 : 0;
-  if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
-  const HexNS H = hex_ns(m, nxp);
-  const RowLaunch nl = node_launch(g);
-  // algorithmic bytes: the nodal fields once, the contributions written and read, the product
-  prof_bytes(m, P_NS_JVP64, (double)ne * 256.0 + (double)m->nn * 8.0 * (13 + (elastic ? 7 * m->ns : 0)));
-  prof_bytes(m, P_NODE_SUM, (double)ne * 256.0 + (double)m->nn * 33.0);
-  auto* kernel = m->ns >= HQ_MANY ? &hq_ns_jvp_kernel<true> : &hq_ns_jvp_kernel<false>;
-  FSI_LAUNCH(m, P_NS_JVP64, kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, dx, m->ke_e, ne, elastic));
-  FSI_LAUNCH(m, P_NODE_SUM,
-             ns_node_kernel<double><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, H.W,
-                                                                         m->mask, m->pin_active, dx, nullptr, nullptr, y));
+  double* E = nullptr;
+  HexNS H = hex_ns(m, nxp);
+  if (int rc = elem_layers(m, (int64_t)nxp * g.ny, &E, &H.layers)) return rc;
+  const int step = H.layers == g.nz ? g.nz : H.layers - 1;
+  for (int z0 = 0; z0 < g.nz; z0 += step) {
+    const int z1 = std::min(g.nz, z0 + step);
+    if (int rc = launch(E, H, (unsigned)z0 * g.ny * g.nx, (unsigned)z1 * g.ny * g.nx, z0, z1 == g.nz ? z1 + 1 : z1))
+      return rc;
+  }
   return FSI_OK;
+}
+
+// Dirichlet rows: dx, less vD where given
+static int hq_ns_sums(fsi_mesh* m, const double* E, const HexNS& H, int k0, int k1, const double* dx, const double* vD,
+                      double* y) {
+  const Geom& g = m->g;
+  const RowLaunch nl = node_launch(g, k0, k1);
+  FSI_LAUNCH(m, P_NODE_SUM,
+             ns_node_kernel<double><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp, H.layers, k0,
+                                                                         k1, m->nn, H.W, m->mask, m->pin_active, dx, nullptr,
+                                                                         vD, y));
+  return FSI_OK;
+}
+
+template <int NC>
+static int hq_sums(fsi_mesh* m, const double* E, const HexNS& H, int k0, int k1, double* y) {
+  const Geom& g = m->g;
+  const RowLaunch nl = node_launch(g, k0, k1);
+  FSI_LAUNCH(m, P_NODE_SUM, em_node_kernel<NC><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp,
+                                                                                    H.layers, k0, k1, m->nn, y));
+  return FSI_OK;
+}
+
+int hq_ns_jvp(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
+  const double ne = (double)m->g.nx * m->g.ny * m->g.nz;
+  const int elastic = (flags & FSI_ELASTIC_AUG) && m->ns > 0 ? 1 : 0;
+  // algorithmic bytes: the nodal fields once, the contributions written and read, the product
+  prof_bytes(m, P_NS_JVP64, ne * 256.0 + (double)m->nn * 8.0 * (13 + (elastic ? 7 * m->ns : 0)));
+  prof_bytes(m, P_NODE_SUM, ne * 256.0 + (double)m->nn * 33.0);
+  auto* kernel = m->ns >= HQ_MANY ? &hq_ns_jvp_kernel<true> : &hq_ns_jvp_kernel<false>;
+  return hq_slabs(m, [&](double* E, const HexNS& H, unsigned e0, unsigned e1, int k0, int k1) -> int {
+    FSI_LAUNCH(m, P_NS_JVP64, kernel<<<hq_blocks(e1 - e0), HQ_THREADS, 0, m->stream>>>(H, dx, E, e0, e1, elastic));
+    return hq_ns_sums(m, E, H, k0, k1, dx, nullptr, y);
+  });
 }
 
 int hq_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y) {
-  const Geom& g = m->g;
-  const int nxp = cq_pitch(m);
-  const int64_t nxyp = (int64_t)nxp * g.ny;
-  const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
-  if (int rc = ensure_elem_scratch(m, 8 * b.nc, nxyp)) return rc;
-  const HexNS H = hex_ns(m, nxp);
-  const RowLaunch nl = node_launch(g);
-  prof_bytes(m, P_NODE_SUM, (double)ne * 64 * b.nc + (double)m->nn * 8 * b.nc);
-  if (b.kind == 1) {
-    prof_bytes(m, P_AC_JVP64, (double)ne * 64.0 + (double)m->nn * 40.0);
-    FSI_LAUNCH(m, P_AC_JVP64, hq_ac_jvp_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(
-                                  H, b.index, m->gamma[b.index], m->beta[b.index], dx, m->ke_e, ne));
-    FSI_LAUNCH(m, P_NODE_SUM,
-               em_node_kernel<1><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, y));
-  } else {
-    prof_bytes(m, P_B_JVP64, (double)ne * 384.0 + (double)m->nn * 80.0);
-    FSI_LAUNCH(m, P_B_JVP64, hq_b_jvp_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, b.index, dx, m->ke_e, ne));
-    FSI_LAUNCH(m, P_NODE_SUM,
-               em_node_kernel<6><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, y));
-  }
-  return FSI_OK;
+  const double ne = (double)m->g.nx * m->g.ny * m->g.nz;
+  prof_bytes(m, P_NODE_SUM, ne * 64 * b.nc + (double)m->nn * 8 * b.nc);
+  prof_bytes(m, b.kind == 1 ? P_AC_JVP64 : P_B_JVP64, ne * 64 * b.nc + (double)m->nn * (b.kind == 1 ? 40.0 : 80.0));
+  return hq_slabs(m, [&](double* E, const HexNS& H, unsigned e0, unsigned e1, int k0, int k1) -> int {
+    if (b.kind == 1) {
+      FSI_LAUNCH(m, P_AC_JVP64, hq_ac_jvp_kernel<<<hq_blocks(e1 - e0), HQ_THREADS, 0, m->stream>>>(
+                                    H, b.index, m->gamma[b.index], m->beta[b.index], dx, E, e0, e1));
+      return hq_sums<1>(m, E, H, k0, k1, y);
+    }
+    FSI_LAUNCH(m, P_B_JVP64,
+               hq_b_jvp_kernel<<<hq_blocks(e1 - e0), HQ_THREADS, 0, m->stream>>>(H, b.index, dx, E, e0, e1));
+    return hq_sums<6>(m, E, H, k0, k1, y);
+  });
 }
 
 int hq_residual(fsi_mesh* m, const BlockInfo& b, double* r) {
-  const Geom& g = m->g;
-  const int nxp = cq_pitch(m);
-  const int64_t nxyp = (int64_t)nxp * g.ny;
-  const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
-  const int nc = b.nc;
-  if (int rc = ensure_elem_scratch(m, 8 * nc, nxyp)) return rc;
-  const HexNS H = hex_ns(m, nxp);
-  const RowLaunch nl = node_launch(g);
-  prof_bytes(m, P_NODE_SUM, (double)ne * 64 * nc + (double)m->nn * 8 * nc);
-  if (b.kind == 0) {
-    FSI_LAUNCH(m, P_NS_RES, hq_ns_res_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, m->ke_e, ne));
-    FSI_LAUNCH(m, P_NODE_SUM,
-               ns_node_kernel<double><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, H.W,
-                                                                           m->mask, m->pin_active, m->staged_x, nullptr,
-                                                                           m->vD, r));
-  } else if (b.kind == 1) {
-    FSI_LAUNCH(m, P_AC_RES, hq_ac_res_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(
-                                H, b.index, m->gamma[b.index], m->beta[b.index], m->ke_e, ne));
-    FSI_LAUNCH(m, P_NODE_SUM,
-               em_node_kernel<1><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, r));
-  } else {
-    FSI_LAUNCH(m, P_B_RES, hq_b_res_kernel<<<hq_blocks(ne), HQ_THREADS, 0, m->stream>>>(H, b.index, m->ke_e, ne));
-    FSI_LAUNCH(m, P_NODE_SUM,
-               em_node_kernel<6><<<nl.grid, nl.block, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, r));
-  }
-  return FSI_OK;
+  prof_bytes(m, P_NODE_SUM, (double)m->g.nx * m->g.ny * m->g.nz * 64 * b.nc + (double)m->nn * 8 * b.nc);
+  return hq_slabs(m, [&](double* E, const HexNS& H, unsigned e0, unsigned e1, int k0, int k1) -> int {
+    const unsigned grid = hq_blocks(e1 - e0);
+    if (b.kind == 0) {
+      FSI_LAUNCH(m, P_NS_RES, hq_ns_res_kernel<<<grid, HQ_THREADS, 0, m->stream>>>(H, E, e0, e1));
+      return hq_ns_sums(m, E, H, k0, k1, m->staged_x, m->vD, r);
+    }
+    if (b.kind == 1) {
+      FSI_LAUNCH(m, P_AC_RES, hq_ac_res_kernel<<<grid, HQ_THREADS, 0, m->stream>>>(H, b.index, m->gamma[b.index],
+                                                                                  m->beta[b.index], E, e0, e1));
+      return hq_sums<1>(m, E, H, k0, k1, r);
+    }
+    FSI_LAUNCH(m, P_B_RES, hq_b_res_kernel<<<grid, HQ_THREADS, 0, m->stream>>>(H, b.index, E, e0, e1));
+    return hq_sums<6>(m, E, H, k0, k1, r);
+  });
 }
 
 // ------------------------------------------------------------------ gamma, beta
 // Sections 2.2.1 and 2.2.2 as CoefOp (ops.cuh) has them: the corner contributions of the lumped
 // projection of q = grad phi^T grad v grad phi / |grad phi|^2, unweighted (its denominator is W times
-// the node's elements), and the CTA's partial integrals of F' and sqrt F over its elements.
+// the node's elements), and the CTA's partial integrals of F' and sqrt F over its elements, added to those
+// of the slabs before.
 __global__ void __launch_bounds__(HQ_THREADS) hq_coef_kernel(const __grid_constant__ HexNS H, int phase,
-                                                             double* __restrict__ E, double* __restrict__ part, unsigned ne) {
+                                                             double* __restrict__ E, double* __restrict__ part, unsigned e0,
+                                                             unsigned e1) {
   const double* phi = H.xa + (int64_t)(4 + phase) * H.nn;
-  const int64_t es = (int64_t)H.g.nz * H.nxyp, nt = (int64_t)ne * 8;
+  const int64_t es = H.stride(), nt = (int64_t)(e1 - e0) * 8;
   double sF = 0.0, sS = 0.0;
   // whole warps stay in the loop together (32 lanes: four elements)
   for (int64_t t = (int64_t)blockIdx.x * HQ_THREADS + threadIdx.x; t - (threadIdx.x & 31) < nt;
        t += (int64_t)gridDim.x * HQ_THREADS) {
     HexLane l;
-    l.set(H.g, H.rh, H.nxp, 0, ne, t);
+    l.set(H.g, H.rh, e0, e1, t);
     const VG<double> ph = l.vg(phi[l.n]);
     const double g[3] = {ph.gx, ph.gy, ph.gz};
     double num = 0.0;
@@ -367,7 +383,7 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_coef_kernel(const __grid_consta
     const double n2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
     const double c = l.val(n2 < 1e-30 ? 0.0 : num / n2);
     if (l.ok) {
-      E[l.q * es + l.e] = c;
+      E[l.q * es + H.at(l)] = c;
       sF += ph.v * ph.v * ph.v - ph.v;
       sS += 0.5 * fabs(ph.v * ph.v - 1.0);
     }
@@ -386,18 +402,20 @@ __global__ void __launch_bounds__(HQ_THREADS) hq_coef_kernel(const __grid_consta
   if (threadIdx.x < 2) {
     double s = 0.0;
     for (int i = 0; i < HQ_THREADS / 32; ++i) s += red[threadIdx.x][i];
-    part[2 * blockIdx.x + threadIdx.x] = H.W * s;
+    double* p = part + 2 * blockIdx.x + threadIdx.x;
+    *p = e0 > 0 ? *p + H.W * s : H.W * s;
   }
 }
 
-// the CTA's partial sum of squared nodal values and count of nodes in the band |phi| <= 0.9
+// the CTA's partial sum of squared nodal values and count of nodes in the band |phi| <= 0.9, over the nodes
+// [n0, n1) and added to those before
 __global__ void __launch_bounds__(NTHREADS) hq_coef_node_kernel(const double* __restrict__ E, int nx, int ny, int nz, int nxp,
-                                                                int64_t nxyp, int64_t nn, const double* __restrict__ phi,
-                                                                double* __restrict__ part) {
+                                                                int64_t nxyp, int layers, int64_t n0, int64_t n1,
+                                                                const double* __restrict__ phi, double* __restrict__ part) {
   __shared__ double scratch[NTHREADS / 32];
-  const int64_t es = (int64_t)nz * nxyp;
+  const int64_t es = (int64_t)layers * nxyp;
   double v2 = 0.0, cnt = 0.0;
-  for (int64_t n = (int64_t)blockIdx.x * NTHREADS + threadIdx.x; n < nn; n += (int64_t)gridDim.x * NTHREADS) {
+  for (int64_t n = n0 + (int64_t)blockIdx.x * NTHREADS + threadIdx.x; n < n1; n += (int64_t)gridDim.x * NTHREADS) {
     if (!(fabs(phi[n]) <= 0.9)) continue;
     const unsigned row = (unsigned)n / (unsigned)(nx + 1);
     const int i = (int)((unsigned)n - row * (unsigned)(nx + 1)), k = (int)(row / (unsigned)(ny + 1));
@@ -408,7 +426,7 @@ __global__ void __launch_bounds__(NTHREADS) hq_coef_node_kernel(const double* __
         for (int ax = 1; ax >= 0; --ax) {
           const int ex = i - ax, ey = j - ay, ez = k - az;
           if (ex < 0 || ex >= nx || ey < 0 || ey >= ny || ez < 0 || ez >= nz) continue;
-          s += E[(ax + 2 * ay + 4 * az) * es + (int64_t)ez * nxyp + (int64_t)ey * nxp + ex];
+          s += E[(ax + 2 * ay + 4 * az) * es + (int64_t)(ez < layers ? ez : ez % layers) * nxyp + (int64_t)ey * nxp + ex];
           elems += 1.0;
         }
     const double v = fabs(s / elems);
@@ -418,8 +436,9 @@ __global__ void __launch_bounds__(NTHREADS) hq_coef_node_kernel(const double* __
   const double a = block_sum(v2, scratch);
   const double b = block_sum(cnt, scratch);
   if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = a;
-    part[2 * blockIdx.x + 1] = b;
+    double* p = part + 2 * blockIdx.x;
+    p[0] = n0 > 0 ? p[0] + a : a;
+    p[1] = n0 > 0 ? p[1] + b : b;
   }
 }
 
@@ -449,10 +468,7 @@ __global__ void __launch_bounds__(NTHREADS) hq_coef_final_kernel(const double* _
 int op_coeffs(fsi_mesh* m, int phase, double* gb) {
   if (m->tet) return tet_coeffs(m, phase, gb);
   const Geom& g = m->g;
-  const int nxp = cq_pitch(m);
-  const int64_t nxyp = (int64_t)nxp * g.ny;
   const unsigned ne = (unsigned)g.nx * g.ny * g.nz;
-  if (int rc = ensure_elem_scratch(m, 8, nxyp)) return rc;
   const int ge = (int)std::min<unsigned>(hq_blocks(ne), 152 * 8), gn = (int)std::min<int64_t>((m->nn + NTHREADS - 1) / NTHREADS, 152 * 4);
   if (m->n_partials < ge + gn) {
     cudaFree(m->partials);
@@ -463,8 +479,14 @@ int op_coeffs(fsi_mesh* m, int phase, double* gb) {
   }
   double* pn = m->partials + 2 * ge;
   const double* phi = m->staged_xa + (int64_t)(4 + phase) * m->nn;
-  FSI_LAUNCH(m, P_COEF, hq_coef_kernel<<<ge, HQ_THREADS, 0, m->stream>>>(hex_ns(m, nxp), phase, m->ke_e, m->partials, ne));
-  FSI_LAUNCH(m, P_COEF, hq_coef_node_kernel<<<gn, NTHREADS, 0, m->stream>>>(m->ke_e, g.nx, g.ny, g.nz, nxp, nxyp, m->nn, phi, pn));
+  const int64_t plane = (int64_t)(g.nx + 1) * (g.ny + 1);
+  const int rc = hq_slabs(m, [&](double* E, const HexNS& H, unsigned e0, unsigned e1, int k0, int k1) -> int {
+    FSI_LAUNCH(m, P_COEF, hq_coef_kernel<<<ge, HQ_THREADS, 0, m->stream>>>(H, phase, E, m->partials, e0, e1));
+    FSI_LAUNCH(m, P_COEF, hq_coef_node_kernel<<<gn, NTHREADS, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp, H.layers,
+                                                                             k0 * plane, k1 * plane, phi, pn));
+    return FSI_OK;
+  });
+  if (rc) return rc;
   FSI_LAUNCH(m, P_COEF, hq_coef_final_kernel<<<1, NTHREADS, 0, m->stream>>>(m->partials, ge, pn, gn, m->P.eta, m->red));
   FSI_CUDA(cudaMemcpyAsync(m->red_host, m->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
   FSI_CUDA(cudaStreamSynchronize(m->stream));

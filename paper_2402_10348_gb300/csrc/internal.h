@@ -87,7 +87,7 @@ struct fsi_mesh {
   double* ke64 = nullptr;            // element matrices: some layers, on tetrahedra a slab (or all)
   int64_t ke_len = 0;
   double* ke_e = nullptr;            // [slots][elements] corner contributions of the element-centric products
-  int64_t ke_e_len = 0;
+  double* ke_s = nullptr;            // the same for some layers (ops_f64.cu), on large meshes
   int64_t f64_gen = -1, f64_count = 0;  // float64 products applied at staging f64_gen ...
   int32_t f64_block = -1;               // ... on this kind and index of block
   // assembled float64 Allen-Cahn and B operators (stencil.cu) of one indicator and one solid
@@ -213,8 +213,10 @@ int nsq_batch_launch(bool f64, const NSQBatchRec* recs, const int4* eitems, int 
 // The coefficient products take NSQ_TILE consecutive elements (x fastest) of a layer per CTA
 constexpr int NSQ_TILE = 128;
 __host__ __device__ inline int nsq_tiles(const Geom& g) { return (int)(((int64_t)g.nx * g.ny + NSQ_TILE - 1) / NSQ_TILE); }
-// [slots][elements] scratch of the element-centric products, grown on demand (ops_f64.cu)
-int ensure_elem_scratch(fsi_mesh* m, int slots, int64_t nxyp);
+// [32][elements] scratch of the element-centric products, allocated on first use, and [48][layers] of those that
+// go by slabs (32 without solids; all layers on all but large meshes); ops_f64.cu
+int ensure_elem_scratch(fsi_mesh* m, int64_t nxyp);
+int elem_layers(fsi_mesh* m, int64_t nxyp, double** E, int* layers);
 // assembled float64 NS operator of the staged state (built when stale): build, product and
 // diagonal (nsa.cu)
 int nsa_build(fsi_mesh* m, unsigned flags);

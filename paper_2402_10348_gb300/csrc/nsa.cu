@@ -113,7 +113,7 @@ template <bool MANY>
 __global__ void __launch_bounds__(HQ_THREADS) nsa_elem_kernel(const __grid_constant__ HexNS H, double* __restrict__ K,
                                                               unsigned e0, unsigned e1, int slots, int elastic) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, e0, e1);
+  l.set(H.g, H.rh, e0, e1);
   Walsh w;
   w.q = l.q;
 #pragma unroll

@@ -267,7 +267,7 @@ int nsq_batch_record(fsi_mesh* m, unsigned flags, bool f64, const double* dx, do
   const Geom& g = m->g;
   const int nxp = cq_pitch(m);
   const int64_t nxyp = (int64_t)nxp * g.ny;
-  if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
+  if (int rc = ensure_elem_scratch(m, nxyp)) return rc;
   if (!m->tma_err) {
     FSI_CUDA(cudaMalloc(&m->tma_err, sizeof(int)));
     FSI_CUDA(cudaMemsetAsync(m->tma_err, 0, sizeof(int), m->stream));
@@ -329,7 +329,7 @@ int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
   const int nxp = cq_pitch(m);
   const int64_t nxyp = (int64_t)nxp * g.ny, nn = m->nn;
   const int elastic = ((flags & FSI_ELASTIC_AUG) && m->ns > 0) ? 1 : 0;
-  if (int rc = ensure_elem_scratch(m, 32, nxyp)) return rc;
+  if (int rc = ensure_elem_scratch(m, nxyp)) return rc;
   float* E = reinterpret_cast<float*>(m->ke_e);
   if (!m->tma_err) {
     FSI_CUDA(cudaMalloc(&m->tma_err, sizeof(int)));
@@ -352,9 +352,9 @@ int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
              (nsq_tma_kernel<<<(unsigned)nblk, TBE, smem, m->stream>>>(static_cast<const float*>(m->cq32.p), ncoef, tiles,
                                                                        m->dx32, E, g.nx, g.ny, g.nz, nxp, nxyp, nn, al, cm,
                                                                        rx, ry, rz, m->tma_err)));
-  const RowLaunch nl = node_launch(g);
+  const RowLaunch nl = node_launch(g, 0, g.nz + 1);
   FSI_LAUNCH(m, P_NODE_SUM,
-             ns_node_kernel<float><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, nxp, nxyp, nn,
+             ns_node_kernel<float><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, nxp, nxyp, g.nz, 0, g.nz + 1, nn,
                                                                         g.hx * g.hy * g.hz / 8.0, m->mask,
                                                                         m->pin_active, dx, m->dx32, nullptr, y));
   return FSI_OK;

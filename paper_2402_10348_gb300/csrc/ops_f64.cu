@@ -5,18 +5,32 @@ namespace fsi {
 
 template int launch_ns<double>(fsi_mesh*, int, const double*, double*, unsigned);
 
-// E[slots][nz * nxyp] scratch of the element contributions (NS, AC and B in turn).  Taken for the largest
-// block at once: batched launches keep its address between solves.
-int ensure_elem_scratch(fsi_mesh* m, int slots, int64_t nxyp) {
-  slots = std::max(slots, m->ns > 0 ? 48 : 32);
-  const int64_t elen = (int64_t)slots * m->g.nz * nxyp;
-  if (m->ke_e_len < elen) {
-    cudaFree(m->ke_e);
-    m->ke_e = nullptr;
-    m->ke_e_len = 0;
-    FSI_CUDA(cudaMalloc(&m->ke_e, sizeof(double) * (size_t)elen));
-    m->ke_e_len = elen;
+// Scratch of the element contributions.  Meshes whose largest block (48 slots an element with a solid, else 32)
+// fits ELEM_SCRATCH have one for everything, taken at once: its address never changes.  On larger ones
+// the float64 products, residuals and gamma/beta go slab by slab of layers through that much of their
+// own (they ran without any before they were element-centric), and the products of a whole mesh take
+// their 32 slots.
+constexpr int64_t ELEM_SCRATCH = (int64_t)1 << 30;
+static int most_slots(const fsi_mesh* m) { return m->ns > 0 ? 48 : 32; }
+static bool one_scratch(const fsi_mesh* m, int64_t nxyp) { return 8 * most_slots(m) * m->g.nz * nxyp <= ELEM_SCRATCH; }
+
+int ensure_elem_scratch(fsi_mesh* m, int64_t nxyp) {
+  if (m->ke_e) return FSI_OK;
+  FSI_CUDA(cudaMalloc(&m->ke_e, sizeof(double) * (size_t)(one_scratch(m, nxyp) ? most_slots(m) : 32) * m->g.nz * nxyp));
+  return FSI_OK;
+}
+
+int elem_layers(fsi_mesh* m, int64_t nxyp, double** E, int* layers) {
+  *layers = m->g.nz;
+  if (one_scratch(m, nxyp)) {
+    if (int rc = ensure_elem_scratch(m, nxyp)) return rc;
+    *E = m->ke_e;
+    return FSI_OK;
   }
+  const int64_t layer = most_slots(m) * nxyp;
+  *layers = (int)std::min<int64_t>(m->g.nz, std::max<int64_t>(2, ELEM_SCRATCH / (8 * layer)));
+  if (!m->ke_s) FSI_CUDA(cudaMalloc(&m->ke_s, sizeof(double) * (size_t)(*layers * layer)));
+  *E = m->ke_s;
   return FSI_OK;
 }
 

@@ -217,23 +217,26 @@ inline RowLaunch row_launch(int len, int64_t rows) {
   const int64_t nbx = (len + bx - 1) / bx, nby = (rows + by - 1) / by;
   return RowLaunch{dim3((unsigned)(nbx * nby)), dim3(bx, by)};
 }
-inline RowLaunch node_launch(const Geom& g) { return row_launch(g.nx + 1, (int64_t)(g.ny + 1) * (g.nz + 1)); }
+// the nodes of the planes [k0, k1)
+inline RowLaunch node_launch(const Geom& g, int k0, int k1) { return row_launch(g.nx + 1, (int64_t)(g.ny + 1) * (k1 - k0)); }
 
 // NS node sums: y = W * sum of the element slots, the Dirichlet rows (velocity; pressure
 // at the pin node when pinned) take the increment itself (dx, or its float32 copy dx32), less
-// the prescribed velocity vD when that is given (a residual: dx is x^{n+1})
+// the prescribed velocity vD when that is given (a residual: dx is x^{n+1}).  The planes [k0, k1); E holds
+// `layers` layers of elements, layer ez at ez % layers.
 template <typename T>
 __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, int nx, int ny, int nz, int nxp,
-                                                      int64_t nxyp, int64_t nn, double W, const uint8_t* __restrict__ mask,
+                                                      int64_t nxyp, int layers, int k0, int k1, int64_t nn, double W,
+                                                      const uint8_t* __restrict__ mask,
                                                       int pin, const double* __restrict__ dx,
                                                       const float* __restrict__ dx32, const double* __restrict__ vD,
                                                       double* __restrict__ y) {
   int i;
-  const int64_t jk = row_index(nx + 1, &i);
-  if (i > nx || jk >= (int64_t)(ny + 1) * (nz + 1)) return;
+  const int64_t jk = row_index(nx + 1, &i) + (int64_t)k0 * (ny + 1);
+  if (i > nx || jk >= (int64_t)(ny + 1) * k1) return;
   const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
   const int64_t n = i + (int64_t)(nx + 1) * (j + (int64_t)(ny + 1) * k);
-  const int64_t es = (int64_t)nz * nxyp;
+  const int64_t es = (int64_t)layers * nxyp;
   T s[4] = {T(0), T(0), T(0), T(0)};
   // elements (z, y, x) descending; an element outside adds a zero, so that the loads of all eight are in
   // flight together (with early exits the sums of the 64^3 float32 product took 19 us, now 16)
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
   for (int a = 0; a < 8; ++a) {  // this node's corner in element (ex, ey, ez), from 7 down
     const int c = 7 - a, ex = i - (c & 1), ey = j - ((c >> 1) & 1), ez = k - (c >> 2);
     const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
-    const int64_t e = ok ? (int64_t)ez * nxyp + (int64_t)ey * nxp + ex : 0;
+    const int64_t e = ok ? (int64_t)(ez < layers ? ez : ez % layers) * nxyp + (int64_t)ey * nxp + ex : 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const T v = ok ? E[(8 * f + c) * es + e] : T(0);
@@ -264,13 +267,14 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
 // the same sums of NC components without Dirichlet rows or weight
 template <int NC>
 __global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__ E, int nx, int ny, int nz, int nxp,
-                                                      int64_t nxyp, int64_t nn, double* __restrict__ y) {
+                                                      int64_t nxyp, int layers, int k0, int k1, int64_t nn,
+                                                      double* __restrict__ y) {
   int i;
-  const int64_t jk = row_index(nx + 1, &i);
-  if (i > nx || jk >= (int64_t)(ny + 1) * (nz + 1)) return;
+  const int64_t jk = row_index(nx + 1, &i) + (int64_t)k0 * (ny + 1);
+  if (i > nx || jk >= (int64_t)(ny + 1) * k1) return;
   const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
   const int64_t n = i + (int64_t)(nx + 1) * (j + (int64_t)(ny + 1) * k);
-  const int64_t es = (int64_t)nz * nxyp;
+  const int64_t es = (int64_t)layers * nxyp;
   double s[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) s[c] = 0.0;
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__
   for (int a = 0; a < 8; ++a) {
     const int q = 7 - a, ex = i - (q & 1), ey = j - ((q >> 1) & 1), ez = k - (q >> 2);
     const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
-    const int64_t e = ok ? (int64_t)ez * nxyp + (int64_t)ey * nxp + ex : 0;
+    const int64_t e = ok ? (int64_t)(ez < layers ? ez : ez % layers) * nxyp + (int64_t)ey * nxp + ex : 0;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       const double v = ok ? E[(8 * c + q) * es + e] : 0.0;

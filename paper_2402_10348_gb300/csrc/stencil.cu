@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(HQ_THREADS) ac_elem_kernel(const __grid_consta
                                                              double bet, const __grid_constant__ Diffusion D,
                                                              double* __restrict__ K, unsigned e0, unsigned e1, int slots) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, e0, e1);
+  l.set(H.g, H.rh, e0, e1);
   const Phys& P = H.P;
   double v[3];
 #pragma unroll
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(HQ_THREADS) ac_elem_kernel(const __grid_consta
 __global__ void __launch_bounds__(HQ_THREADS) b_elem_kernel(const __grid_constant__ HexNS H, int solid,
                                                             double* __restrict__ K, unsigned e0, unsigned e1, int slots) {
   HexLane l;
-  l.set(H.g, H.rh, H.nxp, e0, e1);
+  l.set(H.g, H.rh, e0, e1);
   const Phys& P = H.P;
   const int64_t nn = H.nn;
   double v[3], L[3][3];
