@@ -5,6 +5,16 @@ namespace fsi {
 
 template int launch_ns<double>(fsi_mesh*, int, const double*, double*, unsigned);
 
+// cudaMalloc that is allowed while a stream is being captured too (it is no part of the graph)
+static cudaError_t scratch_malloc(double** p, int64_t len) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  e = cudaMalloc(p, sizeof(double) * (size_t)len);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
+}
+
 // Scratch of the element contributions.  Meshes whose largest block (48 slots an element with a solid, else 32)
 // fits ELEM_SCRATCH have one for everything, taken at once: its address never changes.  On larger ones
 // the float64 products, residuals and gamma/beta go slab by slab of layers through that much of their
@@ -16,7 +26,7 @@ static bool one_scratch(const fsi_mesh* m, int64_t nxyp) { return 8 * most_slots
 
 int ensure_elem_scratch(fsi_mesh* m, int64_t nxyp) {
   if (m->ke_e) return FSI_OK;
-  FSI_CUDA(cudaMalloc(&m->ke_e, sizeof(double) * (size_t)(one_scratch(m, nxyp) ? most_slots(m) : 32) * m->g.nz * nxyp));
+  FSI_CUDA(scratch_malloc(&m->ke_e, (int64_t)(one_scratch(m, nxyp) ? most_slots(m) : 32) * m->g.nz * nxyp));
   return FSI_OK;
 }
 
@@ -29,7 +39,7 @@ int elem_layers(fsi_mesh* m, int64_t nxyp, double** E, int* layers) {
   }
   const int64_t layer = most_slots(m) * nxyp;
   *layers = (int)std::min<int64_t>(m->g.nz, std::max<int64_t>(2, ELEM_SCRATCH / (8 * layer)));
-  if (!m->ke_s) FSI_CUDA(cudaMalloc(&m->ke_s, sizeof(double) * (size_t)(*layers * layer)));
+  if (!m->ke_s) FSI_CUDA(scratch_malloc(&m->ke_s, *layers * layer));
   *E = m->ke_s;
   return FSI_OK;
 }

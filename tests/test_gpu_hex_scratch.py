@@ -1,12 +1,14 @@
-"""Scratch of the element-centric float64 calls on hexahedra: meshes whose contributions exceed
-it (2^30 bytes; 48 slots of 8 bytes an element with a solid) go slab by slab of layers.
+"""Scratch of the element-centric float64 calls on hexahedra: calls that are captured before anything ran on
+their mesh, and meshes whose contributions exceed it (2^30 bytes; 48 slots of 8 bytes an element with a
+solid), which go slab by slab of layers.
 
 A window of layers of the large mesh is a mesh of its own: away from the window's first and last plane
 every entry is the same sum of the same terms in the same order, so the bits agree.  gamma and beta are held
 to fsi_gamma_beta_noalloc, other kernels, at 1e-11 (tests/test_gpu_operators.py)."""
+import numpy as np
 import pytest
 
-from tests.gpu_helpers import DEV
+from tests.gpu_helpers import DEV, Gpu, T
 
 pytestmark = pytest.mark.gpu
 
@@ -14,8 +16,31 @@ import torch  # noqa: E402
 
 from paper_2402_10348_gb300 import fsi  # noqa: E402
 from tests.helpers import desc_small  # noqa: E402
+from workloads import random_state  # noqa: E402
 
 BLOCKS = [(fsi.FSI_BLOCK_NS, 4), (fsi.FSI_BLOCK_AC(0), 1), (fsi.FSI_BLOCK_B(0), 6)]
+
+
+@pytest.mark.parametrize("block,nc", BLOCKS)
+def test_first_call_on_a_mesh_inside_a_capture(block, nc):
+    d = desc_small(n=(9, 7, 6))
+    st = random_state(d, 2)
+    ref = Gpu(d, *st)
+    fsi.fsi_set_ac_coeffs(ref.mesh, 0, 0.37, -0.21)
+    want = ref.residual(block, nc * d.nn)
+    g = Gpu(d, *st)
+    fsi.fsi_set_ac_coeffs(g.mesh, 0, 0.37, -0.21)
+    r = torch.zeros(nc * d.nn, dtype=torch.float64, device=DEV)
+    stream = torch.cuda.Stream()
+    fsi.fsi_set_stream(g.mesh, stream)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        fsi.fsi_residual(g.mesh, block, *g.st(), r)
+    assert float(r.abs().max()) == 0.0
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(r.cpu().numpy(), want)
 
 
 NX, NZ, H = 220, 130, 1.0 / 256
