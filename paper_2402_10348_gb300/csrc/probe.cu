@@ -2,8 +2,10 @@
 // denominators of the operators' rooflines (timing support; the paper has none).
 //
 // FMA rate: every thread runs 8 independent fused multiply-add chains (enough to
-// cover the pipeline latency) for a fixed count, on a grid of 8 CTAs of 256 threads
-// per SM; flops = 2 x chains x count x threads.  Read bandwidth: a grid-stride sum
+// cover the pipeline latency) for a fixed count, on a grid of 4 (float32: 8) CTAs of 256 threads
+// per SM; flops = 2 x chains x count x threads.  The chains' operands are what each type runs fastest with:
+// float64 with operands of each chain's own (0.628 T FMA/s at 2070 MHz, 2 a clock and SM; 0.529 with two that
+// all chains share, which products of the library exceed), float32 with shared ones (38.5; distinct 26).  Read bandwidth: a grid-stride sum
 // of a 2 GiB float4 buffer (only reads reach HBM; the sums are written once per
 // thread).  Copy bandwidth: the same buffer copied into a second one (read + write
 // bytes counted).  Each figure is the best of five timed launches after a warm-up.
@@ -22,9 +24,23 @@ __global__ void __launch_bounds__(256) fma_kernel(T a, T b, int count, T* sink) 
   T x[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) x[i] = a + T(threadIdx.x + i);
-  for (int k = 0; k < count; ++k) {
+  if constexpr (sizeof(T) == 8) {
+    T p[8], q[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = fma(x[i], b, a);
+    for (int i = 0; i < 8; ++i) {
+      p[i] = b + T(7 * threadIdx.x + i) * T(1e-3);
+      q[i] = a * T(threadIdx.x + 3 * i) * T(1e-6);
+    }
+#pragma unroll 8
+    for (int k = 0; k < count; ++k) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = fma(p[i], q[i], x[i]);
+    }
+  } else {
+    for (int k = 0; k < count; ++k) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = fma(x[i], b, a);
+    }
   }
   T s = T(0);
 #pragma unroll
@@ -80,19 +96,18 @@ extern "C" int fsi_probe_peaks(double* fp32_tflops, double* fp64_tflops, double*
   int dev = 0, sms = 0;
   FSI_CUDA(cudaGetDevice(&dev));
   FSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int blocks = sms * 8, threads = 256;
-  const double thr = (double)blocks * threads;
+  const int blocks = sms * 8, blocks64 = sms * 4, threads = 256;
   float* sink = nullptr;
   FSI_CUDA(cudaMalloc(&sink, 64));
   float ms = 0.f;
   int rc;
-  const int n32 = 4096, n64 = 256;
+  const int n32 = 4096, n64 = 1024;
   if ((rc = best_ms([&] { fma_kernel<float><<<blocks, threads>>>(1.0f, 0.999f, n32, sink); }, &ms))) goto done;
-  *fp32_tflops = 2.0 * 8 * n32 * thr / (ms * 1e-3) / 1e12;
-  if ((rc = best_ms([&] { fma_kernel<double><<<blocks, threads>>>(1.0, 0.999, n64, reinterpret_cast<double*>(sink)); },
+  *fp32_tflops = 2.0 * 8 * n32 * blocks * threads / (ms * 1e-3) / 1e12;
+  if ((rc = best_ms([&] { fma_kernel<double><<<blocks64, threads>>>(1.0, 0.999, n64, reinterpret_cast<double*>(sink)); },
                     &ms)))
     goto done;
-  *fp64_tflops = 2.0 * 8 * n64 * thr / (ms * 1e-3) / 1e12;
+  *fp64_tflops = 2.0 * 8 * n64 * blocks64 * threads / (ms * 1e-3) / 1e12;
   {
     const int64_t bytes = (int64_t)2 << 30;  // 2 GiB per buffer
     float4 *a = nullptr, *b = nullptr;
