@@ -247,12 +247,6 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
       FSI_LAUNCH(m, P_KRY_CONV, to_float_kernel<<<vec_grid(b.n), 256, 0, m->stream>>>(dx, m->dx32, b.n));
   }
   flags &= ~OP_DX32_READY;
-  if (m->rec) {  // recorded (batched) launches take the per-element kernels
-    flags &= ~OP_REUSED;
-    if (b.kind == 0) return f32 ? launch_ns<float>(m, 1, dx, y, flags) : launch_ns<double>(m, 1, dx, y, flags);
-    if (b.kind == 1) return f32 ? launch_ac<float>(m, 1, b.index, dx, y) : launch_ac<double>(m, 1, b.index, dx, y);
-    return f32 ? launch_b<float>(m, 1, b.index, dx, y) : launch_b<double>(m, 1, b.index, dx, y);
-  }
   if (f32) {
     if (b.kind == 0) return launch_nsq32(m, dx, y, flags);
     return b.kind == 1 ? launch_ac<float>(m, 1, b.index, dx, y) : launch_b<float>(m, 1, b.index, dx, y);
@@ -273,10 +267,9 @@ int op_jvp(fsi_mesh* m, const BlockInfo& b, const double* dx, double* y, unsigne
 int op_diag(fsi_mesh* m, const BlockInfo& b, double* d, unsigned flags) {
   if (m->tet) return tet_op(m, b, 2, nullptr, d, flags);
   const bool f32 = flags & FSI_FP32;
-  if (!f32 && !m->rec && (flags & OP_REUSED)) return b.kind == 0 ? nsa_diag(m, d, flags) : stencil_diag(m, b, d);
+  if (!f32 && (flags & OP_REUSED)) return b.kind == 0 ? nsa_diag(m, d, flags) : stencil_diag(m, b, d);
   flags &= ~OP_REUSED;
-  if (b.kind == 0)
-    return f32 ? launch_ns<float>(m, 2, nullptr, d, flags) : launch_ns<double>(m, 2, nullptr, d, flags);
+  if (b.kind == 0) return f32 ? launch_ns_diag<float>(m, d, flags) : launch_ns_diag<double>(m, d, flags);
   if (b.kind == 1)
     return f32 ? launch_ac<float>(m, 2, b.index, nullptr, d) : launch_ac<double>(m, 2, b.index, nullptr, d);
   return f32 ? launch_b<float>(m, 2, b.index, nullptr, d) : launch_b<double>(m, 2, b.index, nullptr, d);

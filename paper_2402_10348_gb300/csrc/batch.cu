@@ -936,8 +936,7 @@ int record_set(fsi_batch* b, OpSet* set, unsigned flags, const double* dx_base, 
     m->dx32 = b->dx32_own + b->off[i];
     const double* dx = dx_base + b->off[i];
     double* y = y_base + b->off[i];
-    if (bi.kind == 0) rc = f32 ? launch_ns<float>(m, 1, dx, y, flags) : launch_ns<double>(m, 1, dx, y, flags);
-    else if (bi.kind == 1) rc = f32 ? launch_ac<float>(m, 1, bi.index, dx, y) : launch_ac<double>(m, 1, bi.index, dx, y);
+    if (bi.kind == 1) rc = f32 ? launch_ac<float>(m, 1, bi.index, dx, y) : launch_ac<double>(m, 1, bi.index, dx, y);
     else rc = f32 ? launch_b<float>(m, 1, bi.index, dx, y) : launch_b<double>(m, 1, bi.index, dx, y);
     m->dx32 = mesh_dx32;
     m->rec = nullptr;

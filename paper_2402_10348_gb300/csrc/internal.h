@@ -172,11 +172,11 @@ int op_diag(fsi_mesh* m, const BlockInfo& b, double* d, unsigned flags);
 int op_coeffs(fsi_mesh* m, int phase, double* gamma_beta);  // synchronises
 // Final fixed-order sum of the gamma/beta per-CTA partials {sum val^2, n_band, int F',
 // int sqrt F} into out[0] = gamma, out[1] = beta (ops_f64.cu; one CTA of NTHREADS).
-// Shared by fsi_update_ac_coeffs and fsi_gamma_beta_noalloc.
+// fsi_update_ac_coeffs on tetrahedra and fsi_gamma_beta_noalloc.
 __global__ void coef_finalize(const double* partials, int64_t n, double eta, double* out);
 
 template <typename T>
-int launch_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags);
+int launch_ns_diag(fsi_mesh* m, double* d, unsigned flags);
 // quadrature-point coefficients of the NS product at the staged state (built when stale)
 int ns_build(fsi_mesh* m, unsigned flags, bool f64);  // hexq_ops.cu
 // float64 NS product at a state that is used a few times (hexq_ops.cu)

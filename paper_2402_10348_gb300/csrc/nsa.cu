@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(HQ_THREADS) nsa_elem_kernel(const __grid_const
 // blockDim (NAT, 4), one CTA per 128 nodes.
 __global__ void __launch_bounds__(4 * NAT) nsa_gather_kernel(const double* __restrict__ K, int nx, int ny, int nz, int nxp,
                                                              int64_t nxyp, int slots, int64_t n0, int64_t n1,
-                                                             double* __restrict__ A, float* __restrict__ A32) {
+                                                             double* __restrict__ A) {
   const int64_t n = n0 + (int64_t)blockIdx.x * NAT + threadIdx.x;
   if (n >= n1) return;
   const int r = threadIdx.y;
@@ -299,20 +299,17 @@ __global__ void __launch_bounds__(4 * NAT) nsa_gather_kernel(const double* __res
         }
         const int o = (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          A[dst + (int64_t)(16 * o + c) * NAT] = acc[c];
-          if (A32) A32[dst + (int64_t)(16 * o + c) * NAT] = (float)acc[c];
-        }
+        for (int c = 0; c < 4; ++c) A[dst + (int64_t)(16 * o + c) * NAT] = acc[c];
       }
 }
 
 // y = A x: blockDim (NAT, 4), one thread per (node, row field), one tile per CTA.  A missing
 // neighbour's block is zero and its values are read at the node itself.  Dirichlet rows (velocity;
 // pressure at the pin node when pinned) take the increment itself.
-template <typename T>
-__global__ void __launch_bounds__(4 * NAT) nsa_apply_kernel(const T* __restrict__ A, const T* __restrict__ x, int nx, int ny,
-                                                            int nz, int64_t nn, const uint8_t* __restrict__ mask, int pin,
-                                                            const double* __restrict__ dx, double* __restrict__ y) {
+__global__ void __launch_bounds__(4 * NAT) nsa_apply_kernel(const double* __restrict__ A, const double* __restrict__ x,
+                                                            int nx, int ny, int nz, int64_t nn,
+                                                            const uint8_t* __restrict__ mask, int pin,
+                                                            double* __restrict__ y) {
   const int64_t n = (int64_t)blockIdx.x * NAT + threadIdx.x;
   if (n >= nn) return;
   const int r = threadIdx.y;
@@ -320,8 +317,8 @@ __global__ void __launch_bounds__(4 * NAT) nsa_apply_kernel(const T* __restrict_
   const int i = (int)(n - (int64_t)row * (nx + 1)), k = (int)(row / (unsigned)(ny + 1));
   const int j = (int)(row - (unsigned)k * (ny + 1));
   const int64_t sy = nx + 1, sz = sy * (ny + 1);
-  const T* a = A + ((int64_t)blockIdx.x * 27 * 16 + 4 * r) * NAT + threadIdx.x;
-  T acc[4] = {T(0), T(0), T(0), T(0)};
+  const double* a = A + ((int64_t)blockIdx.x * 27 * 16 + 4 * r) * NAT + threadIdx.x;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
   const bool okx[3] = {i > 0, true, i < nx};
 #pragma unroll 1
   for (int dz = -1; dz <= 1; ++dz) {
@@ -332,7 +329,7 @@ __global__ void __launch_bounds__(4 * NAT) nsa_apply_kernel(const T* __restrict_
 #pragma unroll
       for (int ddx = -1; ddx <= 1; ++ddx) {
         const int64_t nb = okyz && okx[ddx + 1] ? n + ddx + sy * dy + sz * dz : n;
-        const T* ao = a + (int64_t)16 * ((ddx + 1) + 3 * (dy + 1) + 9 * (dz + 1)) * NAT;
+        const double* ao = a + (int64_t)16 * ((ddx + 1) + 3 * (dy + 1) + 9 * (dz + 1)) * NAT;
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[c] += __ldcs(ao + c * NAT) * __ldg(x + c * nn + nb);
       }
@@ -340,7 +337,7 @@ __global__ void __launch_bounds__(4 * NAT) nsa_apply_kernel(const T* __restrict_
   }
   const bool dir = ((mask[n] >> r) & 1) && (r < 3 || pin);
   const int64_t q = (int64_t)r * nn + n;
-  y[q] = dir ? (dx ? dx[q] : (double)x[q]) : (double)((acc[0] + acc[1]) + (acc[2] + acc[3]));
+  y[q] = dir ? x[q] : (acc[0] + acc[1]) + (acc[2] + acc[3]);
 }
 
 // The same with three threads per (node, row field), one per neighbour plane, summed through shared
@@ -443,7 +440,7 @@ int nsa_build(fsi_mesh* m, unsigned flags) {
     const int64_t n0 = z0 * plane, n1 = (z1 == g.nz ? z1 + 1 : z1) * plane;
     FSI_LAUNCH(m, P_NS_BUILD,
                nsa_gather_kernel<<<(unsigned)((n1 - n0 + NAT - 1) / NAT), dim3(NAT, 4), 0, m->stream>>>(
-                   m->ke64, g.nx, g.ny, g.nz, nxp, nxyp, slots, n0, n1, m->na64, nullptr));
+                   m->ke64, g.nx, g.ny, g.nz, nxp, nxyp, slots, n0, n1, m->na64));
   }
   m->na_gen = m->stage_gen;
   m->na_flags = eflags;
@@ -465,8 +462,8 @@ int launch_nsa(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
     return FSI_OK;
   }
   FSI_LAUNCH(m, P_NS_JVP64E,
-             nsa_apply_kernel<double><<<(unsigned)((m->nn + NAT - 1) / NAT), dim3(NAT, 4), 0, m->stream>>>(
-                 m->na64, dx, g.nx, g.ny, g.nz, m->nn, m->mask, m->pin_active, dx, y));
+             nsa_apply_kernel<<<(unsigned)((m->nn + NAT - 1) / NAT), dim3(NAT, 4), 0, m->stream>>>(
+                 m->na64, dx, g.nx, g.ny, g.nz, m->nn, m->mask, m->pin_active, y));
   return FSI_OK;
 }
 

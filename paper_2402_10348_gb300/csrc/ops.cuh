@@ -71,8 +71,6 @@ __host__ __device__ constexpr int sym_idx(int k, int l) {
 
 struct OutDesc {
   double* y;            // output block [NC][nn]
-  const double* dx;     // JVP input block (Dirichlet rows copy it), or null
-  const float* dx32;    // its float copy: the rows copy this one when dx is null
   const uint8_t* mask;  // Dirichlet mask (NS only): bits 0-2 velocity, bit 3 pressure
   int accumulate;       // add into y instead of writing (later solid passes)
   int dirichlet;        // apply Dirichlet rows
@@ -81,9 +79,9 @@ struct OutDesc {
 };
 
 // ----------------------------------------------------------------- NS block
-// Field layout (NSField): state v(3), p, dv/dt(3), rho, mu, then per solid in the
-// pass: alpha^s, B^s(6); JVP: the input dv(3), dp first.
-template <typename TT, int MODE>  // MODE 1: JVP, 2: diagonal (residuals: hexq_ops.cu)
+// The Jacobi diagonal (residuals and float64 products: hexq_ops.cu, float32 products: nsq_tma.cu).  Field
+// layout: state v(3), p, dv/dt(3), rho, mu, then per solid in the pass: alpha^s, B^s(6).
+template <typename TT>
 struct NSOp {
   using T = TT;
   static constexpr int NC = 4;
@@ -92,7 +90,7 @@ struct NSOp {
   int nf;           // staged field count
   int s0, s1;       // solids in this pass
   int fluid;        // 1: include the fluid/pressure terms (first pass)
-  int elastic_aug;  // JVP/diagonal: add the solid-stress linearization
+  int elastic_aug;  // add the solid-stress linearization
   Phys P;
   double rh[3], W;
   OutDesc out;
@@ -104,8 +102,7 @@ struct NSOp {
 
   __device__ void element(const Corners<T>& cr, const ElemCtx&, T (&c)[NC][8], Red&) const {
     const T rhx = T(rh[0]), rhy = T(rh[1]), rhz = T(rh[2]);
-    const int base = (MODE == 1) ? 4 : 0;  // JVP: fields 0..3 are dv, dp
-    const int fv = base, fp = base + 3, fvd = base + 4, frho = base + 7, fmu = base + 8, fsol = base + 9;
+    const int fv = 0, fp = 3, fvd = 4, frho = 7, fmu = 8, fsol = 9;
     const T alpha = T(P.alpha), cm = T(P.c_mass), cel = T(P.c_el);
     T u[8];
 #pragma unroll 1
@@ -137,138 +134,66 @@ struct NSOp {
       const T tau_m = T(1) / sqrt(dt2 + vGv + T(P.c_i) * nu * nu * T(P.GG));
       const T tau_c = T(1) / (T(P.trG) * tau_m);
 
-      if (MODE == 1) {
-        T dv[3], dL[3][3];
+      // trial = test = N_a e_k
+      // per-solid terms of the augmentation: a_s, B^s and its divergence-like row sums
+      T aB[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};  // sum_s a_s B^s
+      T aG[3][3];                                      // sum_s a_s d_k B^s_kj  (row k, j)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          cr.get(k, u);
-          const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
-          dv[k] = r.v; dL[k][0] = alpha * r.gx; dL[k][1] = alpha * r.gy; dL[k][2] = alpha * r.gz;
-        }
-        cr.get(3, u);
-        const VG<T> dpr = interp_vg(u, w, rhx, rhy, rhz);
-        T vt[3], dRm[3];
+      for (int k = 0; k < 3; ++k)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) vt[k] = alpha * dv[k];
+        for (int j = 0; j < 3; ++j) aG[k][j] = T(0);
+      if (elastic_aug) {
+        for (int s = s0; s < s1; ++s) {
+          const int fs = fsol + 7 * (s - s0);
+          cr.get(fs, u);
+          const T a = interp_v(u, w) * T(P.muL[P.solid_phase[s]]) * cel * alpha;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const T dacc = cm * dv[k] + vt[0] * L[k][0] + vt[1] * L[k][1] + vt[2] * L[k][2] +
-                         v[0] * dL[k][0] + v[1] * dL[k][1] + v[2] * dL[k][2];
-          dRm[k] = rho * dacc;
-        }
-        const T dgp[3] = {dpr.gx, dpr.gy, dpr.gz};
-        T dE[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-        if (elastic_aug) {
-          for (int s = s0; s < s1; ++s) {
-            const int fs = fsol + 7 * (s - s0);
-            cr.get(fs, u);
-            const T a = interp_v(u, w) * T(P.muL[P.solid_phase[s]]) * cel;
-            T B[6], dd[6];
-#pragma unroll
-            for (int cc = 0; cc < 6; ++cc) {
-              cr.get(fs + 1 + cc, u);
-              const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
-              B[cc] = r.v;
-              dd[cc] = vt[0] * r.gx + vt[1] * r.gy + vt[2] * r.gz;
-            }
-            // P = grad(vt) B ; dE += a ( -dd + P + P^T )
-#pragma unroll
-            for (int cc = 0; cc < 6; ++cc) {
-              const int k = sym_k(cc), l = sym_l(cc);
-              T pkl = T(0), plk = T(0);
-#pragma unroll
-              for (int m = 0; m < 3; ++m) {
-                pkl += dL[k][m] * B[sym_idx(m, l)];
-                plk += dL[l][m] * B[sym_idx(m, k)];
-              }
-              dE[cc] += a * (pkl + plk - dd[cc]);
-            }
+          for (int cc = 0; cc < 6; ++cc) {
+            cr.get(fs + 1 + cc, u);
+            const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
+            aB[cc] += a * r.v;
+            const int k = sym_k(cc), l = sym_l(cc);
+            const T gk[3] = {r.gx, r.gy, r.gz};
+            aG[k][l] += a * gk[k];
+            if (k != l) aG[l][k] += a * gk[l];
           }
         }
-        const T W = T(this->W);
-        if (fluid) {
-          const T dRc = dL[0][0] + dL[1][1] + dL[2][2];
+      }
+      const T W = T(this->W);
 #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            T gk[3];
+      for (int a = 0; a < 8; ++a) {
+        const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
+        const T N = w.wx[ax] * w.wy[ay] * w.wz[az];
+        const T gN[3] = {(ax ? T(1) : T(-1)) * rhx * w.wy[ay] * w.wz[az],
+                         (ay ? T(1) : T(-1)) * rhy * w.wx[ax] * w.wz[az],
+                         (az ? T(1) : T(-1)) * rhz * w.wx[ax] * w.wy[ay]};
+        const T vgN = v[0] * gN[0] + v[1] * gN[1] + v[2] * gN[2];
+        const T gN2 = gN[0] * gN[0] + gN[1] * gN[1] + gN[2] * gN[2];
+        // grad N^T (sum a_s B) grad N
+        T BNN = T(0);
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) BNN += gN[m] * aB[sym_idx(m, j)] * gN[j];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const T da = cm * N + alpha * N * L[k][k] + alpha * vgN;
+          T d = T(0);
+          if (fluid)
+            d = N * rho * da + alpha * mu * (gN2 + gN[k] * gN[k]) + tau_m * alpha * N * Rm[k] * gN[k] +
+                tau_m * vgN * rho * da + tau_c * rho * alpha * gN[k] * gN[k];
+          if (elastic_aug) {
+            T divrow = T(0), Bk = T(0);
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-              T s = dE[sym_idx(k, j)] + mu * (dL[k][j] + dL[j][k]) + tau_m * (vt[j] * Rm[k] + v[j] * (dRm[k] + dgp[k]));
-              if (j == k) s += -dpr.v + tau_c * rho * dRc;
-              gk[j] = W * s;
+              divrow += aG[k][j] * gN[j];
+              Bk += aB[sym_idx(k, j)] * gN[j];
             }
-            scatter_vg(c[k], w, W * dRm[k], gk[0], gk[1], gk[2], rhx, rhy, rhz);
+            d += -N * divrow + BNN + Bk * gN[k];
           }
-          const T r = W * tau_m / rho;
-          scatter_vg(c[3], w, W * dRc, r * (dRm[0] + dgp[0]), r * (dRm[1] + dgp[1]), r * (dRm[2] + dgp[2]),
-                     rhx, rhy, rhz);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 3; ++k)
-            scatter_vg(c[k], w, T(0), W * dE[sym_idx(k, 0)], W * dE[sym_idx(k, 1)], W * dE[sym_idx(k, 2)],
-                       rhx, rhy, rhz);
+          c[k][a] += W * d;
         }
-      } else {  // MODE 2: diagonal, trial = test = N_a e_k
-        // per-solid terms of the augmentation: a_s, B^s and its divergence-like row sums
-        T aB[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};  // sum_s a_s B^s
-        T aG[3][3];                                      // sum_s a_s d_k B^s_kj  (row k, j)
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) aG[k][j] = T(0);
-        if (elastic_aug) {
-          for (int s = s0; s < s1; ++s) {
-            const int fs = fsol + 7 * (s - s0);
-            cr.get(fs, u);
-            const T a = interp_v(u, w) * T(P.muL[P.solid_phase[s]]) * cel * alpha;
-#pragma unroll
-            for (int cc = 0; cc < 6; ++cc) {
-              cr.get(fs + 1 + cc, u);
-              const VG<T> r = interp_vg(u, w, rhx, rhy, rhz);
-              aB[cc] += a * r.v;
-              const int k = sym_k(cc), l = sym_l(cc);
-              const T gk[3] = {r.gx, r.gy, r.gz};
-              aG[k][l] += a * gk[k];
-              if (k != l) aG[l][k] += a * gk[l];
-            }
-          }
-        }
-        const T W = T(this->W);
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
-          const T N = w.wx[ax] * w.wy[ay] * w.wz[az];
-          const T gN[3] = {(ax ? T(1) : T(-1)) * rhx * w.wy[ay] * w.wz[az],
-                           (ay ? T(1) : T(-1)) * rhy * w.wx[ax] * w.wz[az],
-                           (az ? T(1) : T(-1)) * rhz * w.wx[ax] * w.wy[ay]};
-          const T vgN = v[0] * gN[0] + v[1] * gN[1] + v[2] * gN[2];
-          const T gN2 = gN[0] * gN[0] + gN[1] * gN[1] + gN[2] * gN[2];
-          // grad N^T (sum a_s B) grad N
-          T BNN = T(0);
-#pragma unroll
-          for (int m = 0; m < 3; ++m)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) BNN += gN[m] * aB[sym_idx(m, j)] * gN[j];
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const T da = cm * N + alpha * N * L[k][k] + alpha * vgN;
-            T d = T(0);
-            if (fluid)
-              d = N * rho * da + alpha * mu * (gN2 + gN[k] * gN[k]) + tau_m * alpha * N * Rm[k] * gN[k] +
-                  tau_m * vgN * rho * da + tau_c * rho * alpha * gN[k] * gN[k];
-            if (elastic_aug) {
-              T divrow = T(0), Bk = T(0);
-#pragma unroll
-              for (int j = 0; j < 3; ++j) {
-                divrow += aG[k][j] * gN[j];
-                Bk += aB[sym_idx(k, j)] * gN[j];
-              }
-              d += -N * divrow + BNN + Bk * gN[k];
-            }
-            c[k][a] += W * d;
-          }
-          if (fluid) c[3][a] += W * tau_m / rho * gN2;
-        }
+        if (fluid) c[3][a] += W * tau_m / rho * gN2;
       }
     }
   }
@@ -281,12 +206,7 @@ struct NSOp {
       double* y = out.y + (int64_t)k * nn + nc.n;
       const bool dir = ((m >> k) & 1) && (k < 3 || out.pin);
       if (dir) {
-        if (!out.dirichlet) continue;
-        if (MODE == 1) {
-          *y = out.dx ? out.dx[(int64_t)k * nn + nc.n] : (double)out.dx32[(int64_t)k * nn + nc.n];
-        } else {
-          *y = 1.0;
-        }
+        if (out.dirichlet) *y = 1.0;
       } else {
         *y = out.accumulate ? *y + (double)acc[k] : (double)acc[k];
       }

@@ -3,7 +3,7 @@
 
 namespace fsi {
 
-template int launch_ns<double>(fsi_mesh*, int, const double*, double*, unsigned);
+template int launch_ns_diag<double>(fsi_mesh*, double*, unsigned);
 
 // cudaMalloc that is allowed while a stream is being captured too (it is no part of the graph)
 static cudaError_t scratch_malloc(double** p, int64_t len) {

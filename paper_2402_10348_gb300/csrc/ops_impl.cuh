@@ -99,15 +99,10 @@ int run_tile(fsi_mesh* m, const Op& op, int cls) {
   return FSI_OK;
 }
 
-template <typename T>
-constexpr int jvp_class(int kind) {
-  return kind == 0 ? (sizeof(T) == 8 ? P_NS_JVP64 : P_NS_JVP32)
-                   : (kind == 1 ? (sizeof(T) == 8 ? P_AC_JVP64 : P_AC_JVP32) : (sizeof(T) == 8 ? P_B_JVP64 : P_B_JVP32));
-}
 template <typename T, int MODE>
-constexpr int op_class(int kind) {
-  return MODE == 1 ? jvp_class<T>(kind)
-                   : (kind == 0 ? P_NS_DIAG : (kind == 1 ? P_AC_DIAG : P_B_DIAG));
+constexpr int op_class(int kind) {  // Allen-Cahn (1) and B (2): products, else diagonals
+  return MODE == 1 ? (kind == 1 ? (sizeof(T) == 8 ? P_AC_JVP64 : P_AC_JVP32) : (sizeof(T) == 8 ? P_B_JVP64 : P_B_JVP32))
+                   : (kind == 1 ? P_AC_DIAG : P_B_DIAG);
 }
 
 // The increment of a product: float64 kernels read dx itself, float32 kernels the
@@ -127,19 +122,16 @@ inline int solids_per_pass(int nf_fixed) {
   return (int)((SMEM_LIMIT - fixed) / per);
 }
 
-template <typename T, int MODE>
-int ns_pass(fsi_mesh* m, const double* dx, double* y, unsigned flags, int s0, int s1, bool first) {
-  NSOp<T, MODE> op;
+template <typename T>
+int ns_pass(fsi_mesh* m, double* y, unsigned flags, int s0, int s1, bool first) {
+  NSOp<T> op;
   memset(&op, 0, sizeof(op));
   const T* xa = Staged<T>::xa(m);
   const T* xd = Staged<T>::xd(m);
   const T* mat = Staged<T>::mat(m);
   const int64_t nn = m->nn;
-  if ((MODE == 1 ? 4 : 0) + 9 + 7 * (s1 - s0) > MAXF) return set_error(FSI_EINVAL, "NS operator: too many staged fields");
+  if (9 + 7 * (s1 - s0) > MAXF) return set_error(FSI_EINVAL, "NS operator: too many staged fields");
   int f = 0;
-  if (MODE == 1) {
-    for (int k = 0; k < 4; ++k) put_dx<T>(op.F, f++, m, dx, k * nn);
-  }
   for (int k = 0; k < 3; ++k) put<T>(op.F, f++, xa + k * nn);   // v
   put<T>(op.F, f++, xa + 3 * nn);                                 // p^{n+1}
   for (int k = 0; k < 3; ++k) put<T>(op.F, f++, xd + k * nn);   // dv/dt
@@ -158,31 +150,25 @@ int ns_pass(fsi_mesh* m, const double* dx, double* y, unsigned flags, int s0, in
   op.P = m->P;
   fill_common(m, op.rh, &op.W);
   op.out.y = y;
-  op.out.dx = dx;
-  op.out.dx32 = sizeof(T) == 4 ? m->dx32 : nullptr;
   op.out.mask = m->mask;
   op.out.accumulate = first ? 0 : 1;
   op.out.dirichlet = first ? 1 : 0;
   op.out.pin = m->pin_active;
   op.nn_ = nn;
-  return run_tile(m, op, op_class<T, MODE>(0));
+  return run_tile(m, op, P_NS_DIAG);
 }
 
 template <typename T>
-int launch_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
+int launch_ns_diag(fsi_mesh* m, double* y, unsigned flags) {
   const int ns = (flags & FSI_ELASTIC_AUG) ? m->ns : 0;
-  const int fixed = (mode == 1 ? 4 : 0) + 9;
   // bounded by shared memory and by the MAXF staged-field slots of Fields
-  const int per = std::min(solids_per_pass<T>(fixed), (MAXF - fixed) / 7);
+  const int per = std::min(solids_per_pass<T>(9), (MAXF - 9) / 7);
   if (per < 1 && ns > 0) return set_error(FSI_EINVAL, "NS operator: shared memory too small for one solid");
   int s0 = 0;
   bool first = true;
   do {
     const int s1 = ns == 0 ? 0 : std::min(ns, s0 + per);
-    int rc;
-    if (mode == 1) rc = ns_pass<T, 1>(m, dx, y, flags, s0, s1, first);
-    else rc = ns_pass<T, 2>(m, dx, y, flags, s0, s1, first);
-    if (rc) return rc;
+    if (int rc = ns_pass<T>(m, y, flags, s0, s1, first)) return rc;
     first = false;
     s0 = s1;
   } while (s0 < ns);

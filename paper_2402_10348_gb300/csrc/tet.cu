@@ -712,7 +712,7 @@ int tet_ns(fsi_mesh* m, int mode, const double* dx, double* y, unsigned flags) {
       return FSI_OK;
     }
   }
-  if (mode == 1 && !m->rec) {
+  if (mode == 1) {
     // direct products for the first few at a state, as on hexahedra
     if (t->c_stage != m->stage_gen) {
       t->c_stage = m->stage_gen;
