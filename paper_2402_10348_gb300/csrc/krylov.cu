@@ -1080,9 +1080,10 @@ int gmres_solve(fsi_mesh* m, const BlockInfo& blk, const double* rhs, double* x,
   fsi_pc* harvest = ((o.flags & FSI_HARVEST) && blk.kind == 0 && m->pc && m->pc->cap > 0) ? m->pc : nullptr;
   unsigned opflags = o.flags & ~(FSI_HARVEST | FSI_PC_ALTERNATE | FSI_NO_STALL_STOP | FSI_PINNED_SOLVE | OP_DX32_READY |
                                  OP_REUSED);
-  // a float64 solve that may take many products assembles the operator before the first one (its
-  // diagonal comes with it)
-  if (o.precision == FSI_PREC_FP64 && o.max_iter > (blk.kind == 0 ? NSA_AFTER : STENCIL_AFTER)) opflags |= OP_REUSED;
+  // a float64 solve that may take many products (one an iteration, one a cycle for the true residual)
+  // assembles the operator before the first one (its diagonal comes with it)
+  const int64_t products = o.max_iter + ((int64_t)o.max_iter + mm - 1) / mm;
+  if (o.precision == FSI_PREC_FP64 && products > (blk.kind == 0 ? NSA_AFTER : STENCIL_AFTER)) opflags |= OP_REUSED;
   // read by the solver loop only: network/Jacobi alternation, and no stop on stagnation
   const unsigned alt = o.flags & (FSI_PC_ALTERNATE | FSI_NO_STALL_STOP);
   const bool stall_stop = (o.flags & FSI_NO_STALL_STOP) == 0;
