@@ -1557,8 +1557,13 @@ int fsi_batch_gmres(fsi_batch* b, const fsi_state* states, const double* rhs, do
       if ((rc = upload_live(b, live))) return rc;
       BK_LAUNCH(b, P_KRYLOV, bk_axpy<<<NI, BVB, 0, s>>>(b->items_dev, b->live, b->off_dev, b->nloc_dev, 1.0, b->d, x));
       if (direct) {
-        for (int i = 0; i < nb; ++i)
-          if (live[i] && (rc = hq_ns_jvp(b->meshes[i], x + b->off[i], b->t + b->off[i], base))) return rc;
+        for (int i = 0; i < nb; ++i) {
+          if (!live[i]) continue;
+          const int64_t* c = b->meshes[i]->prof.launches;
+          const int64_t l0 = c[P_NS_JVP64] + c[P_NODE_SUM];
+          if ((rc = hq_ns_jvp(b->meshes[i], x + b->off[i], b->t + b->off[i], base))) return rc;
+          b->launches += c[P_NS_JVP64] + c[P_NODE_SUM] - l0;
+        }
       } else if ((rc = run_set(b, b->jvp_outer, 2))) {
         return rc;
       }
