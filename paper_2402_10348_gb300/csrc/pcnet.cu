@@ -530,12 +530,14 @@ __global__ void __launch_bounds__(32 * WGR) wgrad_reduce_kernel(const float* __r
 // A work unit is 8 x 16 voxels of 1 or 2 z planes: its input planes and one on either side, with their
 // halo (180 x 16 bytes an octet), and the gradient's are copied by cp.async into one of two stages while
 // the other's MMAs (72 a plane) run; warp 0 issues those, the other eight copy.  Each CTA walks a
-// contiguous range of units with the nine accumulators in TMEM (144 columns) and writes them once, as
-// rows of consecutive M that wgrad_reduce_kernel sums in a fixed order.  Bound by the MMAs: the two
+// contiguous range of units with the nine accumulators in TMEM (144 columns) and adds them up in its partial
+// sums, rows of consecutive M that wgrad_reduce_kernel sums in a fixed order.  Bound by the MMAs: the two
 // CTAs of an SM issue one every 48 cycles, 3 CIN of whose 128 rows are used.
+// The tensor core's float32 accumulation cuts low bits off (n MMAs of positive products come out about n 2^-25
+// too small), so the accumulators are emptied after every `turn` units, at most wgm_chain MMAs each.
 // Staging the 27 shifted copies of every voxel, transposed by shuffles, took 72 us on 64^3 (16
-// channels) and 177 (32); now 38 and 41.  (Units of 4 planes: 44, three units on the
-// busiest CTA against 2.5 on average, and 61, one CTA per SM.)
+// channels) and 177 (32); now 45 and 47, 38 and 41 without the readings in between.  (Units of 4 planes: 44,
+// three units on the busiest CTA against 2.5 on average, and 61, one CTA per SM.)
 constexpr int WGM_LOADERS = 256;
 constexpr int WGM_THREADS = 32 + WGM_LOADERS;
 
@@ -556,16 +558,25 @@ struct WgmCfg {
 
 struct WgmGrid {
   int tx, ty, p, panels, units;  // tiles, z planes of a unit, units of a tile and in all
+  int turn;                      // units between two readings of the accumulators
 };
 // p: the fewest z planes (1, 2) with which a grid of `slots` CTAs takes all units at once, a CTA's MMAs
 // being a chain of 72 a plane (5^3 to 33^3 voxels: 15 us a kernel with 4 planes, 9 to 13 so); else the most
-static WgmGrid wgm_grid(const TView& g, int most, int slots) {
+// MMAs in turn on one accumulator: as if 912 CTAs (456 for 32 channels) shared the voxels, 16 at a time (the
+// split of the staged form before).  65^3: 19 (38), units one (two) at a time: sums of positive terms are 3.8e-7
+// (7.7e-7) off, 2.6e-6 with all of a CTA's 78 MMAs in turn; 129 x 129 x 97: 3.5e-6 (9.5e-6) against 2.4e-5.
+static int64_t wgm_chain(const TView& g, int cin) {
+  const int64_t share = 16 * (cin == 16 ? 912 : 456);
+  return ((int64_t)g.nx * g.ny * g.nz + share - 1) / share;
+}
+static WgmGrid wgm_grid(const TView& g, int cin, int most, int slots) {
   WgmGrid w;
   w.tx = (g.nx + TILE_X - 1) / TILE_X, w.ty = (g.ny + TILE_Y - 1) / TILE_Y;
   w.p = 1;
   while (w.p < most && (int64_t)w.tx * w.ty * ((g.nz + w.p - 1) / w.p) > slots) w.p *= 2;
   w.panels = (g.nz + w.p - 1) / w.p;
   w.units = w.tx * w.ty * w.panels;
+  w.turn = (int)std::max<int64_t>(1, wgm_chain(g, cin) / (TILE_Y / 2 * w.p));
   return w;
 }
 
@@ -589,7 +600,7 @@ __device__ __forceinline__ void wgm_load(const TView& x, const TView& g, const W
 }
 
 template <int CIN>
-__global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g, WgmGrid w, float* __restrict__ part,
+__global__ void __launch_bounds__(WGM_THREADS, 2) wgrad_mma_kernel(TView x, TView g, WgmGrid w, float* __restrict__ part,
                                                                 int* err) {
   using C = WgmCfg<CIN>;
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -614,6 +625,24 @@ __global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g
   // M/N-major A and B
   constexpr uint32_t IDESC = idesc_bf16(16, 128) | (1u << 15) | (1u << 16);
   bool bad = false;
+  // warps 1 to 8, two a lane quarter: the accumulators into the CTA's partial sums (its first, or added)
+  auto drain = [&](bool add) {
+    const int quarter = warp & 3, m = quarter * 32 + lane;
+    if (quarter * 32 >= 3 * CIN) return;
+    float* dst = part + (int64_t)blockIdx.x * (16 * CIN * 27) + m;
+#pragma unroll 1
+    for (int a = (warp - 1) >> 2; a < 9; a += 2) {
+      float sum[16];
+#pragma unroll
+      for (int co = 0; co < 16; ++co) sum[co] = add && m < 3 * CIN ? dst[(a * 16 + co) * 3 * CIN] : 0.0f;
+      uint32_t r[16];
+      tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 16), r);
+      if (m < 3 * CIN) {
+#pragma unroll
+        for (int co = 0; co < 16; ++co) dst[(a * 16 + co) * 3 * CIN] = sum[co] + __uint_as_float(r[co]);
+      }
+    }
+  };
   for (int i = 0; i < nu; ++i) {
     const int s = i & 1;
     cp_async_commit();
@@ -635,7 +664,7 @@ __global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g
           for (int kk = 0; kk < TILE_Y / 2; ++kk) {
             const uint64_t db = sdesc(gb + (z * 2) * C::GOCT + kk * 2 * TILE_X * 16, TILE_X * 16, C::GOCT);
             const uint64_t da = sdesc(xb + z * C::SLOT + 2 * kk * SX * 16, SX * 16, OCT_BYTES);
-            const uint32_t acc = i > 0 || z > 0 || kk > 0 ? 1u : 0u;
+            const uint32_t acc = i % w.turn > 0 || z > 0 || kk > 0 ? 1u : 0u;
 #pragma unroll
             for (int a = 0; a < 9; ++a)  // (the start address is the descriptor's lowest field, in 16 bytes)
               mma_bf16(tmem + 16 * a, da + (uint64_t)(a / 3 * SX + a % 3), db, IDESC, acc);
@@ -647,6 +676,15 @@ __global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g
       // the other stage is free once the MMAs of unit i - 1 are done
       if (i >= 1 && !mbar_wait(smem_u32(&bars[s ^ 1]), (uint32_t)(((i - 1) >> 1) & 1))) bad = true;
       if (!bad) wgm_load<CIN>(x, g, w, u0 + i + 1, base + (s ^ 1) * C::STAGE, tid - 32);
+      if ((i + 1) % w.turn == 0) {  // (warp 0 starts on empty accumulators after the next barrier)
+        if (!mbar_wait(smem_u32(&bars[s]), (uint32_t)((i >> 1) & 1))) bad = true;
+        if (__any_sync(0xffffffffu, bad)) {
+          bad = true;
+        } else {
+          tc_fence_after();
+          drain(i >= w.turn);
+        }
+      }
     }
   }
   if (!bad) {
@@ -655,19 +693,7 @@ __global__ void __launch_bounds__(WGM_THREADS) wgrad_mma_kernel(TView x, TView g
   }
   if (!bad) {
     tc_fence_after();
-    if (warp < 4) {
-      const int m = warp * 32 + lane;
-      float* dst = part + (int64_t)blockIdx.x * (16 * CIN * 27) + m;
-#pragma unroll 1
-      for (int a = 0; a < 9; ++a) {
-        uint32_t r[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * 16), r);
-        if (m < 3 * CIN) {
-#pragma unroll
-          for (int co = 0; co < 16; ++co) dst[(a * 16 + co) * 3 * CIN] = __uint_as_float(r[co]);
-        }
-      }
-    }
+    if (warp > 0) drain(nu > w.turn);
   } else if (tid == 0) {
     atomicExch(err, 1);
   }
@@ -927,7 +953,7 @@ int launch_wgrad_mma(fsi_pc* pc, const TView& x, const TView& g, int* nblk_out) 
   fsi_mesh* m = pc->m;
   if (int rc = ensure_smem_attr(reinterpret_cast<const void*>(&wgrad_mma_kernel<CIN>), C::SMEM)) return rc;
   static_assert(2 * (C::SMEM + 1024) <= 228 * 1024 && 2 * C::NCOLS <= 512, "two CTAs per SM");
-  const WgmGrid w = wgm_grid(g, C::P, 2 * 152);
+  const WgmGrid w = wgm_grid(g, CIN, C::P, 2 * 152);
   const int nblk = std::min(w.units, 2 * 152);
   if ((int64_t)nblk * 16 * CIN * 27 > pc->wpart_n) return set_error(FSI_EINVAL, "pc: weight-gradient scratch too small");
   FSI_LAUNCH(m, P_PC_WGRAD, (wgrad_mma_kernel<CIN><<<nblk, WGM_THREADS, C::SMEM, m->stream>>>(x, g, w, pc->wpart, pc->err)));
