@@ -666,12 +666,13 @@ __global__ void __launch_bounds__(VB) combine_kernel(double* __restrict__ x, con
   }
 }
 
-// the same from the float32 basis, four adjacent elements a thread (upd_store4_kernel's layout)
+// the same from the float32 basis, four adjacent elements a thread (upd_store4_kernel's layout), each entry in
+// eight sums as lin_comb_chunk has it (30 vectors: 6.3e-8 off, 9.3e-8 in two sums)
 __global__ void __launch_bounds__(VB) combine4_kernel(double* __restrict__ x, const double* __restrict__ dinv,
                                                       const float* __restrict__ V, int M1, int k,
                                                       const KryDev* __restrict__ K, int64_t n) {
-  __shared__ float ys[MMAX];
-  for (int i = threadIdx.x; i < k; i += VB) ys[i] = (float)K->y[i];
+  __shared__ float ys[MMAX + 8];
+  for (int i = threadIdx.x; i < k + 8; i += VB) ys[i] = i < k ? (float)K->y[i] : 0.f;
   __syncthreads();
   const int64_t nch = (n + CH - 1) / CH;
   const int sub = threadIdx.x >> 6, e0 = (threadIdx.x & 63) * 4;
@@ -680,29 +681,38 @@ __global__ void __launch_bounds__(VB) combine4_kernel(double* __restrict__ x, co
     if (j >= n) break;
     const float* blk = V + c * (int64_t)M1 * CH + e0;
     if (j + 4 <= n) {
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-      int i = 0;
-#pragma unroll 4
-      for (; i + 2 <= k; i += 2) {
-        const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
-        const float4 v1 = *reinterpret_cast<const float4*>(blk + (i + 1) * CH);
-        a.x += ys[i] * v0.x; a.y += ys[i] * v0.y; a.z += ys[i] * v0.z; a.w += ys[i] * v0.w;
-        b.x += ys[i + 1] * v1.x; b.y += ys[i + 1] * v1.y; b.z += ys[i + 1] * v1.z; b.w += ys[i + 1] * v1.w;
+      float4 p[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) p[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i0 = 0; i0 < k; i0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          v[u] = i0 + u < k ? *reinterpret_cast<const float4*>(blk + (i0 + u) * CH) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float y = ys[i0 + u];
+          p[u].x = fmaf(y, v[u].x, p[u].x);
+          p[u].y = fmaf(y, v[u].y, p[u].y);
+          p[u].z = fmaf(y, v[u].z, p[u].z);
+          p[u].w = fmaf(y, v[u].w, p[u].w);
+        }
       }
-      if (i < k) {
-        const float4 v0 = *reinterpret_cast<const float4*>(blk + i * CH);
-        a.x += ys[i] * v0.x; a.y += ys[i] * v0.y; a.z += ys[i] * v0.z; a.w += ys[i] * v0.w;
-      }
-      x[j] += dinv[j] * (double)(a.x + b.x);
-      x[j + 1] += dinv[j + 1] * (double)(a.y + b.y);
-      x[j + 2] += dinv[j + 2] * (double)(a.z + b.z);
-      x[j + 3] += dinv[j + 3] * (double)(a.w + b.w);
+#pragma unroll
+      for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+        for (int u = 0; u < h; ++u) {
+          p[u].x += p[u + h].x;
+          p[u].y += p[u + h].y;
+          p[u].z += p[u + h].z;
+          p[u].w += p[u + h].w;
+        }
+      x[j] += dinv[j] * (double)p[0].x;
+      x[j + 1] += dinv[j + 1] * (double)p[0].y;
+      x[j + 2] += dinv[j + 2] * (double)p[0].z;
+      x[j + 3] += dinv[j + 3] * (double)p[0].w;
     } else {
-      for (int e = 0; e < 4 && j + e < n; ++e) {
-        float s = 0.f;
-        for (int i = 0; i < k; ++i) s += ys[i] * blk[i * CH + e];
-        x[j + e] += dinv[j + e] * (double)s;
-      }
+      for (int e = 0; e < 4 && j + e < n; ++e) x[j + e] += dinv[j + e] * (double)lin_comb_chunk<float>(ys, blk + e, k);
     }
   }
 }
