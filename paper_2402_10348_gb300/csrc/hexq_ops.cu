@@ -293,10 +293,10 @@ static int hq_ns_sums(fsi_mesh* m, const double* E, const HexNS& H, int k0, int 
                       double* y) {
   const Geom& g = m->g;
   const RowLaunch nl = node_launch(g, k0, k1);
-  FSI_LAUNCH(m, P_NODE_SUM,
-             ns_node_kernel<double><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp, H.layers, k0,
-                                                                         k1, m->nn, H.W, m->mask, m->pin_active, dx, nullptr,
-                                                                         vD, y));
+  auto* kernel = H.layers < g.nz ? &ns_node_kernel<double, true> : &ns_node_kernel<double, false>;
+  FSI_LAUNCH(m, P_NODE_SUM, kernel<<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp, H.layers, k0, k1,
+                                                                        m->nn, H.W, m->mask, m->pin_active, dx, nullptr, vD,
+                                                                        y));
   return FSI_OK;
 }
 
@@ -304,8 +304,9 @@ template <int NC>
 static int hq_sums(fsi_mesh* m, const double* E, const HexNS& H, int k0, int k1, double* y) {
   const Geom& g = m->g;
   const RowLaunch nl = node_launch(g, k0, k1);
-  FSI_LAUNCH(m, P_NODE_SUM, em_node_kernel<NC><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp,
-                                                                                    H.layers, k0, k1, m->nn, y));
+  auto* kernel = H.layers < g.nz ? &em_node_kernel<NC, true> : &em_node_kernel<NC, false>;
+  FSI_LAUNCH(m, P_NODE_SUM, kernel<<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, H.nxp, H.nxyp, H.layers, k0, k1,
+                                                                        m->nn, y));
   return FSI_OK;
 }
 

@@ -208,9 +208,9 @@ inline RowLaunch node_launch(const Geom& g, int k0, int k1) { return row_launch(
 
 // NS node sums: y = W * sum of the element slots, the Dirichlet rows (velocity; pressure
 // at the pin node when pinned) take the increment itself (dx, or its float32 copy dx32), less
-// the prescribed velocity vD when that is given (a residual: dx is x^{n+1}).  The planes [k0, k1); E holds
-// `layers` layers of elements, layer ez at ez % layers.
-template <typename T>
+// the prescribed velocity vD when that is given (a residual: dx is x^{n+1}).  RING: the planes [k0, k1), and E
+// holds `layers` layers of elements, layer ez at ez % layers; else all (the remainders cost 1.3 us of 7 on 14 x 15 x 12).
+template <typename T, bool RING>
 __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, int nx, int ny, int nz, int nxp,
                                                       int64_t nxyp, int layers, int k0, int k1, int64_t nn, double W,
                                                       const uint8_t* __restrict__ mask,
@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
                                                       const float* __restrict__ dx32, const double* __restrict__ vD,
                                                       double* __restrict__ y) {
   int i;
+  if (!RING) layers = nz, k0 = 0, k1 = nz + 1;
   const int64_t jk = row_index(nx + 1, &i) + (int64_t)k0 * (ny + 1);
   if (i > nx || jk >= (int64_t)(ny + 1) * k1) return;
   const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
   for (int a = 0; a < 8; ++a) {  // this node's corner in element (ex, ey, ez), from 7 down
     const int c = 7 - a, ex = i - (c & 1), ey = j - ((c >> 1) & 1), ez = k - (c >> 2);
     const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
-    const int64_t e = ok ? (int64_t)(ez < layers ? ez : ez % layers) * nxyp + (int64_t)ey * nxp + ex : 0;
+    const int64_t e = ok ? (int64_t)(RING ? ez % layers : ez) * nxyp + (int64_t)ey * nxp + ex : 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const T v = ok ? E[(8 * f + c) * es + e] : T(0);
@@ -251,11 +252,12 @@ __global__ void __launch_bounds__(128) ns_node_kernel(const T* __restrict__ E, i
 }
 
 // the same sums of NC components without Dirichlet rows or weight
-template <int NC>
+template <int NC, bool RING>
 __global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__ E, int nx, int ny, int nz, int nxp,
                                                       int64_t nxyp, int layers, int k0, int k1, int64_t nn,
                                                       double* __restrict__ y) {
   int i;
+  if (!RING) layers = nz, k0 = 0, k1 = nz + 1;
   const int64_t jk = row_index(nx + 1, &i) + (int64_t)k0 * (ny + 1);
   if (i > nx || jk >= (int64_t)(ny + 1) * k1) return;
   const int j = (int)(jk % (ny + 1)), k = (int)(jk / (ny + 1));
@@ -268,7 +270,7 @@ __global__ void __launch_bounds__(128) em_node_kernel(const double* __restrict__
   for (int a = 0; a < 8; ++a) {
     const int q = 7 - a, ex = i - (q & 1), ey = j - ((q >> 1) & 1), ez = k - (q >> 2);
     const bool ok = ex >= 0 && ex < nx && ey >= 0 && ey < ny && ez >= 0 && ez < nz;
-    const int64_t e = ok ? (int64_t)(ez < layers ? ez : ez % layers) * nxyp + (int64_t)ey * nxp + ex : 0;
+    const int64_t e = ok ? (int64_t)(RING ? ez % layers : ez) * nxyp + (int64_t)ey * nxp + ex : 0;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       const double v = ok ? E[(8 * c + q) * es + e] : 0.0;
