@@ -120,7 +120,7 @@ __device__ __forceinline__ void block_reduce_store(double (&acc)[K], int kc, dou
 // iterative refinement (a float32 operator inside float64 refinement: the inner solve
 // only has to reduce its residual by ir_inner_rtol, far above float32 rounding, and the
 // refinement's float64 residual removes what the inner solve leaves).  Products, per-thread sums and,
-// with a float basis, the sums of a warp are taken in VT, those across warps and CTAs in float64.  The
+// with a float basis, the sums of a warp are taken in VT, those across warps and CTAs in float64 (or two floats).  The
 // work vector w, the preconditioner diagonal and every vector outside the basis stay float64.
 
 // Whether this CTA is the last of `total` to get here; its earlier global writes (and, for the last
