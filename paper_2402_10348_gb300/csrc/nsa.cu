@@ -4,8 +4,8 @@
 // (GB300 issues them at 1/64 of the float32 rate), so the form with the fewest is the fastest:
 // 432 FMAs a node here, against 1024 an element for element matrices and about 2400 for the
 // quadrature-point form, and no element contributions to write and sum.  Bytes: 3,456 a
-// node, under the FMA time on this card.  64^3, one product: 224 us (1.06 of the float64 FMA rate
-// that independent chains reach, 4.2 TB/s) against 586 us with element matrices and their node
+// node, under the FMA time on this card.  64^3, one product: 221 us (0.86 of the float64 FMA rate
+// of 0.628 T/s, 4.3 TB/s) against 586 us with element matrices and their node
 // sums; 240 iterations of GMRES(30): 254.4 -> 118.6 ms with the build below.
 //
 // Layout: tiles of NAT = 128 nodes, A[((tile * 27 + o) * 16 + 4 r + c) * NAT + lane] for row
@@ -264,7 +264,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nsa_elem_kernel(const __grid_const
 
 // Rows of the nodes of the planes [k0, k1): one thread per (node, row field); every entry is the sum
 // over the up to 8 elements that hold both nodes, in a fixed order (z, y, x of the element).
-// blockDim (NAT, 4), one CTA per 128 nodes.
+// blockDim (NAT, 4), one CTA per 128 nodes.  The neighbour loops stay rolled (unrolled they
+// spill: 16^3 84 us, 60 so).
 __global__ void __launch_bounds__(4 * NAT) nsa_gather_kernel(const double* __restrict__ K, int nx, int ny, int nz, int nxp,
                                                              int64_t nxyp, int slots, int64_t n0, int64_t n1,
                                                              double* __restrict__ A) {
@@ -275,7 +276,9 @@ __global__ void __launch_bounds__(4 * NAT) nsa_gather_kernel(const double* __res
   const int i = (int)(n - (int64_t)row * (nx + 1)), k = (int)(row / (unsigned)(ny + 1));
   const int j = (int)(row - (unsigned)k * (ny + 1));
   const int64_t dst = ((n / NAT) * 27 * 16 + 4 * r) * NAT + n % NAT;
+#pragma unroll 1
   for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll 1
     for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll 1
       for (int dx = -1; dx <= 1; ++dx) {
