@@ -748,8 +748,7 @@ class Clocks:
 # multiply by the elements of one launch.
 def flops_per_element(kernel: str, n_solid: int) -> float:
     """Assembled float64 products, one FMA per stored entry: 27 blocks of 4 x 4 a node (NS), 27
-    entries (AC, from a solve's third product), 27 x 24 (B, from its first: 12 values, the
-    couplings used twice); taken per
+    entries (AC), 27 x 24 (B: 12 values, the couplings used twice); taken per
     element here (a mesh has a few percent more nodes).  Per quadrature point: the NS
     product from frozen coefficients 486 + 114 with solids (interpolation of dv, dp: 172;
     convective and mass terms 54; stresses 92; the elastic linearization 114;
@@ -1075,16 +1074,18 @@ def run_gpu(args):
         "dtype": "f64" if f64 else "f32",
         "precision": ("float64 throughout (operators, Arnoldi basis, reductions, Hessenberg and Givens)" if f64 else
                       "float32 operator applies and float32 Arnoldi basis inside float64 iterative "
-                      "refinement; float64 residuals, reductions, Hessenberg and Givens"),
+                      "refinement; basis sums float32 inside a warp and float64 across; float64 "
+                      "residuals, Hessenberg and Givens"),
         "data": "synthetic (seeded icosphere surface, initial phases by the grid-cell method)",
         "config": {"workload": WORKLOAD, "nodes": d.nn, "dof_per_node": d.ncomp, "dt": d.dt,
                    "nl_iters_max": wl.k_max,
                    "gmres": f"Jacobi GMRES({args.restart}) rtol 1e-8 (NS block of the enclosed cavity: the pin "
                             "node keeps its continuity equation, pressure shifted to p = 0 there after the solve)"
                    + (f"; inner solves to {args.ir_inner_rtol:g}" if not f64 else ""),
-                   "l2": ("inputs larger than L2: a time step streams the 64^3 state, the quadrature-point "
-                          "coefficients of the NS product "
-                          f"({d.ne * 8 * 44 * (8 if f64 else 4) / 1e6:.0f} MB) and the (m+1) x 1.1M Krylov basis "
+                   "l2": ("inputs larger than L2: a time step streams the 64^3 state, the "
+                          + (f"assembled rows of the NS operator ({d.nn * 27 * 16 * 8 / 1e6:.0f} MB)" if f64 else
+                             f"quadrature-point coefficients of the NS product ({d.ne * 8 * 44 * 4 / 1e6:.0f} MB)")
+                          + " and the (m+1) x 1.1M Krylov basis "
                           f"({(args.restart + 1) * 4 * d.nn * (8 if f64 else 4) / 1e6:.0f} MB) every restart cycle, "
                           "against a 129 MB L2"),
                    "parallelism": f"replicas x{world}"},

@@ -843,7 +843,7 @@ int build_tiles(fsi_batch* b, int target_mult, int grid_mult) {
 }
 
 // the batched float32 NS product from per-instance coefficients (nsq_tma.cu): element
-// launch over every instance's 64 x 2-element tiles, node launch over its 128-node blocks
+// launch over every instance's tiles of 128 elements, node launch over its 128-node blocks
 // work lists of the batched float32 NS product (built when the operator set is recorded,
 // never inside a captured cycle)
 int ensure_nsq_items(fsi_batch* b) {

@@ -3,8 +3,8 @@
 // As for the momentum block (nsa.cu) the float64 FMA rate binds a product, so the operators are
 // summed into node rows once per solve: 27 FMAs a node for an indicator (64 an element before, in
 // element matrices) and 648 for a solid's six components (1,440 an element before).  One product:
-// Allen-Cahn 96 x 96 x 192 102 us (0.93 of the float64 FMA rate) against 517 with the node sums, B 64^3
-// 323 us (1.06 of it) against 929.  Builds: Allen-Cahn 5.0 ms against 19.3 (and 9.2 for the
+// Allen-Cahn 96 x 96 x 192 102 us (0.77 of the float64 FMA rate) against 517 with the node sums, B 64^3
+// 323 us (0.88 of it) against 929.  Builds: Allen-Cahn 5.0 ms against 19.3 (and 9.2 for the
 // diagonal, 15 for the two products before it), B 3.5 ms against 2.0 (and 2.5 for the diagonal).
 //
 // Allen-Cahn (Eq. PPV_AC's linearization, gamma, beta and tau_phi frozen): with
