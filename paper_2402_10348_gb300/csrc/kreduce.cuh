@@ -60,11 +60,10 @@ __device__ __forceinline__ void block_reduce_store_bf(double (&acc)[K], int kc, 
 // The same in float32 up to the warps' sums, which are added in two floats (Knuth's two-sum) and stored as
 // float64: this GPU issues float64 adds at 1/64 of the float32 rate, so a float64 tree over every thread's
 // sums costs more than the float32 basis kernel's streaming, and over the warps' it still took 0.7 us of an
-// 11 us kernel.  (Added in float32,
-// the 12 warps of a fused update gave |w|^2 of 1.1 M entries an error of 4.5e-9 where CTAs of four warps
-// had 1.2e-9; so 1.0e-9.)  Values in groups of 8 by the transposing butterfly (9
-// shuffles a group against 40 for plain trees: with a few basis chunks a thread, the trees took as
-// long as the streaming), the last ones by plain trees.
+// 11 us kernel.  (Added in float32, the 12 warps of a fused update gave |w|^2 of 1.1 M entries an error of
+// 4.5e-9 where CTAs of four warps had 1.2e-9; so 1.0e-9.)  Values in groups of 8 by the transposing
+// butterfly (9 shuffles a group against 40 for plain trees: with a few basis chunks a thread, the trees took
+// as long as the streaming), the last ones by plain trees.
 template <int K, int NT>
 __device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, bool tail, double* out, int stride) {
   __shared__ float smf[K][NT / 32];
@@ -107,7 +106,7 @@ __device__ __forceinline__ void block_reduce_store_f(float (&acc)[K], int kc, bo
       lo += (hi - (t - b)) + (r - b);  // what the addition rounded off, exactly
       hi = t;
     }
-    out[i * stride] = (double)hi + (double)lo;
+    out[i * stride] = isfinite(hi) ? (double)hi + (double)lo : (double)hi;  // (of an infinity, lo is a NaN)
   }
 }
 
