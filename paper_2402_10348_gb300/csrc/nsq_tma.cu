@@ -354,9 +354,9 @@ int launch_nsq32(fsi_mesh* m, const double* dx, double* y, unsigned flags) {
                                                                        rx, ry, rz, m->tma_err)));
   const RowLaunch nl = node_launch(g, 0, g.nz + 1);
   FSI_LAUNCH(m, P_NODE_SUM,
-             ns_node_kernel<float, false><<<nl.grid, nl.block, 0, m->stream>>>(E, g.nx, g.ny, g.nz, nxp, nxyp, g.nz, 0, g.nz + 1, nn,
-                                                                        g.hx * g.hy * g.hz / 8.0, m->mask,
-                                                                        m->pin_active, dx, m->dx32, nullptr, y));
+             (ns_node_kernel<float, false><<<nl.grid, nl.block, 0, m->stream>>>(
+                 E, g.nx, g.ny, g.nz, nxp, nxyp, g.nz, 0, g.nz + 1, nn, g.hx * g.hy * g.hz / 8.0, m->mask, m->pin_active, dx,
+                 m->dx32, nullptr, y)));
   return FSI_OK;
 }
 

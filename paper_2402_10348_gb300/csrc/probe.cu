@@ -5,7 +5,8 @@
 // cover the pipeline latency) for a fixed count, on a grid of 4 (float32: 8) CTAs of 256 threads
 // per SM; flops = 2 x chains x count x threads.  The chains' operands are what each type runs fastest with:
 // float64 with operands of each chain's own (0.628 T FMA/s at 2070 MHz, 2 a clock and SM; 0.529 with two that
-// all chains share, which products of the library exceed), float32 with shared ones (38.5; distinct 26).  Read bandwidth: a grid-stride sum
+// all chains share, which products of the library exceed), float32 with shared ones (38.5; distinct 26).
+// Read bandwidth: a grid-stride sum
 // of a 2 GiB float4 buffer (only reads reach HBM; the sums are written once per
 // thread).  Copy bandwidth: the same buffer copied into a second one (read + write
 // bytes counted).  Each figure is the best of five timed launches after a warm-up.
